@@ -17,6 +17,7 @@
 //   k_halo_face FP32: faces shared with another rank of a partitioned mesh;
 //   k_wall      wall face nodes: mirror state and the wall-stress model (may
 //               run on a side stream beside k_lift and k_face);
+//   k_volume_fx (volume_fx.cuh; FP64 form, KEP fluxes) and
 //   k_volume    one CTA per element: two-point flux differencing (KEP or
 //               entropy-conserving) with the split-form matrix DVS = 2D - B/w
 //               (zero corners), the surface integral, 1/J scaling, body force,
@@ -54,6 +55,11 @@ __device__ __forceinline__ int chk_idx(int i, int n, int* status) {
 #endif
   return i;
 }
+
+// a fixed-point number h 2^31 + l (volume_fx.cuh)
+struct Fx {
+  int h, l;
+};
 
 struct PhysDev {
   double gamma, gm1, R, mu, Pr, cp, kcond, rcp_R;
@@ -121,9 +127,11 @@ struct MeshDev {
   // written by k_prim64 (null unless that lifting is selected)
   const float2* lift_M2;
   float2* lift_W2;
-  // FP64 volume kernel at N = 7: the metric sums a_i + a_m of every pair it
+  // FP64 entropy-conserving volume kernel at N = 7: the metric sums a_i + a_m of every pair it
   // evaluates (pair_main / pair_half below), fixed with the mesh
   const double* pairA;
+  const Fx* JaX;         // FP64 form: [9][K*n3] metrics in fixed point (volume_fx.cuh) and the exponent bounds [K]
+  const int* JaX_exp;
   double* wm_t;          // [n_wall*n2] last wall-law solution per wall node (warm start; may be null)
   int* status;           // device status flags (index checks of the bounds-checking build)
 };
@@ -134,6 +142,7 @@ struct Tables {
   double DVS8[(N + 1) * (N + 1)];   // (2D - B/w) / 8
   double Dvisc[(N + 1) * (N + 1)];  // (w_m / w_i) D_mi
   double iw[N + 1];                 // 1 / w
+  float iw32[N + 1];
   float D32[(N + 1) * (N + 1)];     // D and Dvisc rounded to FP32 (kernel-parameter
   float Dvisc32[(N + 1) * (N + 1)]; // operands of the FP32 line contractions) and
   float D32lo[(N + 1) * (N + 1)];   // their rounding remainders (the double-float
@@ -2161,10 +2170,10 @@ struct VolShape {
   static constexpr int THREADS = 32 * (WARPS_LINES > WARPS_NODES ? WARPS_LINES : WARPS_NODES);
   // shared memory (in units of R): 7 prim slots (9 with the entropy-
   // conserving flux, 10 in the FP32 form of the KEP fluxes: the low parts of
-  // the velocity), 9 metric, 5 residual per node, three coefficient tables, 1/w
-  static constexpr int SMEM_R = 21 * n3 + 3 * n2 + n;
-  static constexpr int SMEM_R_EC = 23 * n3 + 3 * n2 + n;
-  static constexpr int SMEM_R_F32 = 24 * n3 + 3 * n2 + n;
+  // the velocity), 9 metric, 5 residual per node, three coefficient tables
+  static constexpr int SMEM_R = 21 * n3 + 3 * n2;
+  static constexpr int SMEM_R_EC = 23 * n3 + 3 * n2;
+  static constexpr int SMEM_R_F32 = 24 * n3 + 3 * n2;
 };
 
 // Resident CTAs per SM asked of the register allocator: two for CTAs of up to
@@ -2177,13 +2186,368 @@ constexpr int vol_min_blocks() {
   return (N == 7 && !EC && std::is_same<R, float>::value) ? 3 : ((VolShape<N>::THREADS * 64 * 2 <= 65536) ? 2 : 1);
 }
 
+// shared-memory arrays of the volume kernel
+template <typename R>
+struct VolSmem {
+  R* sQ;    // [QS][n3] node values: rho u v w 4p' h|e 2p (KG) (+ FP32: ul vl wl); EC see k_volume
+  R* sA;    // [9][n3] Ja (dir*3+comp)
+  R* sR;    // [5][n3] residual
+  R* sC8;   // [n2] DVS / 8
+  R* sC16;  // [n2] DVS / 16
+  R* sC1;   // [n2] DVS
+};
+
+// The three direction passes over the lines of element e, from the staged node
+// values: leaves each node's sum (with R_v) in sm.sR.
+template <int N, typename R, bool EC, bool PSUM>
+__device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDev<R>& m, const PhysDev& ph,
+                                              const R* __restrict__ Rv, int e, int t) {
+  using Sh = VolShape<N>;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW;
+  constexpr bool F32 = std::is_same<R, float>::value;
+  R *sQ = sm.sQ, *sA = sm.sA, *sR = sm.sR, *sC8 = sm.sC8, *sC16 = sm.sC16, *sC1 = sm.sC1;
+  const size_t S = (size_t)m.K * n3;
+  const bool kg = ph.vol_flux == 1;
+  const bool dif = F32 && !EC && ph.fs_diff;
+  const int warp = t >> 5, lane = t & 31;
+  const int seg = lane / n, pos = lane - seg * n;
+  const int L0 = warp * LPW + seg;
+  const bool active = (seg < LPW) && (L0 < n2);
+  const int L = active ? L0 : 0;
+  const int base = seg * n;  // first lane of the segment
+  const int la = L % n, lb = L / n;
+  // node at position q of this lane's line along dir (a warp holds the same
+  // lines L in every direction)
+  auto node_at = [&](int dir, int q) {
+    return dir == 0 ? q + n * L : (dir == 1 ? la + n * q + n2 * lb : L + n2 * q);
+  };
+  auto load_node = [&](int nd, int dir) {
+    const int node = vslot<N, R>(nd);
+    VolNode<R> X;
+    X.rho = sQ[node]; X.u = sQ[n3 + node]; X.v = sQ[2 * n3 + node]; X.w = sQ[3 * n3 + node];
+    X.p4 = sQ[4 * n3 + node]; X.hh = sQ[5 * n3 + node];
+    X.p2 = (kg || EC) ? sQ[6 * n3 + node] : R(0);
+    X.ib = EC ? sQ[7 * n3 + node] : R(0);
+    X.irh = EC ? sQ[8 * n3 + node] : R(0);
+    if constexpr (!PSUM) {
+      X.a0 = sA[(dir * 3 + 0) * n3 + node]; X.a1 = sA[(dir * 3 + 1) * n3 + node];
+      X.a2 = sA[(dir * 3 + 2) * n3 + node];
+    } else {
+      X.a0 = X.a1 = X.a2 = R(0);
+    }
+    return X;
+  };
+  // symmetric two-point flux F#(A, B) . 4 {Ja} in the scaled form of the
+  // coefficient tables (mass row against DVS / 8, the others against DVS / 16)
+  // (Sa: the sum of the two nodes' metrics, given or formed here)
+  auto sym_flux_s = [&](const VolNode<R>& A, const VolNode<R>& B, R Sa0, R Sa1, R Sa2, R F[5]) {
+    const R Sr = A.rho + B.rho, Su = A.u + B.u, Sv = A.v + B.v, Sw = A.w + B.w;
+    const R Sp = A.p4 + B.p4;
+    const R ua = Su * Sa0 + Sv * Sa1 + Sw * Sa2;  // 4 {u}.{a}
+    if constexpr (EC) {
+      // nodes hold ib = 1 / (2 beta) and irh = 1 / (2 rho), so that with
+      // Sh = ib_A + ib_B (half the sum of the inverse temperatures):
+      //   rho_ln = Sr G / 2;  rgm1 / beta_ln = Sh Qg / 2 (Qg = 2 rgm1 Q);
+      //   1 / (bA + bB) = Sh Rh / 2 (Rh = Rb / 2)
+      const R Dr = A.rho - B.rho, Db = A.hh - B.hh, Sh = A.ib + B.ib;
+      const R tr = Dr * Dr * (A.irh * B.irh);
+      const R tb = Db * Db * (A.ib * B.ib);
+      const R G = tr < LogMeanCut<R>::v ? logmean_G<R>(tr) : R(2) * Dr / (Sr * log1p(Dr / B.rho));
+      R Qg, Rh;
+      if (tb < LogMeanCut<R>::v) {
+        auto qc = [&](int c) { return cR<R>(ph.ec_q[c], ph.f32c.ec_q[c]); };
+        Qg = qc(0) + tb * (qc(1) + tb * (qc(2) + tb * (qc(3) + tb * qc(4))));
+        Rh = R(0.5) + tb * (R(-0.5) + tb * (R(0.5) + tb * (R(-0.5) + tb * R(0.5))));
+      } else {
+        Qg = R(2) * cR<R>(ph.rgm1, ph.f32c.rgm1) * log1p(Db / B.hh) / (Db * Sh);
+        Rh = R(1) / (Sh * (A.hh + B.hh));
+      }
+      const R mf = Sr * G * ua;                 // 8 F_rho
+      const R Spt = Sh * Rh * Sp;               // 8 (p~ - p_ref)
+      F[0] = mf;
+      F[1] = mf * Su + Spt * Sa0;               // 16 F_m
+      F[2] = mf * Sv + Spt * Sa1;
+      F[3] = mf * Sw + Spt * Sa2;
+      // 16 F_E = 2 mf (1 / (2 (gamma-1) beta_ln) + |{u}|^2 - {|u|^2} / 2) + 4 p~ (4 {u}.{a})
+      //        = mf X / 2 + (Spt / 2 + 4 p_ref) (4 {u}.{a})
+      const R X = Sh * Qg + Su * Su + Sv * Sv + Sw * Sw - A.p2 - B.p2;
+      F[4] = R(0.5) * mf * X + (R(0.5) * Spt + R(4) * cR<R>(ph.p_ref, ph.f32c.p_ref)) * ua;
+    } else {
+      const R mf = Sr * ua;                     // 8 F0
+      F[0] = mf;
+      F[1] = mf * Su + Sp * Sa0;                // 16 F1
+      F[2] = mf * Sv + Sp * Sa1;
+      F[3] = mf * Sw + Sp * Sa2;
+      F[4] = mf * (A.hh + B.hh);                // 16 F4
+      if (kg) F[4] += (A.p2 + B.p2) * ua;
+    }
+  };
+  auto sym_flux = [&](const VolNode<R>& A, const VolNode<R>& B, R F[5]) {
+    sym_flux_s(A, B, A.a0 + B.a0, A.a1 + B.a1, A.a2 + B.a2, F);
+  };
+  auto sums_main = [&](int dir, int d, R Sa[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Sa[c] = m.pairA[pair_main(e, dir, c, d, L, pos)];
+  };
+  auto sums_half = [&](int dir, int Lx, int pa, R Sa[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Sa[c] = m.pairA[pair_half(m.K, e, dir, c, Lx, pa)];
+  };
+  // FP64, N = 7: the n/2 pairs at distance n/2 of a line would be formed twice
+  // (once in each lane); instead the distance-n/2 step of the xi pass forms
+  // the xi pairs in lanes pos < n/2 and the eta pairs in lanes pos >= n/2
+  // (swapped by a shuffle), and the one of the eta pass, in the first half
+  // of the warps, the zeta pairs of its own lines (lanes pos < n/2) and of
+  // the lines of warp + WARPS_LINES/2 (lanes pos >= n/2, through shared
+  // memory: the xi metrics, no longer read after the xi pass).  A lane
+  // carries that pair's flux for its next pass's node in `carry`.
+  // A node's sum runs through the passes: the xi pass starts it with the
+  // weak viscous divergence R_v, the eta and zeta passes from the sum the
+  // previous pass stored (with the carried pair's term as its first FMA).
+  constexpr bool HALF = std::is_same<R, double>::value && n == 8 && Sh::WARPS_LINES % 2 == 0;
+  constexpr int DMAX = HALF ? n / 2 - 1 : n / 2;
+  constexpr int HW = Sh::WARPS_LINES / 2, NX = HW * LPW * (n / 2);
+  R* sX = sA;  // [5][NX] zeta pair fluxes handed to the second half of the warps
+  R carry[5] = {R(0), R(0), R(0), R(0), R(0)};
+#pragma unroll 1
+  for (int dir = 0; dir < 3; ++dir) {
+    const int me = node_at(dir, pos);
+    const int ms = vslot<N, R>(me);
+    const VolNode<R> A = load_node(me, dir);
+    // FP32 difference form: the low parts of this lane's node velocity
+    float Aul = 0.f, Avl = 0.f, Awl = 0.f;
+    if constexpr (F32 && !EC) {
+      if (dif) { Aul = sQ[7 * n3 + ms]; Avl = sQ[8 * n3 + ms]; Awl = sQ[9 * n3 + ms]; }
+    }
+    R acc[5];
+    if (dir == 0) {
+      acc[0] = R(0);
+      const R* rv = Rv + (size_t)e * n3 + me;
+#pragma unroll
+      for (int v = 1; v < 5; ++v) acc[v] = ph.viscous ? rv[(size_t)(v - 1) * S] : R(0);
+    } else if constexpr (HALF) {
+      const int px = pos ^ (n / 2);
+      const R c8 = sC8[pos * n + px], c16 = sC16[pos * n + px];
+      if (dir == 2 && warp >= HW) {
+        const int x = ((warp - HW) * LPW + seg) * (n / 2) + (pos & (n / 2 - 1));
+#pragma unroll
+        for (int v = 0; v < 5; ++v) carry[v] = sX[v * NX + x];
+      }
+      acc[0] = fma(c8, carry[0], sR[ms]);
+#pragma unroll
+      for (int v = 1; v < 5; ++v) acc[v] = fma(c16, carry[v], sR[v * n3 + ms]);
+    } else {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) acc[v] = sR[v * n3 + ms];
+    }
+#pragma unroll
+    for (int d = 1; d <= DMAX; ++d) {
+      const int pm = pos + d < n ? pos + d : pos + d - n;
+      const int q = node_at(dir, pm);
+      if constexpr (std::is_same<R, float>::value && !EC) {
+        if (dif) {
+          const NodeF mi{A.rho, A.u, A.v, A.w, A.p4, A.hh, Aul, Avl, Awl};
+          // the partner node's values from the lane that holds it (lane
+          // base + pm of this line's segment)
+          const int lq = base + pm;
+          auto sh = [&](float x) { return __shfl_sync(0xffffffffu, x, lq); };
+          const NodeF mq{sh(A.rho), sh(A.u), sh(A.v), sh(A.w), sh(A.p4), sh(A.hh), sh(Aul), sh(Avl), sh(Awl)};
+          const float aq0 = sh(A.a0), aq1 = sh(A.a1), aq2 = sh(A.a2);
+          float G[5], Gq[5];
+          const float c1 = sC1[pos * n + pm];
+          if (2 * d != n) {
+            // and G(q -> i) for the partner lane (pos + d); receive G(i -> pos - d)
+            flux_delta_pair(mi, mq, A.a0, A.a1, A.a2, aq0, aq1, aq2, ph.f32c.rho_ref, ph.f32c.h_ref, G, Gq);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] += c1 * G[v];
+            const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
+            const float r1 = sC1[pos * n + (src - base)];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] += r1 * __shfl_sync(0xffffffffu, Gq[v], src);
+          } else {
+            flux_delta(mi, mq, A.a0, A.a1, A.a2, aq0 - A.a0, aq1 - A.a1, aq2 - A.a2, ph.f32c.rho_ref,
+                       ph.f32c.h_ref, G);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] += c1 * G[v];
+          }
+          continue;
+        }
+      }
+      R F[5];
+      if constexpr (PSUM) {
+        R Sa[3];
+        sums_main(dir, d, Sa);
+        sym_flux_s(A, load_node(q, dir), Sa[0], Sa[1], Sa[2], F);
+      } else {
+        sym_flux(A, load_node(q, dir), F);
+      }
+      const R c8 = sC8[pos * n + pm], c16 = sC16[pos * n + pm];
+      acc[0] += c8 * F[0];
+#pragma unroll
+      for (int v = 1; v < 5; ++v) acc[v] += c16 * F[v];
+      if (2 * d != n) {
+        // hand the pair flux to the partner lane (pos + d); receive the one
+        // of lane (pos - d)
+        const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
+        const int ps = src - base;
+        const R r8 = sC8[pos * n + ps], r16 = sC16[pos * n + ps];
+        acc[0] += r8 * __shfl_sync(0xffffffffu, F[0], src);
+#pragma unroll
+        for (int v = 1; v < 5; ++v) acc[v] += r16 * __shfl_sync(0xffffffffu, F[v], src);
+      }
+    }
+    if constexpr (HALF) {
+      constexpr int h = n / 2;
+      const int px = pos ^ h;  // partner at distance n/2
+      const R c8 = sC8[pos * n + px], c16 = sC16[pos * n + px];
+      if (dir == 0) {
+        const bool lo = pos < h;
+        const int dd = lo ? 0 : 1, pa = pos & (h - 1);
+        R F[5];
+        if constexpr (PSUM) {
+          R Sa[3];
+          sums_half(dd, L, pa, Sa);
+          sym_flux_s(load_node(node_at(dd, pa), dd), load_node(node_at(dd, pa + h), dd), Sa[0], Sa[1], Sa[2], F);
+        } else {
+          sym_flux(load_node(node_at(dd, pa), dd), load_node(node_at(dd, pa + h), dd), F);
+        }
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          const R Fx = __shfl_xor_sync(0xffffffffu, F[v], h);
+          acc[v] += (v == 0 ? c8 : c16) * (lo ? F[v] : Fx);
+          carry[v] = lo ? Fx : F[v];
+        }
+      } else if (dir == 1 && warp < HW) {
+        const bool lo = pos < h;
+        const int pa = pos & (h - 1);
+        const int Lz = lo ? L : L + HW * LPW;  // zeta line of this warp or of warp + HW
+        R F[5];
+        if constexpr (PSUM) {
+          R Sa[3];
+          sums_half(2, Lz, pa, Sa);
+          sym_flux_s(load_node(Lz + n2 * pa, 2), load_node(Lz + n2 * (pa + h), 2), Sa[0], Sa[1], Sa[2], F);
+        } else {
+          sym_flux(load_node(Lz + n2 * pa, 2), load_node(Lz + n2 * (pa + h), 2), F);
+        }
+        const int x = (warp * LPW + seg) * h + pa;
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          const R Fx = __shfl_xor_sync(0xffffffffu, F[v], h);
+          carry[v] = lo ? F[v] : Fx;
+          if (!lo) sX[v * NX + x] = F[v];
+        }
+      }
+    }
+    if (active) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sR[v * n3 + ms] = acc[v];
+    }
+    __syncthreads();
+  }
+}
+
+// The epilogue, one node per thread: the passes' sums (sums(node, index, acc)
+// gives a node's), the surface integral, the Jacobian scaling and Ut or the
+// register update.
+template <int N, typename R, int MODE, class F>
+__device__ __forceinline__ void volume_epilogue(const double* __restrict__ Uin, const MeshDev<R>& m, const PhysDev& ph,
+                                                const Tables<N>& tab, const R* __restrict__ Fs,
+                                                double* __restrict__ Out, double* __restrict__ dU,
+                                                double* __restrict__ Uout, const StageArgs& st,
+                                                int* __restrict__ status, int e, int t, F sums) {
+  using Sh = VolShape<N>;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS;
+  constexpr bool F32 = std::is_same<R, float>::value;
+  const size_t S = (size_t)m.K * n3;
+  const bool dif = F32 && ph.fs_diff;
+  if (t >= n3) return;
+  // At N = 7 the two warps of a zeta layer
+  // hold the eta rows {0, N, 1, 2} and {3, 4, 5, 6}, so that only the first
+  // runs the (masked) eta-face branch of the surface integral
+  int i, j, k;
+  if constexpr (n == 8 && T == n3) {
+    const int w = t >> 5, r = (t >> 3) & 3;
+    i = t & 7;
+    k = w >> 1;
+    j = (w & 1) ? 3 + r : (r == 0 ? 0 : (r == 1 ? N : r - 1));
+  } else {
+    i = t % n; j = (t / n) % n; k = t / n2;
+  }
+  const int nd = i + n * (j + n * k);
+  const size_t g = (size_t)e * n3 + nd;
+  // the element's own state, for the register update (read again here rather
+  // than kept in registers through the passes)
+  double Uo[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) Uo[v] = Uin[v * S + g];
+  R acc[5];  // the passes' sums (with R_v)
+  sums(nd, g, acc);
+  // surface integral: + sgn * Fs / w_perp on the faces that touch the node
+  auto surf = [&](int l, int ab, R iw) {
+    const int code = m.elem_face[e * 6 + l];
+    const int f = chk_idx(code >> 4, m.F, m.status);
+    const R sg = (code & 1) ? -iw : iw;
+    ab = omap_ab<N>((code >> 1) & 7, ab);  // the node's index in the master's face order
+    // difference form: the face's own side, F* - F(U_side), in rows 5 n2 apart
+    const R* src = dif ? Fs + (size_t)f * 10 * n2 + ((code & 1) ? 5 * n2 : 0) + ab : Fs + (size_t)f * 5 * n2 + ab;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) acc[v] += sg * src[v * n2];
+  };
+  // one branch per direction (masked lanes of a branch cost as much as active ones)
+  if (i == 0 || i == N) surf(i == 0 ? 0 : 1, j + n * k, i == 0 ? cR<R>(tab.iw[0], tab.iw32[0]) : cR<R>(tab.iw[N], tab.iw32[N]));
+  if (j == 0 || j == N) surf(j == 0 ? 2 : 3, i + n * k, j == 0 ? cR<R>(tab.iw[0], tab.iw32[0]) : cR<R>(tab.iw[N], tab.iw32[N]));
+  if (k == 0 || k == N) surf(k == 0 ? 4 : 5, i + n * j, k == 0 ? cR<R>(tab.iw[0], tab.iw32[0]) : cR<R>(tab.iw[N], tab.iw32[N]));
+  // Ut = -(1/J) acc + S, S = (0, f, f . u)
+  const R iJ = m.invJ[g];
+  const bool force = ph.has_force != 0;
+  double src[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  if (force) {
+    const double ir = 1.0 / Uo[0];
+    src[1] = ph.f[0]; src[2] = ph.f[1]; src[3] = ph.f[2];
+    src[4] = (ph.f[0] * Uo[1] + ph.f[1] * Uo[2] + ph.f[2] * Uo[3]) * ir;
+  }
+  if (MODE == 0) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) Out[v * S + g] = -(double)(iJ * acc[v]) + src[v];
+  } else {
+    // dU = A dU + dt Ut = A dU + (-dt / J) acc + dt S;  U = U + B dU
+    // (the FP32-mixed form forms the increment dt Ut in FP32, the accuracy of
+    // its Ut, and keeps the register update in FP64)
+    const double c = -st.dt * (double)iJ;
+    const R cf = F32 ? (R)(-st.dt) * iJ : R(0);
+    bool bad = false;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      double d;
+      if constexpr (F32) d = f2d_bits(cf * acc[v]);
+      else d = c * (double)acc[v];
+      if (force) d = fma(st.dt, src[v], d);
+      if (st.read_dU) d = fma(st.A, dU[v * S + g], d);
+      const double un = fma(st.B, d, Uo[v]);
+      dU[v * S + g] = d;
+      Uout[v * S + g] = un;
+      Uo[v] = un;
+      bad |= !finite_bits(un);
+    }
+    if (bad) atomicOr(status, ST_NONFINITE);
+    // the next stage's FP32 primitives, from the updated FP64 state
+    if constexpr (F32) {
+      if (st.write_w32) {
+        Lo3 l;
+        const Prim<float> q = prim32_shifted(Uo[0], Uo[1], Uo[2], Uo[3], Uo[4], ph, &l);
+        store_prim32(m.W32, S, g, q, l);
+      }
+    }
+  }
+}
+
 template <int N, typename R, int MODE, bool EC>
 __global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, R, EC>()))
 k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, const Tables<N> tab,
          const R* __restrict__ Rv, const R* __restrict__ Fs, double* __restrict__ Out,
          double* __restrict__ dU, double* __restrict__ Uout, const StageArgs st, int* __restrict__ status) {
   using Sh = VolShape<N>;
-  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS, LPW = Sh::LPW;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr bool F32 = std::is_same<R, float>::value;
   // FP64 at N = 7: the pairs' metric sums read from m.pairA
@@ -2195,7 +2559,6 @@ k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, c
   R* sC8 = sR + 5 * n3;                     // [n2]: DVS / 8
   R* sC16 = sC8 + n2;                       // [n2]: DVS / 16
   R* sC1 = sC16 + n2;                       // [n2]: DVS
-  R* siw = sC1 + n2;                        // [n]
   const int e = blockIdx.x, t = threadIdx.x;
   const size_t S = (size_t)m.K * n3;
   const bool kg = ph.vol_flux == 1;
@@ -2207,10 +2570,8 @@ k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, c
     sC16[x] = (R)(0.5 * tab.DVS8[x]);
     sC1[x] = (R)(8.0 * tab.DVS8[x]);
   }
-  if (t < n) siw[t] = (R)tab.iw[t];
   // prologue: node t (the FP32-mixed form reads the stage's FP32 primitives
   // and loads the FP64 state only in the epilogue)
-  double Uo[5];
   if (t < n3) {
     const size_t g = (size_t)e * n3 + t;
     Prim<R> q;
@@ -2256,323 +2617,12 @@ k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, c
     }
   }
   __syncthreads();
-  // three direction passes over the lines
-  {
-    const int warp = t >> 5, lane = t & 31;
-    const int seg = lane / n, pos = lane - seg * n;
-    const int L0 = warp * LPW + seg;
-    const bool active = (seg < LPW) && (L0 < n2);
-    const int L = active ? L0 : 0;
-    const int base = seg * n;  // first lane of the segment
-    const int la = L % n, lb = L / n;
-    // node at position q of this lane's line along dir (a warp holds the same
-    // lines L in every direction)
-    auto node_at = [&](int dir, int q) {
-      return dir == 0 ? q + n * L : (dir == 1 ? la + n * q + n2 * lb : L + n2 * q);
-    };
-    auto load_node = [&](int nd, int dir) {
-      const int node = vslot<N, R>(nd);
-      VolNode<R> X;
-      X.rho = sQ[node]; X.u = sQ[n3 + node]; X.v = sQ[2 * n3 + node]; X.w = sQ[3 * n3 + node];
-      X.p4 = sQ[4 * n3 + node]; X.hh = sQ[5 * n3 + node];
-      X.p2 = (kg || EC) ? sQ[6 * n3 + node] : R(0);
-      X.ib = EC ? sQ[7 * n3 + node] : R(0);
-      X.irh = EC ? sQ[8 * n3 + node] : R(0);
-      if constexpr (!PSUM) {
-        X.a0 = sA[(dir * 3 + 0) * n3 + node]; X.a1 = sA[(dir * 3 + 1) * n3 + node];
-        X.a2 = sA[(dir * 3 + 2) * n3 + node];
-      } else {
-        X.a0 = X.a1 = X.a2 = R(0);
-      }
-      return X;
-    };
-    // symmetric two-point flux F#(A, B) . 4 {Ja} in the scaled form of the
-    // coefficient tables (mass row against DVS / 8, the others against DVS / 16)
-    // (Sa: the sum of the two nodes' metrics, given or formed here)
-    auto sym_flux_s = [&](const VolNode<R>& A, const VolNode<R>& B, R Sa0, R Sa1, R Sa2, R F[5]) {
-      const R Sr = A.rho + B.rho, Su = A.u + B.u, Sv = A.v + B.v, Sw = A.w + B.w;
-      const R Sp = A.p4 + B.p4;
-      const R ua = Su * Sa0 + Sv * Sa1 + Sw * Sa2;  // 4 {u}.{a}
-      if constexpr (EC) {
-        // nodes hold ib = 1 / (2 beta) and irh = 1 / (2 rho), so that with
-        // Sh = ib_A + ib_B (half the sum of the inverse temperatures):
-        //   rho_ln = Sr G / 2;  rgm1 / beta_ln = Sh Qg / 2 (Qg = 2 rgm1 Q);
-        //   1 / (bA + bB) = Sh Rh / 2 (Rh = Rb / 2)
-        const R Dr = A.rho - B.rho, Db = A.hh - B.hh, Sh = A.ib + B.ib;
-        const R tr = Dr * Dr * (A.irh * B.irh);
-        const R tb = Db * Db * (A.ib * B.ib);
-        const R G = tr < LogMeanCut<R>::v ? logmean_G<R>(tr) : R(2) * Dr / (Sr * log1p(Dr / B.rho));
-        R Qg, Rh;
-        if (tb < LogMeanCut<R>::v) {
-          auto qc = [&](int c) { return cR<R>(ph.ec_q[c], ph.f32c.ec_q[c]); };
-          Qg = qc(0) + tb * (qc(1) + tb * (qc(2) + tb * (qc(3) + tb * qc(4))));
-          Rh = R(0.5) + tb * (R(-0.5) + tb * (R(0.5) + tb * (R(-0.5) + tb * R(0.5))));
-        } else {
-          Qg = R(2) * cR<R>(ph.rgm1, ph.f32c.rgm1) * log1p(Db / B.hh) / (Db * Sh);
-          Rh = R(1) / (Sh * (A.hh + B.hh));
-        }
-        const R mf = Sr * G * ua;                 // 8 F_rho
-        const R Spt = Sh * Rh * Sp;               // 8 (p~ - p_ref)
-        F[0] = mf;
-        F[1] = mf * Su + Spt * Sa0;               // 16 F_m
-        F[2] = mf * Sv + Spt * Sa1;
-        F[3] = mf * Sw + Spt * Sa2;
-        // 16 F_E = 2 mf (1 / (2 (gamma-1) beta_ln) + |{u}|^2 - {|u|^2} / 2) + 4 p~ (4 {u}.{a})
-        //        = mf X / 2 + (Spt / 2 + 4 p_ref) (4 {u}.{a})
-        const R X = Sh * Qg + Su * Su + Sv * Sv + Sw * Sw - A.p2 - B.p2;
-        F[4] = R(0.5) * mf * X + (R(0.5) * Spt + R(4) * cR<R>(ph.p_ref, ph.f32c.p_ref)) * ua;
-      } else {
-        const R mf = Sr * ua;                     // 8 F0
-        F[0] = mf;
-        F[1] = mf * Su + Sp * Sa0;                // 16 F1
-        F[2] = mf * Sv + Sp * Sa1;
-        F[3] = mf * Sw + Sp * Sa2;
-        F[4] = mf * (A.hh + B.hh);                // 16 F4
-        if (kg) F[4] += (A.p2 + B.p2) * ua;
-      }
-    };
-    auto sym_flux = [&](const VolNode<R>& A, const VolNode<R>& B, R F[5]) {
-      sym_flux_s(A, B, A.a0 + B.a0, A.a1 + B.a1, A.a2 + B.a2, F);
-    };
-    auto sums_main = [&](int dir, int d, R Sa[3]) {
+  volume_passes<N, R, EC, PSUM>(VolSmem<R>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
+  volume_epilogue<N, R, MODE>(Uin, m, ph, tab, Fs, Out, dU, Uout, st, status, e, t,
+                              [&](int nd, size_t, R acc[5]) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Sa[c] = m.pairA[pair_main(e, dir, c, d, L, pos)];
-    };
-    auto sums_half = [&](int dir, int Lx, int pa, R Sa[3]) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) Sa[c] = m.pairA[pair_half(m.K, e, dir, c, Lx, pa)];
-    };
-    // FP64, N = 7: the n/2 pairs at distance n/2 of a line would be formed twice
-    // (once in each lane); instead the distance-n/2 step of the xi pass forms
-    // the xi pairs in lanes pos < n/2 and the eta pairs in lanes pos >= n/2
-    // (swapped by a shuffle), and the one of the eta pass, in the first half
-    // of the warps, the zeta pairs of its own lines (lanes pos < n/2) and of
-    // the lines of warp + WARPS_LINES/2 (lanes pos >= n/2, through shared
-    // memory: the xi metrics, no longer read after the xi pass).  A lane
-    // carries that pair's flux for its next pass's node in `carry`.
-    // A node's sum runs through the passes: the xi pass starts it with the
-    // weak viscous divergence R_v, the eta and zeta passes from the sum the
-    // previous pass stored (with the carried pair's term as its first FMA).
-    constexpr bool HALF = std::is_same<R, double>::value && n == 8 && Sh::WARPS_LINES % 2 == 0;
-    constexpr int DMAX = HALF ? n / 2 - 1 : n / 2;
-    constexpr int HW = Sh::WARPS_LINES / 2, NX = HW * LPW * (n / 2);
-    R* sX = sA;  // [5][NX] zeta pair fluxes handed to the second half of the warps
-    R carry[5] = {R(0), R(0), R(0), R(0), R(0)};
-#pragma unroll 1
-    for (int dir = 0; dir < 3; ++dir) {
-      const int me = node_at(dir, pos);
-      const int ms = vslot<N, R>(me);
-      const VolNode<R> A = load_node(me, dir);
-      // FP32 difference form: the low parts of this lane's node velocity
-      float Aul = 0.f, Avl = 0.f, Awl = 0.f;
-      if constexpr (F32 && !EC) {
-        if (dif) { Aul = sQ[7 * n3 + ms]; Avl = sQ[8 * n3 + ms]; Awl = sQ[9 * n3 + ms]; }
-      }
-      R acc[5];
-      if (dir == 0) {
-        acc[0] = R(0);
-        const R* rv = Rv + (size_t)e * n3 + me;
-#pragma unroll
-        for (int v = 1; v < 5; ++v) acc[v] = ph.viscous ? rv[(size_t)(v - 1) * S] : R(0);
-      } else if constexpr (HALF) {
-        const int px = pos ^ (n / 2);
-        const R c8 = sC8[pos * n + px], c16 = sC16[pos * n + px];
-        if (dir == 2 && warp >= HW) {
-          const int x = ((warp - HW) * LPW + seg) * (n / 2) + (pos & (n / 2 - 1));
-#pragma unroll
-          for (int v = 0; v < 5; ++v) carry[v] = sX[v * NX + x];
-        }
-        acc[0] = fma(c8, carry[0], sR[ms]);
-#pragma unroll
-        for (int v = 1; v < 5; ++v) acc[v] = fma(c16, carry[v], sR[v * n3 + ms]);
-      } else {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) acc[v] = sR[v * n3 + ms];
-      }
-#pragma unroll
-      for (int d = 1; d <= DMAX; ++d) {
-        const int pm = pos + d < n ? pos + d : pos + d - n;
-        const int q = node_at(dir, pm);
-        if constexpr (std::is_same<R, float>::value && !EC) {
-          if (dif) {
-            const NodeF mi{A.rho, A.u, A.v, A.w, A.p4, A.hh, Aul, Avl, Awl};
-            // the partner node's values from the lane that holds it (lane
-            // base + pm of this line's segment)
-            const int lq = base + pm;
-            auto sh = [&](float x) { return __shfl_sync(0xffffffffu, x, lq); };
-            const NodeF mq{sh(A.rho), sh(A.u), sh(A.v), sh(A.w), sh(A.p4), sh(A.hh), sh(Aul), sh(Avl), sh(Awl)};
-            const float aq0 = sh(A.a0), aq1 = sh(A.a1), aq2 = sh(A.a2);
-            float G[5], Gq[5];
-            const float c1 = sC1[pos * n + pm];
-            if (2 * d != n) {
-              // and G(q -> i) for the partner lane (pos + d); receive G(i -> pos - d)
-              flux_delta_pair(mi, mq, A.a0, A.a1, A.a2, aq0, aq1, aq2, ph.f32c.rho_ref, ph.f32c.h_ref, G, Gq);
-#pragma unroll
-              for (int v = 0; v < 5; ++v) acc[v] += c1 * G[v];
-              const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
-              const float r1 = sC1[pos * n + (src - base)];
-#pragma unroll
-              for (int v = 0; v < 5; ++v) acc[v] += r1 * __shfl_sync(0xffffffffu, Gq[v], src);
-            } else {
-              flux_delta(mi, mq, A.a0, A.a1, A.a2, aq0 - A.a0, aq1 - A.a1, aq2 - A.a2, ph.f32c.rho_ref,
-                         ph.f32c.h_ref, G);
-#pragma unroll
-              for (int v = 0; v < 5; ++v) acc[v] += c1 * G[v];
-            }
-            continue;
-          }
-        }
-        R F[5];
-        if constexpr (PSUM) {
-          R Sa[3];
-          sums_main(dir, d, Sa);
-          sym_flux_s(A, load_node(q, dir), Sa[0], Sa[1], Sa[2], F);
-        } else {
-          sym_flux(A, load_node(q, dir), F);
-        }
-        const R c8 = sC8[pos * n + pm], c16 = sC16[pos * n + pm];
-        acc[0] += c8 * F[0];
-#pragma unroll
-        for (int v = 1; v < 5; ++v) acc[v] += c16 * F[v];
-        if (2 * d != n) {
-          // hand the pair flux to the partner lane (pos + d); receive the one
-          // of lane (pos - d)
-          const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
-          const int ps = src - base;
-          const R r8 = sC8[pos * n + ps], r16 = sC16[pos * n + ps];
-          acc[0] += r8 * __shfl_sync(0xffffffffu, F[0], src);
-#pragma unroll
-          for (int v = 1; v < 5; ++v) acc[v] += r16 * __shfl_sync(0xffffffffu, F[v], src);
-        }
-      }
-      if constexpr (HALF) {
-        constexpr int h = n / 2;
-        const int px = pos ^ h;  // partner at distance n/2
-        const R c8 = sC8[pos * n + px], c16 = sC16[pos * n + px];
-        if (dir == 0) {
-          const bool lo = pos < h;
-          const int dd = lo ? 0 : 1, pa = pos & (h - 1);
-          R F[5];
-          if constexpr (PSUM) {
-            R Sa[3];
-            sums_half(dd, L, pa, Sa);
-            sym_flux_s(load_node(node_at(dd, pa), dd), load_node(node_at(dd, pa + h), dd), Sa[0], Sa[1], Sa[2], F);
-          } else {
-            sym_flux(load_node(node_at(dd, pa), dd), load_node(node_at(dd, pa + h), dd), F);
-          }
-#pragma unroll
-          for (int v = 0; v < 5; ++v) {
-            const R Fx = __shfl_xor_sync(0xffffffffu, F[v], h);
-            acc[v] += (v == 0 ? c8 : c16) * (lo ? F[v] : Fx);
-            carry[v] = lo ? Fx : F[v];
-          }
-        } else if (dir == 1 && warp < HW) {
-          const bool lo = pos < h;
-          const int pa = pos & (h - 1);
-          const int Lz = lo ? L : L + HW * LPW;  // zeta line of this warp or of warp + HW
-          R F[5];
-          if constexpr (PSUM) {
-            R Sa[3];
-            sums_half(2, Lz, pa, Sa);
-            sym_flux_s(load_node(Lz + n2 * pa, 2), load_node(Lz + n2 * (pa + h), 2), Sa[0], Sa[1], Sa[2], F);
-          } else {
-            sym_flux(load_node(Lz + n2 * pa, 2), load_node(Lz + n2 * (pa + h), 2), F);
-          }
-          const int x = (warp * LPW + seg) * h + pa;
-#pragma unroll
-          for (int v = 0; v < 5; ++v) {
-            const R Fx = __shfl_xor_sync(0xffffffffu, F[v], h);
-            carry[v] = lo ? F[v] : Fx;
-            if (!lo) sX[v * NX + x] = F[v];
-          }
-        }
-      }
-      if (active) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) sR[v * n3 + ms] = acc[v];
-      }
-      __syncthreads();
-    }
-  }
-  if (t >= n3) return;
-  // epilogue: one node per thread.  At N = 7 the two warps of a zeta layer
-  // hold the eta rows {0, N, 1, 2} and {3, 4, 5, 6}, so that only the first
-  // runs the (masked) eta-face branch of the surface integral
-  int i, j, k;
-  if constexpr (n == 8 && T == n3) {
-    const int w = t >> 5, r = (t >> 3) & 3;
-    i = t & 7;
-    k = w >> 1;
-    j = (w & 1) ? 3 + r : (r == 0 ? 0 : (r == 1 ? N : r - 1));
-  } else {
-    i = t % n; j = (t / n) % n; k = t / n2;
-  }
-  const int nd = i + n * (j + n * k);
-  const size_t g = (size_t)e * n3 + nd;
-  // the element's own state, for the register update (read again here rather
-  // than kept in registers through the passes)
-#pragma unroll
-  for (int v = 0; v < 5; ++v) Uo[v] = Uin[v * S + g];
-  R acc[5];  // the passes' sums (with R_v)
-#pragma unroll
-  for (int v = 0; v < 5; ++v) acc[v] = sR[v * n3 + vslot<N, R>(nd)];
-  // surface integral: + sgn * Fs / w_perp on the faces that touch the node
-  auto surf = [&](int l, int ab, R iw) {
-    const int code = m.elem_face[e * 6 + l];
-    const int f = chk_idx(code >> 4, m.F, m.status);
-    const R sg = (code & 1) ? -iw : iw;
-    ab = omap_ab<N>((code >> 1) & 7, ab);  // the node's index in the master's face order
-    // difference form: the face's own side, F* - F(U_side), in rows 5 n2 apart
-    const R* src = dif ? Fs + (size_t)f * 10 * n2 + ((code & 1) ? 5 * n2 : 0) + ab : Fs + (size_t)f * 5 * n2 + ab;
-#pragma unroll
-    for (int v = 0; v < 5; ++v) acc[v] += sg * src[v * n2];
-  };
-  // one branch per direction (masked lanes of a branch cost as much as active ones)
-  if (i == 0 || i == N) surf(i == 0 ? 0 : 1, j + n * k, i == 0 ? siw[0] : siw[N]);
-  if (j == 0 || j == N) surf(j == 0 ? 2 : 3, i + n * k, j == 0 ? siw[0] : siw[N]);
-  if (k == 0 || k == N) surf(k == 0 ? 4 : 5, i + n * j, k == 0 ? siw[0] : siw[N]);
-  // Ut = -(1/J) acc + S, S = (0, f, f . u)
-  const R iJ = m.invJ[g];
-  const bool force = ph.has_force != 0;
-  double src[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (force) {
-    const double ir = 1.0 / Uo[0];
-    src[1] = ph.f[0]; src[2] = ph.f[1]; src[3] = ph.f[2];
-    src[4] = (ph.f[0] * Uo[1] + ph.f[1] * Uo[2] + ph.f[2] * Uo[3]) * ir;
-  }
-  if (MODE == 0) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) Out[v * S + g] = -(double)(iJ * acc[v]) + src[v];
-  } else {
-    // dU = A dU + dt Ut = A dU + (-dt / J) acc + dt S;  U = U + B dU
-    // (the FP32-mixed form forms the increment dt Ut in FP32, the accuracy of
-    // its Ut, and keeps the register update in FP64)
-    const double c = -st.dt * (double)iJ;
-    const R cf = F32 ? (R)(-st.dt) * iJ : R(0);
-    bool bad = false;
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      double d;
-      if constexpr (F32) d = f2d_bits(cf * acc[v]);
-      else d = c * (double)acc[v];
-      if (force) d = fma(st.dt, src[v], d);
-      if (st.read_dU) d = fma(st.A, dU[v * S + g], d);
-      const double un = fma(st.B, d, Uo[v]);
-      dU[v * S + g] = d;
-      Uout[v * S + g] = un;
-      Uo[v] = un;
-      bad |= !finite_bits(un);
-    }
-    if (bad) atomicOr(status, ST_NONFINITE);
-    // the next stage's FP32 primitives, from the updated FP64 state
-    if constexpr (F32) {
-      if (st.write_w32) {
-        Lo3 l;
-        const Prim<float> q = prim32_shifted(Uo[0], Uo[1], Uo[2], Uo[3], Uo[4], ph, &l);
-        store_prim32(m.W32, S, g, q, l);
-      }
-    }
-  }
+                                for (int v = 0; v < 5; ++v) acc[v] = sR[v * n3 + vslot<N, R>(nd)];
+                              });
 }
 
 }  // namespace dg

@@ -6,6 +6,7 @@
 namespace dg {
 
 struct PhysDev;
+struct Fx;
 
 struct OpArgs {
   int N, K, F, n_interior, n_wall, n_bc;
@@ -57,6 +58,8 @@ struct OpArgs {
   const float2* lift_M2;
   float2* lift_W2;
   const double* pairA;  // FP64 at N = 7: the volume kernel's pair metric sums (required there)
+  const Fx* JaX;        // FP64 form: [9][K n^3] metrics in fixed point and their exponent bounds [K]
+  const int* JaX_exp;
   double* wm_t;  // wall-law warm-start values per wall node (null: cold solves)
   // partitioned meshes: n_halo halo faces (the last faces), remote traces in
   // halo_U / halo_G, local traces packed into send_U / send_G.  phase selects

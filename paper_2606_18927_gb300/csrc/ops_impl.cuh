@@ -4,11 +4,13 @@
 
 #include <cstring>
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "adjoint.cuh"
 #include "kernels.cuh"
 #include "lift_df.cuh"
+#include "volume_fx.cuh"
 #include "ops.h"
 
 namespace dg {
@@ -19,6 +21,7 @@ static Tables<N> make_tables(const double* D, const double* w) {
   Tables<N> t;
   for (int i = 0; i < n; ++i) {
     t.iw[i] = 1.0 / w[i];
+    t.iw32[i] = (float)t.iw[i];
     for (int m = 0; m < n; ++m) {
       double dvs = 2.0 * D[i * n + m];
       if (i == m && i == 0) dvs += 1.0 / w[0];
@@ -79,6 +82,52 @@ static LiftPk<N> make_lift_pk(const Tables<N>& t) {
   return c;
 }
 
+// the fixed-point volume kernel's line tables, from the LGL nodes (x +- 1 and
+// the roots of P_N') in long double: D_im = P_N(x_i) / (P_N(x_m) (x_i - x_m))
+// and w_i = 2 / (N (N + 1) P_N(x_i)^2) give the antisymmetric
+// w_i D_im = 2 / (N (N + 1) P_N(x_i) P_N(x_m) (x_i - x_m))
+template <int N>
+static FxTab<N> make_fx_tab() {
+  constexpr int n = N + 1;
+  long double x[n], P[n];
+  for (int i = 0; i < n; ++i) {
+    x[i] = i == 0 ? -1.0L : (i == N ? 1.0L : -std::cos(3.14159265358979323846L * i / N));
+    for (int it = 0; it < 60; ++it) {
+      long double p0 = 1.0L, p1 = x[i];
+      for (int k = 2; k <= N; ++k) {
+        const long double p2 = ((2 * k - 1) * x[i] * p1 - (k - 1) * p0) / k;
+        p0 = p1; p1 = p2;
+      }
+      P[i] = p1;
+      if (i == 0 || i == N) break;
+      // (1 - x^2) P_N' = N (P_{N-1} - x P_N);  (1 - x^2) P_N'' = 2 x P_N' - N (N + 1) P_N
+      const long double q = 1.0L - x[i] * x[i], d = N * (p0 - x[i] * p1) / q;
+      const long double step = d * q / (2 * x[i] * d - N * (N + 1) * p1);
+      if (std::fabs(step) < 1e-18L) break;
+      x[i] -= step;
+    }
+  }
+  auto limbs = [](long double v) {
+    const long long r = llroundl(v), c = r + (1LL << 30);
+    return Fx{(int)(c >> 31), (int)(c & 0x7fffffff) - (1 << 30)};
+  };
+  FxTab<N> t;
+  const long double f = 0.5L * N * (N + 1);
+  t.eW = 0;
+  while (f > std::ldexp(1.0L, t.eW)) ++t.eW;  // 1 / w_0 is the largest
+  for (int i = 0; i < n; ++i) {
+    t.iw[i] = limbs(std::ldexp(f * P[i] * P[i], 61 - t.eW));
+    for (int m = 0; m < n; ++m)
+      t.Q[i * n + m] = limbs(i == m ? 0.0L : std::ldexp(1.0L / (f * (P[i] * P[m]) * (x[i] - x[m])), 61));
+  }
+  return t;
+}
+template <int N>
+static const FxTab<N>& fx_tab() {
+  static const FxTab<N> t = make_fx_tab<N>();
+  return t;
+}
+
 template <int N, typename R>
 static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
@@ -97,7 +146,8 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     return (int)cudaErrorInvalidValue;
   m.lift_M2 = a.lift_M2; m.lift_W2 = a.lift_W2;
   m.pairA = a.pairA;
-  if (N == 7 && std::is_same<R, double>::value && !a.pairA) return (int)cudaErrorInvalidValue;
+  m.JaX = a.JaX; m.JaX_exp = a.JaX_exp;
+  if (N == 7 && std::is_same<R, double>::value && ph.vol_flux == 2 && !a.pairA) return (int)cudaErrorInvalidValue;
   m.wm_t = a.wm_t;
   m.n_halo = a.n_halo; m.halo_U = a.halo_U; m.halo_G = static_cast<const R*>(a.halo_G);
   const Tables<N> tab = make_tables<N>(a.D, a.w);
@@ -115,7 +165,7 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   if (ec) {
     cudaFuncSetAttribute(k_volume<N, R, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
     cudaFuncSetAttribute(k_volume<N, R, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
-  } else {
+  } else if constexpr (std::is_same<R, float>::value) {
     cudaFuncSetAttribute(k_volume<N, R, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
     cudaFuncSetAttribute(k_volume<N, R, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
   }
@@ -196,16 +246,29 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     if (a.ev) cudaEventRecord(a.ev[4], s);
   }
   if (a.ev) cudaEventRecord(a.ev[5], s);
+  bool vol_done = false;
+  if constexpr (std::is_same<R, double>::value) {
+    if (!ec) {
+      auto kern = a.mode == 0 ? k_volume_fx<N, 0> : k_volume_fx<N, 1>;
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, VolFxShape<N>::SMEM);
+      kern<<<a.K, vol_threads, VolFxShape<N>::SMEM, s>>>(a.Uin, m, ph, tab, fx_tab<N>(), Rv, Fs, a.Out,
+                                                         a.dU, a.Uout, StageArgs{a.A, a.B, a.dt, a.read_dU, 0},
+                                                         a.status);
+      vol_done = true;
+    }
+  }
   StageArgs st{a.A, a.B, a.dt, a.read_dU, std::is_same<R, float>::value && a.mode == 1 ? 1 : 0};
-  if (a.mode == 0 && !ec)
-    k_volume<N, R, 0, false><<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, a.Out, nullptr, nullptr,
-                                                                st, a.status);
-  else if (a.mode == 0)
+  if constexpr (std::is_same<R, float>::value) {
+    if (!ec) {
+      auto kern = a.mode == 0 ? k_volume<N, R, 0, false> : k_volume<N, R, 1, false>;
+      kern<<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, a.Out, a.dU, a.Uout, st, a.status);
+      vol_done = true;
+    }
+  }
+  if (vol_done) {
+  } else if (a.mode == 0)
     k_volume<N, R, 0, true><<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, a.Out, nullptr, nullptr,
                                                                st, a.status);
-  else if (!ec)
-    k_volume<N, R, 1, false><<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, nullptr, a.dU, a.Uout,
-                                                                st, a.status);
   else
     k_volume<N, R, 1, true><<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, nullptr, a.dU, a.Uout,
                                                                st, a.status);
