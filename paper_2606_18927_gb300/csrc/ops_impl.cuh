@@ -116,7 +116,9 @@ static FxTab<N> make_fx_tab() {
   t.eW = 0;
   while (f > std::ldexp(1.0L, t.eW)) ++t.eW;  // 1 / w_0 is the largest
   for (int i = 0; i < n; ++i) {
-    t.iw[i] = limbs(std::ldexp(f * P[i] * P[i], 61 - t.eW));
+    t.iw[i] = llroundl(std::ldexp(f * P[i] * P[i], 61 - t.eW));
+    t.hd[i] = 0;
+    while (t.iw[i] << (t.hd[i] + 1) <= 1LL << 61) ++t.hd[i];
     for (int m = 0; m < n; ++m)
       t.Q[i * n + m] = limbs(i == m ? 0.0L : std::ldexp(1.0L / (f * (P[i] * P[m]) * (x[i] - x[m])), 61));
   }
@@ -145,9 +147,7 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   if (std::is_same<R, double>::value && ph.viscous && (!a.JaJ || !a.Mj))
     return (int)cudaErrorInvalidValue;
   m.lift_M2 = a.lift_M2; m.lift_W2 = a.lift_W2;
-  m.pairA = a.pairA;
-  m.JaX = a.JaX; m.JaX_exp = a.JaX_exp;
-  if (N == 7 && std::is_same<R, double>::value && ph.vol_flux == 2 && !a.pairA) return (int)cudaErrorInvalidValue;
+  m.JaX = a.JaX; m.JaX_max = a.JaX_max;
   m.wm_t = a.wm_t;
   m.n_halo = a.n_halo; m.halo_U = a.halo_U; m.halo_G = static_cast<const R*>(a.halo_G);
   const Tables<N> tab = make_tables<N>(a.D, a.w);
@@ -155,20 +155,11 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   R* Gf = static_cast<R*>(a.Gf);
   R* Fs = static_cast<R*>(a.Fs);
   const size_t smem_lift = (size_t)(16 * n3 + 26 * n2 + n) * sizeof(R);
-  const size_t smem_vol = (size_t)(ph.vol_flux == 2 ? VolShape<N>::SMEM_R_EC
-                                   : (std::is_same<R, float>::value ? VolShape<N>::SMEM_R_F32 : VolShape<N>::SMEM_R)) *
-                          sizeof(R);
+  const size_t smem_vol = (size_t)(ph.vol_flux == 2 ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * sizeof(R);
   constexpr int vol_threads = VolShape<N>::THREADS;
   // per device and cheap: set on every call
   cudaFuncSetAttribute(k_lift<N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_lift);
   const bool ec = ph.vol_flux == 2;
-  if (ec) {
-    cudaFuncSetAttribute(k_volume<N, R, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
-    cudaFuncSetAttribute(k_volume<N, R, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
-  } else if constexpr (std::is_same<R, float>::value) {
-    cudaFuncSetAttribute(k_volume<N, R, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
-    cudaFuncSetAttribute(k_volume<N, R, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
-  }
   const int phase = a.phase ? a.phase : 7;
   const unsigned halo_blocks = (unsigned)(((long long)a.n_halo * n2 + 255) / 256);
   if ((phase & 1) && a.n_halo > 0 && a.send_U)
@@ -246,32 +237,27 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     if (a.ev) cudaEventRecord(a.ev[4], s);
   }
   if (a.ev) cudaEventRecord(a.ev[5], s);
-  bool vol_done = false;
+  const StageArgs st{a.A, a.B, a.dt, a.read_dU, std::is_same<R, float>::value && a.mode == 1 ? 1 : 0};
   if constexpr (std::is_same<R, double>::value) {
-    if (!ec) {
-      auto kern = a.mode == 0 ? k_volume_fx<N, 0> : k_volume_fx<N, 1>;
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, VolFxShape<N>::SMEM);
-      kern<<<a.K, vol_threads, VolFxShape<N>::SMEM, s>>>(a.Uin, m, ph, tab, fx_tab<N>(), Rv, Fs, a.Out,
-                                                         a.dU, a.Uout, StageArgs{a.A, a.B, a.dt, a.read_dU, 0},
-                                                         a.status);
-      vol_done = true;
-    }
-  }
-  StageArgs st{a.A, a.B, a.dt, a.read_dU, std::is_same<R, float>::value && a.mode == 1 ? 1 : 0};
-  if constexpr (std::is_same<R, float>::value) {
-    if (!ec) {
-      auto kern = a.mode == 0 ? k_volume<N, R, 0, false> : k_volume<N, R, 1, false>;
+    auto volume = [&](auto kern, int smem) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      kern<<<a.K, vol_threads, smem, s>>>(a.Uin, m, ph, tab, fx_tab<N>(), Rv, Fs, a.Out, a.dU, a.Uout, st, a.status);
+    };
+    auto flux = [&](auto vf) {
+      constexpr int VF = decltype(vf)::value;
+      volume(a.mode == 0 ? k_volume_fx<N, 0, VF> : k_volume_fx<N, 1, VF>, VolFxShape<N, VF>::SMEM);
+    };
+    if (ec) flux(std::integral_constant<int, FX_EC>{});
+    else if (ph.vol_flux == 1) flux(std::integral_constant<int, FX_KG>{});
+    else flux(std::integral_constant<int, FX_KEP>{});
+  } else {
+    auto volume = [&](auto kern) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
       kern<<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, a.Out, a.dU, a.Uout, st, a.status);
-      vol_done = true;
-    }
+    };
+    if (ec) volume(a.mode == 0 ? k_volume<N, R, 0, true> : k_volume<N, R, 1, true>);
+    else volume(a.mode == 0 ? k_volume<N, R, 0, false> : k_volume<N, R, 1, false>);
   }
-  if (vol_done) {
-  } else if (a.mode == 0)
-    k_volume<N, R, 0, true><<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, a.Out, nullptr, nullptr,
-                                                               st, a.status);
-  else
-    k_volume<N, R, 1, true><<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, nullptr, a.dU, a.Uout,
-                                                               st, a.status);
   if (a.ev) cudaEventRecord(a.ev[6], s);
   return (int)cudaGetLastError();
 }

@@ -13,11 +13,13 @@
 // product to 53 bits of its own value, in every operation, the additions
 // among them; so the fixed-point sums are the more exact ones wherever a
 // node's fluxes are not far below the element's largest (against the
-// extended-precision oracle the operator's error fell by 5 to 30 % on meshes
-// of degree 2 to 8; with densities 20 apart within an element it tripled).
+// extended-precision oracle the operator's error (2-norm) fell by up to 30 % on
+// meshes of degree 2 to 8, for the three fluxes; with densities 20 apart
+// within an element it tripled).
 // An element in which they may be is summed in FP64 as before (fx_plan:
-// non-finite values, density or enthalpy differing by more than a factor 8
-// over its nodes, or a Mach number so small that the common unit of the
+// non-finite values; density or enthalpy differing by more than a factor 8
+// over its nodes, with the entropy-conserving flux density or internal energy
+// by more than an eighth, where its logarithmic means' series end; or a Mach number so small that the common unit of the
 // momentum flux would cost the velocity bits).
 #pragma once
 #include <cuda_runtime.h>
@@ -54,6 +56,10 @@ struct FxSum {
   __device__ __forceinline__ long long get() const { return madw((int)(x >> 32), 2, hh); }
 };
 __device__ __forceinline__ long long fx_mul(Fx a, Fx b) { return FxSum(a, b).get(); }
+// a b 2^k in the same units, to the nearest 2^-k'th below
+__device__ __forceinline__ long long fx_mul_shl(Fx a, Fx b, int k) {
+  return (mulw(a.h, b.h) << k) + (madw(a.l, b.h, mulw(a.h, b.l)) >> (31 - k));
+}
 
 // limbs of r 2^k
 template <int k>
@@ -62,6 +68,10 @@ __device__ __forceinline__ Fx fx_split(long long r) {
 }
 
 __device__ __forceinline__ int fx_biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// |x| ordered as integers (the high words), and the factor by which the largest
+// lies below its power of two (rounded up)
+__device__ __forceinline__ int fx_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ float fx_mant(int mag) { return (float)((mag & 0xfffff) + 0x100001) * (1.0f / 2097152.0f); }
 
 // x 2^(60 - eb + 1022), |x| < 2^(eb - 1022), truncated, in normalised limbs
 __device__ __forceinline__ Fx fx_of(double x, int eb) {
@@ -90,93 +100,189 @@ __device__ __forceinline__ double fx_double(long long r, int e) {
 
 // Line tables: Q_im = w_i D_im in units of 2^-61 (antisymmetric off the
 // diagonal, where the split form's DVS = 2 D - B / w is 2 D and has zeros at
-// the corners), and 1 / w_i in units of 2^(eW - 61)
+// the corners), 1 / w_i in units of 2^(eW - 61), and the bits hd_i by which
+// 1 / w_i is below 2^eW: a node's sums are kept in units finer by the least of
+// its three positions' (in one unit for all nodes the interior ones, where
+// 1 / w is a tenth of its end value, would lose those bits)
 template <int N>
 struct FxTab {
   Fx Q[(N + 1) * (N + 1)];
-  Fx iw[N + 1];
+  long long iw[N + 1];
+  int hd[N + 1];
   int eW;
 };
 
-// the element's units, from the largest (and, of rho and h, smallest) biased
-// exponents of its nodes
-enum { FX_RHO, FX_U, FX_P, FX_H, FX_NRHO, FX_NH, FX_NUM };
+// Logarithmic means in fixed point (the entropy-conserving flux; see
+// logmean_G): with t = (a - b)^2 / (4 a b) < 2^-8 (a and b within an eighth of
+// each other), T = 256 t in units of 2^-61, the series
+//   1 - t (c1 - t (c2 - t (c3 - t (c4 - t (c5 - t c6)))))
+// to 2^-61 (truncation below 2^-56 at t = 2^-8).  c3 .. c6 in units of 2^-30 by
+// the high limb alone, c1 and c2 in units of 2^-61.
+struct FxSeries {
+  long long c1, c2;
+  int c3, c4, c5, c6;
+};
+constexpr int fx_q30(double x) { return (int)(x * 1073741824.0 + 0.5); }
+// G = tanh(s) / s, Q = 2 s / sinh(2 s) (s = asinh sqrt t), R = 1 / (1 + t)
+constexpr FxSeries FX_G{(1LL << 61) / 3, (1LL << 61) / 45 * 11, fx_q30(191.0 / 945.0), fx_q30(2497.0 / 14175.0),
+                        fx_q30(14797.0 / 93555.0), fx_q30(92427157.0 / 638512875.0)};
+constexpr FxSeries FX_Q{(1LL << 61) / 3 * 2, (1LL << 61) / 15 * 8, fx_q30(16.0 / 35.0), fx_q30(128.0 / 315.0),
+                        fx_q30(256.0 / 693.0), fx_q30(1024.0 / 3003.0)};
+constexpr FxSeries FX_R{1LL << 61, 1LL << 61, 1 << 30, 1 << 30, 1 << 30, 1 << 30};
+
+__device__ __forceinline__ Fx fx_series(Fx T, const FxSeries c) {
+  auto low = [&](int cc, int s) { return cc - ((int)(mulw(T.h, s) >> 32) >> 6); };
+  const int s3 = low(c.c3, low(c.c4, low(c.c5, c.c6)));
+  const Fx s2 = fx_split<0>(c.c2 - (mulw(T.h, s3) >> 7));
+  const Fx s1 = fx_split<0>(c.c1 - (fx_mul(T, s2) >> 7));
+  return fx_split<0>((1LL << 61) - (fx_mul(T, s1) >> 7));
+}
+
+// 256 t in units of 2^-61 from d = a - b (|d| < 2^57) and the nodes' 1 / (2 a),
+// 1 / (2 b); sh = 7 + 2 (e_a + e_i), the exponents of the units of a and 1 / 2a
+__device__ __forceinline__ Fx fx_mean_arg(Fx a, Fx b, Fx ia, Fx ib, int sh) {
+  const int h = a.h - b.h, l = a.l - b.l;
+  const Fx d{h * 8 + (l >> 28), (l & 0x0fffffff) << 3};  // 8 (a - b)
+  const long long t = fx_mul(fx_split<0>(fx_mul(d, d)), fx_split<2>(fx_mul(ia, ib)));
+  return fx_split<0>(t << sh);
+}
+
+// The element's units, from its nodes' largest magnitudes.  Node values: rho,
+// u, p' and h; Kennedy-Gruber: e = E / rho for h, and 2 p; entropy-conserving
+// flux: rho, u, p', e = p / ((gamma - 1) rho),
+// b = 1 / (2 e) and 1 / (2 rho), with b p' in the place of p'.
+enum { FX_KEP, FX_KG, FX_EC };  // the volume flux, as PhysDev::vol_flux
+enum { FX_RHO, FX_U, FX_P, FX_H, FX_NRHO, FX_NH, FX_B, FX_IR, FX_NUM };
 struct FxPlan {
   int ok;              // 0: the element is summed in FP64
-  int bR, bU, bP, bH;  // biased exponent bounds of rho, u, p', h (fx_of)
+  int bR, bU, bP, bH;  // biased exponent bounds of rho, u, p' (EC: b p'), h (EC: e) for fx_of
+  int bB, bI;          // EC: of b and 1 / (2 rho)
   int kp;              // the momentum flux's unit is 2^kp times that of m u
   int e0, em, ee;      // the sums' units: mass, momentum, energy rows
+  int k0, km, ke;      // bits that the sums' bounds leave free: kept when 1 / w is applied
+  int sr, sb;          // EC: shifts of fx_mean_arg for rho and b
+  int bZ;              // Kennedy-Gruber: of 2 p
+  int kt, kd, kz;      // EC: right shifts of e Q, u.u and 4 p~' to the energy bracket's units
+  long long pref;      // EC: 4 p_ref in the bracket's unit
 };
 
-// ex: FX_RHO.. the maxima, FX_NRHO, FX_NH the maxima of 2047 - exponent; bA:
-// exponent bound of the metrics; eW of the table
-__device__ __forceinline__ FxPlan fx_plan(const int* ex, int bA, int eW) {
+// ex: the largest fx_mag of each value (FX_NRHO, FX_NH: of 0x7fffffff - fx_mag);
+// mA: that of the element's metrics; eW of the line table
+template <int VF>
+__device__ __forceinline__ FxPlan fx_plan(const int* ex, int mA, int eW, double p_ref, double gm1) {
+  constexpr bool EC = VF == FX_EC;
   FxPlan f;
-  f.bR = ex[FX_RHO]; f.bH = ex[FX_H];
-  const int eR = f.bR - 1022, eH = f.bH - 1022, eA = bA - 1022, eP = ex[FX_P] - 1022;
+  f.bR = ex[FX_RHO] >> 20;
+  f.bH = ex[FX_H] >> 20;
+  const int eR = f.bR - 1022, eA = (mA >> 20) - 1022, eP = (ex[FX_P] >> 20) - 1022;
+  int eH = f.bH - 1022;
   // p' is summed with rho u u: below 2^(eR + 2 eU - 1) in the unit of m u; a
   // larger p' (low Mach numbers, no reference pressure) raises that unit by
   // 2^kp, and beyond kp = 40 the velocity's
-  const int eUt = ex[FX_U] - 1022;
+  const int eUt = (ex[FX_U] >> 20) - 1022;
   int eU = max(eUt, -200);
   eU = max(eU, (eP - eR + 1 - 40 + 1) >> 1);
   f.bU = eU + 1022;
   f.kp = max(0, eP - (eR + 2 * eU - 1));
-  f.bP = eR + 2 * eU - 1 + f.kp + 1022;
-  const int base = eA + eW - 57;
-  f.e0 = eR + eU + base;
-  f.em = eR + 2 * eU + base + f.kp;
-  f.ee = eR + eU + eH + base;
-  const bool finite = ex[FX_RHO] < 0x7ff && ex[FX_U] < 0x7ff && ex[FX_P] < 0x7ff && ex[FX_H] < 0x7ff;
+  const int ePt = eR + 2 * eU - 1 + f.kp;
+  f.bP = ePt + 1022;
+  const bool finite = f.bR < 0x7ff && (ex[FX_U] >> 20) < 0x7ff && (ex[FX_P] >> 20) < 0x7ff && f.bH < 0x7ff;
   const bool range = abs(eR) < 200 && abs(eH) < 200 && abs(eA) < 200 && eU < 200 && eP < 200;
-  const bool even = f.bR - (2047 - ex[FX_NRHO]) <= 2 && f.bH - (2047 - ex[FX_NH]) <= 2;
-  f.ok = finite && range && even && (eU - eUt <= 5 || ex[FX_U] == 0);
+  // what the largest values leave of the bounds (all below 1)
+  const float mr = fx_mant(ex[FX_RHO]), mh = fx_mant(ex[FX_H]), ma = fx_mant(mA);
+  const float mu = ldexpf(fx_mant(ex[FX_U]), max(eUt - eU, -60));
+  const float mp = ldexpf(fx_mant(ex[FX_P]), max(eP - ePt, -60));
+  const float mass = mr * mu * ma;
+  float energy = mass * mh;
+  bool even;
+  if constexpr (EC) {
+    // rho and e within an eighth over the element (t < 2^-8)
+    auto near = [](int mx, int nmn) {
+      const double hi = __hiloint2double(mx + 1, 0), lo = __hiloint2double(0x7fffffff - nmn, 0);
+      return hi - lo < 0.125 * lo;
+    };
+    even = near(ex[FX_RHO], ex[FX_NRHO]) && near(ex[FX_H], ex[FX_NH]);
+    f.bB = ex[FX_B] >> 20; f.bI = ex[FX_IR] >> 20;
+    f.sr = 7 + 2 * (eR + f.bI - 1022);
+    f.sb = 7 + 2 * (eH + f.bB - 1022);
+    // b p' in the unit that makes (b p' sums) (e sums) / (1 + t) that of p'
+    f.bP = ePt - eH + 1 + 1022;
+    const int e1 = eH - 59, e2 = 2 * eU - 58, eY = max(e1, e2);  // units of e Q and u.u
+    f.kt = min(eY - e1, 63);
+    f.kd = min(eY - e2, 63);
+    energy = mass * fminf(1.0f, (ldexpf(mh, -f.kt) + ldexpf(mu * mu, -f.kd)) * 0.58f);
+    const int eZ = eR + eY + 2;  // of rho (e Q + u.u)
+    f.kz = eZ - (ePt - 60) - 1;
+    even = even && f.kz >= 0 && f.kz < 64 && f.sr >= 7 && f.sr <= 9 && f.sb >= 7 && f.sb <= 9 &&
+           fx_biased_exp(p_ref) + 2 - 1022 <= eZ + 59 && gm1 < 0.7;
+    f.pref = __double2ll_rn(4.0 * p_ref * __hiloint2double((1023 - eZ) << 20, 0));
+    eH = eY + 60;
+  } else {
+    even = f.bR - ((0x7fffffff - ex[FX_NRHO]) >> 20) <= 2 && f.bH - ((0x7fffffff - ex[FX_NH]) >> 20) <= 2;
+    f.bB = f.bI = f.sr = f.sb = f.kt = f.kd = f.kz = 0;
+    f.pref = 0;
+    if constexpr (VF == FX_KG) {
+      // 2 p (below 2 (gamma - 1) rho e) in the unit of rho e
+      f.bZ = eR + eH + 2 + 1022;
+      even = even && gm1 < 0.7 && (ex[FX_B] >> 20) <= f.bZ;
+    }
+  }
+  auto free_bits = [](float x) { return max(0, min(6, -1 - ilogbf(fmaxf(x, 1e-6f)))); };
+  f.k0 = free_bits(mass);
+  f.km = free_bits((ldexpf(mass * mu, -f.kp) + 0.34f * mp * ma) * 0.76f);
+  f.ke = free_bits(energy);
+  const int base = eA + eW - 57;
+  f.e0 = eR + eU + base - f.k0;
+  f.em = eR + 2 * eU + base + f.kp - f.km;
+  f.ee = eR + eU + eH + base - f.ke;
+  f.ok = finite && range && even && (eU - eUt <= 5 || ex[FX_U] >> 20 == 0);
   return f;
 }
 
 // The metrics Ja of every element in its own unit: limbs [9][K n3] and the
-// exponent bounds [K] (|Ja| < 2^(bA - 1023): one bit below fx_of's bound, so
-// that a pair's sum of three products S_u . S_a has room).  One block per
-// element, once per mesh.
+// largest fx_mag [K] (one bit below fx_of's bound, so that a pair's sum of
+// three products S_u . S_a has room).  One block per element, once per mesh.
 static __global__ void k_metric_fx(int n3, long long S, const double* __restrict__ Ja, Fx* __restrict__ JaX,
-                                   int* __restrict__ bA) {
+                                   int* __restrict__ mA) {
   __shared__ int mx;
   if (threadIdx.x == 0) mx = 0;
   __syncthreads();
   const size_t e0 = (size_t)blockIdx.x * n3;
   int b = 0;
   for (int t = threadIdx.x; t < n3; t += blockDim.x)
-    for (int c = 0; c < 9; ++c) b = max(b, fx_biased_exp(Ja[c * S + e0 + t]));
+    for (int c = 0; c < 9; ++c) b = max(b, fx_mag(Ja[c * S + e0 + t]));
   atomicMax(&mx, b);
   __syncthreads();
-  const int eb = max(mx, 100) + 1;
+  const int mg = max(mx, 100 << 20), eb = (mg >> 20) + 1;
   for (int t = threadIdx.x; t < n3; t += blockDim.x)
     for (int c = 0; c < 9; ++c) JaX[c * S + e0 + t] = fx_of(Ja[c * S + e0 + t], eb);
-  if (threadIdx.x == 0) bA[blockIdx.x] = eb - 1;
+  if (threadIdx.x == 0) mA[blockIdx.x] = mg;
 }
 
 
-template <int N>
+template <int N, int VF>
 struct VolFxShape {
   using Sh = VolShape<N>;
   static constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3;
-  // bytes: 7 node values, 9 metrics, 5 sums per node (8 bytes each; six node
-  // values in fixed point, seven in FP64), the line tables (fixed point: Q and
-  // 1 / w; FP64: three coefficient tables)
-  static constexpr int SMEM = (21 * n3 + 3 * n2) * 8;
+  // 8-byte values per node: 6 node values in fixed point (EC: 8), 7 in FP64
+  // (EC: 9), 9 metrics, 5 sums; the line tables (fixed point: Q and 1 / w;
+  // FP64: three coefficient tables)
+  static constexpr int QS = VF == FX_EC ? 9 : 7;
+  static constexpr int SMEM = ((QS + 14) * n3 + 3 * n2) * 8;
 };
 
-// The three direction passes in fixed point: sQ [6][n3] (rho, u, v, w, p', h),
-// sA [9][n3], sR [5][n3] the sums in units 2^em, sT [n2] Q and sW [n] 1 / w.
-// A line's n nodes are on n consecutive lanes; a lane forms the pairs with the
-// nodes at cyclic distance 1 .. n/2 and hands their flux to the partner by
-// shuffle, where it is subtracted (Q is antisymmetric); a pair at distance n/2
-// is formed by both of its lanes.
-template <int N>
-__device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, long long* sR, const Fx* sT, const Fx* sW,
-                                                 int kp, int t) {
+// The three direction passes in fixed point: sQ [6][n3] (rho, u, v, w, p', h;
+// Kennedy-Gruber [7][n3]: e for h, and 2 p; EC [8][n3]: rho, u, v, w, b p', e, b, 1 / (2 rho)), sA [9][n3], sR [5][n3] the
+// sums in the plan's units, sT [n2] Q, sW [n] 1 / w and sH [n] hd.  A line's n nodes are on
+// n consecutive lanes; a lane forms the pairs with the nodes at cyclic distance
+// 1 .. n/2 and hands their flux to the partner by shuffle, where it is
+// subtracted (Q is antisymmetric); a pair at distance n/2 is formed by both of
+// its lanes.
+template <int N, int VF>
+__device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, long long* sR, const Fx* sT,
+                                                 const long long* sW, const int* sH, const FxPlan& f, int t) {
   using Sh = VolShape<N>;
-  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW, NQ = VF == FX_EC ? 8 : 6 + VF;
   const int warp = t >> 5, lane = t & 31;
   const int seg = lane / n, pos = lane - seg * n;
   const int L0 = warp * LPW + seg;
@@ -184,46 +290,71 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
   const int L = active ? L0 : 0;
   const int base = seg * n;
   const int la = L % n, lb = L / n;
-  const Fx wi = sW[pos];
 #pragma unroll 1
   for (int dir = 0; dir < 3; ++dir) {
-    auto slot_at = [&](int q) {
-      return vslot<N, double>(dir == 0 ? q + n * L : (dir == 1 ? la + n * q + n2 * lb : L + n2 * q));
-    };
-    const int ms = slot_at(pos);
+    const int ms = vslot<N, double>(dir == 0 ? pos + n * L : (dir == 1 ? la + n * pos + n2 * lb : L + n2 * pos));
     const Fx* sD = sA + dir * 3 * n3;
-    Fx q[6], a[3];
+    Fx q[NQ], a[3];
 #pragma unroll
-    for (int v = 0; v < 6; ++v) q[v] = sQ[v * n3 + ms];
+    for (int v = 0; v < NQ; ++v) q[v] = sQ[v * n3 + ms];
 #pragma unroll
     for (int c = 0; c < 3; ++c) a[c] = sD[c * n3 + ms];
     long long acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll
     for (int d = 1; d <= n / 2; ++d) {
       const int pm = pos + d < n ? pos + d : pos + d - n;
-      const int sm = slot_at(pm);
+      const int sm = __shfl_sync(0xffffffffu, ms, base + pm);  // the partner's slot, from its lane
       const Fx Q = sT[pos * n + pm];
       const Fx Sa0 = a[0] + sD[sm], Sa1 = a[1] + sD[n3 + sm], Sa2 = a[2] + sD[2 * n3 + sm];
-      const Fx Su = q[1] + sQ[n3 + sm], Sv = q[2] + sQ[2 * n3 + sm], Sw = q[3] + sQ[3 * n3 + sm];
+      const Fx mv1 = sQ[n3 + sm], mv2 = sQ[2 * n3 + sm], mv3 = sQ[3 * n3 + sm];
+      const Fx Su = q[1] + mv1, Sv = q[2] + mv2, Sw = q[3] + mv3;
       FxSum s(Su, Sa0);
       s.add(Sv, Sa1);
       s.add(Sw, Sa2);
-      const Fx ua = fx_split<1>(s.get());                              // 4 {u}.{a}
-      const Fx rq = fx_split<1>(fx_mul(q[0] + sQ[sm], Q));             // 2 Q {rho}
-      const Fx pq = fx_split<0>(fx_mul(q[4] + sQ[4 * n3 + sm], Q));    // 2 Q {p'}
-      const long long m = fx_mul(rq, ua);                              // 8 Q {rho}{u}.{a}
-      const Fx mu = fx_split<1>(m >> kp), mh = fx_split<1>(m);
+      const Fx ua = fx_split<1>(s.get());  // 4 {u}.{a}
       long long F[5];
-      F[0] = m;
+      Fx pq;  // 2 Q {p'} (EC: 2 Q (p~ - p_ref))
+      if constexpr (VF == FX_KEP) {
+        const Fx rq = fx_split<1>(fx_mul(q[0] + sQ[sm], Q));        // 2 Q {rho}
+        pq = fx_split<0>(fx_mul(q[4] + sQ[4 * n3 + sm], Q));
+        F[0] = fx_mul(rq, ua);                                      // 8 Q {rho}{u}.{a}
+        F[4] = fx_mul(fx_split<1>(F[0]), q[5] + sQ[5 * n3 + sm]);   // times 2 {h}
+      } else if constexpr (VF == FX_KG) {
+        const Fx uq = fx_split<1>(fx_mul(ua, Q)), Sr = q[0] + sQ[sm], Sp = q[6] + sQ[6 * n3 + sm];
+        pq = fx_split<0>(fx_mul(q[4] + sQ[4 * n3 + sm], Q));
+        F[0] = fx_mul(Sr, uq);
+        // 16 F_E = 4 {u}.{a} [S_rho S_e + 4 {p}]
+        const long long Z = fx_mul(Sr, q[5] + sQ[5 * n3 + sm]) + (((long long)Sp.h << 31) + Sp.l);
+        F[4] = fx_mul(uq, fx_split<1>(Z));
+      } else {
+        const Fx uq = fx_split<1>(fx_mul(ua, Q));
+        const Fx rm = sQ[sm];
+        // ln-mean of rho: (S_rho / 2) G(t)
+        const Fx Sr = fx_split<1>(fx_mul(q[0] + rm, fx_series(fx_mean_arg(q[0], rm, q[7], sQ[7 * n3 + sm], f.sr), FX_G)));
+        const Fx em = sQ[5 * n3 + sm];
+        const Fx Se = q[5] + em;
+        const Fx tb = fx_mean_arg(q[6], sQ[6 * n3 + sm], q[5], em, f.sb);
+        // 2 (p~ - p_ref) = (b p' sums) (e sums) / (1 + t)
+        const long long pt = fx_mul_shl(q[4] + sQ[4 * n3 + sm], fx_split<1>(fx_mul(Se, fx_series(tb, FX_R))), 3);
+        pq = fx_split<0>(fx_mul(fx_split<0>(pt), Q));
+        F[0] = fx_mul(Sr, uq);  // 8 Q F_rho
+        // 16 F_E = 4 {u}.{a} [S_rho G (S_e Q(t) + u_A.u_B) + 4 (p~ - p_ref) + 4 p_ref]
+        FxSum k(q[1], mv1);
+        k.add(q[2], mv2);
+        k.add(q[3], mv3);
+        const long long Y = (fx_mul(Se, fx_series(tb, FX_Q)) >> f.kt) + (k.get() >> f.kd);
+        const long long Z = fx_mul(Sr, fx_split<0>(Y)) + (pt >> f.kz) + f.pref;
+        F[4] = fx_mul(uq, fx_split<1>(Z));
+      }
+      const Fx mu = fx_split<1>(F[0] >> f.kp);
       auto momentum = [&](Fx S, Fx Sa) {
-        FxSum f(mu, S);
-        f.add(pq, Sa);
-        return f.get();
+        FxSum x(mu, S);
+        x.add(pq, Sa);
+        return x.get();
       };
       F[1] = momentum(Su, Sa0);
       F[2] = momentum(Sv, Sa1);
       F[3] = momentum(Sw, Sa2);
-      F[4] = fx_mul(mh, q[5] + sQ[5 * n3 + sm]);
 #pragma unroll
       for (int v = 0; v < 5; ++v) acc[v] += F[v];
       if (2 * d != n) {
@@ -233,9 +364,10 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
       }
     }
     if (active) {
+      const Fx wi = fx_split<0>(sW[pos] << min(sH[pos], min(sH[la], sH[lb])));
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const long long r = fx_mul(fx_split<0>(acc[v]), wi);
+        const long long r = fx_mul_shl(fx_split<0>(acc[v]), wi, v == 0 ? f.k0 : (v == 4 ? f.ke : f.km));
         sR[v * n3 + ms] = dir == 0 ? r : r + sR[v * n3 + ms];
       }
     }
@@ -244,11 +376,11 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
 }
 
 // an element summed in FP64 (fx_plan); rare, so kept out of line
-template <int N>
+template <int N, int VF>
 __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<double>& m, const PhysDev& ph,
                                                 const Tables<N>& tab, const double* __restrict__ Rv, int e, int t) {
   constexpr int n3 = VolShape<N>::n3, n2 = VolShape<N>::n2, T = VolShape<N>::THREADS;
-  double *sQ = smem, *sA = sQ + 7 * n3, *sR = sA + 9 * n3, *sC8 = sR + 5 * n3, *sC16 = sC8 + n2, *sC1 = sC16 + n2;
+  double *sQ = smem, *sA = sQ + VolFxShape<N, VF>::QS * n3, *sR = sA + 9 * n3, *sC8 = sR + 5 * n3, *sC16 = sC8 + n2, *sC1 = sC16 + n2;
   for (int x = t; x < n2; x += T) {
     sC8[x] = tab.DVS8[x];
     sC16[x] = 0.5 * tab.DVS8[x];
@@ -260,65 +392,89 @@ __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<doub
     for (int c = 0; c < 9; ++c) sA[c * n3 + ts] = m.Ja[(size_t)c * ((size_t)m.K * n3) + (size_t)e * n3 + t];
   }
   __syncthreads();
-  volume_passes<N, double, false, false>(VolSmem<double>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
+  volume_passes<N, double, VF == FX_EC>(VolSmem<double>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
 }
 
-// k_volume of the FP64 form with the KEP fluxes: one CTA per element, the
-// passes in fixed point (Kennedy-Gruber's flux and elements out of fx_plan's
-// range: in FP64), the epilogue in FP64.  Measured at N = 7, 32^3 elements:
-// 10.08 ms with FP64 pair fluxes (FP64 pipe 90 % busy), 3.07 ms in fixed point
-// (issue 52 %, integer pipes 37 %, FP64 pipe 30 %).
-template <int N, int MODE>
-__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, double, false>()))
+// k_volume of the FP64 form: one CTA per element, the passes in fixed point
+// (elements out of fx_plan's range: in FP64), the epilogue in FP64.  Measured at N = 7, 32^3 elements: KEP flux 10.08 ms with
+// FP64 pair fluxes (FP64 pipe 90 % busy), 3.07 ms in fixed point (issue 52 %,
+// integer pipes 37 %, FP64 pipe 30 %).
+template <int N, int MODE, int VF>
+__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, double, VF == FX_EC>()))
 k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysDev ph, const Tables<N> tab,
             const FxTab<N> ft, const double* __restrict__ Rv, const double* __restrict__ Fs, double* __restrict__ Out,
             double* __restrict__ dU, double* __restrict__ Uout, const StageArgs st, int* __restrict__ status) {
   using Sh = VolShape<N>;
-  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS, QS = VolFxShape<N, VF>::QS;
+  constexpr bool EC = VF == FX_EC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int sEx[FX_NUM];
+  __shared__ FxPlan sF;
   Fx* sQ = reinterpret_cast<Fx*>(smem_raw);
-  Fx* sA = sQ + 7 * n3;
+  Fx* sA = sQ + QS * n3;
   long long* sR = reinterpret_cast<long long*>(sA + 9 * n3);
   Fx* sT = reinterpret_cast<Fx*>(sR + 5 * n3);
-  Fx* sW = sT + n2;
+  long long* sW = reinterpret_cast<long long*>(sT + n2);
+  int* sH = reinterpret_cast<int*>(sW + n);
   const int e = blockIdx.x, t = threadIdx.x;
   const size_t S = (size_t)m.K * n3;
   const size_t g = (size_t)e * n3 + t;
   Prim<double> q{1.0, 0.0, 0.0, 0.0, 0.0, 1.0};
+  // EC: e = p / ((gamma - 1) rho), 1 / (2 e), 1 / (2 rho); Kennedy-Gruber: E / rho, 2 p
+  double en = 1.0, be = 0.5, irh = 0.5;
   if (t < n3) {
     q = m.W64 ? load_prim64(m.W64, S, g) : primitive<double>(Uin[g], Uin[S + g], Uin[2 * S + g], Uin[3 * S + g], Uin[4 * S + g], ph);
     const int ts = vslot<N, double>(t);
 #pragma unroll
     for (int c = 0; c < 9; ++c) sA[c * n3 + ts] = m.JaX[(size_t)c * S + g];
+    if constexpr (EC) {
+      const double ir = rcp_pos(q.rho);
+      // (the quotient's remainder added back: half an ulp instead of two)
+      const double pf = q.p + ph.p_ref, a = ph.rgm1 * pf;
+      en = a * ir;
+      en = fma(fma(-en, q.rho, a) + fma(ph.rgm1, pf, -a), ir, en);
+      be = 0.5 * rcp_pos(en);
+      irh = 0.5 * ir;
+    }
+    if constexpr (VF == FX_KG) {
+      const double ir = rcp_pos(q.rho);
+      be = q.p + ph.p_ref;  // p
+      const double pr = be * ir;
+      en = q.h - fma(fma(-pr, q.rho, be), ir, pr);  // e = h - p / rho
+      be *= 2.0;
+    }
   }
   if (t < FX_NUM) sEx[t] = 0;
   for (int x = t; x < n2; x += T) sT[x] = ft.Q[x];
-  if (t < n) sW[t] = ft.iw[t];
-  const int eA = m.JaX_exp[e];
+  if (t < n) { sW[t] = ft.iw[t]; sH[t] = ft.hd[t]; }
   __syncthreads();
   {
-    const int bR = fx_biased_exp(q.rho), bH = fx_biased_exp(q.h);
+    // (EC: rho and e are positive, else the element is out of range)
+    const bool pos = !EC || (q.rho > 0.0 && en > 0.0);
     int ex[FX_NUM];
-    ex[FX_RHO] = bR;
-    ex[FX_U] = max(max(fx_biased_exp(q.u), fx_biased_exp(q.v)), fx_biased_exp(q.w));
-    ex[FX_P] = fx_biased_exp(q.p);
-    ex[FX_H] = bH;
-    ex[FX_NRHO] = 2047 - bR;
-    ex[FX_NH] = 2047 - bH;
+    ex[FX_RHO] = pos ? fx_mag(q.rho) : 0x7ff00000;
+    ex[FX_H] = fx_mag(VF == FX_KEP ? q.h : en);
+    ex[FX_NRHO] = 0x7fffffff - fx_mag(q.rho);
+    ex[FX_NH] = 0x7fffffff - ex[FX_H];
+    ex[FX_U] = max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w));
+    ex[FX_P] = fx_mag(q.p);
+    ex[FX_B] = fx_mag(be);
+    ex[FX_IR] = fx_mag(irh);
     if (t >= n3) {
 #pragma unroll
       for (int x = 0; x < FX_NUM; ++x) ex[x] = 0;
     }
 #pragma unroll
-    for (int x = 0; x < FX_NUM; ++x) {
+    for (int x = 0; x < (EC ? FX_NUM : FX_B + VF); ++x) {
       const int mx = __reduce_max_sync(0xffffffffu, ex[x]);
       if ((t & 31) == 0) atomicMax(&sEx[x], mx);
     }
   }
   __syncthreads();
-  const FxPlan f = fx_plan(sEx, eA, ft.eW);
-  const bool fx = f.ok && ph.vol_flux == 0;
+  if (t == 0) sF = fx_plan<VF>(sEx, m.JaX_max[e], ft.eW, ph.p_ref, ph.gm1);
+  __syncthreads();
+  const FxPlan f = sF;
+  const bool fx = f.ok != 0;
   if (t < n3) {
     const int ts = vslot<N, double>(t);
     if (fx) {
@@ -326,30 +482,32 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
       sQ[n3 + ts] = fx_of(q.u, f.bU);
       sQ[2 * n3 + ts] = fx_of(q.v, f.bU);
       sQ[3 * n3 + ts] = fx_of(q.w, f.bU);
-      sQ[4 * n3 + ts] = fx_of(q.p, f.bP);
-      sQ[5 * n3 + ts] = fx_of(q.h, f.bH);
-    } else {
-      double* d = reinterpret_cast<double*>(smem_raw) + ts;
-      d[0] = q.rho; d[n3] = q.u; d[2 * n3] = q.v; d[3 * n3] = q.w; d[4 * n3] = 4.0 * q.p;
-      d[5 * n3] = q.h;
-      if (ph.vol_flux == 1) {
-        const double pf = q.p + ph.p_ref;
-        d[5 * n3] = q.h - pf / q.rho;
-        d[6 * n3] = 2.0 * pf;
+      if constexpr (EC) {
+        sQ[4 * n3 + ts] = fx_of(be * q.p, f.bP);
+        sQ[5 * n3 + ts] = fx_of(en, f.bH);
+        sQ[6 * n3 + ts] = fx_of(be, f.bB);
+        sQ[7 * n3 + ts] = fx_of(irh, f.bI);
+      } else {
+        sQ[4 * n3 + ts] = fx_of(q.p, f.bP);
+        sQ[5 * n3 + ts] = fx_of(VF == FX_KEP ? q.h : en, f.bH);
+        if constexpr (VF == FX_KG) sQ[6 * n3 + ts] = fx_of(be, f.bZ);
       }
+    } else {
+      stage_node<N, double, EC>(reinterpret_cast<double*>(smem_raw), ts, q, ph, false);
     }
   }
   if (fx) {
     __syncthreads();
-    volume_passes_fx<N>(sQ, sA, sR, sT, sW, f.kp, t);
+    volume_passes_fx<N, VF>(sQ, sA, sR, sT, sW, sH, f, t);
   } else {
-    volume_passes_fp64<N>(reinterpret_cast<double*>(smem_raw), m, ph, tab, Rv, e, t);
+    volume_passes_fp64<N, VF>(reinterpret_cast<double*>(smem_raw), m, ph, tab, Rv, e, t);
   }
   volume_epilogue<N, double, MODE>(
       Uin, m, ph, tab, Fs, Out, dU, Uout, st, status, e, t, [&](int nd, size_t gn, double acc[5]) {
         const int ts = vslot<N, double>(nd);
         if (fx) {
-          const int eu[5] = {f.e0, f.em, f.em, f.em, f.ee};
+          const int k = min(sH[nd % n], min(sH[nd / n % n], sH[nd / n2]));
+          const int eu[5] = {f.e0 - k, f.em - k, f.em - k, f.em - k, f.ee - k};
 #pragma unroll
           for (int v = 0; v < 5; ++v) acc[v] = fx_double(sR[v * n3 + ts], eu[v]);
           if (ph.viscous) {

@@ -45,22 +45,35 @@ CASES = [(N, "flow", {}, {}, 1e-12) for N in range(1, 9)] + [
     (7, "density contrast in FP64", dict(contrast=2.5), {}, 2e-12),
     (4, "density contrast in FP64", dict(contrast=2.5), {}, 2e-12),
 ]
+# entropy-conserving flux: in range while density and internal energy vary by
+# less than an eighth over an element
+EC_CASES = [(N, "flow", {}, {}, 1e-12) for N in (1, 2, 4, 5, 7, 8)] + [
+    (7, "density steps", dict(contrast=0.02), {}, 1e-12),
+    (5, "no reference pressure", {}, dict(p_ref=0.0), 1e-10),
+    (7, "density contrast in FP64", dict(contrast=1.0), {}, 2e-12),
+]
+
+KG_CASES = [(N, "flow", {}, {}, 1e-12) for N in (1, 4, 7)] + [(5, "density contrast in FP64", dict(contrast=2.5), {}, 2e-12)]
 
 
-@pytest.mark.parametrize("N,label,state,phys_over,bound", CASES, ids=["n%d %s" % c[:2] for c in CASES])
-def test_fixed_point_volume_term(ora, N, label, state, phys_over, bound):
+@pytest.mark.parametrize("vol,N,label,state,phys_over,bound",
+                         [(0,) + c for c in CASES] + [(2,) + c for c in EC_CASES] + [(1,) + c for c in KG_CASES],
+                         ids=["kep n%d %s" % c[:2] for c in CASES] + ["ec n%d %s" % c[:2] for c in EC_CASES]
+                         + ["kg n%d %s" % c[:2] for c in KG_CASES])
+def test_fixed_point_volume_term(ora, vol, N, label, state, phys_over, bound):
     torch = torch_cuda()
     phys = dict(I.phys_params(Ma=0.3, Re=1600.0), **phys_over)
-    o, g, U = build(ora, I.BoxSpec(N, 3, 2, 2, geometry="sine", amplitude=0.1), phys, flow(**state))
+    o, g, U = build(ora, I.BoxSpec(N, 3, 2, 2, geometry="sine", amplitude=0.1), phys, flow(**state), vol_flux=vol)
     e = parity_per_var(gpu_ut(torch, g, U), o.time_derivative(U))
     print(N, label, ["%.1e" % x for x in e])
     assert max(e) <= bound, e
 
 
-def test_elements_in_and_out_of_range_side_by_side(ora):
+@pytest.mark.parametrize("vol", [0, 2])
+def test_elements_in_and_out_of_range_side_by_side(ora, vol):
     torch = torch_cuda()
     phys = I.phys_params(Ma=0.3, Re=1600.0)
-    o, g, U = build(ora, I.BoxSpec(5, 4, 2, 2), phys, flow())
+    o, g, U = build(ora, I.BoxSpec(5, 4, 2, 2), phys, flow(), vol_flux=vol)
     U = U.reshape(5, -1, 216)
     U[0, 3] *= np.exp(2.3 * np.linspace(-1.0, 1.0, 216))  # element 3: a contrast of 100
     U = np.ascontiguousarray(U)
