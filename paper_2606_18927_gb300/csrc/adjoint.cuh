@@ -88,8 +88,14 @@ __device__ __forceinline__ void law_param_derivs(int law, double w, double kap, 
 }
 
 // qw (may be null): the wall heat flux of isothermal walls (0 for adiabatic ones)
+// The law-of-the-wall solve depends on the values alone: with `sv` it is done
+// once (sv->have false: here, then kept in *sv) and serves every direction.
+struct WallSolve {
+  bool have, ok;
+  double ut, L, wdL, Lk, LB;
+};
 static __device__ void wall_stress_jvp(const PhysDev& ph, const DualD Us[5], double dk, double dB, double nx,
-                                double ny, double nz, DualD tau[3], bool* ok, DualD* qw = nullptr) {
+                                double ny, double nz, DualD tau[3], WallSolve* sv, DualD* qw = nullptr) {
   const DualD rho = Us[0], ir = 1.0 / rho;
   const DualD u = Us[1] * ir, v = Us[2] * ir, w = Us[3] * ir;
   const DualD p = ph.gm1 * (Us[4] - 0.5 * rho * (u * u + v * v + w * w));
@@ -99,7 +105,7 @@ static __device__ void wall_stress_jvp(const PhysDev& ph, const DualD Us[5], dou
   const DualD u2 = ux * ux + uy * uy + uz * uz;
   tau[0] = tau[1] = tau[2] = DualD(0.0);
   if (qw) *qw = DualD(0.0);
-  *ok = true;
+  if (!sv->have) { sv->ok = true; sv->ut = sv->wdL = sv->Lk = sv->LB = 0.0; sv->L = 1.0; }
   if (!(u2.v > 0.0)) return;
   const DualD um = sqrt(u2);
   const double r = cbrt(ph.Pr);
@@ -123,12 +129,15 @@ static __device__ void wall_stress_jvp(const PhysDev& ph, const DualD Us[5], dou
   // wall viscosity: constant, or Sutherland's law at the wall temperature
   const DualD muw = ph.sutherland ? ph.suth_C * Tw * sqrt(Tw) / (Tw + ph.suth_S) : DualD(ph.mu);
   const DualD nuw = muw / rhow;
-  const double ut = solve_utau(ph.law, uvd.v, ph.hwm, nuw.v, ph.kappa, ph.B, ph.wm_maxit, ok);
-  // explicit variable of the law at the solution
-  const double wv = ph.law == 1 ? ut * ph.hwm / nuw.v : uvd.v / ut;
-  double L, wdL, Lk, LB;
-  law_eval(ph.law, wv, ph.kappa, ph.B, &L, &wdL);
-  law_param_derivs(ph.law, wv, ph.kappa, ph.B, &Lk, &LB);
+  if (!sv->have) {
+    sv->ut = solve_utau(ph.law, uvd.v, ph.hwm, nuw.v, ph.kappa, ph.B, ph.wm_maxit, &sv->ok);
+    // explicit variable of the law at the solution
+    const double wv = ph.law == 1 ? sv->ut * ph.hwm / nuw.v : uvd.v / sv->ut;
+    law_eval(ph.law, wv, ph.kappa, ph.B, &sv->L, &sv->wdL);
+    law_param_derivs(ph.law, wv, ph.kappa, ph.B, &sv->Lk, &sv->LB);
+    sv->have = true;
+  }
+  const double ut = sv->ut, L = sv->L, wdL = sv->wdL, Lk = sv->Lk, LB = sv->LB;
   const double Ft = 1.0 + wdL / L;
   const double dlnRe = uvd.d / uvd.v - nuw.d / nuw.v;
   const double dt = -((Lk * dk + LB * dB) / L - dlnRe) / Ft;
@@ -485,34 +494,45 @@ k_adj_face(const double* __restrict__ U, const double* __restrict__ lam, const M
 }
 
 // ---------------------------------------------------------------------------
-// k_adj_wall: one thread per node of a wall face.  Also accumulates
-// g_theta = sum_nodes (dFs/dtheta)^T gFs.
+// k_adj_wall: nodes of the wall faces, 32 per block of ADJ_WALL_WARPS warps, a
+// node per lane (few nodes, long chains; see k_wall): the warps share the
+// planes of the sample's interpolation, the last takes the Riemann flux's
+// reverse mode, the first the law-of-the-wall solve, and then the warps 0 .. 6
+// one direction each of the wall model's derivative (the sample state's five
+// components, kappa, B).  Also accumulates g_theta = sum_nodes
+// (dFs/dtheta)^T gFs.
 // ---------------------------------------------------------------------------
+constexpr int ADJ_WALL_WARPS = 8;
+
 template <int N>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * ADJ_WALL_WARPS)
 k_adj_wall(const double* __restrict__ U, const double* __restrict__ lam, const MeshDev<double> m,
            const PhysDev ph, double iw, double* __restrict__ gUf, double* __restrict__ gGf,
            double* __restrict__ gUs, double* __restrict__ gtheta, int* __restrict__ status) {
-  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int wf = tid / n2, ab = tid - wf * n2;
-  double gk = 0.0, gb = 0.0;
-  if (wf < m.n_wall) {
-    const int f = m.n_interior + wf;
-    int4 fc = m.faces[f];
-    fc.x = chk_idx(fc.x, m.K, m.status);
-    const size_t S = (size_t)m.K * n3;
-    const size_t gM = (size_t)fc.x * n3 + fnode<N>(fc.y, ab % n, ab / n);
-    const double jM = m.invJ[gM];
-    double gFs[5], UA[5];
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, W = ADJ_WALL_WARPS;
+  __shared__ double sUs[W][5][32];
+  __shared__ WallSolve sSv[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int tid = blockIdx.x * 32 + lane;
+  const bool valid = tid < m.n_wall * n2;
+  const int wf = valid ? tid / n2 : 0, ab = valid ? tid - wf * n2 : 0;
+  const int f = m.n_interior + wf;
+  int4 fc = m.faces[f];
+  fc.x = chk_idx(fc.x, m.K, m.status);
+  const size_t S = (size_t)m.K * n3;
+  const size_t gM = (size_t)fc.x * n3 + fnode<N>(fc.y, ab % n, ab / n);
+  const double jM = m.invJ[gM];
+  double gFs[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      gFs[v] = -lam[v * S + gM] * jM * iw;
-      UA[v] = U[v * S + gM];
-    }
-    const size_t FN = (size_t)m.F * n2, fg = (size_t)f * n2 + ab;
-    const double nx = m.fgeo[fg], ny = m.fgeo[FN + fg], nz = m.fgeo[2 * FN + fg], s = m.fgeo[3 * FN + fg];
-    if (ph.viscous) {
+  for (int v = 0; v < 5; ++v) gFs[v] = -lam[v * S + gM] * jM * iw;
+  const size_t FN = (size_t)m.F * n2, fg = (size_t)f * n2 + ab;
+  const double nx = m.fgeo[fg], ny = m.fgeo[FN + fg], nz = m.fgeo[2 * FN + fg], s = m.fgeo[3 * FN + fg];
+  const size_t slot = (size_t)wf * n2 + ab;
+  if (w == W - 1) {
+    double UA[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) UA[v] = U[v * S + gM];
+    if (ph.viscous && valid) {
       double* dM = gGf + ((size_t)fc.x * 6 + fc.y) * 4 * n2 + ab;
 #pragma unroll
       for (int v = 0; v < 4; ++v) dM[v * n2] = 0.0;
@@ -520,72 +540,71 @@ k_adj_wall(const double* __restrict__ U, const double* __restrict__ lam, const M
     // inviscid flux through the mirror state U_B = (rho, m - 2 (m.n) n, E):
     // gU = gA + (dU_B/dU)^T gB
     double g[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, gB[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, gF[5], UB[5];
-    {
-      const double mn = UA[1] * nx + UA[2] * ny + UA[3] * nz;
-      UB[0] = UA[0]; UB[1] = UA[1] - 2.0 * mn * nx; UB[2] = UA[2] - 2.0 * mn * ny; UB[3] = UA[3] - 2.0 * mn * nz;
-      UB[4] = UA[4];
+    const double mn = UA[1] * nx + UA[2] * ny + UA[3] * nz;
+    UB[0] = UA[0]; UB[1] = UA[1] - 2.0 * mn * nx; UB[2] = UA[2] - 2.0 * mn * ny; UB[3] = UA[3] - 2.0 * mn * nz;
+    UB[4] = UA[4];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) gF[v] = gFs[v] * s;
-      face_flux_vjp(ph, UA, UB, nx, ny, nz, gF, g, gB);
-      const double gbn = gB[1] * nx + gB[2] * ny + gB[3] * nz;
-      g[0] += gB[0]; g[4] += gB[4];
-      g[1] += gB[1] - 2.0 * gbn * nx; g[2] += gB[2] - 2.0 * gbn * ny; g[3] += gB[3] - 2.0 * gbn * nz;
+    for (int v = 0; v < 5; ++v) gF[v] = gFs[v] * s;
+    face_flux_vjp(ph, UA, UB, nx, ny, nz, gF, g, gB);
+    const double gbn = gB[1] * nx + gB[2] * ny + gB[3] * nz;
+    g[0] += gB[0]; g[4] += gB[4];
+    g[1] += gB[1] - 2.0 * gbn * nx; g[2] += gB[2] - 2.0 * gbn * ny; g[3] += gB[3] - 2.0 * gbn * nz;
+    if (valid) {
+      double* oM = gUf + ((size_t)fc.x * 6 + fc.y) * 5 * n2 + ab;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) oM[v * n2] = g[v];
     }
-    double* oM = gUf + ((size_t)fc.x * 6 + fc.y) * 5 * n2 + ab;
-#pragma unroll
-    for (int v = 0; v < 5; ++v) oM[v * n2] = g[v];
-    // wall model: Fs_mom += tau s
-    const size_t slot = (size_t)wf * n2 + ab;
-    if (ph.viscous) {
-      const int es = chk_idx(m.ws_elem[slot], m.K, m.status);
-      const double* L = m.ws_lag + slot * 3 * n;
-      double Us[5] = {0, 0, 0, 0, 0};
-      for (int kk = 0; kk < n; ++kk)
-        for (int jj = 0; jj < n; ++jj) {
-          const double ljk = L[n + jj] * L[2 * n + kk];
-          double row[5] = {0, 0, 0, 0, 0};
-          for (int ii = 0; ii < n; ++ii) {
-            const size_t gs = (size_t)es * n3 + ii + n * (jj + n * kk);
-#pragma unroll
-            for (int v = 0; v < 5; ++v) row[v] += L[ii] * U[v * S + gs];
-          }
-#pragma unroll
-          for (int v = 0; v < 5; ++v) Us[v] += ljk * row[v];
-        }
-      const double gt0 = gFs[1] * s, gt1 = gFs[2] * s, gt2 = gFs[3] * s, gt4 = -gFs[4] * s;
-      bool ok = true;
-#pragma unroll 1
-      for (int k = 0; k < 7; ++k) {
-        DualD Ud[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) Ud[v] = DualD(Us[v], k == v ? 1.0 : 0.0);
-        DualD tau[3], qwd;
-        bool okk;
-        wall_stress_jvp(ph, Ud, k == 5 ? 1.0 : 0.0, k == 6 ? 1.0 : 0.0, nx, ny, nz, tau, &okk, &qwd);
-        ok = ok && okk;
-        // (the wall flux: Fs_mom += tau s, Fs_E -= q_w s)
-        const double gdot = tau[0].d * gt0 + tau[1].d * gt1 + tau[2].d * gt2 + qwd.d * gt4;
-        if (k < 5) gUs[slot * 5 + k] = gdot;
-        else if (k == 5) gk = gdot;
-        else gb = gdot;
-      }
-      if (!ok) atomicOr(status, ST_WM_NOCONV);
-    } else {
+  }
+  if (!ph.viscous) {
+    if (w == 0 && valid) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) gUs[slot * 5 + v] = 0.0;
     }
+    return;
   }
-  // block reduction of the two parameter cotangents
-  if (gtheta) {
+  // wall model: Fs_mom += tau s
+  {
+    double Us[5];
+    sample_planes<N, W>(U, S, chk_idx(m.ws_elem[slot], m.K, m.status), m.ws_lag + slot * 3 * n, w, Us);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      gk += __shfl_down_sync(0xffffffffu, gk, o);
-      gb += __shfl_down_sync(0xffffffffu, gb, o);
-    }
-    if ((threadIdx.x & 31) == 0 && (gk != 0.0 || gb != 0.0)) {
-      atomicAdd(&gtheta[0], gk);
-      atomicAdd(&gtheta[1], gb);
-    }
+    for (int v = 0; v < 5; ++v) sUs[w][v][lane] = Us[v];
+  }
+  __syncthreads();
+  double Us[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    Us[v] = sUs[0][v][lane];
+#pragma unroll
+    for (int x = 1; x < W; ++x) Us[v] += sUs[x][v][lane];
+  }
+  // direction w: d U_s,w (w < 5), d kappa (5), d B (6)
+  DualD Ud[5], tau[3], qwd;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) Ud[v] = DualD(Us[v], w == v ? 1.0 : 0.0);
+  const double dk = w == 5 ? 1.0 : 0.0, dB = w == 6 ? 1.0 : 0.0;
+  WallSolve sv{false};
+  if (w == 0) {
+    wall_stress_jvp(ph, Ud, dk, dB, nx, ny, nz, tau, &sv, &qwd);
+    sv.have = true;
+    sSv[lane] = sv;
+    if (!sv.ok && valid) atomicOr(status, ST_WM_NOCONV);
+  }
+  __syncthreads();
+  if (w > 6) return;
+  if (w > 0) {
+    sv = sSv[lane];
+    wall_stress_jvp(ph, Ud, dk, dB, nx, ny, nz, tau, &sv, &qwd);
+  }
+  // (the wall flux: Fs_mom += tau s, Fs_E -= q_w s)
+  double gdot = (tau[0].d * gFs[1] + tau[1].d * gFs[2] + tau[2].d * gFs[3] - qwd.d * gFs[4]) * s;
+  if (w < 5) {
+    if (valid) gUs[slot * 5 + w] = gdot;
+  } else if (gtheta) {
+    // the warp's sum of a parameter's cotangent
+    gdot = valid ? gdot : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) gdot += __shfl_down_sync(0xffffffffu, gdot, o);
+    if (lane == 0 && gdot != 0.0) atomicAdd(&gtheta[w - 5], gdot);
   }
 }
 
@@ -1238,29 +1257,42 @@ k_adj_gather(const double* __restrict__ U, const MeshDev<double> m, const PhysDe
 }
 
 // ---------------------------------------------------------------------------
-// k_adj_scatter: wall-model sample cotangents to the sample element's nodes.
+// k_adj_scatter: wall-model sample cotangents to the sample elements' nodes,
+// one block per wall face.  A face's nodes sample one element or a few: for
+// each, a thread adds up its node's share of all of them and gives it to gU by
+// one atomic addition (one per wall node and sample-element node before, 86 us
+// on the 12 x 6 x 8 channel at N = 5).
 // ---------------------------------------------------------------------------
 template <int N>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(256)
 k_adj_scatter(const MeshDev<double> m, const double* __restrict__ gUs, double* __restrict__ gU) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
-  const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= m.n_wall * n2) return;
-  const size_t S = (size_t)m.K * n3;
-  const int es = chk_idx(m.ws_elem[slot], m.K, m.status);
-  const double* L = m.ws_lag + (size_t)slot * 3 * n;
-  double gs[5];
+  __shared__ double sL[n2][3 * n], sG[n2][5];
+  __shared__ int sE[n2];
+  const size_t S = (size_t)m.K * n3, slot0 = (size_t)blockIdx.x * n2;
+  for (int x = threadIdx.x; x < n2 * 3 * n; x += blockDim.x) (&sL[0][0])[x] = m.ws_lag[slot0 * 3 * n + x];
+  for (int x = threadIdx.x; x < n2 * 5; x += blockDim.x) (&sG[0][0])[x] = gUs[slot0 * 5 + x];
+  for (int x = threadIdx.x; x < n2; x += blockDim.x) sE[x] = chk_idx(m.ws_elem[slot0 + x], m.K, m.status);
+  __syncthreads();
+  for (int q0 = 0; q0 < n2; ++q0) {
+    const int es = sE[q0];
+    bool first = true;  // the first node that samples es takes all that do
+    for (int x = 0; x < q0; ++x) first = first && sE[x] != es;
+    if (!first) continue;
+    for (int p = threadIdx.x; p < n3; p += blockDim.x) {
+      const int i = p % n, j = (p / n) % n, k = p / n2;
+      double g[5] = {0, 0, 0, 0, 0};
+      for (int x = q0; x < n2; ++x) {
+        if (sE[x] != es) continue;
+        const double wgt = sL[x][i] * sL[x][n + j] * sL[x][2 * n + k];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) gs[v] = gUs[(size_t)slot * 5 + v];
-  if (gs[0] == 0.0 && gs[1] == 0.0 && gs[2] == 0.0 && gs[3] == 0.0 && gs[4] == 0.0) return;
-  for (int kk = 0; kk < n; ++kk)
-    for (int jj = 0; jj < n; ++jj)
-      for (int ii = 0; ii < n; ++ii) {
-        const double wgt = L[ii] * L[n + jj] * L[2 * n + kk];
-        const size_t gn = (size_t)es * n3 + ii + n * (jj + n * kk);
-#pragma unroll
-        for (int v = 0; v < 5; ++v) atomicAdd(&gU[v * S + gn], wgt * gs[v]);
+        for (int v = 0; v < 5; ++v) g[v] = fma(wgt, sG[x][v], g[v]);
       }
+#pragma unroll
+      for (int v = 0; v < 5; ++v)
+        if (g[v] != 0.0) atomicAdd(&gU[v * S + (size_t)es * n3 + p], g[v]);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1299,7 +1331,7 @@ k_wall_loss(const double* __restrict__ U, const MeshDev<double> m, const PhysDev
         for (int v = 0; v < 5; ++v) Us[v] += ljk * row[v];
       }
     const double wgt = wq[slot] * inv_total;
-    bool ok = true;
+    WallSolve sv{false};
     const int seeds = grad ? 7 : 1;
 #pragma unroll 1
     for (int k = 0; k < seeds; ++k) {
@@ -1307,9 +1339,7 @@ k_wall_loss(const double* __restrict__ U, const MeshDev<double> m, const PhysDev
 #pragma unroll
       for (int v = 0; v < 5; ++v) Ud[v] = DualD(Us[v], grad && k == v ? 1.0 : 0.0);
       DualD tau[3];
-      bool okk;
-      wall_stress_jvp(ph, Ud, grad && k == 5 ? 1.0 : 0.0, grad && k == 6 ? 1.0 : 0.0, nx, ny, nz, tau, &okk);
-      ok = ok && okk;
+      wall_stress_jvp(ph, Ud, grad && k == 5 ? 1.0 : 0.0, grad && k == 6 ? 1.0 : 0.0, nx, ny, nz, tau, &sv);
       if (k == 0) lv = wgt * tau[0].v;
       if (grad) {
         if (k < 5) gUs[(size_t)slot * 5 + k] = wgt * tau[0].d;
@@ -1317,7 +1347,7 @@ k_wall_loss(const double* __restrict__ U, const MeshDev<double> m, const PhysDev
         else gb = wgt * tau[0].d;
       }
     }
-    if (!ok) atomicOr(status, ST_WM_NOCONV);
+    if (!sv.ok) atomicOr(status, ST_WM_NOCONV);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

@@ -959,8 +959,8 @@ __device__ __forceinline__ void law_eval(int law, double w, double kap, double B
 // steps from the laminar estimate t = ln(Re_h)/2, then Newton with bisection
 // whenever a step would leave the bracket.  Returns u_tau (and *ok).  F is
 // increasing in t; its value at the starting point is evaluated once.
-static __device__ double solve_utau(int law, double u, double h, double nu, double kap, double B, int maxit,
-                                    bool* ok) {
+static __device__ double solve_utau_bracket(int law, double u, double h, double nu, double kap, double B, int maxit,
+                                            bool* ok) {
   *ok = true;
   if (!(u > 0.0)) return 0.0;
   const double lnRe = log(h * u / nu);
@@ -1001,15 +1001,24 @@ static __device__ double solve_utau(int law, double u, double h, double nu, doub
   return law == 1 ? exp(t) * nu / h : u / exp(t);
 }
 
-// Warm-started solve: up to four Newton steps from t_prev (the node's solution
-// at its previous evaluation, NaN if none), stopping by the same rule as the
-// bracketed solve; if they do not converge, the bracketed solve from scratch.
-// *t_out receives the converged t.  The state changes little between stages, so
-// one or two evaluations of F usually suffice instead of about eight.
+static __device__ float solve_utau_f(int law, float u, float h, float nu, float kap, float B, int maxit, bool* ok);
+
+// Started solve: up to four Newton steps from t_prev (the node's solution at
+// its previous evaluation), or from the FP32 solution when there is none (NaN),
+// stopping by the same rule as the bracketed solve; if they do not converge,
+// the bracketed solve from scratch.  The state changes little between stages
+// and the FP32 solution is good to 1e-6, so two evaluations of F usually
+// suffice instead of about eight (an evaluation is some 170 FP64 operations,
+// the solve a serial chain).  *t_out receives the converged t.
 static __device__ double solve_utau_warm(int law, double u, double h, double nu, double kap, double B, int maxit,
                                          double t_prev, double* t_out, bool* ok) {
   *ok = true;
   if (!(u > 0.0)) { *t_out = t_prev; return 0.0; }
+  if (!(t_prev == t_prev)) {
+    bool okf;
+    const float utf = solve_utau_f(law, (float)u, (float)h, (float)nu, (float)kap, (float)B, maxit, &okf);
+    if (okf) t_prev = law == 1 ? logf(utf * (float)h / (float)nu) : logf((float)u / utf);
+  }
   if (t_prev == t_prev && fabs(t_prev) < 1e3) {
     const double lnRe = log(h * u / nu);
     const double cst = law_const(law, kap, B);
@@ -1028,9 +1037,13 @@ static __device__ double solve_utau_warm(int law, double u, double h, double nu,
       if (step <= 1e-12 * fmax(1.0, fabs(t))) { *t_out = t; return law == 1 ? exp(t) * nu / h : u / exp(t); }
     }
   }
-  const double ut = solve_utau(law, u, h, nu, kap, B, maxit, ok);
+  const double ut = solve_utau_bracket(law, u, h, nu, kap, B, maxit, ok);
   *t_out = law == 1 ? log(ut * h / nu) : log(u / ut);
   return ut;
+}
+static __device__ double solve_utau(int law, double u, double h, double nu, double kap, double B, int maxit, bool* ok) {
+  double t;
+  return solve_utau_warm(law, u, h, nu, kap, B, maxit, __longlong_as_double(-1LL), &t, ok);  // (NaN: no start)
 }
 
 // FP32 form of the wall model for the FP32-mixed kernels: the same steps in
@@ -1940,68 +1953,105 @@ k_bc(const double* __restrict__ U, const MeshDev<R> m, const PhysDev ph, const R
 }
 
 // ---------------------------------------------------------------------------
-// k_wall: one thread per node of a wall face (slip wall + wall model).
-// The work per node is long (sample interpolation over n^3 nodes, Newton
-// iterations of transcendental functions) and the nodes are few, so blocks
-// are one warp: the launch spreads over all SMs instead of filling a few.
+// k_wall: nodes of the wall faces (slip wall + wall model), 32 per block of
+// WALL_WARPS warps, a node per lane.  The work per node is a long serial chain
+// (sample interpolation over n^3 nodes, Newton iterations of transcendental
+// functions) and the nodes are few, so a node's chain is cut: the warps share
+// the planes of its interpolation, the last one also takes the mirror state's
+// Riemann flux, the first the law-of-the-wall solve.
 // ---------------------------------------------------------------------------
 constexpr int WALL_THREADS = 32;
+constexpr int WALL_WARPS = 4;
+
+// the planes kk = w, w + W, .. of a wall node's sample state at h_wm: tensor-
+// product Lagrange interpolation of U
+template <int N, int W>
+__device__ __forceinline__ void sample_planes(const double* __restrict__ U, size_t S, int es,
+                                              const double* __restrict__ L, int w, double Us[5]) {
+  constexpr int n = N + 1, n3 = n * n * n;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) Us[v] = 0.0;
+  for (int kk = w; kk < n; kk += W)
+    for (int jj = 0; jj < n; ++jj) {
+      const double ljk = L[n + jj] * L[2 * n + kk];
+      double row[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+      for (int ii = 0; ii < n; ++ii) {
+        const size_t gs = (size_t)es * n3 + ii + n * (jj + n * kk);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) row[v] += L[ii] * U[v * S + gs];
+      }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) Us[v] += ljk * row[v];
+    }
+}
 
 template <int N, typename R>
-__global__ void __launch_bounds__(WALL_THREADS)
+__global__ void __launch_bounds__(32 * WALL_WARPS)
 k_wall(const double* __restrict__ U, const MeshDev<R> m, const PhysDev ph, R* __restrict__ Fs,
        double* __restrict__ tau_out, int* __restrict__ status) {
-  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int wf = tid / n2, ab = tid - wf * n2;
-  if (wf >= m.n_wall) return;
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, W = WALL_WARPS;
+  constexpr bool F32 = std::is_same<R, float>::value;
+  __shared__ R sUs[W][5][32];  // the warps' shares of the sample state
+  __shared__ R sF[5][32];      // inviscid flux
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int tid = blockIdx.x * 32 + lane;
+  const bool valid = tid < m.n_wall * n2;
+  const int wf = valid ? tid / n2 : 0, ab = valid ? tid - wf * n2 : 0;
   const int f = m.n_interior + wf;
-  int4 fc = m.faces[f];
-  fc.x = chk_idx(fc.x, m.K, m.status);
+  const size_t slot = (size_t)wf * n2 + ab;
   const size_t S = (size_t)m.K * n3;
-  const size_t gM = (size_t)fc.x * n3 + fnode<N>(fc.y, ab % n, ab / n);
   const size_t FN = (size_t)m.F * n2, fg = (size_t)f * n2 + ab;
   const double nxd = m.fgeo[fg], nyd = m.fgeo[FN + fg], nzd = m.fgeo[2 * FN + fg], sd = m.fgeo[3 * FN + fg];
-  double UA[5], UB[5];
+  const bool dif = F32 && ph.fs_diff;
+  if (w == W - 1) {
+    int4 fc = m.faces[f];
+    fc.x = chk_idx(fc.x, m.K, m.status);
+    const size_t gM = (size_t)fc.x * n3 + fnode<N>(fc.y, ab % n, ab / n);
+    double UA[5], UB[5];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) UA[v] = U[v * S + gM];
-  const double mn = UA[1] * nxd + UA[2] * nyd + UA[3] * nzd;
-  UB[0] = UA[0]; UB[1] = UA[1] - 2.0 * mn * nxd; UB[2] = UA[2] - 2.0 * mn * nyd;
-  UB[3] = UA[3] - 2.0 * mn * nzd; UB[4] = UA[4];
-  Prim<R> As, Bs;  // FP32: the storage form, for the flux-difference form
-  Lo3 la, lb;
-  const Prim<R> A = trace_prims<R>(UA, ph, &As, &la), B = trace_prims<R>(UB, ph, &Bs, &lb);
-  R F[5];
-  int fss = 5;  // surface-flux values per face node (10: FP32 difference form)
-  if constexpr (std::is_same<R, float>::value) {
-    if (ph.fs_diff) {
-      float dU[5], DB[5];
+    for (int v = 0; v < 5; ++v) UA[v] = U[v * S + gM];
+    const double mn = UA[1] * nxd + UA[2] * nyd + UA[3] * nzd;
+    UB[0] = UA[0]; UB[1] = UA[1] - 2.0 * mn * nxd; UB[2] = UA[2] - 2.0 * mn * nyd;
+    UB[3] = UA[3] - 2.0 * mn * nzd; UB[4] = UA[4];
+    Prim<R> As, Bs;  // FP32: the storage form, for the flux-difference form
+    Lo3 la, lb;
+    const Prim<R> A = trace_prims<R>(UA, ph, &As, &la), B = trace_prims<R>(UB, ph, &Bs, &lb);
+    R F[5];
+    if constexpr (F32) {
+      if (dif) {
+        float dU[5], DB[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) dU[v] = d2f_bits(UB[v] - UA[v]);
-      face_flux_delta(ph, As, Bs, la, lb, dU, (R)nxd, (R)nyd, (R)nzd, F, DB);
-      fss = 10;
+        for (int v = 0; v < 5; ++v) dU[v] = d2f_bits(UB[v] - UA[v]);
+        face_flux_delta(ph, As, Bs, la, lb, dU, (R)nxd, (R)nyd, (R)nzd, F, DB);
+      }
     }
+    if (!dif) riemann<R, double>(ph, A, UA, B, UB, (R)nxd, (R)nyd, (R)nzd, F);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) sF[v][lane] = F[v];
   }
-  if (fss == 5) riemann<R, double>(ph, A, UA, B, UB, (R)nxd, (R)nyd, (R)nzd, F);
-  double tau[3] = {0.0, 0.0, 0.0}, qw = 0.0;
-  if constexpr (std::is_same<R, float>::value) {
-    if (ph.viscous) {
+  if (ph.viscous) {
+    const int es = chk_idx(m.ws_elem[slot], m.K, m.status);
+    if constexpr (F32) {
       // FP32 form: interpolation of the conservative state formed from the
       // stage's FP32 primitives, with the energy taken relative to
       // p_ref / (gamma - 1) (the interpolation weights sum to one), then the
       // FP32 wall model
-      const size_t slot = (size_t)wf * n2 + ab;
-      const int es = chk_idx(m.ws_elem[slot], m.K, m.status);
       const double* Ld = m.ws_lag + slot * 3 * n;
       float L[3 * n];
 #pragma unroll
       for (int x = 0; x < 3 * n; ++x) L[x] = (float)Ld[x];
       const float rg = ph.f32c.rgm1;
       float Us[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-      for (int kk = 0; kk < n; ++kk)
+#pragma unroll
+      for (int kk = 0; kk < n; ++kk) {
+        if (kk % W != w) continue;
         for (int jj = 0; jj < n; ++jj) {
-          const float ljk = L[n + jj] * L[2 * n + kk];
+          float ljk = 0.f;
+#pragma unroll
+          for (int x = 0; x < n; ++x) ljk = x == jj ? L[n + x] * L[2 * n + kk] : ljk;
           float row[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
           for (int ii = 0; ii < n; ++ii) {
             const Prim<float> q = load_prim32_full(m.W32, S, (size_t)es * n3 + ii + n * (jj + n * kk), ph);
             const float li = L[ii];
@@ -2014,39 +2064,37 @@ k_wall(const double* __restrict__ U, const MeshDev<R> m, const PhysDev ph, R* __
 #pragma unroll
           for (int v = 0; v < 5; ++v) Us[v] += ljk * row[v];
         }
+      }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sUs[w][v][lane] = Us[v];
+    } else {
+      double Us[5];
+      sample_planes<N, W>(U, S, es, m.ws_lag + slot * 3 * n, w, Us);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sUs[w][v][lane] = Us[v];
+    }
+  }
+  __syncthreads();
+  if (w != 0 || !valid) return;
+  double tau[3] = {0.0, 0.0, 0.0}, qw = 0.0;
+  if (ph.viscous) {
+    R Us[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      Us[v] = sUs[0][v][lane];
+#pragma unroll
+      for (int x = 1; x < W; ++x) Us[v] += sUs[x][v][lane];
+    }
+    bool ok;
+    if constexpr (F32) {
       const float ir = 1.0f / Us[0];
-      const float u = Us[1] * ir, v = Us[2] * ir, w = Us[3] * ir;
-      const float pp = (float)ph.gm1 * (Us[4] - 0.5f * Us[0] * (u * u + v * v + w * w));  // p - p_ref
+      const float u = Us[1] * ir, v = Us[2] * ir, ww = Us[3] * ir;
+      const float pp = (float)ph.gm1 * (Us[4] - 0.5f * Us[0] * (u * u + v * v + ww * ww));  // p - p_ref
       const float Ts = (pp + ph.f32c.p_ref) * ph.f32c.rcp_R * ir;
       float tf[3], qf;
-      bool ok;
-      wall_stress_f(ph, Us[0], u, v, w, Ts, (float)nxd, (float)nyd, (float)nzd, tf, &qf, &ok);
-      if (!ok) atomicOr(status, ST_WM_NOCONV);
+      wall_stress_f(ph, Us[0], u, v, ww, Ts, (float)nxd, (float)nyd, (float)nzd, tf, &qf, &ok);
       tau[0] = tf[0]; tau[1] = tf[1]; tau[2] = tf[2]; qw = qf;
-      if (tau_out) {
-        tau_out[slot * 3 + 0] = tau[0]; tau_out[slot * 3 + 1] = tau[1]; tau_out[slot * 3 + 2] = tau[2];
-      }
-    }
-  } else if (ph.viscous) {
-    // sample state at h_wm: tensor-product Lagrange interpolation of U
-    const size_t slot = (size_t)wf * n2 + ab;
-    const int es = chk_idx(m.ws_elem[slot], m.K, m.status);
-    const double* L = m.ws_lag + slot * 3 * n;
-    double Us[5] = {0, 0, 0, 0, 0};
-    for (int kk = 0; kk < n; ++kk)
-      for (int jj = 0; jj < n; ++jj) {
-        const double ljk = L[n + jj] * L[2 * n + kk];
-        double row[5] = {0, 0, 0, 0, 0};
-        for (int ii = 0; ii < n; ++ii) {
-          const size_t gs = (size_t)es * n3 + ii + n * (jj + n * kk);
-#pragma unroll
-          for (int v = 0; v < 5; ++v) row[v] += L[ii] * U[v * S + gs];
-        }
-#pragma unroll
-        for (int v = 0; v < 5; ++v) Us[v] += ljk * row[v];
-      }
-    bool ok;
-    if (m.wm_t) {
+    } else if (m.wm_t) {
       double tw = m.wm_t[slot];
       wall_stress(ph, Us, nxd, nyd, nzd, tau, &qw, &ok, &tw);
       m.wm_t[slot] = tw;
@@ -2059,13 +2107,13 @@ k_wall(const double* __restrict__ U, const MeshDev<R> m, const PhysDev ph, R* __
     }
   }
   // viscous wall flux Fv . n = (0, -tau_w t, 0): the wall decelerates the flow
-  R* out = Fs + (size_t)f * fss * n2 + ab;
+  R* out = Fs + (size_t)f * (dif ? 10 : 5) * n2 + ab;
   const R s = (R)sd;
-  out[0] = F[0] * s;
-  out[n2] = F[1] * s + (R)(tau[0] * sd);
-  out[2 * n2] = F[2] * s + (R)(tau[1] * sd);
-  out[3 * n2] = F[3] * s + (R)(tau[2] * sd);
-  out[4 * n2] = F[4] * s - (R)(qw * sd);  // viscous energy flux along the outward normal: q_w
+  out[0] = sF[0][lane] * s;
+  out[n2] = sF[1][lane] * s + (R)(tau[0] * sd);
+  out[2 * n2] = sF[2][lane] * s + (R)(tau[1] * sd);
+  out[3 * n2] = sF[3][lane] * s + (R)(tau[2] * sd);
+  out[4 * n2] = sF[4][lane] * s - (R)(qw * sd);  // viscous energy flux along the outward normal: q_w
 }
 
 // ---------------------------------------------------------------------------

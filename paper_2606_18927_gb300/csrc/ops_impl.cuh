@@ -182,9 +182,7 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   const cudaStream_t ws = fork ? a.side : s;
   auto wall = [&]() {
     if (a.n_wall == 0) return;
-    const int threads = WALL_THREADS;
-    const long long work = (long long)a.n_wall * n2;
-    k_wall<N, R><<<(unsigned)((work + threads - 1) / threads), threads, 0, ws>>>(a.Uin, m, ph, Fs, a.tau, a.status);
+    k_wall<N, R><<<spread_blocks((long long)a.n_wall * n2, 32), 32 * WALL_WARPS, 0, ws>>>(a.Uin, m, ph, Fs, a.tau, a.status);
   };
   if (phase & 2) {
     // the FP32 primitives first: the FP32 wall kernel reads them
@@ -323,8 +321,7 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
       k_adj_face<N><<<spread_blocks(work, threads), threads, 0, s>>>(a.Uin, a.lam, m, ph, iw, a.gUf, a.gGf, sendU,
                                                                    sendG);
     if (a.n_wall > 0) {
-      const long long ww = (long long)a.n_wall * n2;
-      k_adj_wall<N><<<(unsigned)((ww + WALL_THREADS - 1) / WALL_THREADS), WALL_THREADS, 0, s>>>(
+      k_adj_wall<N><<<spread_blocks((long long)a.n_wall * n2, 32), 32 * ADJ_WALL_WARPS, 0, s>>>(
           a.Uin, a.lam, m, ph, iw, a.gUf, a.gGf, a.gUs, a.gtheta, a.status);
     }
     if (a.n_bc > 0) {
@@ -343,8 +340,7 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     k_adj_gather<N><<<spread_blocks(S, threads), threads, 0, s>>>(a.Uin, m, ph, a.gUf, a.gWf,
                                                                  part ? a.halo_U : nullptr, a.gU);
     if (a.n_wall > 0 && ph.viscous) {
-      const long long work = (long long)a.n_wall * n2;
-      k_adj_scatter<N><<<(unsigned)((work + 127) / 128), 128, 0, s>>>(m, a.gUs, a.gU);
+      k_adj_scatter<N><<<(unsigned)a.n_wall, std::min(256, (n3 + 31) / 32 * 32), 0, s>>>(m, a.gUs, a.gU);
     }
   }
   return (int)cudaGetLastError();
@@ -367,7 +363,7 @@ static int run_wall_loss_typed(const OpArgs& a, const PhysDev& ph, const double*
   if (grad) {
     const long long S = 5LL * a.K * n3;
     k_axpby<<<(unsigned)((S + 255) / 256), 256, 0, s>>>(S, 0.0, a.gU, 0.0, a.gU);
-    k_adj_scatter<N><<<(unsigned)((work + 127) / 128), 128, 0, s>>>(m, a.gUs, a.gU);
+    k_adj_scatter<N><<<(unsigned)a.n_wall, std::min(256, (n3 + 31) / 32 * 32), 0, s>>>(m, a.gUs, a.gU);
   }
   return (int)cudaGetLastError();
 }
