@@ -11,9 +11,11 @@
 //                wall-model derivative (forward-mode duals over the sample
 //                state; implicit function theorem for the law of the wall)
 //                with respect to the sample state and (kappa, B);
-//   k_adj_element one CTA per element: transposed split-form volume integral
-//                (hand-derived, symmetric pairs with shuffles), transposed
-//                viscous divergence and viscous flux, transposed BR1 lifting,
+//   k_adj_volume (adjoint_fx.cuh) one CTA per element: the KEP flux's
+//                transposed split-form volume integral in fixed point;
+//   k_adj_element one CTA per element: with the entropy-conserving flux its
+//                transposed volume integral (hand-derived, symmetric pairs
+//                with shuffles), transposed viscous divergence and viscous flux, transposed BR1 lifting,
 //                transposed primitive recovery, source term;
 //   k_adj_gather  adds the per-face contributions of the face kernels and of
 //                the neighbours' lifting to every node;
@@ -165,6 +167,14 @@ __device__ __forceinline__ void prim_vjp(const double U[5], const PhysDev& ph, c
   gU[2] += gQ[2] * ir - gp * g1 * v - gh * g1 * v * ir;
   gU[3] += gQ[3] * ir - gp * g1 * w - gh * g1 * w * ir;
   gU[4] += gp * g1 + gh * (1.0 + g1) * ir;
+}
+
+// the body force's source S_E = f . m / rho: gU += (dS/dU)^T lam
+__device__ __forceinline__ void source_vjp(const double U[5], const PhysDev& ph, double l4, double gU[5]) {
+  if (ph.f[0] == 0.0 && ph.f[1] == 0.0 && ph.f[2] == 0.0) return;
+  const double ir = 1.0 / U[0];
+  gU[0] -= l4 * (ph.f[0] * U[1] + ph.f[1] * U[2] + ph.f[2] * U[3]) * ir * ir;
+  gU[1] += l4 * ph.f[0] * ir; gU[2] += l4 * ph.f[1] * ir; gU[3] += l4 * ph.f[2] * ir;
 }
 
 // W = (u, v, w, T): gU += (dW/dU)^T gW
@@ -694,6 +704,136 @@ struct AdjShape {
   static constexpr int SMEM_D = 36 * n3 + 24 * n2 + 3 * n2 + n;
 };
 
+// The transposed split-form volume integral in FP64 (symmetric pairs): adds
+// up the cotangents sGQ [6][n3] of (rho, u, v, w, p', h) from the primitives sQ
+// [6][n3] and the scaled cotangents sL [5][n3] (lam~ = -lam / J); sLt [5][n3] is
+// scratch, sDVS [n2] w_a DVS_ab, siw [n] 1 / w.  metrics(dir, node, active)
+// gives Ja^dir [3][n3], readable after the next barrier.
+template <int N, bool EC, class M>
+__device__ __forceinline__ void adj_pairs_fp64(const double* sQ, const double* sL, double* sLt, double* sGQ,
+                                               const double* sDVS, const double* siw, const PhysDev& ph, int t,
+                                               M metrics) {
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, LPW = VolShape<N>::LPW;
+  const int warp = t >> 5, lane = t & 31;
+  const int seg = lane / n, pos = lane - seg * n;
+  const int L0 = warp * LPW + seg;
+  const bool active = (seg < LPW) && (L0 < n2);
+  const int L = active ? L0 : 0;
+  const int base = seg * n;
+  // The pair terms are linear in the combined cotangent
+  //   mu = DVS_im lam~_i + DVS_mi lam~_m = w_i DVS_im (lam~_i / w_i - lam~_m / w_m)
+  // (w_i DVS_im = -w_m DVS_mi off the diagonal, the SBP property), so each
+  // pass first stores lam~ / w along its direction and a pair forms the
+  // difference; the factor w_i DVS_im (table sDVS) scales its terms as they
+  // are summed, for the partner lane's pair w_m DVS_mi.
+#pragma unroll 1
+  for (int dir = 0; dir < 3; ++dir) {
+    const int a = L % n, b = L / n;
+    auto node = [&](int q) {
+      return dir == 0 ? q + n * L : (dir == 1 ? a + n * q + n2 * b : L + n2 * q);
+    };
+    const int me = node(pos);
+    if (active) {
+      const double iwp = siw[pos];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sLt[v * n3 + me] = sL[v * n3 + me] * iwp;
+    }
+    const double* sAd = metrics(dir, me, active);
+    __syncthreads();
+    // the pair terms below carry constant factors (1/8 for rho, u, v, w,
+    // 1/4 for p, 1/16 for h) that are applied once per node after the sums
+    double g0 = 0, g1 = 0, g2 = 0, g3 = 0, g4 = 0, g5 = 0;
+    if constexpr (EC) {
+      // entropy-conserving flux: the two nodes of a pair get different
+      // cotangents (the logarithmic means are symmetric, their partial
+      // derivatives are not); the lane keeps its node's share and hands the
+      // partner's share (pos + d) over by a shuffle
+#pragma unroll 1
+      for (int d = 1; d <= n / 2; ++d) {
+        const int pm = pos + d < n ? pos + d : pos + d - n;
+        const int q = node(pm);
+        const Prim<double> Pa{sQ[me], sQ[n3 + me], sQ[2 * n3 + me], sQ[3 * n3 + me], sQ[4 * n3 + me], 0.0};
+        const Prim<double> Pb{sQ[q], sQ[n3 + q], sQ[2 * n3 + q], sQ[3 * n3 + q], sQ[4 * n3 + q], 0.0};
+        const double a0 = 0.5 * (sAd[0 * n3 + me] + sAd[0 * n3 + q]);
+        const double a1 = 0.5 * (sAd[1 * n3 + me] + sAd[1 * n3 + q]);
+        const double a2 = 0.5 * (sAd[2 * n3 + me] + sAd[2 * n3 + q]);
+        double mu[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) mu[v] = sLt[v * n3 + me] - sLt[v * n3 + q];
+        double gA[5] = {0, 0, 0, 0, 0}, gB[5] = {0, 0, 0, 0, 0};
+        ec_flux_vjp(ph, Pa, Pb, a0, a1, a2, mu, gA, gB);
+        const double cw = sDVS[pos * n + pm];
+        g0 = fma(cw, gA[0], g0); g1 = fma(cw, gA[1], g1); g2 = fma(cw, gA[2], g2);
+        g3 = fma(cw, gA[3], g3); g4 = fma(cw, gA[4], g4);
+        if (2 * d != n) {
+          const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
+          const double cs = sDVS[(src - base) * n + pos];
+          g0 = fma(cs, __shfl_sync(0xffffffffu, gB[0], src), g0);
+          g1 = fma(cs, __shfl_sync(0xffffffffu, gB[1], src), g1);
+          g2 = fma(cs, __shfl_sync(0xffffffffu, gB[2], src), g2);
+          g3 = fma(cs, __shfl_sync(0xffffffffu, gB[3], src), g3);
+          g4 = fma(cs, __shfl_sync(0xffffffffu, gB[4], src), g4);
+        }
+      }
+    } else {
+#pragma unroll
+    for (int d = 1; d <= n / 2; ++d) {
+      const int pm = pos + d < n ? pos + d : pos + d - n;
+      const int q = node(pm);
+      // sums of the two nodes' values: {x} = Sx / 2
+      const double Sr = sQ[me] + sQ[q];
+      const double Su = sQ[n3 + me] + sQ[n3 + q], Sv = sQ[2 * n3 + me] + sQ[2 * n3 + q],
+                   Sw = sQ[3 * n3 + me] + sQ[3 * n3 + q];
+      const double Sh = sQ[5 * n3 + me] + sQ[5 * n3 + q];
+      const double Sa0 = sAd[0 * n3 + me] + sAd[0 * n3 + q];
+      const double Sa1 = sAd[1 * n3 + me] + sAd[1 * n3 + q];
+      const double Sa2 = sAd[2 * n3 + me] + sAd[2 * n3 + q];
+      double mu[5];  // mu / (w_i DVS_im)
+#pragma unroll
+      for (int v = 0; v < 5; ++v) mu[v] = sLt[v * n3 + me] - sLt[v * n3 + q];
+      // F0 = {rho} qa, Fk = {rho} qa {u_k} + {p} {a_k}, F4 = {rho} qa {h}, qa = {u}.{a} = Q / 4;
+      // tt = mu . dF/d({rho} qa) = mu0 + (mu1 Su + mu2 Sv + mu3 Sw + mu4 Sh) / 2;
+      // half of each average's cotangent goes to each node:
+      //   g_rho = Q tt / 8, g_u_k = Sr (tt Sa_k + Q mu_k / 2) / 8, g_p = (mu . Sa) / 4,
+      //   g_h = Sr Q mu4 / 16
+      const double Q = Su * Sa0 + Sv * Sa1 + Sw * Sa2;
+      const double tt = fma(0.5, mu[1] * Su + mu[2] * Sv + mu[3] * Sw + mu[4] * Sh, mu[0]);
+      const double hQ = 0.5 * Q;
+      const double h0 = Q * tt;
+      const double h1 = Sr * fma(tt, Sa0, hQ * mu[1]);
+      const double h2 = Sr * fma(tt, Sa1, hQ * mu[2]);
+      const double h3 = Sr * fma(tt, Sa2, hQ * mu[3]);
+      const double h4 = mu[1] * Sa0 + mu[2] * Sa1 + mu[3] * Sa2;
+      const double h5 = Sr * Q * mu[4];
+      const double cw = sDVS[pos * n + pm];
+      g0 = fma(cw, h0, g0); g1 = fma(cw, h1, g1); g2 = fma(cw, h2, g2);
+      g3 = fma(cw, h3, g3); g4 = fma(cw, h4, g4); g5 = fma(cw, h5, g5);
+      if (2 * d != n) {
+        const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
+        const double cs = sDVS[(src - base) * n + pos];
+        g0 = fma(cs, __shfl_sync(0xffffffffu, h0, src), g0);
+        g1 = fma(cs, __shfl_sync(0xffffffffu, h1, src), g1);
+        g2 = fma(cs, __shfl_sync(0xffffffffu, h2, src), g2);
+        g3 = fma(cs, __shfl_sync(0xffffffffu, h3, src), g3);
+        g4 = fma(cs, __shfl_sync(0xffffffffu, h4, src), g4);
+        g5 = fma(cs, __shfl_sync(0xffffffffu, h5, src), g5);
+      }
+    }
+    g0 *= 0.125; g1 *= 0.125; g2 *= 0.125; g3 *= 0.125; g4 *= 0.25; g5 *= 0.0625;
+    }  // Pirozzoli
+    if (active) {
+      if (dir == 0) {
+        sGQ[me] = g0; sGQ[n3 + me] = g1; sGQ[2 * n3 + me] = g2; sGQ[3 * n3 + me] = g3;
+        sGQ[4 * n3 + me] = g4; sGQ[5 * n3 + me] = g5;
+      } else {
+        sGQ[me] += g0; sGQ[n3 + me] += g1; sGQ[2 * n3 + me] += g2; sGQ[3 * n3 + me] += g3;
+        sGQ[4 * n3 + me] += g4; sGQ[5 * n3 + me] += g5;
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // EC: the entropy-conserving volume flux; SUTH: Sutherland's law (own
 // instantiations: the reverse mode of the entropy-conserving pair flux and
 // the temperature-dependent viscosity need registers that the Pirozzoli,
@@ -701,10 +841,10 @@ struct AdjShape {
 template <int N, bool EC, bool SUTH>
 __global__ void __launch_bounds__(AdjShape<N>::THREADS)
 k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, const MeshDev<double> m,
-              const PhysDev ph, const Tables<N> tab, const double* __restrict__ gGf, double* __restrict__ gU,
-              double* __restrict__ gWf, double* __restrict__ gHaloU) {
+              const PhysDev ph, const Tables<N> tab, const double* __restrict__ gGf, const double* __restrict__ gV,
+              double* __restrict__ gU, double* __restrict__ gWf, double* __restrict__ gHaloU) {
   using Sh = AdjShape<N>;
-  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS, LPW = VolShape<N>::LPW;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* sQ = reinterpret_cast<double*>(smem_raw);  // [6][n3] (pair phase)
   double* sH = sQ;                                     // [3][4][n3] (viscous phase, reuses Q)
@@ -723,7 +863,7 @@ k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, cons
   // lifting kernel): sD holds the tables of D and of D^T, sDv that of Dvisc^T
   constexpr bool EO = (n == 8) && (T == n3);
   for (int x = t; x < n2; x += T) {
-    sDVS[x] = 8.0 * tab.DVS8[x] / tab.iw[x / n];
+    if constexpr (EC) sDVS[x] = 8.0 * tab.DVS8[x] / tab.iw[x / n];
     if constexpr (EO) {
       if (x < n * (n / 2)) {
         sD[x] = LineEO<N>::coef(tab.D, x);
@@ -741,9 +881,11 @@ k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, cons
     double Uo[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) Uo[v] = U[v * S + g];
-    const Prim<double> q = primitive<double>(Uo[0], Uo[1], Uo[2], Uo[3], Uo[4], ph);
-    sQ[t] = q.rho; sQ[n3 + t] = q.u; sQ[2 * n3 + t] = q.v; sQ[3 * n3 + t] = q.w;
-    sQ[4 * n3 + t] = q.p; sQ[5 * n3 + t] = q.h;
+    if constexpr (EC) {
+      const Prim<double> q = primitive<double>(Uo[0], Uo[1], Uo[2], Uo[3], Uo[4], ph);
+      sQ[t] = q.rho; sQ[n3 + t] = q.u; sQ[2 * n3 + t] = q.v; sQ[3 * n3 + t] = q.w;
+      sQ[4 * n3 + t] = q.p; sQ[5 * n3 + t] = q.h;
+    }
     const double iJ = m.invJ[g];
 #pragma unroll
     for (int v = 0; v < 5; ++v) sL[v * n3 + t] = -lam[v * S + g] * iJ;
@@ -754,127 +896,11 @@ k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, cons
     sW[t] = uu; sW[n3 + t] = vv; sW[2 * n3 + t] = ww; sW[3 * n3 + t] = TT;
   }
   __syncthreads();
-  // ---- transposed split-form volume integral (symmetric pairs)
-  {
-    const int warp = t >> 5, lane = t & 31;
-    const int seg = lane / n, pos = lane - seg * n;
-    const int L0 = warp * LPW + seg;
-    const bool active = (seg < LPW) && (L0 < n2);
-    const int L = active ? L0 : 0;
-    const int base = seg * n;
-    // The pair terms are linear in the combined cotangent
-    //   mu = DVS_im lam~_i + DVS_mi lam~_m = w_i DVS_im (lam~_i / w_i - lam~_m / w_m)
-    // (w_i DVS_im = -w_m DVS_mi off the diagonal, the SBP property), so each
-    // pass first stores lam~ / w along its direction and a pair forms the
-    // difference; the factor w_i DVS_im (table sDVS) scales its terms as they
-    // are summed, for the partner lane's pair w_m DVS_mi.
-    double* sLt = sQ + 6 * n3;  // [5][n3] lam~ / w (the unused half of the Q slots)
-#pragma unroll 1
-    for (int dir = 0; dir < 3; ++dir) {
-      const int a = L % n, b = L / n;
-      auto node = [&](int q) {
-        return dir == 0 ? q + n * L : (dir == 1 ? a + n * q + n2 * b : L + n2 * q);
-      };
-      const int me = node(pos);
-      if (active) {
-        const double iwp = siw[pos];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) sLt[v * n3 + me] = sL[v * n3 + me] * iwp;
-      }
-      __syncthreads();
-      // the pair terms below carry constant factors (1/8 for rho, u, v, w,
-      // 1/4 for p, 1/16 for h) that are applied once per node after the sums
-      double g0 = 0, g1 = 0, g2 = 0, g3 = 0, g4 = 0, g5 = 0;
-      if constexpr (EC) {
-        // entropy-conserving flux: the two nodes of a pair get different
-        // cotangents (the logarithmic means are symmetric, their partial
-        // derivatives are not); the lane keeps its node's share and hands the
-        // partner's share (pos + d) over by a shuffle
-#pragma unroll 1
-        for (int d = 1; d <= n / 2; ++d) {
-          const int pm = pos + d < n ? pos + d : pos + d - n;
-          const int q = node(pm);
-          const Prim<double> Pa{sQ[me], sQ[n3 + me], sQ[2 * n3 + me], sQ[3 * n3 + me], sQ[4 * n3 + me], 0.0};
-          const Prim<double> Pb{sQ[q], sQ[n3 + q], sQ[2 * n3 + q], sQ[3 * n3 + q], sQ[4 * n3 + q], 0.0};
-          const double a0 = 0.5 * (sA[(dir * 3 + 0) * n3 + me] + sA[(dir * 3 + 0) * n3 + q]);
-          const double a1 = 0.5 * (sA[(dir * 3 + 1) * n3 + me] + sA[(dir * 3 + 1) * n3 + q]);
-          const double a2 = 0.5 * (sA[(dir * 3 + 2) * n3 + me] + sA[(dir * 3 + 2) * n3 + q]);
-          double mu[5];
-#pragma unroll
-          for (int v = 0; v < 5; ++v) mu[v] = sLt[v * n3 + me] - sLt[v * n3 + q];
-          double gA[5] = {0, 0, 0, 0, 0}, gB[5] = {0, 0, 0, 0, 0};
-          ec_flux_vjp(ph, Pa, Pb, a0, a1, a2, mu, gA, gB);
-          const double cw = sDVS[pos * n + pm];
-          g0 = fma(cw, gA[0], g0); g1 = fma(cw, gA[1], g1); g2 = fma(cw, gA[2], g2);
-          g3 = fma(cw, gA[3], g3); g4 = fma(cw, gA[4], g4);
-          if (2 * d != n) {
-            const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
-            const double cs = sDVS[(src - base) * n + pos];
-            g0 = fma(cs, __shfl_sync(0xffffffffu, gB[0], src), g0);
-            g1 = fma(cs, __shfl_sync(0xffffffffu, gB[1], src), g1);
-            g2 = fma(cs, __shfl_sync(0xffffffffu, gB[2], src), g2);
-            g3 = fma(cs, __shfl_sync(0xffffffffu, gB[3], src), g3);
-            g4 = fma(cs, __shfl_sync(0xffffffffu, gB[4], src), g4);
-          }
-        }
-      } else {
-#pragma unroll
-      for (int d = 1; d <= n / 2; ++d) {
-        const int pm = pos + d < n ? pos + d : pos + d - n;
-        const int q = node(pm);
-        // sums of the two nodes' values: {x} = Sx / 2
-        const double Sr = sQ[me] + sQ[q];
-        const double Su = sQ[n3 + me] + sQ[n3 + q], Sv = sQ[2 * n3 + me] + sQ[2 * n3 + q],
-                     Sw = sQ[3 * n3 + me] + sQ[3 * n3 + q];
-        const double Sh = sQ[5 * n3 + me] + sQ[5 * n3 + q];
-        const double Sa0 = sA[(dir * 3 + 0) * n3 + me] + sA[(dir * 3 + 0) * n3 + q];
-        const double Sa1 = sA[(dir * 3 + 1) * n3 + me] + sA[(dir * 3 + 1) * n3 + q];
-        const double Sa2 = sA[(dir * 3 + 2) * n3 + me] + sA[(dir * 3 + 2) * n3 + q];
-        double mu[5];  // mu / (w_i DVS_im)
-#pragma unroll
-        for (int v = 0; v < 5; ++v) mu[v] = sLt[v * n3 + me] - sLt[v * n3 + q];
-        // F0 = {rho} qa, Fk = {rho} qa {u_k} + {p} {a_k}, F4 = {rho} qa {h}, qa = {u}.{a} = Q / 4;
-        // tt = mu . dF/d({rho} qa) = mu0 + (mu1 Su + mu2 Sv + mu3 Sw + mu4 Sh) / 2;
-        // half of each average's cotangent goes to each node:
-        //   g_rho = Q tt / 8, g_u_k = Sr (tt Sa_k + Q mu_k / 2) / 8, g_p = (mu . Sa) / 4,
-        //   g_h = Sr Q mu4 / 16
-        const double Q = Su * Sa0 + Sv * Sa1 + Sw * Sa2;
-        const double tt = fma(0.5, mu[1] * Su + mu[2] * Sv + mu[3] * Sw + mu[4] * Sh, mu[0]);
-        const double hQ = 0.5 * Q;
-        const double h0 = Q * tt;
-        const double h1 = Sr * fma(tt, Sa0, hQ * mu[1]);
-        const double h2 = Sr * fma(tt, Sa1, hQ * mu[2]);
-        const double h3 = Sr * fma(tt, Sa2, hQ * mu[3]);
-        const double h4 = mu[1] * Sa0 + mu[2] * Sa1 + mu[3] * Sa2;
-        const double h5 = Sr * Q * mu[4];
-        const double cw = sDVS[pos * n + pm];
-        g0 = fma(cw, h0, g0); g1 = fma(cw, h1, g1); g2 = fma(cw, h2, g2);
-        g3 = fma(cw, h3, g3); g4 = fma(cw, h4, g4); g5 = fma(cw, h5, g5);
-        if (2 * d != n) {
-          const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
-          const double cs = sDVS[(src - base) * n + pos];
-          g0 = fma(cs, __shfl_sync(0xffffffffu, h0, src), g0);
-          g1 = fma(cs, __shfl_sync(0xffffffffu, h1, src), g1);
-          g2 = fma(cs, __shfl_sync(0xffffffffu, h2, src), g2);
-          g3 = fma(cs, __shfl_sync(0xffffffffu, h3, src), g3);
-          g4 = fma(cs, __shfl_sync(0xffffffffu, h4, src), g4);
-          g5 = fma(cs, __shfl_sync(0xffffffffu, h5, src), g5);
-        }
-      }
-      g0 *= 0.125; g1 *= 0.125; g2 *= 0.125; g3 *= 0.125; g4 *= 0.25; g5 *= 0.0625;
-      }  // Pirozzoli
-      if (active) {
-        if (dir == 0) {
-          sGQ[me] = g0; sGQ[n3 + me] = g1; sGQ[2 * n3 + me] = g2; sGQ[3 * n3 + me] = g3;
-          sGQ[4 * n3 + me] = g4; sGQ[5 * n3 + me] = g5;
-        } else {
-          sGQ[me] += g0; sGQ[n3 + me] += g1; sGQ[2 * n3 + me] += g2; sGQ[3 * n3 + me] += g3;
-          sGQ[4 * n3 + me] += g4; sGQ[5 * n3 + me] += g5;
-        }
-      }
-      __syncthreads();
-    }
-  }
+  // ---- transposed split-form volume integral (entropy-conserving flux; the
+  // KEP flux's is k_adj_volume's, whose result gV this kernel adds to)
+  if constexpr (EC)
+    adj_pairs_fp64<N, true>(sQ, sL, sQ + 6 * n3, sGQ, sDVS, siw, ph, t,
+                            [&](int dir, int, bool) { return sA + dir * 3 * n3; });
   // ---- viscous part: recompute the lifted gradients, then transpose
   // this thread's node from here on (N = 7: warp a + 4 b holds the xi lines at
   // eta in {a, N - a} and zeta in {b, N - b}, so that a node's mirror nodes
@@ -1186,19 +1212,19 @@ k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, cons
   double Uo[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) Uo[v] = U[v * S + g];
-  double gQ[6];
-#pragma unroll
-  for (int v = 0; v < 6; ++v) gQ[v] = sGQ[v * n3 + p];
   double out[5] = {0, 0, 0, 0, 0};
-  prim_vjp(Uo, ph, gQ, out);
+  if constexpr (EC) {
+    double gQ[6];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) gQ[v] = sGQ[v * n3 + p];
+    prim_vjp(Uo, ph, gQ, out);
+    source_vjp(Uo, ph, lam[4 * S + g], out);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) out[v] = gV[v * S + g];
+  }
   if (ph.viscous) vt_vjp(Uo, ph, gWo, out);
   if (gText != 0.0) out[0] -= gText * ph.p_out * ph.rcp_R / (Uo[0] * Uo[0]);
-  if (ph.f[0] != 0.0 || ph.f[1] != 0.0 || ph.f[2] != 0.0) {
-    // S_E = f . m / rho
-    const double l4 = lam[4 * S + g], ir = 1.0 / Uo[0];
-    out[0] -= l4 * (ph.f[0] * Uo[1] + ph.f[1] * Uo[2] + ph.f[2] * Uo[3]) * ir * ir;
-    out[1] += l4 * ph.f[0] * ir; out[2] += l4 * ph.f[1] * ir; out[3] += l4 * ph.f[2] * ir;
-  }
 #pragma unroll
   for (int v = 0; v < 5; ++v) gU[v * S + g] = out[v];
 }

@@ -1,0 +1,299 @@
+// adjoint_fx.cuh -- the KEP flux's transposed volume integral in fixed point.
+//
+// The pair terms of the adjoint (45 FP64 operations each, 540 of the element
+// kernel's 1124 FP64 instructions per node) run on the integer pipes in the
+// arithmetic of volume_fx.cuh: the state and the cotangents lam~ = -lam / J are
+// 62-bit integers in units of the element, one for the density's cotangent, one
+// for the momentum's and one for the energy's.  In the terms that add them, mu0 +
+// (mu_m . S_u + mu_4 S_h) / 2, each is shifted to the coarsest of the three
+// units.  Cotangents are of either sign and any size, so the terms lie further
+// below their bounds than the forward fluxes do; a line's sums therefore keep
+// 28 more bits (the full product of the last factors), the sum of the three is
+// normalised in each lane before it is multiplied, and the directions' sums are
+// added in FP64: the error against the extended-precision oracle's J^T lam
+// stays at FP64's.  Elements out of range (non-finite values, exponents beyond
+// 2^200) are summed in FP64.
+#pragma once
+#include "adjoint.cuh"
+#include "volume_fx.cuh"
+
+namespace dg {
+
+enum { AX_RHO, AX_U, AX_H, AX_L0, AX_LM, AX_LE, AX_NUM };
+struct AdjFxPlan {
+  int ok;
+  int bR, bU, bH, bL0, bLM, bLE;  // biased exponent bounds for fx_of
+  int s0, s1, s2;                 // right shifts of mu0, mu_m . S_u, mu_4 S_h to their common unit
+  int eg[4];                      // the units of the sums rho, u, p, h
+};
+
+// ex: the largest fx_mag of each value; mA: that of the element's metrics; eW:
+// lam~ / w is in units 2^eW times lam~'s.  Bounds in units of 2^60, times Q for the
+// pair terms: the sum of the three parts 3 (half of 6, by the extra shift), rho
+// and u 1.1, p 1.5, h 0.75; a line's sum of |Q| is below 3.7.
+__device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, int mA, int eW) {
+  AdjFxPlan f;
+  int eX[AX_NUM];
+  bool ok = true;
+#pragma unroll
+  for (int x = 0; x < AX_NUM; ++x) {
+    const int e = (ex[x] >> 20) - 1022;
+    eX[x] = max(e, -200);  // (smaller values, zeros among them, in that unit)
+    ok = ok && e < 200;
+  }
+  const int eA = (mA >> 20) - 1022;
+  f.bR = eX[AX_RHO] + 1022; f.bU = eX[AX_U] + 1022; f.bH = eX[AX_H] + 1022;
+  f.bL0 = eX[AX_L0] + 1022; f.bLM = eX[AX_LM] + 1022; f.bLE = eX[AX_LE] + 1022;
+  // units of the three parts of mu0 + (mu_m . S_u + mu_4 S_h) / 2
+  const int e0 = eX[AX_L0] + eW - 60, e1 = eX[AX_LM] + eX[AX_U] + eW - 59, e2 = eX[AX_LE] + eX[AX_H] + eW - 59;
+  const int et = max(e0, max(e1, e2)) + 1;
+  f.s0 = min(et - e0, 63); f.s1 = min(et - e1, 63); f.s2 = min(et - e2, 63);
+  f.eg[0] = et + eX[AX_U] + eA + 3;
+  f.eg[1] = et + eX[AX_RHO] + eA + 2;
+  f.eg[2] = eX[AX_LM] + eW + eA - 58;
+  f.eg[3] = eX[AX_U] + eA + eX[AX_LE] + eW + eX[AX_RHO] - 57;
+  f.ok = ok && abs(eA) < 200;
+  return f;
+}
+
+// a product in units of 2^62 of the factors' units and its next 32 bits (lo in
+// units of 2^-31: the sum of lo's may carry)
+struct Fx96 {
+  long long hi;
+  unsigned lo;
+};
+__device__ __forceinline__ Fx96 fx_mul96(Fx a, Fx b) {
+  const long long ll = mulw(a.l, b.l);
+  const long long x = madw((int)(ll >> 32), 2, madw(a.l, b.h, mulw(a.h, b.l)));
+  return Fx96{madw((int)(x >> 32), 2, mulw(a.h, b.h)), (unsigned)x};
+}
+
+template <int N>
+struct AdjFxShape {
+  static constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
+  // 8-byte values per node: 6 node values (fixed point 5), 5 cotangents, 5 of
+  // them over w, 3 metrics of the pass's direction, 6 sums
+  static constexpr int SMEM = (25 * n3 + n2 + 2 * n) * 8;
+  // lam~ / w is kept in units 2^(eW + 1 - LSH) times lam~'s: at N = 8 the largest
+  // 1 / w, 36, leaves almost a bit of 2^eW = 64 unused
+  static constexpr int LSH = N == 8 ? 2 : 1;
+};
+
+// The three direction passes: sQ [5][n3] (rho, u, v, w, h), sL [5][n3], sLt
+// [5][n3] scratch, sA [3][n3] scratch, sG [6][n3] the sums of (rho, u, v, w, p', h),
+// in FP64.
+// Lanes, pairs and shuffles as in volume_passes_fx; a pair's terms are the same
+// for its two nodes.
+template <int N>
+__device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sLt, Fx* sA, double* sG, const Fx* sT,
+                                              const long long* sW, const Fx* __restrict__ JaX, size_t S, size_t e0,
+                                              const AdjFxPlan& f, int t) {
+  using Sh = VolShape<N>;
+  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW;
+  const int warp = t >> 5, lane = t & 31;
+  const int seg = lane / n, pos = lane - seg * n;
+  const int L0 = warp * LPW + seg;
+  const bool active = (seg < LPW) && (L0 < n2);
+  const int L = active ? L0 : 0;
+  const int base = seg * n;
+  const int la = L % n, lb = L / n;
+#pragma unroll 1
+  for (int dir = 0; dir < 3; ++dir) {
+    const int me = dir == 0 ? pos + n * L : (dir == 1 ? la + n * pos + n2 * lb : L + n2 * pos);
+    const int ms = vslot<N, double>(me);
+    Fx q[5], a[3], l[5];
+    {
+      // lam~ / w
+      const Fx wi = fx_split<0>(sW[pos]);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        l[v] = fx_split<0>(fx_mul_shl(sL[v * n3 + ms], wi, AdjFxShape<N>::LSH));
+        if (active) sLt[v * n3 + ms] = l[v];
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        a[c] = JaX[(size_t)(dir * 3 + c) * S + e0 + me];
+        if (active) sA[c * n3 + ms] = a[c];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) q[v] = sQ[v * n3 + ms];
+    __syncthreads();
+    long long acc[6] = {0, 0, 0, 0, 0, 0};
+    unsigned low[6] = {0, 0, 0, 0, 0, 0};  // their next 28 bits, units of 2^-27
+#pragma unroll
+    for (int d = 1; d <= n / 2; ++d) {
+      const int pm = pos + d < n ? pos + d : pos + d - n;
+      const int sm = __shfl_sync(0xffffffffu, ms, base + pm);
+      const Fx Q = sT[pos * n + pm];
+      auto dif = [&](int v) {
+        const Fx x = sLt[v * n3 + sm];
+        return Fx{l[v].h - x.h, l[v].l - x.l};
+      };
+      const Fx Sa0 = a[0] + sA[sm], Sa1 = a[1] + sA[n3 + sm], Sa2 = a[2] + sA[2 * n3 + sm];
+      const Fx Su = q[1] + sQ[n3 + sm], Sv = q[2] + sQ[2 * n3 + sm], Sw = q[3] + sQ[3 * n3 + sm];
+      const Fx m1 = dif(1), m2 = dif(2), m3 = dif(3), m4 = dif(4);
+      FxSum k(Su, Sa0);
+      k.add(Sv, Sa1);
+      k.add(Sw, Sa2);
+      const long long qv = k.get();  // S_u . S_a
+      FxSum x(m1, Su);
+      x.add(m2, Sv);
+      x.add(m3, Sw);
+      const Fx m0 = dif(0);
+      const long long tt = ((((long long)m0.h << 31) + m0.l) >> f.s0) + (x.get() >> f.s1) +
+                           (fx_mul(m4, q[4] + sQ[4 * n3 + sm]) >> f.s2);
+      const Fx Qv = fx_split<1>(qv);
+      const long long sq = fx_mul(q[0] + sQ[sm], Q);  // S_rho Q
+      // tt (and S_u . S_a / 2 beside it) shifted up in this lane as far as both
+      // have room, S_rho Q down by as much
+      auto room = [](long long r) { return __clzll(r ^ (r >> 63)) - 3; };
+      const int up = max(0, min(min(room(tt), room(qv) + f.s1), 20));
+      const Fx Tn = fx_split<0>(tt << up);
+      const Fx Qs = fx_split<0>(up > f.s1 ? qv << (up - f.s1) : qv >> (f.s1 - up));
+      const Fx Sr = fx_split<1>(sq), Sn = fx_split<1>(sq >> up);
+      Fx96 F[6];
+      F[0] = fx_mul96(fx_split<0>(tt), fx_split<0>(fx_mul(Qv, Q)));
+      auto vel = [&](Fx Sa, Fx mk) {
+        FxSum y(Tn, Sa);
+        y.add(Qs, mk);
+        return fx_mul96(Sn, fx_split<1>(y.get()));
+      };
+      F[1] = vel(Sa0, m1);
+      F[2] = vel(Sa1, m2);
+      F[3] = vel(Sa2, m3);
+      FxSum z(m1, Sa0);
+      z.add(m2, Sa1);
+      z.add(m3, Sa2);
+      F[4] = fx_mul96(fx_split<1>(z.get()), Q);
+      F[5] = fx_mul96(Sr, fx_split<0>(fx_mul(Qv, m4)));
+#pragma unroll
+      for (int v = 0; v < 6; ++v) {
+        F[v].lo >>= 4;
+        acc[v] += F[v].hi;
+        low[v] += F[v].lo;
+      }
+      if (2 * d != n) {
+        const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
+#pragma unroll
+        for (int v = 0; v < 6; ++v) {
+          acc[v] += __shfl_sync(0xffffffffu, F[v].hi, src);
+          low[v] += __shfl_sync(0xffffffffu, F[v].lo, src);
+        }
+      }
+    }
+    if (active) {
+#pragma unroll
+      for (int v = 0; v < 6; ++v) {
+        // to FP64, with as many of the low bits as there is room for
+        const long long r = acc[v] + (low[v] >> 27);
+        const int k = min(max(__clzll(r ^ (r >> 63)) - 2, 0), 27);
+        const long long w = (r << k) + ((low[v] & 0x7ffffffu) >> (27 - k));
+        const double x = fx_double(w, f.eg[v == 0 ? 0 : (v < 4 ? 1 : v - 2)] - k);
+        sG[v * n3 + ms] = dir == 0 ? x : x + sG[v * n3 + ms];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// an element summed in FP64 (adj_fx_plan); rare, so kept out of line
+template <int N>
+__device__ __noinline__ void adj_volume_fp64(double* smem, const MeshDev<double>& m, const PhysDev& ph,
+                                             const Tables<N>& tab, int e, int t) {
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, T = VolShape<N>::THREADS;
+  double *sQ = smem, *sL = sQ + 6 * n3, *sLt = sL + 5 * n3, *sA = sLt + 5 * n3, *sG = sA + 3 * n3, *sDVS = sG + 6 * n3,
+         *siw = sDVS + n2;
+  for (int x = t; x < n2; x += T) sDVS[x] = 8.0 * tab.DVS8[x] / tab.iw[x / n];
+  if (t < n) siw[t] = tab.iw[t];
+  __syncthreads();
+  adj_pairs_fp64<N, false>(sQ, sL, sLt, sG, sDVS, siw, ph, t, [&](int dir, int me, bool active) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (active) sA[c * n3 + me] = m.Ja[(size_t)(dir * 3 + c) * ((size_t)m.K * n3) + (size_t)e * n3 + me];
+    return (const double*)sA;
+  });
+}
+
+// k_adj_volume: one CTA per element; gV = the volume integral's and the body
+// force's part of gU (through the primitives).  Measured at N = 7, 10^3
+// elements: the element kernel with the pairs in FP64 1181 us (FP64 pipe 86 %
+// busy); 495 us without them and 233 us here (issue 47 %, integer pipes 36 %,
+// FP64 pipe 32 %, of which the recovery of the primitives and its transpose).
+template <int N>
+__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, double, false>()))
+k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const MeshDev<double> m, const PhysDev ph,
+             const Tables<N> tab, const FxTab<N> ft, double* __restrict__ gV) {
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, T = VolShape<N>::THREADS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int sEx[AX_NUM];
+  __shared__ AdjFxPlan sF;
+  Fx* sQ = reinterpret_cast<Fx*>(smem_raw);
+  Fx* sL = sQ + 6 * n3;
+  Fx* sLt = sL + 5 * n3;
+  Fx* sA = sLt + 5 * n3;
+  double* sG = reinterpret_cast<double*>(sA + 3 * n3);
+  Fx* sT = reinterpret_cast<Fx*>(sG + 6 * n3);
+  long long* sW = reinterpret_cast<long long*>(sT + n2);
+  const int e = blockIdx.x, t = threadIdx.x;
+  const size_t S = (size_t)m.K * n3, e0 = (size_t)e * n3, g = e0 + t;
+  Prim<double> q{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  double l[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  if (t < n3) {
+    q = primitive<double>(U[g], U[S + g], U[2 * S + g], U[3 * S + g], U[4 * S + g], ph);
+    const double iJ = m.invJ[g];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) l[v] = -lam[v * S + g] * iJ;
+  }
+  if (t < AX_NUM) sEx[t] = 0;
+  for (int x = t; x < n2; x += T) sT[x] = ft.Q[x];
+  if (t < n) sW[t] = ft.iw[t];
+  __syncthreads();
+  {
+    const int ex[AX_NUM] = {fx_mag(q.rho), max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w)), fx_mag(q.h), fx_mag(l[0]),
+                            max(max(fx_mag(l[1]), fx_mag(l[2])), fx_mag(l[3])), fx_mag(l[4])};
+#pragma unroll
+    for (int x = 0; x < AX_NUM; ++x) {
+      const int mx = __reduce_max_sync(0xffffffffu, ex[x]);
+      if ((t & 31) == 0) atomicMax(&sEx[x], mx);
+    }
+  }
+  __syncthreads();
+  if (t == 0) sF = adj_fx_plan(sEx, m.JaX_max[e], ft.eW + 1 - AdjFxShape<N>::LSH);
+  __syncthreads();
+  const AdjFxPlan f = sF;
+  // node slots: swizzled in fixed point (vslot), natural in FP64
+  if (t < n3) {
+    const int ts = f.ok ? vslot<N, double>(t) : t;
+    const double x[6] = {q.rho, q.u, q.v, q.w, f.ok ? q.h : q.p, q.h};
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      if (!f.ok) reinterpret_cast<double*>(sQ)[v * n3 + ts] = x[v];
+      else if (v < 5) sQ[v * n3 + ts] = fx_of(x[v], v == 0 ? f.bR : (v < 4 ? f.bU : f.bH));
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      if (!f.ok) reinterpret_cast<double*>(sL)[v * n3 + ts] = l[v];
+      else sL[v * n3 + ts] = fx_of(l[v], v == 0 ? f.bL0 : (v < 4 ? f.bLM : f.bLE));
+    }
+  }
+  if (f.ok) {
+    __syncthreads();
+    adj_passes_fx<N>(sQ, sL, sLt, sA, sG, sT, sW, m.JaX, S, e0, f, t);
+  } else {
+    adj_volume_fp64<N>(reinterpret_cast<double*>(smem_raw), m, ph, tab, e, t);
+  }
+  if (t >= n3) return;
+  double gQ[6], Uo[5], out[5] = {0, 0, 0, 0, 0};
+  const int ts = f.ok ? vslot<N, double>(t) : t;
+#pragma unroll
+  for (int v = 0; v < 6; ++v) gQ[v] = sG[v * n3 + ts];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) Uo[v] = U[v * S + g];
+  prim_vjp(Uo, ph, gQ, out);
+  source_vjp(Uo, ph, lam[4 * S + g], out);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) gV[v * S + g] = out[v];
+}
+
+}  // namespace dg

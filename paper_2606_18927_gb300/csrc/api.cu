@@ -96,6 +96,7 @@ struct dg_ctx {
   double* wJ = nullptr;        // w_i w_j w_k J per node (kinetic-energy integral)
   double vol = 0.0;
   // adjoint scratch (allocated on the first dg_vjp)
+  double* gV = nullptr;
   double* gUf = nullptr;
   double* gGf = nullptr;
   double* gWf = nullptr;
@@ -163,7 +164,7 @@ void free_all(dg_ctx* c) {
   c->cp_in = c->cp_out = nullptr;
   void* ptrs[] = {c->U, c->dU, c->io, c->io2, c->Ja, c->invJ, c->fgeo, c->nbr, c->elem_face, c->faces,
                   c->ws_elem, c->ws_lag, c->Rv, c->Gf, c->Fs, c->tau, c->status,
-                  c->gUf, c->gGf, c->gWf, c->gUs, c->gtheta, c->wq, c->ro_ckpt, c->ro_stage, c->ro_work,
+                  c->gV, c->gUf, c->gGf, c->gWf, c->gUs, c->gtheta, c->wq, c->ro_ckpt, c->ro_stage, c->ro_work,
                   c->ro_scalar, c->wJ, c->W32, c->W64, c->JaJ, c->Mj, c->lift_M2, c->lift_W2, c->JaX, c->JaX_max, c->halo_U, c->send_U,
                   c->halo_G, c->send_G,
                   c->wm_t};
@@ -902,6 +903,7 @@ static int ensure_adjoint_scratch(dg_ctx* c) {
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   const size_t kn2 = (size_t)c->K * 6 * c->n2;
+  if (c->opts.vol_flux != DG_VOL_EC_CHANDRASHEKAR) chk(alloc(&c->gV, 5 * c->S));
   chk(alloc(&c->gUf, 5 * kn2));
   chk(alloc(&c->gGf, 4 * kn2));
   chk(alloc(&c->gWf, 4 * kn2));
@@ -919,8 +921,9 @@ static dg::OpArgs adjoint_args(dg_ctx* c, const double* U, const double* lam, do
   a.faces = c->faces; a.ws_elem = c->ws_elem; a.ws_lag = c->ws_lag;
   a.D = c->geo.basis.D.data(); a.w = c->geo.basis.w.data();
   a.Uin = U; a.status = c->status;
-  a.lam = lam; a.gU = gU; a.gUf = c->gUf; a.gGf = c->gGf; a.gWf = c->gWf; a.gUs = c->gUs; a.gtheta = gth;
+  a.lam = lam; a.gU = gU; a.gV = c->gV; a.gUf = c->gUf; a.gGf = c->gGf; a.gWf = c->gWf; a.gUs = c->gUs; a.gtheta = gth;
   a.JaJ = c->JaJ; a.Mj = c->Mj;
+  a.JaX = c->JaX; a.JaX_max = c->JaX_max;
   a.n_halo = c->geo.n_halo;
   a.halo_U = c->halo_U; a.halo_G = c->halo_G; a.send_U = c->send_U; a.send_G = c->send_G;
   return a;

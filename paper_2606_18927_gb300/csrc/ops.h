@@ -73,6 +73,7 @@ struct OpArgs {
   // adjoint (FP64): cotangent lam of Ut, output gU, and scratch
   const double* lam;
   double* gU;
+  double* gV;               // [5][K n3] the KEP volume integral's part of gU
   double* gUf;              // [K][6][5][n2] face-kernel state cotangents
   double* gGf;              // [K][6][4][n2] cotangents of the own face viscous fluxes
   double* gWf;              // [K][6][4][n2] lifting cotangents for the neighbour's face nodes

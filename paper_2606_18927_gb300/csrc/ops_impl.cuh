@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "adjoint.cuh"
+#include "adjoint_fx.cuh"
 #include "kernels.cuh"
 #include "lift_df.cuh"
 #include "volume_fx.cuh"
@@ -283,6 +284,7 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   m.ws_elem = a.ws_elem; m.ws_lag = a.ws_lag;
   m.status = a.status;
   m.JaJ = a.JaJ; m.Mj = a.Mj;
+  m.JaX = a.JaX; m.JaX_max = a.JaX_max;
   m.n_halo = a.n_halo; m.halo_U = a.halo_U; m.halo_G = static_cast<const double*>(a.halo_G);
   if (ph.viscous && !a.JaJ) return (int)cudaErrorInvalidValue;
   const Tables<N> tab = make_tables<N>(a.D, a.w);
@@ -332,7 +334,12 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   }
   if (phase == 3 || phase == 14) {
     if (part && ph.viscous) k_adj_halo_in<N><<<halo_blocks, 128, 0, s>>>(m, m.halo_G, a.gGf);
-    kel<<<a.K, AdjShape<N>::THREADS, smem, s>>>(a.Uin, a.lam, m, ph, tab, a.gGf, a.gU, a.gWf, sendU);
+    if (!ec) {
+      cudaFuncSetAttribute(k_adj_volume<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, AdjFxShape<N>::SMEM);
+      k_adj_volume<N><<<a.K, VolShape<N>::THREADS, AdjFxShape<N>::SMEM, s>>>(a.Uin, a.lam, m, ph, tab, fx_tab<N>(),
+                                                                             a.gV);
+    }
+    kel<<<a.K, AdjShape<N>::THREADS, smem, s>>>(a.Uin, a.lam, m, ph, tab, a.gGf, a.gV, a.gU, a.gWf, sendU);
   }
   if (phase == 4 || phase == 14) {
     const long long S = (long long)a.K * n3;
