@@ -221,7 +221,7 @@ __device__ __noinline__ void adj_volume_fp64(double* smem, const MeshDev<double>
 // busy); 495 us without them and 233 us here (issue 47 %, integer pipes 36 %,
 // FP64 pipe 32 %, of which the recovery of the primitives and its transpose).
 template <int N>
-__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, double, false>()))
+__global__ void __launch_bounds__(VolShape<N>::THREADS, (resident_ctas(VolShape<N>::THREADS, AdjFxShape<N>::SMEM, 1024)))
 k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const MeshDev<double> m, const PhysDev ph,
              const Tables<N> tab, const FxTab<N> ft, double* __restrict__ gV) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, T = VolShape<N>::THREADS;

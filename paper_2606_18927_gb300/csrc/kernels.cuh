@@ -56,6 +56,22 @@ __device__ __forceinline__ int chk_idx(int i, int n, int* status) {
   return i;
 }
 
+// Resident CTAs per SM asked of the register allocator for an element kernel of
+// `threads` threads and `smem` bytes of shared memory: those of `resident`
+// threads per SM, as far as the shared memory goes.  The fixed-point and
+// double-float kernels take 1024 (64 registers), the FP32-mixed ones 1536 (40):
+// left to itself the compiler takes 70 to 126 registers at the lower degrees,
+// and their memory and barrier waits show.  Measured per stage, in place of two
+// CTAs: k_volume_fx N = 4 0.95 -> 0.59 ms, N = 6 1.29 -> 0.78 (in the sine box of
+// 32^3 and 22^3 elements); FP32-mixed k_volume N = 5 0.66 -> 0.35, N = 4 0.56 ->
+// 0.35, N = 6 0.87 -> 0.39 (26^3, 32^3, 22^3); more threads (2048) spill: 0.45,
+// 0.40, 0.50.
+constexpr int resident_ctas(int threads, int smem, int resident) {
+  const int warps = (threads + 31) / 32 * 32, by_smem = 232448 / (smem + 1024);
+  const int n = resident / warps < by_smem ? resident / warps : by_smem;
+  return n < 1 ? 1 : (n > 32 ? 32 : n);
+}
+
 // a fixed-point number h 2^31 + l (volume_fx.cuh)
 struct Fx {
   int h, l;
@@ -1356,13 +1372,14 @@ struct LiftPk {
   f32x2 d[(N + 1) * (N + 1)], dv[(N + 1) * (N + 1)];
 };
 
-// Resident CTAs per SM asked of the register allocator for the lifting
-// kernel: two for CTAs of up to 512 threads, three for the FP32 kernel at
-// N = 7 (42 registers; its line phases leave the other threads waiting at a
-// barrier, which a third CTA per SM covers)
+// Resident CTAs per SM asked of the register allocator for the lifting kernel:
+// two in FP64 (bound by the FP64 pipe), FP32 resident_ctas (its line phases
+// leave the other threads waiting at a barrier, which more CTAs cover: N = 5
+// 0.195 -> 0.177 ms at 26^3, N = 3 0.248 -> 0.157 at 40^3)
 template <int N, typename R>
 constexpr int lift_min_blocks() {
-  return ((N + 1) * (N + 1) * (N + 1) > 512) ? 1 : ((N == 7 && std::is_same<R, float>::value) ? 3 : 2);
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
+  return std::is_same<R, float>::value ? resident_ctas(n3, (16 * n3 + 26 * n2 + n) * 4, 1536) : (n3 > 512 ? 1 : 2);
 }
 
 template <int N, typename R>
@@ -2185,16 +2202,6 @@ struct VolShape {
   static constexpr int SMEM_R_F32 = 24 * n3 + 3 * n2;
 };
 
-// Resident CTAs per SM asked of the register allocator: two for CTAs of up to
-// 512 threads (64 registers at N = 7; measured 5 % faster in FP64 than one CTA
-// at 106 registers, 1.6x faster for the FP32 entropy-conserving kernel than one
-// CTA at 104, and 1.3 % faster for the FP64 entropy-conserving kernel than one
-// CTA at 126 registers, in spite of its spills).
-template <int N, typename R, bool EC>
-constexpr int vol_min_blocks() {
-  return (N == 7 && !EC && std::is_same<R, float>::value) ? 3 : ((VolShape<N>::THREADS * 64 * 2 <= 65536) ? 2 : 1);
-}
-
 // shared-memory arrays of the volume kernel
 template <typename R>
 struct VolSmem {
@@ -2543,7 +2550,9 @@ __device__ __forceinline__ void stage_node(R* sQ, int ts, const Prim<R>& q, cons
 }
 
 template <int N, typename R, int MODE, bool EC>
-__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, R, EC>()))
+__global__ void __launch_bounds__(VolShape<N>::THREADS,
+                                  (resident_ctas(VolShape<N>::THREADS,
+                                                 (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4, 1536)))
 k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, const Tables<N> tab,
          const R* __restrict__ Rv, const R* __restrict__ Fs, double* __restrict__ Out,
          double* __restrict__ dU, double* __restrict__ Uout, const StageArgs st, int* __restrict__ status) {

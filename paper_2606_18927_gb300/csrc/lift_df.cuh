@@ -196,7 +196,8 @@ __device__ __forceinline__ int df_slot(int node) {
 // divergence R_v, both FP64 in memory) with the line contractions on two
 // threads per line, two variables each.
 template <int N>
-__global__ void __launch_bounds__((N + 1) * (N + 1) * (N + 1), ((N + 1) * (N + 1) * (N + 1) <= 512 ? 2 : 1))
+__global__ void __launch_bounds__((N + 1) * (N + 1) * (N + 1),
+                                  (resident_ctas((N + 1) * (N + 1) * (N + 1), LiftDfShape<N>::SMEM_F2 * 8, 1024)))
 k_lift_df(const double* __restrict__ U, const MeshDev<double> m, const PhysDev ph, const Tables<N> tab,
           const LiftDfCoef<N> cf, double* __restrict__ Rv, double* __restrict__ Gf) {
   static_assert(N % 2 == 1, "the double-float lifting kernel needs an even node count");

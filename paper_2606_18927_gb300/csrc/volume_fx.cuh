@@ -400,7 +400,7 @@ __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<doub
 // FP64 pair fluxes (FP64 pipe 90 % busy), 3.07 ms in fixed point (issue 52 %,
 // integer pipes 37 %, FP64 pipe 30 %).
 template <int N, int MODE, int VF>
-__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, double, VF == FX_EC>()))
+__global__ void __launch_bounds__(VolShape<N>::THREADS, (resident_ctas(VolShape<N>::THREADS, VolFxShape<N, VF>::SMEM, 1024)))
 k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysDev ph, const Tables<N> tab,
             const FxTab<N> ft, const double* __restrict__ Rv, const double* __restrict__ Fs, double* __restrict__ Out,
             double* __restrict__ dU, double* __restrict__ Uout, const StageArgs st, int* __restrict__ status) {
