@@ -437,7 +437,8 @@ int dg_time_derivative_phase(dg_ctx* c, int phase, const double* U, double* Ut);
  * dg_profile_enable(c, 1) records events around the lift, face, wall and
  * volume kernels of every subsequent operator evaluation (in the FP64
  * viscous form the lift window also holds the kernel that forms the input
- * state's primitives, when they are not already stored); dg_profile_read
+ * state's primitives, when they are not already stored: a stage stores those
+ * of the state it writes); dg_profile_read
  * synchronises the stream, returns the summed milliseconds ms[4] and the
  * launch counts launches[4] (order: lift, face, wall, volume) since the last
  * read, and resets them. */

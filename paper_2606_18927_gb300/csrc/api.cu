@@ -175,6 +175,12 @@ void free_all(dg_ctx* c) {
 // profiling events per operator evaluation (see OpArgs::ev)
 constexpr size_t kEventsPerLaunch = 7;
 
+// whether s is being captured (the legacy default stream cannot be)
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return s && cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
 int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double B, double dt, int read_dU,
            double* Uout, double* dU = nullptr, int phase = 7) {
   if (phase == 7 && c->geo.n_halo > 0)
@@ -210,7 +216,12 @@ int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double
   a.W32 = c->W32;
   a.w32_valid = (a.fp32 && Uin == c->U && c->w32_of_U) ? 1 : 0;
   a.W64 = c->W64;
-  a.w64_valid = (c->W64 && !a.fp32 && Uin == c->U && c->w64_of_U) ? 1 : 0;
+  // A graph of the caller's replays after states this context cannot foresee
+  // (dg_set_state between replays): every evaluation in it forms its own
+  // primitives.  (dg_rk_steps_graph refreshes them before its replays.)
+  const bool user_capture = c->W64 && c->stream != c->cap_stream && capturing(c->stream);
+  a.w64_valid = (c->W64 && !a.fp32 && Uin == c->U && c->w64_of_U && !user_capture) ? 1 : 0;
+  a.keep_w64 = Uout == c->U ? 1 : 0;
   a.JaJ = c->JaJ; a.Mj = c->Mj;
   a.lift_M2 = c->lift_M2; a.lift_W2 = c->lift_W2;
   a.JaX = c->JaX; a.JaX_max = c->JaX_max;
@@ -224,19 +235,27 @@ int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double
   // the FP32 primitives now belong to the stage's output (mode 1) or input
   if (a.fp32 && (phase & 4)) c->w32_of_U = mode == 1 ? (Uout == c->U) : (Uin == c->U);
   else if (a.fp32 && (phase & 2)) c->w32_of_U = (Uin == c->U);
-  // the FP64 primitives: those of the input once phase 2 ran, stale once a
-  // stage has updated the state in place
+  // the FP64 primitives: those of the input once phase 2 ran, of the updated
+  // state after a stage on the context's state
   if (!a.fp32 && c->W64 && c->opts.viscous) {
-    if ((phase & 4) && mode == 1 && Uout == c->U) c->w64_of_U = false;
+    if ((phase & 4) && mode == 1 && Uout == c->U) c->w64_of_U = true;
     else if (phase & 2) c->w64_of_U = (Uin == c->U);
+    if (user_capture) c->w64_of_U = false;  // nothing has run yet
   }
   return DG_OK;
 }
 
-// FP32-mixed form: form the primitives of the context's state if they are stale
-int refresh_w32(dg_ctx* c) {
-  if (c->opts.precision != DG_FP32_MIXED || c->w32_of_U) return DG_OK;
+// form the stored primitives of the context's state if they are stale
+int refresh_primitives(dg_ctx* c) {
   const long long S = (long long)c->S;
+  if (c->W64 && c->opts.viscous && !c->w64_of_U) {
+    dg::k_prim64<<<(unsigned)std::min<long long>((S + 255) / 256, 152 * 16), 256, 0, c->stream>>>(
+        S, c->U, c->ph, c->W64, c->ph.lift_df ? c->lift_W2 : nullptr);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(c, e, "primitive refresh");
+    c->w64_of_U = true;
+  }
+  if (c->opts.precision != DG_FP32_MIXED || c->w32_of_U) return DG_OK;
   dg::k_prim32<<<(unsigned)std::min<long long>((S + 255) / 256, 152 * 16), 256, 0, c->stream>>>(S, c->U, c->ph,
                                                                                                  c->W32);
   cudaError_t e = cudaGetLastError();
@@ -503,6 +522,7 @@ int dg_init_mesh(dg_ctx** out, const dg_mesh_desc* m, const dg_phys* p, const dg
   ph.T_wall = p->T_wall;
   ph.wm_maxit = kWallSolveMaxIter;
   ph.lift_df = 0;
+  ph.T_lift = p->rho_ref > 0.0 ? p->p_ref * ph.rcp_R / p->rho_ref : 0.0;
   ph.sutherland = ph.suth_S > 0.0 ? 1 : 0;
   ph.fs_diff = (o->precision == DG_FP32_MIXED && o->vol_flux == DG_VOL_KEP_PIROZZOLI) ? 1 : 0;
   ph.has_force = (ph.f[0] != 0.0 || ph.f[1] != 0.0 || ph.f[2] != 0.0) ? 1 : 0;
@@ -1210,7 +1230,7 @@ int dg_rk_steps_graph(dg_ctx* c, double t, double dt, int nsteps) {
   (void)t;  // the operator is autonomous
   if (!c || nsteps < 0) return c ? fail(c, DG_ERR_ARG, "dg_rk_steps_graph: nsteps < 0") : DG_ERR_ARG;
   if (!c->state_set) return fail(c, DG_ERR_NOT_INIT, "dg_rk_steps_graph: state not set");
-  int rc0 = refresh_w32(c);
+  int rc0 = refresh_primitives(c);
   if (rc0 != DG_OK) return rc0;
   cudaError_t e = cudaSuccess;
   if (!c->step_graph || c->step_graph_dt != dt) {
@@ -1225,9 +1245,6 @@ int dg_rk_steps_graph(dg_ctx* c, double t, double dt, int nsteps) {
     cudaStream_t user = c->stream;
     c->profiling = false;
     c->stream = c->cap_stream;
-    // every replay starts from a state its previous step updated: the first
-    // stage must form the FP64 primitives
-    c->w64_of_U = false;
     e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     int rc = DG_OK;
     if (e == cudaSuccess)
@@ -1251,7 +1268,6 @@ int dg_rk_steps_graph(dg_ctx* c, double t, double dt, int nsteps) {
     e = cudaGraphLaunch(c->step_graph, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "dg_rk_steps_graph: launch");
   }
-  if (nsteps > 0) c->w64_of_U = false;  // the state changed under the stored primitives
   return DG_OK;
 }
 

@@ -95,6 +95,7 @@ struct PhysDev {
   double T_wall;              // isothermal wall temperature (<= 0: adiabatic walls)
   int wm_maxit;               // iteration cap of the law-of-the-wall solve (bracket growth + Newton)
   int lift_df;                // FP64 viscous form at odd N: lifting in double-float arithmetic (k_lift_df)
+  double T_lift;              // its temperatures' reference: rho_ref > 0: p_ref / (rho_ref R), else 0
   // FP32 copies of the constants the FP32 kernels use (a double-to-float
   // conversion is an FP64-pipe instruction)
   struct {
@@ -518,26 +519,34 @@ __device__ __forceinline__ void store_prim64(double* __restrict__ W, size_t S, s
   W[4 * S + g] = q.p; W[5 * S + g] = q.h; W[6 * S + g] = T;
 }
 
-// the primitives of the input state, stored for the operator's kernels (FP64
-// viscous form); run before the lifting kernel whenever they are stale
-// (W2: the double-float lifting's (u, v, w, T - T_ref) as (hi, lo) float
-// pairs, or null)
+// one node's primitives into W64, and with W2 the double-float lifting's
+// (u, v, w, T - T_ref) as (hi, lo) float pairs
+__device__ __forceinline__ void form_prim64(size_t S, size_t g, const double U[5], const PhysDev& ph,
+                                            double* __restrict__ W, float2* __restrict__ W2) {
+  double T;
+  const Prim<double> q = primitive_T(U[0], U[1], U[2], U[3], U[4], ph, T);
+  store_prim64(W, S, g, q, T);
+  if (W2) {
+    const double x[4] = {q.u, q.v, q.w, T - ph.T_lift};
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      float lo;
+      const float hi = d2f_bits(x[v], &lo);
+      W2[v * S + g] = make_float2(hi, lo);
+    }
+  }
+}
+
+// The primitives of the input state, stored for the operator's kernels (FP64
+// viscous form); run before the lifting kernel when they are stale: a stage
+// leaves those of the state it writes (volume_epilogue, whose FP64 pipe has
+// room beside the integer passes: a step of 16^3 elements at N = 7 takes 4.70
+// instead of 4.89 ms, of 24^3 15.3 instead of 15.9 ms).
 static __global__ void k_prim64(long long S, const double* __restrict__ U, const PhysDev ph, double* __restrict__ W,
                                 float2* __restrict__ W2) {
-  const double Tref = ph.rho_ref > 0.0 ? ph.p_ref * ph.rcp_R / ph.rho_ref : 0.0;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < S; g += (long long)gridDim.x * blockDim.x) {
-    double T;
-    const Prim<double> q = primitive_T(U[g], U[S + g], U[2 * S + g], U[3 * S + g], U[4 * S + g], ph, T);
-    store_prim64(W, (size_t)S, (size_t)g, q, T);
-    if (W2) {
-      const double x[4] = {q.u, q.v, q.w, T - Tref};
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        float lo;
-        const float hi = d2f_bits(x[v], &lo);
-        W2[v * S + g] = make_float2(hi, lo);
-      }
-    }
+    const double x[5] = {U[g], U[S + g], U[2 * S + g], U[3 * S + g], U[4 * S + g]};
+    form_prim64((size_t)S, (size_t)g, x, ph, W, W2);
   }
 }
 
@@ -2182,6 +2191,7 @@ struct StageArgs {
   double A, B, dt;
   int read_dU;
   int write_w32;  // FP32-mixed form: store the updated state's primitives into W32
+  int write_w64;  // FP64 viscous form: 1 into W64, 2 also their pairs into lift_W2
 };
 
 // Shared-memory slot of a node in the volume kernel's per-node arrays.  A
@@ -2540,13 +2550,15 @@ __device__ __forceinline__ void volume_epilogue(const double* __restrict__ Uin, 
       bad |= !finite_bits(un);
     }
     if (bad) atomicOr(status, ST_NONFINITE);
-    // the next stage's FP32 primitives, from the updated FP64 state
+    // the next stage's primitives, from the updated FP64 state
     if constexpr (F32) {
       if (st.write_w32) {
         Lo3 l;
         const Prim<float> q = prim32_shifted(Uo[0], Uo[1], Uo[2], Uo[3], Uo[4], ph, &l);
         store_prim32(m.W32, S, g, q, l);
       }
+    } else if (st.write_w64) {
+      form_prim64(S, g, Uo, ph, m.W64, st.write_w64 == 2 ? m.lift_W2 : nullptr);
     }
   }
 }

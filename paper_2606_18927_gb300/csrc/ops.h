@@ -49,6 +49,7 @@ struct OpArgs {
   // forms them before the lifting kernel)
   double* W64;
   int w64_valid;
+  int keep_w64;  // a stage leaves the primitives of Uout in W64 (and lift_W2)
   // FP64 viscous form: the lifting kernel's metric products, [9][K n^3] Ja / J
   // and [6][K n^3] (Ja Ja^T) / J (order 00, 11, 22, 01, 02, 12)
   const double* JaJ;

@@ -249,7 +249,8 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     if (a.ev) cudaEventRecord(a.ev[4], s);
   }
   if (a.ev) cudaEventRecord(a.ev[5], s);
-  const StageArgs st{a.A, a.B, a.dt, a.read_dU, std::is_same<R, float>::value && a.mode == 1 ? 1 : 0};
+  const StageArgs st{a.A, a.B, a.dt, a.read_dU, std::is_same<R, float>::value && a.mode == 1 ? 1 : 0,
+                     a.mode == 1 && m.W64 && a.keep_w64 ? (ph.lift_df && N % 2 == 1 && a.lift_W2 ? 2 : 1) : 0};
   if constexpr (std::is_same<R, double>::value) {
     auto volume = [&](auto kern, int smem) {
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
