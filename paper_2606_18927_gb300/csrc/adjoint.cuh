@@ -8,9 +8,8 @@
 //                (face_flux_vjp), and the cotangents of the two sides'
 //                viscous face fluxes;
 //   k_adj_wall   wall face nodes: the same through the mirror state, and the
-//                wall-model derivative (forward-mode duals over the sample
-//                state; implicit function theorem for the law of the wall)
-//                with respect to the sample state and (kappa, B);
+//                wall model in reverse mode (implicit function theorem for
+//                the law of the wall) to the sample state and (kappa, B);
 //   k_adj_volume (adjoint_fx.cuh) one CTA per element: the KEP flux's
 //                transposed split-form volume integral in fixed point;
 //   k_adj_element one CTA per element: with the entropy-conserving flux its
@@ -26,51 +25,7 @@
 
 namespace dg {
 
-// ---------------------------------------------------------------------------
-// forward-mode dual number (value, one directional derivative)
-// ---------------------------------------------------------------------------
-struct DualD {
-  double v, d;
-  __device__ DualD() : v(0.0), d(0.0) {}
-  __device__ DualD(double x) : v(x), d(0.0) {}
-  __device__ DualD(double x, double dx) : v(x), d(dx) {}
-};
-__device__ __forceinline__ DualD operator+(DualD a, DualD b) { return DualD(a.v + b.v, a.d + b.d); }
-__device__ __forceinline__ DualD operator-(DualD a, DualD b) { return DualD(a.v - b.v, a.d - b.d); }
-__device__ __forceinline__ DualD operator-(DualD a) { return DualD(-a.v, -a.d); }
-__device__ __forceinline__ DualD operator*(DualD a, DualD b) { return DualD(a.v * b.v, a.d * b.v + a.v * b.d); }
-__device__ __forceinline__ DualD operator/(DualD a, DualD b) {
-  const double r = a.v / b.v;
-  return DualD(r, (a.d - r * b.d) / b.v);
-}
-__device__ __forceinline__ DualD operator+(DualD a, double b) { return DualD(a.v + b, a.d); }
-__device__ __forceinline__ DualD operator+(double a, DualD b) { return DualD(a + b.v, b.d); }
-__device__ __forceinline__ DualD operator-(DualD a, double b) { return DualD(a.v - b, a.d); }
-__device__ __forceinline__ DualD operator-(double a, DualD b) { return DualD(a - b.v, -b.d); }
-__device__ __forceinline__ DualD operator*(DualD a, double b) { return DualD(a.v * b, a.d * b); }
-__device__ __forceinline__ DualD operator*(double a, DualD b) { return DualD(a * b.v, a * b.d); }
-__device__ __forceinline__ DualD operator/(DualD a, double b) { return DualD(a.v / b, a.d / b); }
-__device__ __forceinline__ DualD operator/(double a, DualD b) {
-  const double r = a / b.v;
-  return DualD(r, -r * b.d / b.v);
-}
-__device__ __forceinline__ DualD& operator+=(DualD& a, DualD b) { a = a + b; return a; }
-__device__ __forceinline__ DualD& operator-=(DualD& a, DualD b) { a = a - b; return a; }
-__device__ __forceinline__ bool operator<(DualD a, DualD b) { return a.v < b.v; }
-__device__ __forceinline__ bool operator>=(DualD a, DualD b) { return a.v >= b.v; }
-__device__ __forceinline__ DualD sqrt(DualD a) {
-  const double s = ::sqrt(a.v);
-  return DualD(s, a.d / (2.0 * s));
-}
-__device__ __forceinline__ DualD fabs(DualD a) { return a.v < 0.0 ? -a : a; }
-__device__ __forceinline__ DualD asin(DualD a) { return DualD(::asin(a.v), a.d / ::sqrt(1.0 - a.v * a.v)); }
-
-// ---------------------------------------------------------------------------
-// wall-model JVP: tau (3) with its derivative along the duals of Us and
-// (dk, dB) for the law constants.  u_tau comes from the primal solver; its
-// derivative from the implicit function theorem on F(t) = t + ln L(e^t) -
-// ln Re_h = 0, Re_h = h u_VD / nu_w.
-// ---------------------------------------------------------------------------
+// d ln-law / d(kappa, B) of L at the explicit variable w
 __device__ __forceinline__ void law_param_derivs(int law, double w, double kap, double B, double* Lk,
                                                  double* LB) {
   if (law == 1) {
@@ -89,65 +44,102 @@ __device__ __forceinline__ void law_param_derivs(int law, double w, double kap, 
   }
 }
 
-// qw (may be null): the wall heat flux of isothermal walls (0 for adiabatic ones)
-// The law-of-the-wall solve depends on the values alone: with `sv` it is done
-// once (sv->have false: here, then kept in *sv) and serves every direction.
-struct WallSolve {
-  bool have, ok;
-  double ut, L, wdL, Lk, LB;
-};
-static __device__ void wall_stress_jvp(const PhysDev& ph, const DualD Us[5], double dk, double dB, double nx,
-                                double ny, double nz, DualD tau[3], WallSolve* sv, DualD* qw = nullptr) {
-  const DualD rho = Us[0], ir = 1.0 / rho;
-  const DualD u = Us[1] * ir, v = Us[2] * ir, w = Us[3] * ir;
-  const DualD p = ph.gm1 * (Us[4] - 0.5 * rho * (u * u + v * v + w * w));
-  const DualD T = p * ph.rcp_R * ir;
-  const DualD un = u * nx + v * ny + w * nz;
-  const DualD ux = u - un * nx, uy = v - un * ny, uz = w - un * nz;
-  const DualD u2 = ux * ux + uy * uy + uz * uz;
-  tau[0] = tau[1] = tau[2] = DualD(0.0);
-  if (qw) *qw = DualD(0.0);
-  if (!sv->have) { sv->ok = true; sv->ut = sv->wdL = sv->Lk = sv->LB = 0.0; sv->L = 1.0; }
-  if (!(u2.v > 0.0)) return;
-  const DualD um = sqrt(u2);
+// Wall model in reverse mode: from the cotangents gt of tau and gq of the wall heat
+// flux (isothermal walls), gU = (d(tau, q_w)/dU_s)^T and gth = (d/d(kappa, B))^T;
+// returns tau_x in *tx.  The model is a function of the scalars rho, T and the
+// wall-parallel speed um, and u_tau follows from the implicit function theorem on
+// F(t) = t + ln L(e^t) - ln Re_h = 0, Re_h = h u_VD / nu_w: with alpha = 1 / F' =
+// L / (L + w L'), in Reichardt's law (explicit in u_tau)
+//   d ln u_tau = alpha d ln u_VD + (1 - alpha) d ln nu_w - alpha (L_k dk + L_B dB) / L,
+// in the other law (explicit in u_VD / u_tau) with alpha and 1 - alpha exchanged and
+// the last term's sign turned.
+static __device__ __noinline__ void wall_stress_vjp(const PhysDev& ph, const double U[5], double nx, double ny,
+                                                    double nz, const double gt[3], double gq, double gU[5],
+                                                    double gth[2], double* tx, bool* ok) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) gU[v] = 0.0;
+  gth[0] = gth[1] = *tx = 0.0;
+  *ok = true;
+  const double rho = U[0], ir = 1.0 / rho;
+  const double u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
+  const double q2 = u * u + v * v + w * w;
+  const double p = ph.gm1 * (U[4] - 0.5 * rho * q2);
+  const double T = p * ph.rcp_R * ir;
+  const double un = u * nx + v * ny + w * nz;
+  const double ux = u - un * nx, uy = v - un * ny, uz = w - un * nz;
+  const double u2 = ux * ux + uy * uy + uz * uz;
+  if (!(u2 > 0.0)) return;
+  const double um = sqrt(u2), ium = 1.0 / um;
   const double r = cbrt(ph.Pr);
-  const DualD Taw = T + r * u2 / (2.0 * ph.cp);
-  // the Van Driest transform: adiabatic (T_w = T_aw) or, at an isothermal
-  // wall, the closed form of the Crocco-Busemann integral (as wall_stress)
-  DualD Tw, uvd;
-  if (ph.T_wall > 0.0) {
-    Tw = DualD(ph.T_wall);
-    const DualD b = (Taw - Tw) / (Tw * um);
-    const DualD a2 = r / (2.0 * ph.cp * Tw);
-    const DualD aa = sqrt(a2);
-    const DualD q = sqrt(b * b + 4.0 * a2);
-    uvd = (asin((2.0 * a2 * um - b) / q) + asin(b / q)) / aa;
+  const double Taw = T + r * u2 / (2.0 * ph.cp);
+  const bool iso = ph.T_wall > 0.0;
+  // the Van Driest transform (as wall_stress) with its derivatives: by um, by Tw
+  // at adiabatic walls, by T_aw at isothermal ones
+  double Tw, uvd, dum, dTw = 0.0, dTaw = 0.0;
+  if (iso) {
+    Tw = ph.T_wall;
+    const double b = (Taw - Tw) * ium / Tw;
+    const double a2 = r / (2.0 * ph.cp * Tw), aa = sqrt(a2);
+    const double q = sqrt(b * b + 4.0 * a2), iq = 1.0 / q;
+    const double X = (2.0 * a2 * um - b) * iq, Y = b * iq;
+    uvd = (asin(X) + asin(Y)) / aa;
+    const double cx = 1.0 / sqrt(1.0 - X * X);
+    const double db = (2.0 * aa * iq - cx * (1.0 + X * Y)) * iq / aa;
+    dum = 2.0 * aa * cx * iq - db * b * ium;
+    dTaw = db * ium / Tw;
   } else {
     Tw = Taw;
-    const DualD a = sqrt(r / (2.0 * ph.cp * Tw));
+    const double a = sqrt(r / (2.0 * ph.cp * Tw));
     uvd = asin(a * um) / a;
+    dum = 1.0 / sqrt(1.0 - a * um * (a * um));
+    dTw = 0.5 * (uvd - um * dum) / Tw;
   }
-  const DualD rhow = rho * T / Tw;
+  const double iTw = 1.0 / Tw, rhow = rho * T * iTw;
   // wall viscosity: constant, or Sutherland's law at the wall temperature
-  const DualD muw = ph.sutherland ? ph.suth_C * Tw * sqrt(Tw) / (Tw + ph.suth_S) : DualD(ph.mu);
-  const DualD nuw = muw / rhow;
-  if (!sv->have) {
-    sv->ut = solve_utau(ph.law, uvd.v, ph.hwm, nuw.v, ph.kappa, ph.B, ph.wm_maxit, &sv->ok);
-    // explicit variable of the law at the solution
-    const double wv = ph.law == 1 ? sv->ut * ph.hwm / nuw.v : uvd.v / sv->ut;
-    law_eval(ph.law, wv, ph.kappa, ph.B, &sv->L, &sv->wdL);
-    law_param_derivs(ph.law, wv, ph.kappa, ph.B, &sv->Lk, &sv->LB);
-    sv->have = true;
+  const double muw = ph.sutherland ? ph.suth_C * Tw * sqrt(Tw) / (Tw + ph.suth_S) : ph.mu;
+  const double nuw = muw / rhow;
+  const double ut = solve_utau(ph.law, uvd, ph.hwm, nuw, ph.kappa, ph.B, ph.wm_maxit, ok);
+  // explicit variable of the law at the solution
+  const double wv = ph.law == 1 ? ut * ph.hwm / nuw : uvd / ut;
+  double L, wdL, Lk, LB;
+  law_eval(ph.law, wv, ph.kappa, ph.B, &L, &wdL);
+  law_param_derivs(ph.law, wv, ph.kappa, ph.B, &Lk, &LB);
+  const double is = 1.0 / (L + wdL), alpha = L * is, beta = wdL * is;  // beta = 1 - alpha
+  const double tw = rhow * ut * ut * ium;  // tau = tw u_parallel
+  *tx = tw * ux;
+  // reverse
+  double gtw = gt[0] * ux + gt[1] * uy + gt[2] * uz, gTaw = 0.0;
+  if (iso) {  // q_w = -(cp / Pr) tw (T_aw - T_w)
+    const double c = -(ph.cp / ph.Pr) * gq;
+    gtw += c * (Taw - Tw);
+    gTaw = c * tw;
   }
-  const double ut = sv->ut, L = sv->L, wdL = sv->wdL, Lk = sv->Lk, LB = sv->LB;
-  const double Ft = 1.0 + wdL / L;
-  const double dlnRe = uvd.d / uvd.v - nuw.d / nuw.v;
-  const double dt = -((Lk * dk + LB * dB) / L - dlnRe) / Ft;
-  const double dut = ph.law == 1 ? ut * (dt + nuw.d / nuw.v) : ut * (uvd.d / uvd.v - dt);
-  const DualD utD(ut, dut);
-  const DualD tw = rhow * utD * utD / um;
-  tau[0] = tw * ux; tau[1] = tw * uy; tau[2] = tw * uz;
-  if (qw && ph.T_wall > 0.0) *qw = -(ph.cp / ph.Pr) * (rhow * utD * utD) * (Taw - Tw) / um;
+  const double Lm = gtw * tw;  // cotangent of ln tw = ln rho_w + 2 ln u_tau - ln um
+  const double gl = 2.0 * Lm, gth_c = (ph.law == 1 ? -is : is) * gl;
+  gth[0] = gth_c * Lk;
+  gth[1] = gth_c * LB;
+  const double guvd = gl * (ph.law == 1 ? alpha : beta) / uvd, gnu = gl * (ph.law == 1 ? beta : alpha);
+  const double grw = Lm - gnu;  // of ln rho_w (ln nu_w = ln mu_w - ln rho_w)
+  double gum = guvd * dum - Lm * ium;
+  if (iso) {
+    gTaw += guvd * dTaw;
+  } else {
+    gTaw = guvd * dTw - grw * iTw;
+    if (ph.sutherland) gTaw += gnu * (1.5 * iTw - 1.0 / (Tw + ph.suth_S));
+  }
+  gum += gTaw * r * um / ph.cp;
+  const double gT = gTaw + grw / T;
+  // tau = tw u_parallel, um = |u_parallel|, u_parallel = u - (u . n) n
+  const double c = gum * ium;
+  const double px = tw * gt[0] + c * ux, py = tw * gt[1] + c * uy, pz = tw * gt[2] + c * uz;
+  const double pn = px * nx + py * ny + pz * nz;
+  const double gu = px - pn * nx, gv = py - pn * ny, gw = pz - pn * nz;
+  const double gp = gT * ph.rcp_R * ir * ph.gm1;
+  gU[0] = (grw - gT * T - (gu * u + gv * v + gw * w)) * ir + 0.5 * gp * q2;
+  gU[1] = gu * ir - gp * u;
+  gU[2] = gv * ir - gp * v;
+  gU[3] = gw * ir - gp * w;
+  gU[4] = gp;
 }
 
 // ---------------------------------------------------------------------------
@@ -507,10 +499,11 @@ k_adj_face(const double* __restrict__ U, const double* __restrict__ lam, const M
 // k_adj_wall: nodes of the wall faces, 32 per block of ADJ_WALL_WARPS warps, a
 // node per lane (few nodes, long chains; see k_wall): the warps share the
 // planes of the sample's interpolation, the last takes the Riemann flux's
-// reverse mode, the first the law-of-the-wall solve, and then the warps 0 .. 6
-// one direction each of the wall model's derivative (the sample state's five
-// components, kappa, B).  Also accumulates g_theta = sum_nodes
-// (dFs/dtheta)^T gFs.
+// reverse mode, the first the wall model's (wall_stress_vjp).  Also accumulates
+// g_theta = sum_nodes (dFs/dtheta)^T gFs.  6912 nodes at N = 5: 158 us, 212 with
+// seven forward-mode sweeps (the sample state's components, kappa, B), one per
+// warp, which filled the FP64 pipe; what is left is the chain of the sample,
+// the solve and the sweep.
 // ---------------------------------------------------------------------------
 constexpr int ADJ_WALL_WARPS = 8;
 
@@ -521,7 +514,6 @@ k_adj_wall(const double* __restrict__ U, const double* __restrict__ lam, const M
            double* __restrict__ gUs, double* __restrict__ gtheta, int* __restrict__ status) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, W = ADJ_WALL_WARPS;
   __shared__ double sUs[W][5][32];
-  __shared__ WallSolve sSv[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int tid = blockIdx.x * 32 + lane;
   const bool valid = tid < m.n_wall * n2;
@@ -580,6 +572,7 @@ k_adj_wall(const double* __restrict__ U, const double* __restrict__ lam, const M
     for (int v = 0; v < 5; ++v) sUs[w][v][lane] = Us[v];
   }
   __syncthreads();
+  if (w != 0) return;
   double Us[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -587,34 +580,25 @@ k_adj_wall(const double* __restrict__ U, const double* __restrict__ lam, const M
 #pragma unroll
     for (int x = 1; x < W; ++x) Us[v] += sUs[x][v][lane];
   }
-  // direction w: d U_s,w (w < 5), d kappa (5), d B (6)
-  DualD Ud[5], tau[3], qwd;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) Ud[v] = DualD(Us[v], w == v ? 1.0 : 0.0);
-  const double dk = w == 5 ? 1.0 : 0.0, dB = w == 6 ? 1.0 : 0.0;
-  WallSolve sv{false};
-  if (w == 0) {
-    wall_stress_jvp(ph, Ud, dk, dB, nx, ny, nz, tau, &sv, &qwd);
-    sv.have = true;
-    sSv[lane] = sv;
-    if (!sv.ok && valid) atomicOr(status, ST_WM_NOCONV);
-  }
-  __syncthreads();
-  if (w > 6) return;
-  if (w > 0) {
-    sv = sSv[lane];
-    wall_stress_jvp(ph, Ud, dk, dB, nx, ny, nz, tau, &sv, &qwd);
-  }
   // (the wall flux: Fs_mom += tau s, Fs_E -= q_w s)
-  double gdot = (tau[0].d * gFs[1] + tau[1].d * gFs[2] + tau[2].d * gFs[3] - qwd.d * gFs[4]) * s;
-  if (w < 5) {
-    if (valid) gUs[slot * 5 + w] = gdot;
-  } else if (gtheta) {
-    // the warp's sum of a parameter's cotangent
-    gdot = valid ? gdot : 0.0;
+  const double gt[3] = {gFs[1] * s, gFs[2] * s, gFs[3] * s};
+  double g[5], gth[2], tx;
+  bool ok;
+  wall_stress_vjp(ph, Us, nx, ny, nz, gt, -gFs[4] * s, g, gth, &tx, &ok);
+  if (valid) {
+    if (!ok) atomicOr(status, ST_WM_NOCONV);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gdot += __shfl_down_sync(0xffffffffu, gdot, o);
-    if (lane == 0 && gdot != 0.0) atomicAdd(&gtheta[w - 5], gdot);
+    for (int v = 0; v < 5; ++v) gUs[slot * 5 + v] = g[v];
+  }
+  if (gtheta) {
+    // the warp's sum of the parameters' cotangents
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      double x = valid ? gth[c] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0 && x != 0.0) atomicAdd(&gtheta[c], x);
+    }
   }
 }
 
@@ -1357,23 +1341,17 @@ k_wall_loss(const double* __restrict__ U, const MeshDev<double> m, const PhysDev
         for (int v = 0; v < 5; ++v) Us[v] += ljk * row[v];
       }
     const double wgt = wq[slot] * inv_total;
-    WallSolve sv{false};
-    const int seeds = grad ? 7 : 1;
-#pragma unroll 1
-    for (int k = 0; k < seeds; ++k) {
-      DualD Ud[5];
+    const double gt[3] = {wgt, 0.0, 0.0};
+    double g[5], gth[2], tx;
+    bool ok;
+    wall_stress_vjp(ph, Us, nx, ny, nz, gt, 0.0, g, gth, &tx, &ok);
+    lv = wgt * tx;
+    if (grad) {
 #pragma unroll
-      for (int v = 0; v < 5; ++v) Ud[v] = DualD(Us[v], grad && k == v ? 1.0 : 0.0);
-      DualD tau[3];
-      wall_stress_jvp(ph, Ud, grad && k == 5 ? 1.0 : 0.0, grad && k == 6 ? 1.0 : 0.0, nx, ny, nz, tau, &sv);
-      if (k == 0) lv = wgt * tau[0].v;
-      if (grad) {
-        if (k < 5) gUs[(size_t)slot * 5 + k] = wgt * tau[0].d;
-        else if (k == 5) gk = wgt * tau[0].d;
-        else gb = wgt * tau[0].d;
-      }
+      for (int v = 0; v < 5; ++v) gUs[(size_t)slot * 5 + v] = g[v];
+      gk = gth[0]; gb = gth[1];
     }
-    if (!sv.ok) atomicOr(status, ST_WM_NOCONV);
+    if (!ok) atomicOr(status, ST_WM_NOCONV);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
