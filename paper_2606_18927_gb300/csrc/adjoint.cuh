@@ -145,43 +145,46 @@ static __device__ __noinline__ void wall_stress_vjp(const PhysDev& ph, const dou
 // ---------------------------------------------------------------------------
 // transposed primitive recoveries
 // ---------------------------------------------------------------------------
-// Q = (rho, u, v, w, p - p_ref, h): gU += (dQ/dU)^T gQ
+// Q = (rho, u, v, w, p - p_ref, h): gU += (dQ/dU)^T gQ.  1 / rho by rcp_pos, as
+// the forward recovery takes it (below 1 ulp, 4 FP64 FMAs; an IEEE division is
+// some ten operations, and the adjoint's face kernel is bound by the FP64 pipe:
+// with rcp_pos, sqrt_pos and shared reciprocals here and in face_flux_vjp it takes
+// 158 instead of 189 us on 10^3 elements at N = 7)
 __device__ __forceinline__ void prim_vjp(const double U[5], const PhysDev& ph, const double gQ[6], double gU[5]) {
-  const double ir = 1.0 / U[0];
+  const double ir = rcp_pos(U[0]);
   const double u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
-  const double q2 = u * u + v * v + w * w;
-  const double p = ph.gm1 * (U[4] - 0.5 * U[0] * q2);
+  const double p = ph.gm1 * (U[4] - 0.5 * (U[1] * u + U[2] * v + U[3] * w));
   const double h = (U[4] + p) * ir;
-  const double g1 = ph.gm1;
-  const double gp = gQ[4], gh = gQ[5];
-  gU[0] += gQ[0] - (gQ[1] * u + gQ[2] * v + gQ[3] * w) * ir + gp * 0.5 * g1 * q2 + gh * (0.5 * g1 * q2 - h) * ir;
-  gU[1] += gQ[1] * ir - gp * g1 * u - gh * g1 * u * ir;
-  gU[2] += gQ[2] * ir - gp * g1 * v - gh * g1 * v * ir;
-  gU[3] += gQ[3] * ir - gp * g1 * w - gh * g1 * w * ir;
-  gU[4] += gp * g1 + gh * (1.0 + g1) * ir;
+  const double a1 = gQ[1] * ir, a2 = gQ[2] * ir, a3 = gQ[3] * ir, ah = gQ[5] * ir;
+  const double gp = ph.gm1 * (gQ[4] + ah);  // of E - |m|^2 / (2 rho)
+  gU[0] += gQ[0] - (a1 * u + a2 * v + a3 * w) + 0.5 * gp * (u * u + v * v + w * w) - ah * h;
+  gU[1] += a1 - gp * u;
+  gU[2] += a2 - gp * v;
+  gU[3] += a3 - gp * w;
+  gU[4] += gp + ah;
 }
 
 // the body force's source S_E = f . m / rho: gU += (dS/dU)^T lam
 __device__ __forceinline__ void source_vjp(const double U[5], const PhysDev& ph, double l4, double gU[5]) {
   if (ph.f[0] == 0.0 && ph.f[1] == 0.0 && ph.f[2] == 0.0) return;
-  const double ir = 1.0 / U[0];
+  const double ir = rcp_pos(U[0]);
   gU[0] -= l4 * (ph.f[0] * U[1] + ph.f[1] * U[2] + ph.f[2] * U[3]) * ir * ir;
   gU[1] += l4 * ph.f[0] * ir; gU[2] += l4 * ph.f[1] * ir; gU[3] += l4 * ph.f[2] * ir;
 }
 
 // W = (u, v, w, T): gU += (dW/dU)^T gW
 __device__ __forceinline__ void vt_vjp(const double U[5], const PhysDev& ph, const double gW[4], double gU[5]) {
-  const double ir = 1.0 / U[0];
+  const double ir = rcp_pos(U[0]);
   const double u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
-  const double q2 = u * u + v * v + w * w;
-  const double p = ph.gm1 * (U[4] - 0.5 * U[0] * q2);
-  const double T = p * ph.rcp_R * ir;
-  const double c = ph.gm1 * ph.rcp_R * ir;  // dT/dE
-  gU[0] += -(gW[0] * u + gW[1] * v + gW[2] * w) * ir + gW[3] * (0.5 * q2 * c - T * ir);
-  gU[1] += gW[0] * ir - gW[3] * c * u;
-  gU[2] += gW[1] * ir - gW[3] * c * v;
-  gU[3] += gW[2] * ir - gW[3] * c * w;
-  gU[4] += gW[3] * c;
+  const double p = ph.gm1 * (U[4] - 0.5 * (U[1] * u + U[2] * v + U[3] * w));
+  const double a1 = gW[0] * ir, a2 = gW[1] * ir, a3 = gW[2] * ir;
+  const double aT = gW[3] * ph.rcp_R * ir;  // of p (T = p / (rho R))
+  const double gp = ph.gm1 * aT;
+  gU[0] += 0.5 * gp * (u * u + v * v + w * w) - (a1 * u + a2 * v + a3 * w) - aT * (p * ir);
+  gU[1] += a1 - gp * u;
+  gU[2] += a2 - gp * v;
+  gU[3] += a3 - gp * w;
+  gU[4] += gp;
 }
 
 // ---------------------------------------------------------------------------
@@ -289,7 +292,8 @@ static __device__ void face_flux_vjp(const PhysDev& ph, const double UA[5], cons
   if (ph.surf_flux == 1) {
     // F -= lam (U_B - U_A), lam = max(|u_n| + c) / 2 over the sides
     const double pref = ph.p_ref, gam = ph.gamma;
-    const double cA = ::sqrt(gam * (A.p + pref) / A.rho), cB = ::sqrt(gam * (B.p + pref) / B.rho);
+    const double irA = rcp_pos(A.rho), irB = rcp_pos(B.rho);
+    const double cA = sqrt_pos(gam * (A.p + pref) * irA), cB = sqrt_pos(gam * (B.p + pref) * irB);
     const double unA = A.u * nx + A.v * ny + A.w * nz, unB = B.u * nx + B.v * ny + B.w * nz;
     const double lA = ::fabs(unA) + cA, lB = ::fabs(unB) + cB;
     const double lam = 0.5 * (lA >= lB ? lA : lB);
@@ -303,49 +307,49 @@ static __device__ void face_flux_vjp(const PhysDev& ph, const double UA[5], cons
     const bool a_side = lA >= lB;
     double* q = a_side ? qA : qB;
     const double un = a_side ? unA : unB, c = a_side ? cA : cB;
-    const Prim<double>& X = a_side ? A : B;
+    const double ir = a_side ? irA : irB;
     const double gl = 0.5 * glam, gn = gl * sgn1(un);
     q[1] += gn * nx; q[2] += gn * ny; q[3] += gn * nz;
     // c = sqrt(gamma (p + p_ref) / rho)
-    q[4] += gl * gam / (2.0 * c * X.rho);
-    q[0] -= gl * c / (2.0 * X.rho);
+    q[4] += gl * gam * 0.5 * ir * rcp_pos(c);
+    q[0] -= gl * c * 0.5 * ir;
   } else if (ph.surf_flux == 2) {
     // forward sweep of the Roe dissipation with Harten's fix (F -= D / 2)
     const double gam = ph.gamma;
-    const double sA = ::sqrt(A.rho), sB = ::sqrt(B.rho);
-    const double is = 1.0 / (sA + sB);
+    const double sA = sqrt_pos(A.rho), sB = sqrt_pos(B.rho);
+    const double is = rcp_pos(sA + sB);
     const double rt = sA * sB;
     const double Nu = sA * A.u + sB * B.u, Nv = sA * A.v + sB * B.v, Nw = sA * A.w + sB * B.w;
     const double NH = sA * A.h + sB * B.h;
     const double u = Nu * is, v = Nv * is, w = Nw * is, H = NH * is;
     const double q2 = u * u + v * v + w * w;
     const double c2 = (gam - 1.0) * (H - 0.5 * q2);
-    const double c = ::sqrt(c2);
+    const double c = sqrt_pos(c2), ic2 = rcp_pos(c2), ic = c * ic2;
     const double un = u * nx + v * ny + w * nz;
     const double dr = B.rho - A.rho, dp = B.p - A.p;
     const double du = B.u - A.u, dv = B.v - A.v, dw = B.w - A.w;
     const double dun = du * nx + dv * ny + dw * nz;
-    const double i2c2 = 0.5 / c2;
+    const double i2c2 = 0.5 * ic2;
     const double P1 = dp - rt * c * dun, P5 = dp + rt * c * dun;
-    const double a1 = P1 * i2c2, a2 = dr - dp / c2, a5 = P5 * i2c2;
+    const double a1 = P1 * i2c2, a2 = dr - dp * ic2, a5 = P5 * i2c2;
     const double l1o = ::fabs(un - c), l2 = ::fabs(un), l5o = ::fabs(un + c);
-    const double del = 0.1 * c;
+    const double del = 0.1 * c, idel = 10.0 * ic;
     const bool h1 = l1o < del, h5 = l5o < del;
-    const double l1 = h1 ? (l1o * l1o + del * del) / (2.0 * del) : l1o;
-    const double l5 = h5 ? (l5o * l5o + del * del) / (2.0 * del) : l5o;
+    const double l1 = h1 ? 0.5 * (l1o * l1o * idel + del) : l1o;
+    const double l5 = h5 ? 0.5 * (l5o * l5o * idel + del) : l5o;
     const double w1 = l1 * a1, w2 = l2 * a2, w5 = l5 * a5, ws = l2 * rt;
     const double dut = du - dun * nx, dvt = dv - dun * ny, dwt = dw - dun * nz;
     const double X4 = u * du + v * dv + w * dw - un * dun;
     // backward sweep
     const double g0 = -0.5 * gF[0], g1 = -0.5 * gF[1], g2 = -0.5 * gF[2], g3 = -0.5 * gF[3], g4 = -0.5 * gF[4];
     const double g13 = g1 * nx + g2 * ny + g3 * nz;  // sum_d gD_d n_d
-    double gw1 = g0 + g1 * (u - c * nx) + g2 * (v - c * ny) + g3 * (w - c * nz) + g4 * (H - c * un);
-    double gw2 = g0 + g1 * u + g2 * v + g3 * w + g4 * (0.5 * q2);
-    double gw5 = g0 + g1 * (u + c * nx) + g2 * (v + c * ny) + g3 * (w + c * nz) + g4 * (H + c * un);
+    const double gu_ = g0 + g1 * u + g2 * v + g3 * w;
+    const double E0 = gu_ + g4 * H, Ec = c * (g13 + g4 * un);
+    const double gw1 = E0 - Ec, gw2 = gu_ + g4 * (0.5 * q2), gw5 = E0 + Ec;
     const double gws = g1 * dut + g2 * dvt + g3 * dwt + g4 * X4;
     const double wsum = w1 + w2 + w5;
     double gu = g1 * wsum + g4 * ws * du, gv = g2 * wsum + g4 * ws * dv, gw = g3 * wsum + g4 * ws * dw;
-    double gc = g13 * (w5 - w1) + g4 * un * (w5 - w1);
+    double gc = (g13 + g4 * un) * (w5 - w1);
     double gun = g4 * c * (w5 - w1) - g4 * ws * dun;
     double gH = g4 * (w1 + w5);
     double gq2 = g4 * 0.5 * w2;
@@ -357,36 +361,36 @@ static __device__ void face_flux_vjp(const PhysDev& ph, const double UA[5], cons
     const double ga1 = gw1 * l1, ga2 = gw2 * l2, ga5 = gw5 * l5;
     // Harten: l = (l_o^2 + del^2) / (2 del) below del
     double gdel = 0.0;
-    if (h1) { gdel += gl1 * (0.5 - l1o * l1o / (2.0 * del * del)); gl1 *= l1o / del; }
-    if (h5) { gdel += gl5 * (0.5 - l5o * l5o / (2.0 * del * del)); gl5 *= l5o / del; }
+    if (h1) { const double x = l1o * idel; gdel += gl1 * (0.5 - 0.5 * x * x); gl1 *= x; }
+    if (h5) { const double x = l5o * idel; gdel += gl5 * (0.5 - 0.5 * x * x); gl5 *= x; }
     gc += 0.1 * gdel;
     // l1 = |un - c|, l2 = |un|, l5 = |un + c|
     const double s1 = sgn1(un - c), s5 = sgn1(un + c);
     gun += gl1 * s1 + gl2 * sgn1(un) + gl5 * s5;
     gc += -gl1 * s1 + gl5 * s5;
     // a1 = P1 i2c2, a5 = P5 i2c2, a2 = dr - dp / c2
-    double gdp = (ga1 + ga5) * i2c2 - ga2 / c2;
+    double gdp = (ga1 + ga5) * i2c2 - ga2 * ic2;
     const double gdr = ga2;
     const double gP = (ga5 - ga1) * i2c2;  // d/d(rt c dun) of P5 and -P1
     grt += gP * c * dun;
     gc += gP * rt * dun;
     gdun += gP * rt * c;
     const double gi2c2 = ga1 * P1 + ga5 * P5;
-    double gc2 = ga2 * dp / (c2 * c2) - gi2c2 * 0.5 / (c2 * c2);
+    double gc2 = (ga2 * dp - 0.5 * gi2c2) * ic2 * ic2;
     // dun, un
     gdu += gdun * nx; gdv += gdun * ny; gdw += gdun * nz;
     gu += gun * nx; gv += gun * ny; gw += gun * nz;
     // c = sqrt(c2), c2 = (gamma - 1)(H - q2 / 2), q2 = |u|^2
-    gc2 += gc / (2.0 * c);
+    gc2 += 0.5 * gc * ic;
     gH += gc2 * (gam - 1.0);
     gq2 -= 0.5 * (gam - 1.0) * gc2;
     gu += 2.0 * u * gq2; gv += 2.0 * v * gq2; gw += 2.0 * w * gq2;
     // Roe averages x = N_x is, N_x = sA x_A + sB x_B
-    const double gis = gu * Nu + gv * Nv + gw * Nw + gH * NH;
-    double gsA = (gu * A.u + gv * A.v + gw * A.w + gH * A.h) * is + grt * sB - gis * is * is;
-    double gsB = (gu * B.u + gv * B.v + gw * B.w + gH * B.h) * is + grt * sA - gis * is * is;
-    qA[1] += gu * sA * is; qA[2] += gv * sA * is; qA[3] += gw * sA * is; qA[5] += gH * sA * is;
-    qB[1] += gu * sB * is; qB[2] += gv * sB * is; qB[3] += gw * sB * is; qB[5] += gH * sB * is;
+    const double wA = sA * is, wB = sB * is, gis = (gu * Nu + gv * Nv + gw * Nw + gH * NH) * is;
+    const double gsA = (gu * A.u + gv * A.v + gw * A.w + gH * A.h - gis) * is + grt * sB;
+    const double gsB = (gu * B.u + gv * B.v + gw * B.w + gH * B.h - gis) * is + grt * sA;
+    qA[1] += gu * wA; qA[2] += gv * wA; qA[3] += gw * wA; qA[5] += gH * wA;
+    qB[1] += gu * wB; qB[2] += gv * wB; qB[3] += gw * wB; qB[5] += gH * wB;
     // jumps
     qB[0] += gdr; qA[0] -= gdr;
     qB[4] += gdp; qA[4] -= gdp;
@@ -394,8 +398,8 @@ static __device__ void face_flux_vjp(const PhysDev& ph, const double UA[5], cons
     qB[2] += gdv; qA[2] -= gdv;
     qB[3] += gdw; qA[3] -= gdw;
     // s = sqrt(rho)
-    qA[0] += gsA / (2.0 * sA);
-    qB[0] += gsB / (2.0 * sB);
+    qA[0] += 0.5 * gsA * sA * rcp_pos(A.rho);
+    qB[0] += 0.5 * gsB * sB * rcp_pos(B.rho);
   }
   prim_vjp(UA, ph, qA, gUA);
   prim_vjp(UB, ph, qB, gUB);
@@ -1054,7 +1058,7 @@ k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, cons
       if constexpr (SUTH) {
         const double Tn = sW[3 * n3 + p];
         mu = sutherland<double>(ph, Tn);
-        dmu = mu * (1.5 / Tn - 1.0 / (Tn + ph.suth_S));
+        dmu = mu * (1.5 * rcp_pos(Tn) - rcp_pos(Tn + ph.suth_S));
         kc = mu * ph.cp_Pr;
       }
       const double div = q[0][0] + q[1][1] + q[2][2];
@@ -1214,7 +1218,7 @@ k_adj_element(const double* __restrict__ U, const double* __restrict__ lam, cons
 }
 
 // ---------------------------------------------------------------------------
-// k_adj_gather: one thread per node; adds the face kernels' state cotangents
+// k_adj_gather: one thread per node (interior nodes leave at once); adds the face kernels' state cotangents
 // and the neighbours' lifting cotangents (through W(U) of this node).
 // ---------------------------------------------------------------------------
 template <int N>
@@ -1228,6 +1232,7 @@ k_adj_gather(const double* __restrict__ U, const MeshDev<double> m, const PhysDe
   if (g >= S) return;
   const int e = (int)(g / n3), t = (int)(g - (size_t)e * n3);
   const int i = t % n, j = (t / n) % n, k = t / n2;
+  if (i > 0 && i < N && j > 0 && j < N && k > 0 && k < N) return;  // no face: nothing to add
   double add[5] = {0, 0, 0, 0, 0}, gW[4] = {0, 0, 0, 0};
   bool any_w = false;
   auto face = [&](int l, int ab) {
