@@ -343,9 +343,9 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     kel<<<a.K, AdjShape<N>::THREADS, smem, s>>>(a.Uin, a.lam, m, ph, tab, a.gGf, a.gV, a.gU, a.gWf, sendU);
   }
   if (phase == 4 || phase == 14) {
-    const long long S = (long long)a.K * n3;
-    const int threads = spread_threads(S, 256);
-    k_adj_gather<N><<<spread_blocks(S, threads), threads, 0, s>>>(a.Uin, m, ph, a.gUf, a.gWf,
+    const long long work = (long long)a.K * SurfaceNodes<N>::COUNT;
+    const int threads = spread_threads(work, 256);
+    k_adj_gather<N><<<spread_blocks(work, threads), threads, 0, s>>>(a.Uin, m, ph, a.gUf, a.gWf,
                                                                  part ? a.halo_U : nullptr, a.gU);
     if (a.n_wall > 0 && ph.viscous) {
       k_adj_scatter<N><<<(unsigned)a.n_wall, std::min(256, (n3 + 31) / 32 * 32), 0, s>>>(m, a.gUs, a.gU);
