@@ -1298,40 +1298,50 @@ k_adj_gather(const double* __restrict__ U, const MeshDev<double> m, const PhysDe
 
 // ---------------------------------------------------------------------------
 // k_adj_scatter: wall-model sample cotangents to the sample elements' nodes,
-// one block per wall face.  A face's nodes sample one element or a few: for
-// each, a thread adds up its node's share of all of them and gives it to gU by
-// one atomic addition (one per wall node and sample-element node before, 86 us
-// on the 12 x 6 x 8 channel at N = 5).
+// SCATTER_THREADS of them per block and as many blocks per wall face.  A face's
+// nodes sample one element or a few: for each, a thread adds up its node's share
+// of all of them and gives it to gU by one atomic addition (one per wall node
+// and sample-element node before, 86 us on the 12 x 6 x 8 channel at N = 5).
+// Latency-bound with one block per face, which also searched the list of sample
+// elements in every thread (48 us); the blocks now cover a face's nodes side by
+// side and each thread marks one entry of the list: 33 us.
 // ---------------------------------------------------------------------------
+constexpr int SCATTER_THREADS = 64;
+
 template <int N>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(SCATTER_THREADS)
 k_adj_scatter(const MeshDev<double> m, const double* __restrict__ gUs, double* __restrict__ gU) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
   __shared__ double sL[n2][3 * n], sG[n2][5];
-  __shared__ int sE[n2];
+  __shared__ int sE[n2], sFirst[n2];
   const size_t S = (size_t)m.K * n3, slot0 = (size_t)blockIdx.x * n2;
   for (int x = threadIdx.x; x < n2 * 3 * n; x += blockDim.x) (&sL[0][0])[x] = m.ws_lag[slot0 * 3 * n + x];
   for (int x = threadIdx.x; x < n2 * 5; x += blockDim.x) (&sG[0][0])[x] = gUs[slot0 * 5 + x];
   for (int x = threadIdx.x; x < n2; x += blockDim.x) sE[x] = chk_idx(m.ws_elem[slot0 + x], m.K, m.status);
   __syncthreads();
+  for (int x = threadIdx.x; x < n2; x += blockDim.x) {
+    bool first = true;  // the first node that samples an element takes all that do
+    for (int y = 0; y < x; ++y) first = first && sE[y] != sE[x];
+    sFirst[x] = first;
+  }
+  __syncthreads();
+  const int p = blockIdx.y * SCATTER_THREADS + threadIdx.x;
+  if (p >= n3) return;
+  const int i = p % n, j = (p / n) % n, k = p / n2;
   for (int q0 = 0; q0 < n2; ++q0) {
+    if (!sFirst[q0]) continue;
     const int es = sE[q0];
-    bool first = true;  // the first node that samples es takes all that do
-    for (int x = 0; x < q0; ++x) first = first && sE[x] != es;
-    if (!first) continue;
-    for (int p = threadIdx.x; p < n3; p += blockDim.x) {
-      const int i = p % n, j = (p / n) % n, k = p / n2;
-      double g[5] = {0, 0, 0, 0, 0};
-      for (int x = q0; x < n2; ++x) {
-        if (sE[x] != es) continue;
-        const double wgt = sL[x][i] * sL[x][n + j] * sL[x][2 * n + k];
+    double g[5] = {0, 0, 0, 0, 0};
+#pragma unroll 4
+    for (int x = q0; x < n2; ++x) {
+      if (sE[x] != es) continue;
+      const double wgt = sL[x][i] * sL[x][n + j] * sL[x][2 * n + k];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) g[v] = fma(wgt, sG[x][v], g[v]);
-      }
-#pragma unroll
-      for (int v = 0; v < 5; ++v)
-        if (g[v] != 0.0) atomicAdd(&gU[v * S + (size_t)es * n3 + p], g[v]);
+      for (int v = 0; v < 5; ++v) g[v] = fma(wgt, sG[x][v], g[v]);
     }
+#pragma unroll
+    for (int v = 0; v < 5; ++v)
+      if (g[v] != 0.0) atomicAdd(&gU[v * S + (size_t)es * n3 + p], g[v]);
   }
 }
 

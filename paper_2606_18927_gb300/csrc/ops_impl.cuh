@@ -348,7 +348,8 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     k_adj_gather<N><<<spread_blocks(work, threads), threads, 0, s>>>(a.Uin, m, ph, a.gUf, a.gWf,
                                                                  part ? a.halo_U : nullptr, a.gU);
     if (a.n_wall > 0 && ph.viscous) {
-      k_adj_scatter<N><<<(unsigned)a.n_wall, std::min(256, (n3 + 31) / 32 * 32), 0, s>>>(m, a.gUs, a.gU);
+      k_adj_scatter<N><<<dim3((unsigned)a.n_wall, (n3 + SCATTER_THREADS - 1) / SCATTER_THREADS), SCATTER_THREADS, 0, s>>>(
+          m, a.gUs, a.gU);
     }
   }
   return (int)cudaGetLastError();
@@ -371,7 +372,8 @@ static int run_wall_loss_typed(const OpArgs& a, const PhysDev& ph, const double*
   if (grad) {
     const long long S = 5LL * a.K * n3;
     k_axpby<<<(unsigned)((S + 255) / 256), 256, 0, s>>>(S, 0.0, a.gU, 0.0, a.gU);
-    k_adj_scatter<N><<<(unsigned)a.n_wall, std::min(256, (n3 + 31) / 32 * 32), 0, s>>>(m, a.gUs, a.gU);
+    k_adj_scatter<N><<<dim3((unsigned)a.n_wall, (n3 + SCATTER_THREADS - 1) / SCATTER_THREADS), SCATTER_THREADS, 0, s>>>(
+          m, a.gUs, a.gU);
   }
   return (int)cudaGetLastError();
 }
