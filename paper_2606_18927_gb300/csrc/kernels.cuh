@@ -72,6 +72,20 @@ constexpr int resident_ctas(int threads, int smem, int resident) {
   return n < 1 ? 1 : (n > 32 ? 32 : n);
 }
 
+// The FP32-mixed kernels of `threads` threads exist twice: dense, with the 40
+// registers of 1536 resident threads, and with the 70 to 90 that they need
+// without spills (some 819 threads per SM).  The first pays when the K elements
+// are more than those CTAs, by 1.1 to 1.6; below it the spills (36 to 144 bytes)
+// only lengthen the kernels: FP32-mixed steps of 64 to 729 elements were up to
+// 13 % slower (N = 5, entropy-conserving, 6^3 elements: k_volume 14.8 against 16.8
+// us).  The entropy-conserving kernel spills most and needs five elements per SM
+// at least (dense against the other: N = 4 1.02 at 8.8 elements per SM, N = 5 0.96
+// at 4.8 and 1.02 at 18, N = 6 0.88 at 3.4 and 1.0 at 11).
+constexpr bool dense_mesh(long long K, int threads, bool ec) {
+  const int ctas = 819 / threads, least = ec ? 5 : 1;
+  return K > 152LL * (ctas > least ? ctas : least);
+}
+
 // a fixed-point number h 2^31 + l (volume_fx.cuh)
 struct Fx {
   int h, l;
@@ -1410,17 +1424,17 @@ struct LiftPk {
 };
 
 // Resident CTAs per SM asked of the register allocator for the lifting kernel:
-// two in FP64 (bound by the FP64 pipe), FP32 resident_ctas (its line phases
+// two in FP64 (bound by the FP64 pipe) and on small meshes (dense_mesh), else FP32 resident_ctas (its line phases
 // leave the other threads waiting at a barrier, which more CTAs cover: N = 5
 // 0.195 -> 0.177 ms at 26^3, N = 3 0.248 -> 0.157 at 40^3)
-template <int N, typename R>
+template <int N, typename R, bool DENSE>
 constexpr int lift_min_blocks() {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
-  return std::is_same<R, float>::value ? resident_ctas(n3, (16 * n3 + 26 * n2 + n) * 4, 1536) : (n3 > 512 ? 1 : 2);
+  return std::is_same<R, float>::value && DENSE ? resident_ctas(n3, (16 * n3 + 26 * n2 + n) * 4, 1536) : (n3 > 512 ? 1 : 2);
 }
 
-template <int N, typename R>
-__global__ void __launch_bounds__((N + 1) * (N + 1) * (N + 1), (lift_min_blocks<N, R>()))
+template <int N, typename R, bool DENSE = false>
+__global__ void __launch_bounds__((N + 1) * (N + 1) * (N + 1), (lift_min_blocks<N, R, DENSE>()))
 k_lift(const double* __restrict__ U, const MeshDev<R> m, const PhysDev ph, const Tables<N> tab,
        const LiftPk<N> pk, R* __restrict__ Rv, R* __restrict__ Gf) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
@@ -2588,10 +2602,14 @@ __device__ __forceinline__ void stage_node(R* sQ, int ts, const Prim<R>& q, cons
   }
 }
 
-template <int N, typename R, int MODE, bool EC>
-__global__ void __launch_bounds__(VolShape<N>::THREADS,
-                                  (resident_ctas(VolShape<N>::THREADS,
-                                                 (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4, 1536)))
+template <int N, bool EC, bool DENSE>
+constexpr int vol_min_blocks() {
+  constexpr int T = VolShape<N>::THREADS;
+  return DENSE ? resident_ctas(T, (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4, 1536) : (T > 512 ? 1 : 2);
+}
+
+template <int N, typename R, int MODE, bool EC, bool DENSE>
+__global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, EC, DENSE>()))
 k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, const Tables<N> tab,
          const R* __restrict__ Rv, const R* __restrict__ Fs, double* __restrict__ Out,
          double* __restrict__ dU, double* __restrict__ Uout, const StageArgs st, int* __restrict__ status) {

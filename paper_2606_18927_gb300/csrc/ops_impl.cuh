@@ -170,7 +170,11 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   const size_t smem_vol = (size_t)(ph.vol_flux == 2 ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * sizeof(R);
   constexpr int vol_threads = VolShape<N>::THREADS;
   // per device and cheap: set on every call
-  cudaFuncSetAttribute(k_lift<N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_lift);
+  auto kl = k_lift<N, R>;
+  if constexpr (std::is_same<R, float>::value) {
+    if (dense_mesh(a.K, n3, false)) kl = k_lift<N, R, true>;
+  }
+  cudaFuncSetAttribute(kl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_lift);
   const bool ec = ph.vol_flux == 2;
   const int phase = a.phase ? a.phase : 7;
   const unsigned halo_blocks = (unsigned)(((long long)a.n_halo * n2 + 255) / 256);
@@ -220,7 +224,7 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
           done = true;
         }
       }
-      if (!done) k_lift<N, R><<<a.K, n3, smem_lift, s>>>(a.Uin, m, ph, tab, make_lift_pk<N>(tab), Rv, Gf);
+      if (!done) kl<<<a.K, n3, smem_lift, s>>>(a.Uin, m, ph, tab, make_lift_pk<N>(tab), Rv, Gf);
     }
     if (a.ev) cudaEventRecord(a.ev[1], s);
     if (a.n_halo > 0 && a.send_G && ph.viscous)
@@ -268,8 +272,13 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_vol);
       kern<<<a.K, vol_threads, smem_vol, s>>>(a.Uin, m, ph, tab, Rv, Fs, a.Out, a.dU, a.Uout, st, a.status);
     };
-    if (ec) volume(a.mode == 0 ? k_volume<N, R, 0, true> : k_volume<N, R, 1, true>);
-    else volume(a.mode == 0 ? k_volume<N, R, 0, false> : k_volume<N, R, 1, false>);
+    auto form = [&](auto dense) {
+      constexpr bool D = decltype(dense)::value;
+      if (ec) volume(a.mode == 0 ? k_volume<N, R, 0, true, D> : k_volume<N, R, 1, true, D>);
+      else volume(a.mode == 0 ? k_volume<N, R, 0, false, D> : k_volume<N, R, 1, false, D>);
+    };
+    if (dense_mesh(a.K, VolShape<N>::THREADS, ec)) form(std::true_type{});
+    else form(std::false_type{});
   }
   if (a.ev) cudaEventRecord(a.ev[6], s);
   return (int)cudaGetLastError();
