@@ -28,7 +28,7 @@
 // the mixed form); the state U, dU, the pressure recovery and the RK update
 // are always double.  The FP32 form also keeps per-stage FP32 primitives
 // relative to a reference state (k_prim32 / the stage epilogue) and, with the
-// Pirozzoli flux, sums flux differences (flux_delta_pair16, flux_delta_pair) instead of fluxes.
+// Pirozzoli flux, sums flux differences (flux_delta) instead of fluxes.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -810,25 +810,17 @@ struct NodeF {
 //   16 G'_m = 8 G'_rho (u_i + u_m) + 4 (rho_i (u_i.A) du + dp A),
 //   16 G'_E = 8 G'_rho (h_i + h_m) + 4 rho_i (u_i.A) dh,
 // gi receives 16 G' (its mass row 8 G'), against DVS / 16 (and DVS / 8).  G'(m -> i)
-// has the differences' signs turned; gm receives its negative.  u_i.A is formed
-// as 2 u_i.a_i + u_i.(a_m - a_i) from the node's own product uia: its rounding
-// then is the same in all of a node's pairs and cancels like a derivative (a
-// fresh u_i.A per pair raised the momentum rows' error by up to 6 % on curved
-// meshes, u_m.A as u_i.A + du.A by 10 to 20 %).  Issue-bound: both
-// orientations share sums, differences and pressure terms; against each formed
-// from {a} and its own products, a step of 24^3 elements at N = 7 takes 4.99
-// instead of 5.31 ms.  Error against the oracle: density and energy rows 4 to
-// 10 % lower (density at even N: equal), momentum rows equal to 1 to 2 %.
-__device__ __forceinline__ void flux_delta_pair16(const NodeF& i, const NodeF& m, float ai0, float ai1, float ai2,
-                                                  float am0, float am1, float am2, float uia, float uma, float rho2,
-                                                  float h2, float gi[5], float gm[5]) {
-  const float A0 = ai0 + am0, A1 = ai1 + am1, A2 = ai2 + am2;
-  const float e0 = am0 - ai0, e1 = am1 - ai1, e2 = am2 - ai2;
+// has the differences' signs turned; gm receives its negative.  u_m.A is formed
+// from u_m, not as u_i.A + du.A: its rounding then is the same in all of a node's
+// pairs on an affine element and cancels like a derivative (the sum raised the
+// momentum rows' error by 10 to 20 %).  The two orientations take 55 FP32
+// operations (about 90 when each was formed from {a} and its own products).
+__device__ __forceinline__ void flux_delta_pair16(const NodeF& i, const NodeF& m, float A0, float A1, float A2,
+                                                  float rho2, float h2, float gi[5], float gm[5]) {
   const float du = (m.u - i.u) + (m.ul - i.ul), dv = (m.v - i.v) + (m.vl - i.vl), dw = (m.w - i.w) + (m.wl - i.wl);
   const float dr = m.rho - i.rho, dp4 = 4.0f * (m.p - i.p), dh = m.h - i.h;
   const float su = i.u + m.u, sv = i.v + m.v, sw = i.w + m.w, sh = (i.h + m.h) + h2;
-  const float ua = fmaf(2.0f, uia, i.u * e0 + i.v * e1 + i.w * e2);
-  const float um = fmaf(2.0f, uma, -(m.u * e0 + m.v * e1 + m.w * e2));
+  const float ua = i.u * A0 + i.v * A1 + i.w * A2;
   const float da = du * A0 + dv * A1 + dw * A2;
   const float t = dr * fmaf(2.0f, ua, da);
   const float P0 = dp4 * A0, P1 = dp4 * A1, P2 = dp4 * A2;
@@ -841,7 +833,7 @@ __device__ __forceinline__ void flux_delta_pair16(const NodeF& i, const NodeF& m
     gi[4] = fmaf(g, sh, q * dh);
   }
   {
-    const float r = fmaf(2.0f, m.rho, rho2), g = fmaf(r, da, t), q = 2.0f * r * um;
+    const float r = fmaf(2.0f, m.rho, rho2), g = fmaf(r, da, t), q = 2.0f * r * (m.u * A0 + m.v * A1 + m.w * A2);
     // the negatives (the partner lane subtracts)
     gm[0] = g;
     gm[1] = fmaf(g, su, fmaf(q, du, P0));
@@ -2368,9 +2360,8 @@ __device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDe
     const int ms = vslot<N, R>(me);
     const VolNode<R> A = load_node(me, dir);
     // FP32 difference form: the low parts of this lane's node velocity
-    float Aul = 0.f, Avl = 0.f, Awl = 0.f, uia = 0.f;
+    float Aul = 0.f, Avl = 0.f, Awl = 0.f;
     if constexpr (F32 && !EC) {
-      uia = A.u * A.a0 + A.v * A.a1 + A.w * A.a2;
       if (dif) { Aul = sQ[7 * n3 + ms]; Avl = sQ[8 * n3 + ms]; Awl = sQ[9 * n3 + ms]; }
     }
     R acc[5];
@@ -2406,11 +2397,11 @@ __device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDe
           const int lq = base + pm;
           auto sh = [&](float x) { return __shfl_sync(0xffffffffu, x, lq); };
           const NodeF mq{sh(A.rho), sh(A.u), sh(A.v), sh(A.w), sh(A.p4), sh(A.hh), sh(Aul), sh(Avl), sh(Awl)};
-          const float aq0 = sh(A.a0), aq1 = sh(A.a1), aq2 = sh(A.a2);
+          const float A0 = A.a0 + sh(A.a0), A1 = A.a1 + sh(A.a1), A2 = A.a2 + sh(A.a2);
           const float rho2 = 2.0f * ph.f32c.rho_ref, h2 = 2.0f * ph.f32c.h_ref;
           float G[5], Gq[5];
           const float c8 = sC8[pos * n + pm], c16 = sC16[pos * n + pm];
-          flux_delta_pair16(mi, mq, A.a0, A.a1, A.a2, aq0, aq1, aq2, uia, sh(uia), rho2, h2, G, Gq);
+          flux_delta_pair16(mi, mq, A0, A1, A2, rho2, h2, G, Gq);
           acc[0] = fmaf(c8, G[0], acc[0]);
 #pragma unroll
           for (int v = 1; v < 5; ++v) acc[v] = fmaf(c16, G[v], acc[v]);
@@ -2628,7 +2619,7 @@ k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, c
   const size_t S = (size_t)m.K * n3;
   const bool kg = ph.vol_flux == 1;
   // FP32 Pirozzoli form: flux differences G(i -> m) and per-side surface
-  // differences F* - F(U_i) (see flux_delta_pair16)
+  // differences F* - F(U_i) (see flux_delta)
   const bool dif = std::is_same<R, float>::value && !EC && ph.fs_diff;
   for (int x = t; x < n2; x += T) {
     sC8[x] = (R)tab.DVS8[x];

@@ -1,6 +1,7 @@
-"""The FP32-mixed volume sums: every degree, odd and even line lengths, against
-the oracle (the form's bound, 1e-5 relative L2), and results written over their
-input, bitwise the same as into an array of their own."""
+"""The FP32-mixed volume sums by line threads (volume_line.cuh): every degree
+against the oracle (the form's bound, 1e-5 relative L2), and results written over
+their input (the sums' storage must not be the state that the source term still
+reads), bitwise the same as into an array of their own."""
 import numpy as np
 import pytest
 
