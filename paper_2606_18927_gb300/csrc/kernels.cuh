@@ -802,45 +802,25 @@ struct NodeF {
   float ul, vl, wl;  // low parts of the velocity (u = u + ul, see prim32_shifted)
 };
 
-// The volume kernel's pairs, both nodes in the storage form of the FP32
-// primitives (rho, h shifted by rho_ref, h_ref: the differences come from the
-// shifted values, the full density and enthalpy are rebuilt where they
-// multiply).  With A = a_i + a_m and the two nodes' sums and differences,
-//   {u}.{a} - u_i.{a} = du.A / 4,   8 G'_rho = 2 rho_i du.A + drho (2 u_i.A + du.A),
-//   16 G'_m = 8 G'_rho (u_i + u_m) + 4 (rho_i (u_i.A) du + dp A),
-//   16 G'_E = 8 G'_rho (h_i + h_m) + 4 rho_i (u_i.A) dh,
-// gi receives 16 G' (its mass row 8 G'), against DVS / 16 (and DVS / 8).  G'(m -> i)
-// has the differences' signs turned; gm receives its negative.  u_m.A is formed
-// from u_m, not as u_i.A + du.A: its rounding then is the same in all of a node's
-// pairs on an affine element and cancels like a derivative (the sum raised the
-// momentum rows' error by 10 to 20 %).  The two orientations take 55 FP32
-// operations (about 90 when each was formed from {a} and its own products).
-__device__ __forceinline__ void flux_delta_pair16(const NodeF& i, const NodeF& m, float A0, float A1, float A2,
-                                                  float rho2, float h2, float gi[5], float gm[5]) {
+// i, m in the storage form of the FP32 primitives (rho, h shifted by
+// rho_ref, h_ref): the differences come from the shifted values, the full
+// density and enthalpy of node i are rebuilt where they multiply
+__device__ __forceinline__ void flux_delta(const NodeF& i, const NodeF& m, float ai0, float ai1, float ai2, float da0,
+                                           float da1, float da2, float rho_ref, float h_ref, float G[5]) {
   const float du = (m.u - i.u) + (m.ul - i.ul), dv = (m.v - i.v) + (m.vl - i.vl), dw = (m.w - i.w) + (m.wl - i.wl);
-  const float dr = m.rho - i.rho, dp4 = 4.0f * (m.p - i.p), dh = m.h - i.h;
-  const float su = i.u + m.u, sv = i.v + m.v, sw = i.w + m.w, sh = (i.h + m.h) + h2;
-  const float ua = i.u * A0 + i.v * A1 + i.w * A2;
-  const float da = du * A0 + dv * A1 + dw * A2;
-  const float t = dr * fmaf(2.0f, ua, da);
-  const float P0 = dp4 * A0, P1 = dp4 * A1, P2 = dp4 * A2;
-  {
-    const float r = fmaf(2.0f, i.rho, rho2), g = fmaf(r, da, t), q = 2.0f * r * ua;  // r = 2 rho_i
-    gi[0] = g;
-    gi[1] = fmaf(g, su, fmaf(q, du, P0));
-    gi[2] = fmaf(g, sv, fmaf(q, dv, P1));
-    gi[3] = fmaf(g, sw, fmaf(q, dw, P2));
-    gi[4] = fmaf(g, sh, q * dh);
-  }
-  {
-    const float r = fmaf(2.0f, m.rho, rho2), g = fmaf(r, da, t), q = 2.0f * r * (m.u * A0 + m.v * A1 + m.w * A2);
-    // the negatives (the partner lane subtracts)
-    gm[0] = g;
-    gm[1] = fmaf(g, su, fmaf(q, du, P0));
-    gm[2] = fmaf(g, sv, fmaf(q, dv, P1));
-    gm[3] = fmaf(g, sw, fmaf(q, dw, P2));
-    gm[4] = fmaf(g, sh, q * dh);
-  }
+  const float dr = m.rho - i.rho, dp = m.p - i.p, dh = m.h - i.h;
+  const float ri = rho_ref + i.rho;
+  const float ab0 = fmaf(0.5f, da0, ai0), ab1 = fmaf(0.5f, da1, ai1), ab2 = fmaf(0.5f, da2, ai2);
+  const float uia = i.u * ai0 + i.v * ai1 + i.w * ai2;          // u_i . a_i
+  const float uida = 0.5f * (i.u * da0 + i.v * da1 + i.w * da2);  // u_i . da / 2
+  const float dua = 0.5f * (du * ab0 + dv * ab1 + dw * ab2);      // du/2 . {a}
+  const float g0 = ri * dua + 0.5f * dr * (uia + uida + dua);
+  const float ruia = ri * (uia + uida);  // rho_i (u_i.a_i + u_i . da/2)
+  G[0] = g0;
+  G[1] = g0 * fmaf(0.5f, du, i.u) + 0.5f * (ruia * du + dp * ab0);
+  G[2] = g0 * fmaf(0.5f, dv, i.v) + 0.5f * (ruia * dv + dp * ab1);
+  G[3] = g0 * fmaf(0.5f, dw, i.w) + 0.5f * (ruia * dw + dp * ab2);
+  G[4] = g0 * (h_ref + fmaf(0.5f, dh, i.h)) + 0.5f * ruia * dh;
 }
 
 // both orientations of a pair, G(i -> m) into Gi and G(m -> i) into Gm: the
@@ -2397,21 +2377,23 @@ __device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDe
           const int lq = base + pm;
           auto sh = [&](float x) { return __shfl_sync(0xffffffffu, x, lq); };
           const NodeF mq{sh(A.rho), sh(A.u), sh(A.v), sh(A.w), sh(A.p4), sh(A.hh), sh(Aul), sh(Avl), sh(Awl)};
-          const float A0 = A.a0 + sh(A.a0), A1 = A.a1 + sh(A.a1), A2 = A.a2 + sh(A.a2);
-          const float rho2 = 2.0f * ph.f32c.rho_ref, h2 = 2.0f * ph.f32c.h_ref;
+          const float aq0 = sh(A.a0), aq1 = sh(A.a1), aq2 = sh(A.a2);
           float G[5], Gq[5];
-          const float c8 = sC8[pos * n + pm], c16 = sC16[pos * n + pm];
-          flux_delta_pair16(mi, mq, A0, A1, A2, rho2, h2, G, Gq);
-          acc[0] = fmaf(c8, G[0], acc[0]);
-#pragma unroll
-          for (int v = 1; v < 5; ++v) acc[v] = fmaf(c16, G[v], acc[v]);
+          const float c1 = sC1[pos * n + pm];
           if (2 * d != n) {
-            // -G(q -> i) for the partner lane (pos + d); receive that of lane pos - d
-            const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
-            const float r8 = -sC8[pos * n + (src - base)], r16 = -sC16[pos * n + (src - base)];
-            acc[0] = fmaf(r8, __shfl_sync(0xffffffffu, Gq[0], src), acc[0]);
+            // and G(q -> i) for the partner lane (pos + d); receive G(i -> pos - d)
+            flux_delta_pair(mi, mq, A.a0, A.a1, A.a2, aq0, aq1, aq2, ph.f32c.rho_ref, ph.f32c.h_ref, G, Gq);
 #pragma unroll
-            for (int v = 1; v < 5; ++v) acc[v] = fmaf(r16, __shfl_sync(0xffffffffu, Gq[v], src), acc[v]);
+            for (int v = 0; v < 5; ++v) acc[v] += c1 * G[v];
+            const int src = base + (pos - d >= 0 ? pos - d : pos - d + n);
+            const float r1 = sC1[pos * n + (src - base)];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] += r1 * __shfl_sync(0xffffffffu, Gq[v], src);
+          } else {
+            flux_delta(mi, mq, A.a0, A.a1, A.a2, aq0 - A.a0, aq1 - A.a1, aq2 - A.a2, ph.f32c.rho_ref,
+                       ph.f32c.h_ref, G);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] += c1 * G[v];
           }
           continue;
         }
