@@ -45,10 +45,14 @@ NCU_TRAFFIC_PER_DOF = {("k_volume", "fp64", 7): (830.92e6 + 157.87e6) / 2097152,
 # U read 40 and written 40, dU read and written 80, FP32 primitives and the
 # velocity's low parts read 36 and written 36, Ja + 1/J 40, R_v 16, surface
 # fluxes 3 n^2 / n^3 x 5 x 4 B x 2 sides
+# of the FP64 one: U and dU read and written 160, primitives read 48 and those of
+# the updated state written 56 (at odd N 32 more as float pairs), the fixed-point
+# metrics and 1/J 80, R_v 32, surface fluxes
+FP64_VOLUME_BYTES_PER_DOF = lambda N: 160 + 48 + 56 + (32 if N % 2 else 0) + 80 + 32 + 3.0 / (N + 1) * 5 * 8 * 2
 MIXED_VOLUME_BYTES_PER_DOF = lambda N: 40 + 40 + 80 + 36 + 36 + 40 + 16 + 3.0 / (N + 1) * 5 * 4 * 2
 
 
-def algorithmic_flops_per_dof(N, kernel, viscous=True, surf="roe", stored_prims=None, pair_sums=None):
+def algorithmic_flops_per_dof(N, kernel, viscous=True, surf="roe", stored_prims=None):
     """Algorithmic FP64 flops per DOF and operator evaluation (FMA = 2).
 
     Counted on the formulas of the operator, independent of how a kernel
@@ -56,26 +60,24 @@ def algorithmic_flops_per_dof(N, kernel, viscous=True, surf="roe", stored_prims=
     with a symmetric flux allows).  The primitive recovery is counted where it
     runs: in the FP64 viscous form (stored_prims, the default there) once per
     node in the lifting window, which stores them for the face and volume
-    kernels.  The FP64 volume kernel at N = 7 reads each pair's metric sum,
-    stored with the mesh (pair_sums, the default there): those 3 additions
-    are not counted."""
+    kernels.  (The volume kernel forms its pairs in fixed point on the integer
+    pipes and the lifting in double-float arithmetic on the FP32 pipe: their
+    counts are FP64-equivalent work, and exceed the FP64 peak.)"""
     n = N + 1
     if stored_prims is None:
         stored_prims = viscous
-    if pair_sums is None:
-        pair_sums = N == 7
     if kernel == "volume":
         pairs = 3 * N / 2.0                     # unordered pairs per node, 3 directions
-        pair = 6 + (0 if pair_sums else 3) + 5 + 1 + 9 + 1 + 20  # averages, metric sum, u.a, m, F_m, F_E, 2 x 5 FMA
+        pair = 6 + 3 + 5 + 1 + 9 + 1 + 20       # averages, metric sum, u.a, m, F_m, F_E, 2 x 5 FMA
         prim = 1 if stored_prims else 13        # 4 p' (stored) | 1/rho, u, |u|^2, p, h
         surf_int = (6.0 / n) * 5 * 2            # face nodes per DOF x 5 FMA
         return pairs * pair + prim + (4 if viscous else 0) + surf_int + 5 + 20
     if kernel == "lift":
         if not viscous:
             return 0.0
-        # the event window holds k_prim64 (the primitives of each node, 13,
+        # 13: the primitives of each node (formed by the stage before),
         # read by the lifting kernel at the node and at the neighbours' face
-        # nodes) and k_lift.  12 line contractions of the gradient and 12 of
+        # nodes.  12 line contractions of the gradient and 12 of
         # the weak divergence per node; with an even node count in their
         # even/odd form (D is centro-antisymmetric): n/2 FMA, one addition
         # forming the half-sums, one combining the halves, instead of n FMA;
@@ -497,12 +499,20 @@ def run_ours(args):
     modelled = [k for k in kernels if kernels[k]["flops_per_dof"]] or list(kernels)
     dom = max(modelled, key=lambda k: kernels[k]["ms_per_launch"] * kernels[k]["launches"])
     peaks = load_peaks()
-    if precision == dg.FP64:
+    if precision == dg.FP64 and dom == "volume":
+        # fixed-point pairs on the integer pipes (no FP64 or tensor roofline
+        # applies): against HBM
+        hbm = peaks.get("hbm_gbs", 6800.0)
+        achieved = FP64_VOLUME_BYTES_PER_DOF(wl.spec.N) * dofs / (kernels[dom]["ms_per_launch"] * 1e-3) / 1e9
+        tpd = NCU_TRAFFIC_PER_DOF.get(("k_volume", "fp64", wl.spec.N))
+        roof = {"bound": "hbm", "kernel": "k_volume_fx", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+                "frac": achieved / hbm, "traffic": tpd * dofs if tpd else None,
+                "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
+    elif precision == dg.FP64:
         achieved = kernels[dom]["achieved_tflops"]
-        tpd = NCU_TRAFFIC_PER_DOF.get(("k_" + dom, "fp64", wl.spec.N))
         roof = {"bound": "alu", "kernel": "k_" + dom, "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
                 "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS if achieved else None,
-                "traffic": tpd * dofs if tpd else None,
+                "traffic": None,
                 "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (FP64 pipe)"}
     else:
         # the mixed form's dominant kernel is the volume kernel, against HBM
@@ -513,8 +523,8 @@ def run_ours(args):
         roof = {"bound": "hbm", "kernel": "k_volume", "achieved": ach, "peak": hbm, "unit": "GB/s",
                 "frac": ach / hbm if ach else None, "traffic": tpd * dofs if tpd else None,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
-    # (the FP64 viscous form's lift window holds two launches, k_prim64 and k_lift)
-    launches_per_step = sum(2 if (k == "lift" and precision == dg.FP64) else 1 for k in kernels)
+    # (one launch each: a stage leaves the primitives that the next one's lifting reads)
+    launches_per_step = len(kernels)
     # CPU baseline: the oracle on a bounded sample (rank 0, N = 1 only)
     cpu = None
     if world == 1 and not args.no_cpu_baseline:

@@ -172,10 +172,11 @@ int dg_lgl_nodes(int N, double* xi, double* w);
 /* Builds the geometry (curl-form metrics, Jacobians, face normals, wall-model
  * sampling points) on the host, validates it, allocates the device storage
  * and uploads it.  stream: cudaStream_t (may be 0).  On success *out owns
- * everything; free it with dg_destroy.  Device storage at N = 7: about 500
- * bytes per DOF in the FP64 viscous form (state, RK register, metrics and the
- * stored products Ja / J and (Ja Ja^T) / J, the stored primitives, scratch),
- * about 280 in the FP32-mixed form.  Errors: DG_ERR_ARG, DG_ERR_MESH,
+ * everything; free it with dg_destroy.  Device storage at N = 7: about 800
+ * bytes per DOF in the FP64 viscous form (state, RK register, metrics, also in
+ * fixed point, the stored products Ja / J and (Ja Ja^T) / J, the lifting's float
+ * pairs, the stored primitives, scratch),
+ * about 290 in the FP32-mixed form.  Errors: DG_ERR_ARG, DG_ERR_MESH,
  * DG_ERR_OOM, DG_ERR_CUDA (the message is then available through
  * dg_last_error(NULL)). */
 int dg_init_mesh(dg_ctx** out, const dg_mesh_desc* m, const dg_phys* p, const dg_options* o,
@@ -232,9 +233,9 @@ int dg_rk_steps(dg_ctx* c, double t, double dt, int nsteps);
  * split-form volume integral, viscous flux, BR1 lifting and primitive
  * recovery are written out by hand, and so is the reverse mode of the
  * Riemann flux (one forward sweep keeping the intermediates of the two-point
- * flux and of its dissipation, one backward sweep); the local derivatives of
- * the wall model come from forward-mode dual numbers, with the implicit
- * function theorem for the law-of-the-wall solve (Sec. 3.2).  FP64
+ * flux and of its dissipation, one backward sweep); the wall model's
+ * reverse mode uses the implicit function theorem for the law-of-the-wall
+ * solve (Sec. 3.2).  FP64
  * contexts with the Pirozzoli or the entropy-conserving volume flux (the
  * paper's Sec. 4 scheme, with Roe + Harten faces), constant viscosity or
  * Sutherland's law, adiabatic or isothermal walls (the wall heat flux's
