@@ -39,7 +39,7 @@ L2_BYTES = 129e6  # GB300 L2 (nominal)
 # DRAM bytes (read + write) of one launch of the dominant kernel, from an ncu
 # capture of the same kernel build on a 16^3-element case, scaled to the
 # launch size by the DOF count (traffic is proportional to the DOF count).
-NCU_TRAFFIC_PER_DOF = {("k_volume", "fp64", 7): (830.92e6 + 157.87e6) / 2097152,
+NCU_TRAFFIC_PER_DOF = {("k_volume", "fp64", 7): (537.06e6 + 327.35e6) / 2097152,
                        ("k_volume", "fp32", 7): (308.59e6 + 204.15e6) / 2097152}
 # algorithmic HBM bytes per DOF of the FP32-mixed volume kernel (stage form):
 # U read 40 and written 40, dU read and written 80, FP32 primitives and the
