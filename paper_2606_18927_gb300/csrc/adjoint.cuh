@@ -504,7 +504,7 @@ k_adj_face(const double* __restrict__ U, const double* __restrict__ lam, const M
 // node per lane (few nodes, long chains; see k_wall): the warps share the
 // planes of the sample's interpolation, the last takes the Riemann flux's
 // reverse mode, the first the wall model's (wall_stress_vjp).  Also accumulates
-// g_theta = sum_nodes (dFs/dtheta)^T gFs.  6912 nodes at N = 5: 158 us, 212 with
+// g_theta = sum_nodes (dFs/dtheta)^T gFs.  6912 nodes at N = 5: 149 us, 212 with
 // seven forward-mode sweeps (the sample state's components, kappa, B), one per
 // warp, which filled the FP64 pipe; what is left is the chain of the sample,
 // the solve and the sweep.

@@ -1396,7 +1396,8 @@ struct LiftPk {
 };
 
 // Resident CTAs per SM asked of the register allocator for the lifting kernel:
-// two in FP64 (bound by the FP64 pipe) and on small meshes (dense_mesh), else FP32 resident_ctas (its line phases
+// two in FP64 (bound by the FP64 pipe) and on small meshes (see dense_mesh),
+// else in FP32 resident_ctas (its line phases
 // leave the other threads waiting at a barrier, which more CTAs cover: N = 5
 // 0.195 -> 0.177 ms at 26^3, N = 3 0.248 -> 0.157 at 40^3)
 template <int N, typename R, bool DENSE>
