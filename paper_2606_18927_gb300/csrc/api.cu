@@ -48,6 +48,10 @@ struct dg_ctx {
   // face and volume kernels of the same evaluation
   double* W64 = nullptr;  // FP64 viscous form: primitives [7][S]; w64_of_U says they are those of U
   bool w64_of_U = false;
+  // A graph that the caller captured from this context has W32, W64, lift_W2 or U
+  // written at every replay, which no host flag sees: from the first such capture
+  // on, stored primitives are used only within the call that stored them.
+  bool replayed = false;
   double* JaJ = nullptr;  // FP64 viscous: [9][S] Ja / J
   double* Mj = nullptr;   // FP64 viscous: [6][S] (Ja Ja^T) / J
   // double-float lifting (N = 7, FP64 viscous): (hi, lo) pairs of Ja, Ja / J,
@@ -175,10 +179,15 @@ void free_all(dg_ctx* c) {
 // profiling events per operator evaluation (see OpArgs::ev)
 constexpr size_t kEventsPerLaunch = 7;
 
-// whether s is being captured (the legacy default stream cannot be)
-bool capturing(cudaStream_t s) {
+// whether a graph of the caller's is being captured on the context's stream (the
+// legacy default stream cannot be; cap_stream captures dg_rk_steps_graph's own
+// graph); the context remembers that one has been
+bool user_capture(dg_ctx* c) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return s && cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+  const bool now = c->stream && c->stream != c->cap_stream && cudaStreamIsCapturing(c->stream, &st) == cudaSuccess &&
+                   st != cudaStreamCaptureStatusNone;
+  c->replayed = c->replayed || now;
+  return now;
 }
 
 int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double B, double dt, int read_dU,
@@ -214,13 +223,15 @@ int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double
     c->events_used += kEventsPerLaunch;
   }
   a.W32 = c->W32;
-  a.w32_valid = (a.fp32 && Uin == c->U && c->w32_of_U) ? 1 : 0;
   a.W64 = c->W64;
   // A graph of the caller's replays after states this context cannot foresee
-  // (dg_set_state between replays): every evaluation in it forms its own
-  // primitives.  (dg_rk_steps_graph refreshes them before its replays.)
-  const bool user_capture = c->W64 && c->stream != c->cap_stream && capturing(c->stream);
-  a.w64_valid = (c->W64 && !a.fp32 && Uin == c->U && c->w64_of_U && !user_capture) ? 1 : 0;
+  // (dg_set_state between replays), and between calls that it cannot see: in it
+  // and after it every evaluation forms its own primitives.  (dg_rk_steps_graph
+  // refreshes them before its replays, which follow each other.)
+  user_capture(c);
+  const bool stored = Uin == c->U && (!c->replayed || c->stream == c->cap_stream);
+  a.w32_valid = (a.fp32 && stored && c->w32_of_U) ? 1 : 0;
+  a.w64_valid = (c->W64 && !a.fp32 && stored && c->w64_of_U) ? 1 : 0;
   a.keep_w64 = Uout == c->U ? 1 : 0;
   a.JaJ = c->JaJ; a.Mj = c->Mj;
   a.lift_M2 = c->lift_M2; a.lift_W2 = c->lift_W2;
@@ -240,22 +251,22 @@ int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double
   if (!a.fp32 && c->W64 && c->opts.viscous) {
     if ((phase & 4) && mode == 1 && Uout == c->U) c->w64_of_U = true;
     else if (phase & 2) c->w64_of_U = (Uin == c->U);
-    if (user_capture) c->w64_of_U = false;  // nothing has run yet
   }
   return DG_OK;
 }
 
-// form the stored primitives of the context's state if they are stale
+// form the stored primitives of the context's state if they are, or may be, stale
 int refresh_primitives(dg_ctx* c) {
   const long long S = (long long)c->S;
-  if (c->W64 && c->opts.viscous && !c->w64_of_U) {
+  user_capture(c);
+  if (c->W64 && c->opts.viscous && (!c->w64_of_U || c->replayed)) {
     dg::k_prim64<<<(unsigned)std::min<long long>((S + 255) / 256, 152 * 16), 256, 0, c->stream>>>(
         S, c->U, c->ph, c->W64, c->ph.lift_df ? c->lift_W2 : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "primitive refresh");
     c->w64_of_U = true;
   }
-  if (c->opts.precision != DG_FP32_MIXED || c->w32_of_U) return DG_OK;
+  if (c->opts.precision != DG_FP32_MIXED || (c->w32_of_U && !c->replayed)) return DG_OK;
   dg::k_prim32<<<(unsigned)std::min<long long>((S + 255) / 256, 152 * 16), 256, 0, c->stream>>>(S, c->U, c->ph,
                                                                                                  c->W32);
   cudaError_t e = cudaGetLastError();
@@ -446,7 +457,10 @@ int noalloc_args(dg_ctx* c, const double* U, double* Ut, OpArgs* a, const PhysDe
 // context's W32 now holds the primitives of U (if the launches succeeded), so
 // they are those of the context's state only when U is the state.
 void noalloc_done(dg_ctx* c, const double* U, bool ok) {
-  if (c->opts.precision == DG_FP32_MIXED) c->w32_of_U = ok && (U == c->U);
+  if (c->opts.precision == DG_FP32_MIXED) {
+    user_capture(c);
+    c->w32_of_U = ok && (U == c->U);
+  }
 }
 int noalloc_fail(dg_ctx* c, int code, const std::string& msg) { return fail(c, code, msg); }
 }  // namespace dg
@@ -719,6 +733,7 @@ int dg_sizes(const dg_ctx* c, int* N, int* K, long long* n_state) {
 
 int dg_set_state(dg_ctx* c, const double* U, int on_device) {
   if (!c || !U) return c ? fail(c, DG_ERR_ARG, "dg_set_state: null U") : DG_ERR_ARG;
+  user_capture(c);
   cudaError_t e = cudaMemcpyAsync(c->U, U, 5 * c->S * sizeof(double),
                                   on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "dg_set_state");
