@@ -135,10 +135,13 @@ __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sL
       const Fx m1 = dif(1), m2 = dif(2), m3 = dif(3), m4 = dif(4);
       FxSum k(Su, Sa0);
       k.add(Sv, Sa1);
+      k.fold();
       k.add(Sw, Sa2);
       const long long qv = k.get();  // S_u . S_a
-      FxSum x(m1, Su);
+      FxSum x(m1, Su);  // (differences have limbs as large as sums: one term is up to 4.3 2^60)
+      x.fold();
       x.add(m2, Sv);
+      x.fold();
       x.add(m3, Sw);
       const Fx m0 = dif(0);
       const long long tt = ((((long long)m0.h << 31) + m0.l) >> f.s0) + (x.get() >> f.s1) +
@@ -164,6 +167,7 @@ __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sL
       F[3] = vel(Sa2, m3);
       FxSum z(m1, Sa0);
       z.add(m2, Sa1);
+      z.fold();
       z.add(m3, Sa2);
       F[4] = fx_mul96(fx_split<1>(z.get()), Q);
       F[5] = fx_mul96(Sr, fx_split<0>(fx_mul(Qv, m4)));

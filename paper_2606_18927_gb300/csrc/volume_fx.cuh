@@ -42,6 +42,10 @@ __device__ __forceinline__ Fx operator+(Fx a, Fx b) { return Fx{a.h + b.h, a.l +
 // high limbs' products, x the cross products (units of 2^31; they start at
 // 2^31, half a unit of what is kept).  The low limbs' products, below half a
 // unit, are left out.
+// Bounds of x: limbs are |l| <= 2^31 and |h| <= 2^(b - 31) for values below 2^b, so
+// a pair's S_u S_a (b = 61, 60) adds up to 3 2^60, its two momentum terms together
+// 7 2^60 (|Q| < 1).  Sums of more stay below 2^63 = 8 2^60 by fold() between the
+// terms: two products S_u S_a fit, a third does not.
 struct FxSum {
   long long hh, x;
   __device__ __forceinline__ FxSum(Fx a, Fx b) {
@@ -51,6 +55,11 @@ struct FxSum {
   __device__ __forceinline__ void add(Fx a, Fx b) {
     x = madw(a.l, b.h, madw(a.h, b.l, x));
     hh = madw(a.h, b.h, hh);
+  }
+  // x's high word (it counts twice) into hh; the sum's bits stay the same
+  __device__ __forceinline__ void fold() {
+    hh = madw((int)(x >> 32), 2, hh);
+    x = (long long)(unsigned)x;
   }
   // hh + x / 2^31: the high word of x counts twice
   __device__ __forceinline__ long long get() const { return madw((int)(x >> 32), 2, hh); }
@@ -310,6 +319,7 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
       const Fx Su = q[1] + mv1, Sv = q[2] + mv2, Sw = q[3] + mv3;
       FxSum s(Su, Sa0);
       s.add(Sv, Sa1);
+      s.fold();
       s.add(Sw, Sa2);
       const Fx ua = fx_split<1>(s.get());  // 4 {u}.{a}
       long long F[5];
