@@ -315,7 +315,8 @@ __global__ void k_kinetic_energy(long long S, const double* __restrict__ U, cons
 // the largest matters: a first sweep takes FP32 bounds of every node's value and
 // the largest lower bound (out[1], as float bits), a second one the FP64 value
 // of the nodes whose upper bound reaches it.  A lower bound counts only where
-// the FP64 value is sure to be a number.  565k nodes: dg_time_step 122 -> 52 us.
+// the FP64 value is sure to be a number, an upper one only where no term has left
+// FP32's normal range.  565k nodes: dg_time_step 122 -> 52 us.
 __device__ __forceinline__ float to_f32(double x) { return d2f_bits(x); }
 __device__ __forceinline__ float to_f32(float x) { return x; }
 template <typename R>
@@ -323,28 +324,33 @@ __global__ void k_wave_speed(long long S, const double* __restrict__ U, const R*
                              const R* __restrict__ invJ, double gamma, unsigned long long* __restrict__ out) {
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
   unsigned* const bound = reinterpret_cast<unsigned*>(out + 1);
-  const float gf = (float)gamma;
-  // FP32 bounds: 2e-6 of the sums' absolute terms cover their rounding
+  const float gg = (float)(gamma * (gamma - 1.0));  // (formed in FP64: gamma - 1 may be small)
+  // FP32 bounds: 2e-6 of the sums' absolute terms cover their rounding, provided
+  // that no term that matters leaves FP32's normal range; where one might (in >
+  // 1e-30: what is flushed is below 1e-37), nothing is said about the node
   auto estimate = [&](long long i, float& lo, float& hi) {
     const float r = d2f_bits(U[i]), m0 = d2f_bits(U[S + i]), m1 = d2f_bits(U[2 * S + i]), m2 = d2f_bits(U[3 * S + i]),
                 E = d2f_bits(U[4 * S + i]);
     const float ir = 1.0f / r, u = m0 * ir, v = m1 * ir, w = m2 * ir;
     const float ke = 0.5f * (m0 * u + m1 * v + m2 * w), pe = 2e-6f * (fabsf(E) + fabsf(ke)), p = E - ke;
-    const float g = gf * (gf - 1.0f) * ir;
-    const float ch = sqrtf(g * (p + pe)), cl = sqrtf(g * (p - pe));
+    const float g = gg * ir, c2 = g * (p + pe);
+    const float ch = sqrtf(c2), cl = sqrtf(g * (p - pe));
+    bool in = E > 1e-30f && c2 > 1e-30f && ch * r > 1e-25f;
     float l = 0.0f, h = 0.0f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const float a0 = to_f32(Ja[(size_t)(d * 3) * S + i]), a1 = to_f32(Ja[(size_t)(d * 3 + 1) * S + i]),
                   a2 = to_f32(Ja[(size_t)(d * 3 + 2) * S + i]);
       const float un = fabsf(u * a0 + v * a1 + w * a2), ue = 2e-6f * (fabsf(u * a0) + fabsf(v * a1) + fabsf(w * a2));
-      const float j = sqrtf(a0 * a0 + a1 * a1 + a2 * a2);
+      const float a = a0 * a0 + a1 * a1 + a2 * a2, j = sqrtf(a);
+      in = in && a > 1e-30f && ch * j > 1e-25f;
       h += un + ue + ch * j;
       l += fmaxf(un - ue, 0.0f) + cl * j;
     }
     const float ij = to_f32(invJ[i]);
-    hi = h * ij * 1.000005f;
-    lo = r > 0.0f && p > pe && l * ij < 1e37f ? l * ij * 0.999995f : 0.0f;
+    in = in && ij > 1e-30f && h * ij > 1e-30f && h * ij < 1e30f;
+    hi = in ? h * ij * 1.000005f : __int_as_float(0x7f800000);
+    lo = in && cl > 1e-3f * ch ? l * ij * 0.999995f : 0.0f;
   };
   float best = 0.0f;
   for (long long i = i0; i < S; i += step) {
