@@ -27,11 +27,11 @@ struct AdjFxPlan {
   int eg[4];                      // the units of the sums rho, u, p, h
 };
 
-// ex: the largest fx_mag of each value; mA: that of the element's metrics; eW:
+// ex: the largest fx_mag of each value; mt: the element's metrics; eW:
 // lam~ / w is in units 2^eW times lam~'s.  Bounds in units of 2^60, times Q for the
 // pair terms: the sum of the three parts 3 (half of 6, by the extra shift), rho
 // and u 1.1, p 1.5, h 0.75; a line's sum of |Q| is below 3.7.
-__device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, int mA, int eW) {
+__device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& mt, int eW) {
   AdjFxPlan f;
   int eX[AX_NUM];
   bool ok = true;
@@ -41,7 +41,7 @@ __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, int mA, int eW) 
     eX[x] = max(e, -200);  // (smaller values, zeros among them, in that unit)
     ok = ok && e < 200;
   }
-  const int eA = (mA >> 20) - 1022;
+  const int eA = (mt.col[0] >> 20) - 1022;  // (elements whose columns differ are summed in FP64)
   f.bR = eX[AX_RHO] + 1022; f.bU = eX[AX_U] + 1022; f.bH = eX[AX_H] + 1022;
   f.bL0 = eX[AX_L0] + 1022; f.bLM = eX[AX_LM] + 1022; f.bLE = eX[AX_LE] + 1022;
   // units of the three parts of mu0 + (mu_m . S_u + mu_4 S_h) / 2
@@ -52,7 +52,7 @@ __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, int mA, int eW) 
   f.eg[1] = et + eX[AX_RHO] + eA + 2;
   f.eg[2] = eX[AX_LM] + eW + eA - 58;
   f.eg[3] = eX[AX_U] + eA + eX[AX_LE] + eW + eX[AX_RHO] - 57;
-  f.ok = ok && abs(eA) < 200;
+  f.ok = ok && abs(eA) < 200 && mt.kind == FX_EVEN;
   return f;
 }
 

@@ -59,7 +59,8 @@ struct dg_ctx {
   float2* lift_M2 = nullptr;
   float2* lift_W2 = nullptr;
   dg::Fx* JaX = nullptr;    // FP64: [9][S] metrics in fixed point (volume kernel), and
-  int* JaX_max = nullptr;   // the elements' largest magnitudes [K]
+  dg::FxMetric* JaX_max = nullptr;  // the elements' largest magnitudes and kinds [K]
+  int stretched = 0;        // some element is not FX_EVEN
   double* wm_t = nullptr;  // wall-law warm start per wall node (NaN: none yet)
   // partitioned meshes: halo buffers [n_halo][5][n2] (state traces, FP64) and
   // [n_halo][4][n2] (viscous-flux traces, flux type), received and sent
@@ -235,7 +236,7 @@ int launch(dg_ctx* c, const double* Uin, int mode, double* Out, double A, double
   a.keep_w64 = Uout == c->U ? 1 : 0;
   a.JaJ = c->JaJ; a.Mj = c->Mj;
   a.lift_M2 = c->lift_M2; a.lift_W2 = c->lift_W2;
-  a.JaX = c->JaX; a.JaX_max = c->JaX_max;
+  a.JaX = c->JaX; a.JaX_max = c->JaX_max; a.stretched = c->stretched;
   a.wm_t = c->wm_t;
   int rc = dg::run_operator(a, c->ph, c->stream);
   if (rc != 0) {
@@ -442,7 +443,7 @@ int noalloc_args(dg_ctx* c, const double* U, double* Ut, OpArgs* a, const PhysDe
   a->Ja = c->Ja; a->invJ = c->invJ; a->fgeo = c->fgeo; a->nbr = c->nbr; a->elem_face = c->elem_face;
   a->JaJ = c->JaJ; a->Mj = c->Mj;  // geometry, owned by the context
   a->lift_M2 = nullptr; a->lift_W2 = nullptr;  // (the FP64 lifting: no stored primitives here)
-  a->JaX = c->JaX; a->JaX_max = c->JaX_max;
+  a->JaX = c->JaX; a->JaX_max = c->JaX_max; a->stretched = c->stretched;
   a->faces = c->faces; a->ws_elem = c->ws_elem; a->ws_lag = c->ws_lag;
   a->D = c->geo.basis.D.data(); a->w = c->geo.basis.w.data();
   a->Uin = U; a->status = c->status;
@@ -690,9 +691,14 @@ int dg_init_mesh(dg_ctx** out, const dg_mesh_desc* m, const dg_phys* p, const dg
     chk(alloc(&c->JaX, 9 * S));
     chk(alloc(&c->JaX_max, (size_t)c->K));
     if (e == cudaSuccess) {
+      // (status is free until the first evaluation)
+      chk(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
       dg::k_metric_fx<<<(unsigned)c->K, 128, 0, c->stream>>>(c->n3, (long long)S, static_cast<const double*>(c->Ja),
-                                                            c->JaX, c->JaX_max);
+                                                            c->JaX, c->JaX_max, c->status);
       e = cudaGetLastError();
+      chk(cudaMemcpyAsync(&c->stretched, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+      chk(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
+      chk(cudaStreamSynchronize(c->stream));
     }
     if (e != cudaSuccess) { free_all(c); delete c; return cuda_fail(nullptr, e, "dg_init_mesh: metrics"); }
   }
@@ -1009,7 +1015,7 @@ static dg::OpArgs adjoint_args(dg_ctx* c, const double* U, const double* lam, do
   a.Uin = U; a.status = c->status;
   a.lam = lam; a.gU = gU; a.gV = c->gV; a.gUf = c->gUf; a.gGf = c->gGf; a.gWf = c->gWf; a.gUs = c->gUs; a.gtheta = gth;
   a.JaJ = c->JaJ; a.Mj = c->Mj;
-  a.JaX = c->JaX; a.JaX_max = c->JaX_max;
+  a.JaX = c->JaX; a.JaX_max = c->JaX_max; a.stretched = c->stretched;
   a.n_halo = c->geo.n_halo;
   a.halo_U = c->halo_U; a.halo_G = c->halo_G; a.send_U = c->send_U; a.send_G = c->send_G;
   return a;

@@ -90,6 +90,7 @@ constexpr bool dense_mesh(long long K, int threads, bool ec) {
 struct Fx {
   int h, l;
 };
+struct FxMetric;  // volume_fx.cuh
 
 struct PhysDev {
   double gamma, gm1, R, mu, Pr, cp, kcond, rcp_R;
@@ -159,7 +160,7 @@ struct MeshDev {
   const float2* lift_M2;
   float2* lift_W2;
   const Fx* JaX;         // FP64 form: [9][K*n3] metrics in fixed point (volume_fx.cuh) and their largest
-  const int* JaX_max;    // magnitudes [K]
+  const FxMetric* JaX_max;  // magnitudes [K]
   double* wm_t;          // [n_wall*n2] last wall-law solution per wall node (warm start; may be null)
   int* status;           // device status flags (index checks of the bounds-checking build)
 };

@@ -7,6 +7,7 @@ namespace dg {
 
 struct PhysDev;
 struct Fx;
+struct FxMetric;
 
 struct OpArgs {
   int N, K, F, n_interior, n_wall, n_bc;
@@ -59,7 +60,8 @@ struct OpArgs {
   const float2* lift_M2;
   float2* lift_W2;
   const Fx* JaX;        // FP64 form: [9][K n^3] metrics in fixed point and their largest
-  const int* JaX_max;   // magnitudes [K]
+  const FxMetric* JaX_max;  // magnitudes [K]
+  int stretched;        // some element's metrics are not FX_EVEN
   double* wm_t;  // wall-law warm-start values per wall node (null: cold solves)
   // partitioned meshes: n_halo halo faces (the last faces), remote traces in
   // halo_U / halo_G, local traces packed into send_U / send_G.  phase selects

@@ -262,7 +262,9 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     };
     auto flux = [&](auto vf) {
       constexpr int VF = decltype(vf)::value;
-      volume(a.mode == 0 ? k_volume_fx<N, 0, VF> : k_volume_fx<N, 1, VF>, VolFxShape<N, VF>::SMEM);
+      volume(a.stretched ? (a.mode == 0 ? k_volume_fx<N, 0, VF, true> : k_volume_fx<N, 1, VF, true>)
+                         : (a.mode == 0 ? k_volume_fx<N, 0, VF, false> : k_volume_fx<N, 1, VF, false>),
+             VolFxShape<N, VF>::SMEM);
     };
     if (ec) flux(std::integral_constant<int, FX_EC>{});
     else if (ph.vol_flux == 1) flux(std::integral_constant<int, FX_KG>{});

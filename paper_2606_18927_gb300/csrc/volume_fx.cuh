@@ -12,15 +12,18 @@
 // its largest value and is rounded to the nearest unit.  FP64 rounds the same
 // product to 53 bits of its own value, in every operation, the additions
 // among them; so the fixed-point sums are the more exact ones wherever a
-// node's fluxes are not far below the element's largest (against the
-// extended-precision oracle the operator's error (2-norm) fell by up to 30 % on
-// meshes of degree 2 to 8, for the three fluxes; with densities 20 apart
-// within an element it tripled).
-// An element in which they may be is summed in FP64 as before (fx_plan:
-// non-finite values; density or enthalpy differing by more than a factor 8
+// node's fluxes are not far below the element's largest.  Against the
+// extended-precision oracle the mass row's error (2-norm) is 0.4 to 0.7 of FP64's on
+// straight boxes of degree 3 to 7 with sides 1 : 1 to 1 : 1000, the energy row's 0.5
+// to 0.8, the momentum rows' 0.9 to 1.1; the whole operator's fell by up to 30 % on
+// curved meshes of degree 2 to 8.  Stretched elements have units of their own for
+// every component of u and column of Ja (FxMetric, FxRows).
+// An element whose fluxes may be far below its largest is summed in FP64 as before
+// (fx_plan: non-finite values; density or enthalpy differing by more than a factor 8
 // over its nodes, with the entropy-conserving flux density or internal energy
-// by more than an eighth, where its logarithmic means' series end; or a Mach number so small that the common unit of the
-// momentum flux would cost the velocity bits).
+// by more than an eighth, where its logarithmic means' series end; a Mach number so
+// small that the common unit of the momentum flux would cost the velocity bits; a
+// column of Ja that falls below an eighth of its largest).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -51,6 +54,11 @@ struct FxSum {
   __device__ __forceinline__ FxSum(Fx a, Fx b) {
     x = madw(a.l, b.h, madw(a.h, b.l, 1LL << 31));
     hh = mulw(a.h, b.h);
+  }
+  // with half added to the sum: half = 2^(k - 1) for a sum that is shifted by k
+  __device__ __forceinline__ FxSum(Fx a, Fx b, long long half) {
+    x = madw(a.l, b.h, madw(a.h, b.l, 1LL << 31));
+    hh = madw(a.h, b.h, half);
   }
   __device__ __forceinline__ void add(Fx a, Fx b) {
     x = madw(a.l, b.h, madw(a.h, b.l, x));
@@ -161,7 +169,7 @@ __device__ __forceinline__ Fx fx_mean_arg(Fx a, Fx b, Fx ia, Fx ib, int sh) {
 // flux: rho, u, p', e = p / ((gamma - 1) rho),
 // b = 1 / (2 e) and 1 / (2 rho), with b p' in the place of p'.
 enum { FX_KEP, FX_KG, FX_EC };  // the volume flux, as PhysDev::vol_flux
-enum { FX_RHO, FX_U, FX_P, FX_H, FX_NRHO, FX_NH, FX_B, FX_IR, FX_NUM };
+enum { FX_RHO, FX_U, FX_P, FX_H, FX_NRHO, FX_NH, FX_B, FX_IR, FX_V, FX_W, FX_NUM };
 struct FxPlan {
   int ok;              // 0: the element is summed in FP64
   int bR, bU, bP, bH;  // biased exponent bounds of rho, u, p' (EC: b p'), h (EC: e) for fx_of
@@ -174,13 +182,43 @@ struct FxPlan {
   int kt, kd, kz;      // EC: right shifts of e Q, u.u and 4 p~' to the energy bracket's units
   long long pref;      // EC: 4 p_ref in the bracket's unit
 };
+// Stretched elements: what differs by component c of u, Ja and the momentum
+// (FxPlan's bU, kp, em, km and kd are not used).  The passes read it from shared
+// memory pair by pair (volatile): in registers it spilled (N = 7, sides 1 : 8,
+// 12^3 elements: volume kernel 227 us, so 181; 160 for even elements).
+struct FxRows {
+  int bU[3];                      // biased exponent bounds of u_c
+  int t[3], s1[3], s2[3], kd[3];  // right shifts of S_u S_a, m u_c, p Ja_c and (EC) u_c u_c to the common units
+  long long ht[3], h1[3], h2[3];  // half of what the first three drop
+  int em[3], km[3];
+};
+
+// An element's metrics (k_metric_fx): the largest |Ja^d_c| of each column c over
+// nodes and directions (as fx_mag), and its kind.  FX_EVEN: the columns are within
+// a factor 2 of each other, and the metrics and the velocities have one unit each.
+// FX_STRETCHED: a side is short against another.  The flux S_u . S_a then adds
+// products of large velocities with small metrics and of small velocities with
+// large ones: in common units both lose as many bits as the sides' ratio has (the
+// mass row's error was 3 times FP64's at ratio 10, 280 times at 1000), so every
+// column and every velocity component has its own, and the products are shifted
+// to the largest one's.  FX_GRADED: some column is below an eighth of its largest at
+// some node (thin at one end); its lines there would lose as much: summed in FP64.
+enum { FX_EVEN, FX_STRETCHED, FX_GRADED };
+struct FxMetric {
+  int col[3], kind;
+};
 
 // ex: the largest fx_mag of each value (FX_NRHO, FX_NH: of 0x7fffffff - fx_mag);
-// mA: that of the element's metrics; eW of the line table
-template <int VF>
-__device__ __forceinline__ FxPlan fx_plan(const int* ex, int mA, int eW, double p_ref, double gm1) {
+// mt: the element's metrics; eW of the line table; rows: for stretched elements
+// (GEN: the mesh has some)
+template <int VF, bool GEN>
+__device__ __forceinline__ FxPlan fx_plan(const int* ex, const FxMetric& mt, int eW, double p_ref, double gm1,
+                                          FxRows* rows) {
   constexpr bool EC = VF == FX_EC;
   FxPlan f;
+  const bool st = GEN && mt.kind == FX_STRETCHED;
+  const int mA = max(mt.col[0], max(mt.col[1], mt.col[2]));
+  const int xU = GEN ? max(ex[FX_U], max(ex[FX_V], ex[FX_W])) : ex[FX_U];
   f.bR = ex[FX_RHO] >> 20;
   f.bH = ex[FX_H] >> 20;
   const int eR = f.bR - 1022, eA = (mA >> 20) - 1022, eP = (ex[FX_P] >> 20) - 1022;
@@ -188,20 +226,49 @@ __device__ __forceinline__ FxPlan fx_plan(const int* ex, int mA, int eW, double 
   // p' is summed with rho u u: below 2^(eR + 2 eU - 1) in the unit of m u; a
   // larger p' (low Mach numbers, no reference pressure) raises that unit by
   // 2^kp, and beyond kp = 40 the velocity's
-  const int eUt = (ex[FX_U] >> 20) - 1022;
+  const int eUt = (xU >> 20) - 1022;
   int eU = max(eUt, -200);
-  eU = max(eU, (eP - eR + 1 - 40 + 1) >> 1);
+  if (!st) eU = max(eU, (eP - eR + 1 - 40 + 1) >> 1);
   f.bU = eU + 1022;
   f.kp = max(0, eP - (eR + 2 * eU - 1));
-  const int ePt = eR + 2 * eU - 1 + f.kp;
-  f.bP = ePt + 1022;
-  const bool finite = f.bR < 0x7ff && (ex[FX_U] >> 20) < 0x7ff && (ex[FX_P] >> 20) < 0x7ff && f.bH < 0x7ff;
-  const bool range = abs(eR) < 200 && abs(eH) < 200 && abs(eA) < 200 && eU < 200 && eP < 200;
+  int ePt = eR + 2 * eU - 1 + f.kp, E = eU + eA;  // E: of S_u . S_a
   // what the largest values leave of the bounds (all below 1)
   const float mr = fx_mant(ex[FX_RHO]), mh = fx_mant(ex[FX_H]), ma = fx_mant(mA);
-  const float mu = ldexpf(fx_mant(ex[FX_U]), max(eUt - eU, -60));
+  const float mu = ldexpf(fx_mant(xU), max(eUt - eU, -60));
+  float mass = mr * mu * ma;
+  bool range = abs(eR) < 200 && abs(eH) < 200 && abs(eA) < 200 && eU < 200 && eP < 200;
+  int eC[3], aC[3];  // stretched: exponents of u_c (no further than 2^-40 below the largest) and of Ja_c
+  float uC[3] = {0.0f, 0.0f, 0.0f};
+  if (st) {
+    const int x[3] = {ex[FX_U], ex[FX_V], ex[FX_W]};
+    E = -1000;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int e = (x[c] >> 20) - 1022;
+      eC[c] = max(e, eU - 40);
+      aC[c] = (mt.col[c] >> 20) - 1022;
+      uC[c] = ldexpf(fx_mant(x[c]), max(e - eC[c], -60));
+      E = max(E, eC[c] + aC[c]);
+      range = range && abs(aC[c]) < 200;
+    }
+    // p' in its own unit, but no finer than the least row m u_c needs
+    mass = 0.0f;
+    ePt = 1000;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int t = min(E - eC[c] - aC[c], 62);
+      rows->bU[c] = eC[c] + 1022;
+      rows->t[c] = t;
+      rows->ht[c] = (1LL << t) >> 1;
+      mass += ldexpf(uC[c] * fx_mant(mt.col[c]), -t);
+      ePt = min(ePt, eR + E + eC[c] - 1 - aC[c]);
+    }
+    mass *= mr * (1.0f / 3.0f);
+    ePt = max(ePt, eP);
+  }
+  f.bP = ePt + 1022;
+  const bool finite = f.bR < 0x7ff && (xU >> 20) < 0x7ff && (ex[FX_P] >> 20) < 0x7ff && f.bH < 0x7ff;
   const float mp = ldexpf(fx_mant(ex[FX_P]), max(eP - ePt, -60));
-  const float mass = mr * mu * ma;
   float energy = mass * mh;
   bool even;
   if constexpr (EC) {
@@ -219,6 +286,10 @@ __device__ __forceinline__ FxPlan fx_plan(const int* ex, int mA, int eW, double 
     const int e1 = eH - 59, e2 = 2 * eU - 58, eY = max(e1, e2);  // units of e Q and u.u
     f.kt = min(eY - e1, 63);
     f.kd = min(eY - e2, 63);
+    if (st) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) rows->kd[c] = min(eY - (2 * eC[c] - 58), 63);
+    }
     energy = mass * fminf(1.0f, (ldexpf(mh, -f.kt) + ldexpf(mu * mu, -f.kd)) * 0.58f);
     const int eZ = eR + eY + 2;  // of rho (e Q + u.u)
     f.kz = eZ - (ePt - 60) - 1;
@@ -240,34 +311,69 @@ __device__ __forceinline__ FxPlan fx_plan(const int* ex, int mA, int eW, double 
   f.k0 = free_bits(mass);
   f.km = free_bits((ldexpf(mass * mu, -f.kp) + 0.34f * mp * ma) * 0.76f);
   f.ke = free_bits(energy);
-  const int base = eA + eW - 57;
-  f.e0 = eR + eU + base - f.k0;
-  f.em = eR + 2 * eU + base + f.kp - f.km;
-  f.ee = eR + eU + eH + base - f.ke;
-  f.ok = finite && range && even && (eU - eUt <= 5 || ex[FX_U] >> 20 == 0);
+  f.e0 = eR + E + eW - 57 - f.k0;
+  f.em = eR + eU + E + eW - 57 + f.kp - f.km;
+  f.ee = eR + E + eH + eW - 57 - f.ke;
+  if constexpr (GEN) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (st) {
+        // units of m u_c and p Ja_c; the sums are in the coarser one
+        const int u1 = eR + E + eC[c] - 55, u2 = ePt + aC[c] - 54, T = max(u1, u2);
+        const int s1 = min(T - u1, 62), s2 = min(T - u2, 62);
+        rows->s1[c] = s1;
+        rows->s2[c] = s2;
+        rows->h1[c] = (1LL << s1) >> 1;
+        rows->h2[c] = (1LL << s2) >> 1;
+        rows->km[c] = free_bits((ldexpf(mass * uC[c], -s1) + 0.34f * ldexpf(mp * fx_mant(mt.col[c]), -s2)) * 0.76f);
+        rows->em[c] = T + eW - 2 - rows->km[c];
+      } else {
+        rows->bU[c] = f.bU;
+        rows->em[c] = f.em;
+      }
+    }
+  }
+  f.ok = finite && range && even && mt.kind != FX_GRADED && (eU - eUt <= 5 || xU >> 20 == 0);
   return f;
 }
 
-// The metrics Ja of every element in its own unit: limbs [9][K n3] and the
-// largest fx_mag [K] (one bit below fx_of's bound, so that a pair's sum of
-// three products S_u . S_a has room).  One block per element, once per mesh.
+// The metrics Ja of every element in its units: limbs [9][K n3] and FxMetric [K]
+// (one bit below fx_of's bound, so that a pair's sum of three products S_u . S_a
+// has room).  One block per element, once per mesh; *kinds collects the kinds.
 static __global__ void k_metric_fx(int n3, long long S, const double* __restrict__ Ja, Fx* __restrict__ JaX,
-                                   int* __restrict__ mA) {
-  __shared__ int mx;
-  if (threadIdx.x == 0) mx = 0;
+                                   FxMetric* __restrict__ mt, int* __restrict__ kinds) {
+  __shared__ int mx[3], graded;
+  if (threadIdx.x < 3) mx[threadIdx.x] = 100 << 20;
+  if (threadIdx.x == 3) graded = 0;
   __syncthreads();
   const size_t e0 = (size_t)blockIdx.x * n3;
-  int b = 0;
-  for (int t = threadIdx.x; t < n3; t += blockDim.x)
-    for (int c = 0; c < 9; ++c) b = max(b, fx_mag(Ja[c * S + e0 + t]));
-  atomicMax(&mx, b);
+  auto column = [&](int t, int c) {
+    int b = 0;
+    for (int d = 0; d < 3; ++d) b = max(b, fx_mag(Ja[(d * 3 + c) * S + e0 + t]));
+    return b;
+  };
+  for (int c = 0; c < 3; ++c) {
+    int b = 0;
+    for (int t = threadIdx.x; t < n3; t += blockDim.x) b = max(b, column(t, c));
+    atomicMax(&mx[c], b);
+  }
   __syncthreads();
-  const int mg = max(mx, 100 << 20), eb = (mg >> 20) + 1;
-  for (int t = threadIdx.x; t < n3; t += blockDim.x)
-    for (int c = 0; c < 9; ++c) JaX[c * S + e0 + t] = fx_of(Ja[c * S + e0 + t], eb);
-  if (threadIdx.x == 0) mA[blockIdx.x] = mg;
+  const int most = max(mx[0], max(mx[1], mx[2])), least = min(mx[0], min(mx[1], mx[2]));
+  const bool even = most - least <= 1 << 20;
+  for (int t = threadIdx.x; t < n3; t += blockDim.x) {
+    for (int c = 0; c < 3; ++c) {
+      if (mx[c] - column(t, c) > 3 << 20) graded = 1;
+      const int eb = ((even ? most : mx[c]) >> 20) + 1;
+      for (int d = 0; d < 3; ++d) JaX[(d * 3 + c) * S + e0 + t] = fx_of(Ja[(d * 3 + c) * S + e0 + t], eb);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int kind = graded ? FX_GRADED : (even ? FX_EVEN : FX_STRETCHED);
+    mt[blockIdx.x] = FxMetric{{even ? most : mx[0], even ? most : mx[1], even ? most : mx[2]}, kind};
+    if (kind != FX_EVEN) atomicOr(kinds, 1 << kind);
+  }
 }
-
 
 template <int N, int VF>
 struct VolFxShape {
@@ -286,10 +392,11 @@ struct VolFxShape {
 // n consecutive lanes; a lane forms the pairs with the nodes at cyclic distance
 // 1 .. n/2 and hands their flux to the partner by shuffle, where it is
 // subtracted (Q is antisymmetric); a pair at distance n/2 is formed by both of
-// its lanes.
-template <int N, int VF>
+// its lanes.  ST: a stretched element, with its rows r.
+template <int N, int VF, bool ST>
 __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, long long* sR, const Fx* sT,
-                                                 const long long* sW, const int* sH, const FxPlan& f, int t) {
+                                                 const long long* sW, const int* sH, const FxPlan& f,
+                                                 const volatile FxRows& r, int t) {
   using Sh = VolShape<N>;
   constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW, NQ = VF == FX_EC ? 8 : 6 + VF;
   const int warp = t >> 5, lane = t & 31;
@@ -317,11 +424,17 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
       const Fx Sa0 = a[0] + sD[sm], Sa1 = a[1] + sD[n3 + sm], Sa2 = a[2] + sD[2 * n3 + sm];
       const Fx mv1 = sQ[n3 + sm], mv2 = sQ[2 * n3 + sm], mv3 = sQ[3 * n3 + sm];
       const Fx Su = q[1] + mv1, Sv = q[2] + mv2, Sw = q[3] + mv3;
-      FxSum s(Su, Sa0);
-      s.add(Sv, Sa1);
-      s.fold();
-      s.add(Sw, Sa2);
-      const Fx ua = fx_split<1>(s.get());  // 4 {u}.{a}
+      Fx ua;  // 4 {u}.{a}
+      if constexpr (ST) {
+        ua = fx_split<1>((FxSum(Su, Sa0, r.ht[0]).get() >> r.t[0]) + (FxSum(Sv, Sa1, r.ht[1]).get() >> r.t[1]) +
+                         (FxSum(Sw, Sa2, r.ht[2]).get() >> r.t[2]));
+      } else {
+        FxSum s(Su, Sa0);
+        s.add(Sv, Sa1);
+        s.fold();
+        s.add(Sw, Sa2);
+        ua = fx_split<1>(s.get());
+      }
       long long F[5];
       Fx pq;  // 2 Q {p'} (EC: 2 Q (p~ - p_ref))
       if constexpr (VF == FX_KEP) {
@@ -349,22 +462,32 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
         pq = fx_split<0>(fx_mul(fx_split<0>(pt), Q));
         F[0] = fx_mul(Sr, uq);  // 8 Q F_rho
         // 16 F_E = 4 {u}.{a} [S_rho G (S_e Q(t) + u_A.u_B) + 4 (p~ - p_ref) + 4 p_ref]
-        FxSum k(q[1], mv1);
-        k.add(q[2], mv2);
-        k.add(q[3], mv3);
-        const long long Y = (fx_mul(Se, fx_series(tb, FX_Q)) >> f.kt) + (k.get() >> f.kd);
+        long long uu;
+        if constexpr (ST) {
+          uu = (fx_mul(q[1], mv1) >> r.kd[0]) + (fx_mul(q[2], mv2) >> r.kd[1]) + (fx_mul(q[3], mv3) >> r.kd[2]);
+        } else {
+          FxSum k(q[1], mv1);
+          k.add(q[2], mv2);
+          k.add(q[3], mv3);
+          uu = k.get() >> f.kd;
+        }
+        const long long Y = (fx_mul(Se, fx_series(tb, FX_Q)) >> f.kt) + uu;
         const long long Z = fx_mul(Sr, fx_split<0>(Y)) + (pt >> f.kz) + f.pref;
         F[4] = fx_mul(uq, fx_split<1>(Z));
       }
-      const Fx mu = fx_split<1>(F[0] >> f.kp);
-      auto momentum = [&](Fx S, Fx Sa) {
-        FxSum x(mu, S);
-        x.add(pq, Sa);
-        return x.get();
+      const Fx mu = fx_split<1>(ST ? F[0] : F[0] >> f.kp);
+      auto momentum = [&](Fx S, Fx Sa, int c) {
+        if constexpr (ST) {
+          return (FxSum(mu, S, r.h1[c]).get() >> r.s1[c]) + (FxSum(pq, Sa, r.h2[c]).get() >> r.s2[c]);
+        } else {
+          FxSum x(mu, S);
+          x.add(pq, Sa);
+          return x.get();
+        }
       };
-      F[1] = momentum(Su, Sa0);
-      F[2] = momentum(Sv, Sa1);
-      F[3] = momentum(Sw, Sa2);
+      F[1] = momentum(Su, Sa0, 0);
+      F[2] = momentum(Sv, Sa1, 1);
+      F[3] = momentum(Sw, Sa2, 2);
 #pragma unroll
       for (int v = 0; v < 5; ++v) acc[v] += F[v];
       if (2 * d != n) {
@@ -377,8 +500,9 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
       const Fx wi = fx_split<0>(sW[pos] << min(sH[pos], min(sH[la], sH[lb])));
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const long long r = fx_mul_shl(fx_split<0>(acc[v]), wi, v == 0 ? f.k0 : (v == 4 ? f.ke : f.km));
-        sR[v * n3 + ms] = dir == 0 ? r : r + sR[v * n3 + ms];
+        const int k = v == 0 ? f.k0 : (v == 4 ? f.ke : (ST ? r.km[v - 1] : f.km));
+        const long long x = fx_mul_shl(fx_split<0>(acc[v]), wi, k);
+        sR[v * n3 + ms] = dir == 0 ? x : x + sR[v * n3 + ms];
       }
     }
     __syncthreads();
@@ -409,7 +533,8 @@ __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<doub
 // (elements out of fx_plan's range: in FP64), the epilogue in FP64.  Measured at N = 7, 32^3 elements: KEP flux 10.08 ms with
 // FP64 pair fluxes (FP64 pipe 90 % busy), 3.07 ms in fixed point (issue 52 %,
 // integer pipes 37 %, FP64 pipe 30 %).
-template <int N, int MODE, int VF>
+// GEN: for meshes with stretched elements (their passes beside the others').
+template <int N, int MODE, int VF, bool GEN>
 __global__ void __launch_bounds__(VolShape<N>::THREADS, (resident_ctas(VolShape<N>::THREADS, VolFxShape<N, VF>::SMEM, 1024)))
 k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysDev ph, const Tables<N> tab,
             const FxTab<N> ft, const double* __restrict__ Rv, const double* __restrict__ Fs, double* __restrict__ Out,
@@ -420,6 +545,7 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int sEx[FX_NUM];
   __shared__ FxPlan sF;
+  __shared__ FxRows sRows;
   Fx* sQ = reinterpret_cast<Fx*>(smem_raw);
   Fx* sA = sQ + QS * n3;
   long long* sR = reinterpret_cast<long long*>(sA + 9 * n3);
@@ -466,7 +592,9 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
     ex[FX_H] = fx_mag(VF == FX_KEP ? q.h : en);
     ex[FX_NRHO] = 0x7fffffff - fx_mag(q.rho);
     ex[FX_NH] = 0x7fffffff - ex[FX_H];
-    ex[FX_U] = max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w));
+    ex[FX_U] = GEN ? fx_mag(q.u) : max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w));
+    ex[FX_V] = fx_mag(q.v);
+    ex[FX_W] = fx_mag(q.w);
     ex[FX_P] = fx_mag(q.p);
     ex[FX_B] = fx_mag(be);
     ex[FX_IR] = fx_mag(irh);
@@ -475,13 +603,14 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
       for (int x = 0; x < FX_NUM; ++x) ex[x] = 0;
     }
 #pragma unroll
-    for (int x = 0; x < (EC ? FX_NUM : FX_B + VF); ++x) {
+    for (int x = 0; x < FX_NUM; ++x) {
+      if (x >= FX_V ? !GEN : x >= (EC ? FX_V : FX_B + VF)) continue;
       const int mx = __reduce_max_sync(0xffffffffu, ex[x]);
       if ((t & 31) == 0) atomicMax(&sEx[x], mx);
     }
   }
   __syncthreads();
-  if (t == 0) sF = fx_plan<VF>(sEx, m.JaX_max[e], ft.eW, ph.p_ref, ph.gm1);
+  if (t == 0) sF = fx_plan<VF, GEN>(sEx, m.JaX_max[e], ft.eW, ph.p_ref, ph.gm1, &sRows);
   __syncthreads();
   const FxPlan f = sF;
   const bool fx = f.ok != 0;
@@ -489,9 +618,9 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
     const int ts = vslot<N, double>(t);
     if (fx) {
       sQ[ts] = fx_of(q.rho, f.bR);
-      sQ[n3 + ts] = fx_of(q.u, f.bU);
-      sQ[2 * n3 + ts] = fx_of(q.v, f.bU);
-      sQ[3 * n3 + ts] = fx_of(q.w, f.bU);
+      sQ[n3 + ts] = fx_of(q.u, GEN ? sRows.bU[0] : f.bU);
+      sQ[2 * n3 + ts] = fx_of(q.v, GEN ? sRows.bU[1] : f.bU);
+      sQ[3 * n3 + ts] = fx_of(q.w, GEN ? sRows.bU[2] : f.bU);
       if constexpr (EC) {
         sQ[4 * n3 + ts] = fx_of(be * q.p, f.bP);
         sQ[5 * n3 + ts] = fx_of(en, f.bH);
@@ -508,7 +637,8 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
   }
   if (fx) {
     __syncthreads();
-    volume_passes_fx<N, VF>(sQ, sA, sR, sT, sW, sH, f, t);
+    if (GEN && m.JaX_max[e].kind == FX_STRETCHED) volume_passes_fx<N, VF, GEN>(sQ, sA, sR, sT, sW, sH, f, sRows, t);
+    else volume_passes_fx<N, VF, false>(sQ, sA, sR, sT, sW, sH, f, sRows, t);
   } else {
     volume_passes_fp64<N, VF>(reinterpret_cast<double*>(smem_raw), m, ph, tab, Rv, e, t);
   }
@@ -517,7 +647,8 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
         const int ts = vslot<N, double>(nd);
         if (fx) {
           const int k = min(sH[nd % n], min(sH[nd / n % n], sH[nd / n2]));
-          const int eu[5] = {f.e0 - k, f.em - k, f.em - k, f.em - k, f.ee - k};
+          const int eu[5] = {f.e0 - k, (GEN ? sRows.em[0] : f.em) - k, (GEN ? sRows.em[1] : f.em) - k,
+                             (GEN ? sRows.em[2] : f.em) - k, f.ee - k};
 #pragma unroll
           for (int v = 0; v < 5; ++v) acc[v] = fx_double(sR[v * n3 + ts], eu[v]);
           if (ph.viscous) {
