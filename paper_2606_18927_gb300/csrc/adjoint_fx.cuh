@@ -11,8 +11,9 @@
 // 28 more bits (the full product of the last factors), the sum of the three is
 // normalised in each lane before it is multiplied, and the directions' sums are
 // added in FP64: the error against the extended-precision oracle's J^T lam
-// stays at FP64's.  Elements out of range (non-finite values, exponents beyond
-// 2^200) are summed in FP64.
+// stays at FP64's.  Elements out of range (non-finite values; a value's or a
+// cotangent's largest magnitude beyond 2^200 or below 2^-200 without being zero)
+// are summed in FP64.
 #pragma once
 #include "adjoint.cuh"
 #include "volume_fx.cuh"
@@ -38,14 +39,18 @@ __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& 
 #pragma unroll
   for (int x = 0; x < AX_NUM; ++x) {
     const int e = (ex[x] >> 20) - 1022;
-    eX[x] = max(e, -200);  // (smaller values, zeros among them, in that unit)
-    ok = ok && e < 200;
+    eX[x] = max(e, -200);  // (zeros in that unit)
+    ok = ok && e < 200 && (e > -200 || ex[x] == 0);
   }
   const int eA = (mt.col[0] >> 20) - 1022;  // (elements whose columns differ are summed in FP64)
   f.bR = eX[AX_RHO] + 1022; f.bU = eX[AX_U] + 1022; f.bH = eX[AX_H] + 1022;
   f.bL0 = eX[AX_L0] + 1022; f.bLM = eX[AX_LM] + 1022; f.bLE = eX[AX_LE] + 1022;
-  // units of the three parts of mu0 + (mu_m . S_u + mu_4 S_h) / 2
-  const int e0 = eX[AX_L0] + eW - 60, e1 = eX[AX_LM] + eX[AX_U] + eW - 59, e2 = eX[AX_LE] + eX[AX_H] + eW - 59;
+  // units of the three parts of mu0 + (mu_m . S_u + mu_4 S_h) / 2 (a part that is zero
+  // must not raise the others' unit)
+  auto unit = [](bool zero, int e) { return zero ? -2000 : e; };
+  const int e0 = unit(ex[AX_L0] == 0, eX[AX_L0] + eW - 60),
+            e1 = unit(ex[AX_LM] == 0 || ex[AX_U] == 0, eX[AX_LM] + eX[AX_U] + eW - 59),
+            e2 = unit(ex[AX_LE] == 0 || ex[AX_H] == 0, eX[AX_LE] + eX[AX_H] + eW - 59);
   const int et = max(e0, max(e1, e2)) + 1;
   f.s0 = min(et - e0, 63); f.s1 = min(et - e1, 63); f.s2 = min(et - e2, 63);
   f.eg[0] = et + eX[AX_U] + eA + 3;
