@@ -12,15 +12,16 @@
 // normalised in each lane before it is multiplied, and the directions' sums are
 // added in FP64: the error against the extended-precision oracle's J^T lam
 // stays at FP64's.  Elements out of range (non-finite values; a value's or a
-// cotangent's largest magnitude beyond 2^200 or below 2^-200 without being zero)
-// are summed in FP64.
+// cotangent's largest magnitude beyond 2^200 or below 2^-200 without being zero;
+// density or enthalpy differing by more than a factor 8 over the nodes: the gradients
+// at the light ones are divided by their own density) are summed in FP64.
 #pragma once
 #include "adjoint.cuh"
 #include "volume_fx.cuh"
 
 namespace dg {
 
-enum { AX_RHO, AX_U, AX_H, AX_L0, AX_LM, AX_LE, AX_NUM };
+enum { AX_RHO, AX_U, AX_H, AX_L0, AX_LM, AX_LE, AX_NRHO, AX_NH, AX_NUM };
 struct AdjFxPlan {
   int ok;
   int bR, bU, bH, bL0, bLM, bLE;  // biased exponent bounds for fx_of
@@ -28,16 +29,16 @@ struct AdjFxPlan {
   int eg[4];                      // the units of the sums rho, u, p, h
 };
 
-// ex: the largest fx_mag of each value; mt: the element's metrics; eW:
+// ex: the largest fx_mag of each value (AX_NRHO, AX_NH: of 0x7fffffff - fx_mag); mt: the element's metrics; eW:
 // lam~ / w is in units 2^eW times lam~'s.  Bounds in units of 2^60, times Q for the
 // pair terms: the sum of the three parts 3 (half of 6, by the extra shift), rho
 // and u 1.1, p 1.5, h 0.75; a line's sum of |Q| is below 3.7.
 __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& mt, int eW) {
   AdjFxPlan f;
-  int eX[AX_NUM];
+  int eX[AX_NRHO];
   bool ok = true;
 #pragma unroll
-  for (int x = 0; x < AX_NUM; ++x) {
+  for (int x = 0; x < AX_NRHO; ++x) {
     const int e = (ex[x] >> 20) - 1022;
     eX[x] = max(e, -200);  // (zeros in that unit)
     ok = ok && e < 200 && (e > -200 || ex[x] == 0);
@@ -57,7 +58,9 @@ __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& 
   f.eg[1] = et + eX[AX_RHO] + eA + 2;
   f.eg[2] = eX[AX_LM] + eW + eA - 58;
   f.eg[3] = eX[AX_U] + eA + eX[AX_LE] + eW + eX[AX_RHO] - 57;
-  f.ok = ok && abs(eA) < 200 && mt.kind == FX_EVEN;
+  const bool even = (ex[AX_RHO] >> 20) - ((0x7fffffff - ex[AX_NRHO]) >> 20) <= 2 &&
+                    (ex[AX_H] >> 20) - ((0x7fffffff - ex[AX_NH]) >> 20) <= 2;
+  f.ok = ok && even && abs(eA) < 200 && mt.kind == FX_EVEN;
   return f;
 }
 
@@ -259,8 +262,10 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
   if (t < n) sW[t] = ft.iw[t];
   __syncthreads();
   {
+    const bool in = t < n3;
     const int ex[AX_NUM] = {fx_mag(q.rho), max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w)), fx_mag(q.h), fx_mag(l[0]),
-                            max(max(fx_mag(l[1]), fx_mag(l[2])), fx_mag(l[3])), fx_mag(l[4])};
+                            max(max(fx_mag(l[1]), fx_mag(l[2])), fx_mag(l[3])), fx_mag(l[4]),
+                            in ? 0x7fffffff - fx_mag(q.rho) : 0, in ? 0x7fffffff - fx_mag(q.h) : 0};
 #pragma unroll
     for (int x = 0; x < AX_NUM; ++x) {
       const int mx = __reduce_max_sync(0xffffffffu, ex[x]);

@@ -5,6 +5,7 @@ result is that of the unscaled cotangent to FP64 rounding of two summation order
 import numpy as np
 import pytest
 
+from paper_2606_18927_gb300 import dg, inputs as I
 from gpu_helpers import torch_cuda
 from test_gpu_adjoint_fx import cotangent, operator, vjp
 
@@ -30,3 +31,42 @@ def test_small_cotangents(ora, N, kind, power):
     e = [float(np.abs(a[v] - b[v]).max() / max(np.abs(a[v]).max(), 1e-300)) for v in range(5)]
     print(N, kind, power, ["%.1e" % x for x in e])
     assert max(e) <= 1e-13, e
+
+
+def columns(ora, o, U, lam, cols):
+    """(J^T lam)_c of the extended oracle, and the sum of the magnitudes it adds up."""
+    g, scale, d = np.zeros(len(cols)), np.zeros(len(cols)), np.zeros(U.size)
+    for k, c in enumerate(cols):
+        d[c] = 1.0
+        t = lam * o.jvp(U, d.reshape(U.shape))[1]
+        d[c] = 0.0
+        g[k], scale[k] = t.sum(), np.abs(t).sum()
+    return g, scale
+
+
+@pytest.mark.parametrize("N", [3, 5])
+@pytest.mark.parametrize("contrast", [0.8, 1.9, 3.0, 6.0])
+def test_density_contrast(ora, N, contrast):
+    """A density that differs by e^contrast over an element: the gradients at its light nodes,
+    divided by their own density, against the oracle's columns.  Bound: 4e-15 (some 36 roundings)
+    of the magnitudes that a column adds up."""
+    torch = torch_cuda()
+    spec = I.BoxSpec(N, 2, 1, 1)
+    phys = I.phys_params(Ma=0.3, Re=1600.0)
+    X = I.node_coordinates(spec, ora.lgl(N)[0])
+    x, y, z = X
+    rho = np.exp(0.5 * contrast * np.cos(x))
+    u = np.sin(x) * np.cos(y) + 0.3
+    v = 0.4 - np.cos(x) * np.sin(y)
+    w = 0.5 * np.cos(z - x)
+    U = I.perturb(I.conservative(rho, u, v, w, phys["p0"] + 0.2 * np.cos(2 * x) * np.sin(y), phys["gamma"]), rel=1e-3)
+    g = dg.Operator(N, X, I.connectivity(spec), phys, surf_flux=2)
+    o = ora.Oracle(N, X, I.connectivity(spec), phys, vol_flux=0, surf_flux=2, viscous=1, extended=True)
+    lam = I.random_direction(U.shape, 43)
+    got = vjp(torch, g, U, lam).ravel()
+    light = np.argsort(U[0].ravel())[: U[0].size // 6]
+    cols = np.concatenate([v * U[0].size + light[v::5][:12] for v in range(5)])
+    ref, scale = columns(ora, o, U, lam, cols)
+    e = np.abs(got[cols] - ref) / scale
+    print(N, contrast, e.max(), np.sqrt((e * e).mean()))
+    assert e.max() <= 4e-15
