@@ -21,46 +21,100 @@
 
 namespace dg {
 
-enum { AX_RHO, AX_U, AX_H, AX_L0, AX_LM, AX_LE, AX_NRHO, AX_NH, AX_NUM };
+enum { AX_RHO, AX_U, AX_H, AX_L0, AX_LM, AX_LE, AX_NRHO, AX_NH, AX_V, AX_W, AX_LM1, AX_LM2, AX_NUM };
 struct AdjFxPlan {
   int ok;
   int bR, bU, bH, bL0, bLM, bLE;  // biased exponent bounds for fx_of
   int s0, s1, s2;                 // right shifts of mu0, mu_m . S_u, mu_4 S_h to their common unit
   int eg[4];                      // the units of the sums rho, u, p, h
 };
+// Stretched elements (FxMetric): what differs by component c of u, Ja and the
+// momentum's cotangent (s1, eg[1] and bU, bLM of AdjFxPlan are not used); as FxRows
+struct AdjFxRows {
+  int bU[3], bLM[3];
+  int t[3], s1[3], sz[3];         // right shifts of S_u S_a, mu_c S_u and mu_c S_a to their sums' units
+  int yt[3], yq[3];               // and of tt S_a and (S_u . S_a / 2) mu_c to that of the velocity's term
+  long long ht[3], h1[3], hz[3], hyt[3], hyq[3];  // half of what they drop
+  int eg[3];                      // the units of the sums u
+};
 
 // ex: the largest fx_mag of each value (AX_NRHO, AX_NH: of 0x7fffffff - fx_mag); mt: the element's metrics; eW:
 // lam~ / w is in units 2^eW times lam~'s.  Bounds in units of 2^60, times Q for the
 // pair terms: the sum of the three parts 3 (half of 6, by the extra shift), rho
 // and u 1.1, p 1.5, h 0.75; a line's sum of |Q| is below 3.7.
-__device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& mt, int eW) {
+template <bool GEN>
+__device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& mt, int eW, AdjFxRows* rows) {
   AdjFxPlan f;
+  const bool st = GEN && mt.kind == FX_STRETCHED;
+  const int xU[3] = {ex[AX_U], ex[AX_V], ex[AX_W]}, xM[3] = {ex[AX_LM], ex[AX_LM1], ex[AX_LM2]};
   int eX[AX_NRHO];
+  bool zero[AX_NRHO];
   bool ok = true;
 #pragma unroll
   for (int x = 0; x < AX_NRHO; ++x) {
-    const int e = (ex[x] >> 20) - 1022;
+    int mag = ex[x];
+    if (GEN && x == AX_U) mag = max(mag, max(xU[1], xU[2]));
+    if (GEN && x == AX_LM) mag = max(mag, max(xM[1], xM[2]));
+    const int e = (mag >> 20) - 1022;
     eX[x] = max(e, -200);  // (zeros in that unit)
-    ok = ok && e < 200 && (e > -200 || ex[x] == 0);
+    ok = ok && e < 200 && (e > -200 || mag == 0);
+    zero[x] = mag == 0;
   }
-  const int eA = (mt.col[0] >> 20) - 1022;  // (elements whose columns differ are summed in FP64)
+  const int eA = (max(mt.col[0], max(mt.col[1], mt.col[2])) >> 20) - 1022;
   f.bR = eX[AX_RHO] + 1022; f.bU = eX[AX_U] + 1022; f.bH = eX[AX_H] + 1022;
   f.bL0 = eX[AX_L0] + 1022; f.bLM = eX[AX_LM] + 1022; f.bLE = eX[AX_LE] + 1022;
   // units of the three parts of mu0 + (mu_m . S_u + mu_4 S_h) / 2 (a part that is zero
   // must not raise the others' unit)
   auto unit = [](bool zero, int e) { return zero ? -2000 : e; };
-  const int e0 = unit(ex[AX_L0] == 0, eX[AX_L0] + eW - 60),
-            e1 = unit(ex[AX_LM] == 0 || ex[AX_U] == 0, eX[AX_LM] + eX[AX_U] + eW - 59),
-            e2 = unit(ex[AX_LE] == 0 || ex[AX_H] == 0, eX[AX_LE] + eX[AX_H] + eW - 59);
+  const int e0 = unit(zero[AX_L0], eX[AX_L0] + eW - 60),
+            e2 = unit(zero[AX_LE] || zero[AX_H], eX[AX_LE] + eX[AX_H] + eW - 59);
+  int e1 = unit(zero[AX_LM] || zero[AX_U], eX[AX_LM] + eX[AX_U] + eW - 59);
+  // stretched: exponents of u_c, mu_c (no further than 2^-40 below the largest) and Ja_c
+  int eC[3], eM[3], aC[3], E = eX[AX_U] + eA, Z = -3000;  // E, Z: of S_u . S_a and mu . S_a
+  if (st) {
+    e1 = -2000;
+    E = -3000;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      eC[c] = max((xU[c] >> 20) - 1022, eX[AX_U] - 40);
+      eM[c] = max((xM[c] >> 20) - 1022, eX[AX_LM] - 40);
+      aC[c] = (mt.col[c] >> 20) - 1022;
+      ok = ok && abs(aC[c]) < 200;
+      E = max(E, eC[c] + aC[c]);
+      Z = max(Z, eM[c] + aC[c]);
+      e1 = max(e1, unit(zero[AX_LM] || zero[AX_U], eM[c] + eC[c] + eW - 59));
+    }
+  }
   const int et = max(e0, max(e1, e2)) + 1;
+  if (st) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      auto shift = [](int x) { return min(max(x, 0), 62); };
+      auto half = [](int k) { return (1LL << k) >> 1; };
+      rows->bU[c] = eC[c] + 1022;
+      rows->bLM[c] = eM[c] + 1022;
+      rows->t[c] = shift(E - eC[c] - aC[c]);
+      rows->s1[c] = shift(et - (eM[c] + eC[c] + eW - 59));
+      rows->sz[c] = shift(Z - eM[c] - aC[c]);
+      const int ut = et + aC[c] + 3, uq = unit(zero[AX_LM], E + eM[c] + eW - 56), G = max(ut, uq);
+      rows->yt[c] = shift(G - ut);
+      rows->yq[c] = shift(G - uq);
+      rows->eg[c] = G + eX[AX_RHO] - 1;
+      rows->ht[c] = half(rows->t[c]);
+      rows->h1[c] = half(rows->s1[c]);
+      rows->hz[c] = half(rows->sz[c]);
+      rows->hyt[c] = half(rows->yt[c]);
+      rows->hyq[c] = half(rows->yq[c]);
+    }
+  }
   f.s0 = min(et - e0, 63); f.s1 = min(et - e1, 63); f.s2 = min(et - e2, 63);
-  f.eg[0] = et + eX[AX_U] + eA + 3;
+  f.eg[0] = et + E + 3;
   f.eg[1] = et + eX[AX_RHO] + eA + 2;
-  f.eg[2] = eX[AX_LM] + eW + eA - 58;
-  f.eg[3] = eX[AX_U] + eA + eX[AX_LE] + eW + eX[AX_RHO] - 57;
+  f.eg[2] = (st ? Z : eX[AX_LM] + eA) + eW - 58;
+  f.eg[3] = E + eX[AX_LE] + eW + eX[AX_RHO] - 57;
   const bool even = (ex[AX_RHO] >> 20) - ((0x7fffffff - ex[AX_NRHO]) >> 20) <= 2 &&
                     (ex[AX_H] >> 20) - ((0x7fffffff - ex[AX_NH]) >> 20) <= 2;
-  f.ok = ok && even && abs(eA) < 200 && mt.kind == FX_EVEN;
+  f.ok = ok && even && abs(eA) < 200 && mt.kind != FX_GRADED;
   return f;
 }
 
@@ -91,11 +145,12 @@ struct AdjFxShape {
 // [5][n3] scratch, sA [3][n3] scratch, sG [6][n3] the sums of (rho, u, v, w, p', h),
 // in FP64.
 // Lanes, pairs and shuffles as in volume_passes_fx; a pair's terms are the same
-// for its two nodes.
-template <int N>
+// for its two nodes.  ST: a stretched element, with its rows r (read from shared
+// memory as in volume_passes_fx).
+template <int N, bool ST>
 __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sLt, Fx* sA, double* sG, const Fx* sT,
                                               const long long* sW, const Fx* __restrict__ JaX, size_t S, size_t e0,
-                                              const AdjFxPlan& f, int t) {
+                                              const AdjFxPlan& f, const volatile AdjFxRows& r, int t) {
   using Sh = VolShape<N>;
   constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW;
   const int warp = t >> 5, lane = t & 31;
@@ -141,43 +196,65 @@ __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sL
       const Fx Sa0 = a[0] + sA[sm], Sa1 = a[1] + sA[n3 + sm], Sa2 = a[2] + sA[2 * n3 + sm];
       const Fx Su = q[1] + sQ[n3 + sm], Sv = q[2] + sQ[2 * n3 + sm], Sw = q[3] + sQ[3 * n3 + sm];
       const Fx m1 = dif(1), m2 = dif(2), m3 = dif(3), m4 = dif(4);
-      FxSum k(Su, Sa0);
-      k.add(Sv, Sa1);
-      k.fold();
-      k.add(Sw, Sa2);
-      const long long qv = k.get();  // S_u . S_a
-      FxSum x(m1, Su);  // (differences have limbs as large as sums: one term is up to 4.3 2^60)
-      x.fold();
-      x.add(m2, Sv);
-      x.fold();
-      x.add(m3, Sw);
+      long long qv, mu;  // S_u . S_a; mu_m . S_u in the unit of tt
+      if constexpr (ST) {
+        qv = (FxSum(Su, Sa0, r.ht[0]).get() >> r.t[0]) + (FxSum(Sv, Sa1, r.ht[1]).get() >> r.t[1]) +
+             (FxSum(Sw, Sa2, r.ht[2]).get() >> r.t[2]);
+        mu = (FxSum(m1, Su, r.h1[0]).get() >> r.s1[0]) + (FxSum(m2, Sv, r.h1[1]).get() >> r.s1[1]) +
+             (FxSum(m3, Sw, r.h1[2]).get() >> r.s1[2]);
+      } else {
+        FxSum k(Su, Sa0);
+        k.add(Sv, Sa1);
+        k.fold();
+        k.add(Sw, Sa2);
+        qv = k.get();
+        FxSum x(m1, Su);  // (differences have limbs as large as sums: one term is up to 4.3 2^60)
+        x.fold();
+        x.add(m2, Sv);
+        x.fold();
+        x.add(m3, Sw);
+        mu = x.get() >> f.s1;
+      }
       const Fx m0 = dif(0);
-      const long long tt = ((((long long)m0.h << 31) + m0.l) >> f.s0) + (x.get() >> f.s1) +
-                           (fx_mul(m4, q[4] + sQ[4 * n3 + sm]) >> f.s2);
+      const long long tt =
+          ((((long long)m0.h << 31) + m0.l) >> f.s0) + mu + (fx_mul(m4, q[4] + sQ[4 * n3 + sm]) >> f.s2);
       const Fx Qv = fx_split<1>(qv);
       const long long sq = fx_mul(q[0] + sQ[sm], Q);  // S_rho Q
       // tt (and S_u . S_a / 2 beside it) shifted up in this lane as far as both
       // have room, S_rho Q down by as much
       auto room = [](long long r) { return __clzll(r ^ (r >> 63)) - 3; };
-      const int up = max(0, min(min(room(tt), room(qv) + f.s1), 20));
+      const int s1 = ST ? 0 : f.s1;
+      const int up = max(0, min(min(room(tt), room(qv) + s1), 20));
       const Fx Tn = fx_split<0>(tt << up);
-      const Fx Qs = fx_split<0>(up > f.s1 ? qv << (up - f.s1) : qv >> (f.s1 - up));
+      const Fx Qs = fx_split<0>(up > s1 ? qv << (up - s1) : qv >> (s1 - up));
       const Fx Sr = fx_split<1>(sq), Sn = fx_split<1>(sq >> up);
       Fx96 F[6];
       F[0] = fx_mul96(fx_split<0>(tt), fx_split<0>(fx_mul(Qv, Q)));
-      auto vel = [&](Fx Sa, Fx mk) {
-        FxSum y(Tn, Sa);
-        y.add(Qs, mk);
-        return fx_mul96(Sn, fx_split<1>(y.get()));
+      auto vel = [&](Fx Sa, Fx mk, int c) {
+        if constexpr (ST) {
+          return fx_mul96(Sn, fx_split<1>((FxSum(Tn, Sa, r.hyt[c]).get() >> r.yt[c]) +
+                                          (FxSum(Qs, mk, r.hyq[c]).get() >> r.yq[c])));
+        } else {
+          FxSum y(Tn, Sa);
+          y.add(Qs, mk);
+          return fx_mul96(Sn, fx_split<1>(y.get()));
+        }
       };
-      F[1] = vel(Sa0, m1);
-      F[2] = vel(Sa1, m2);
-      F[3] = vel(Sa2, m3);
-      FxSum z(m1, Sa0);
-      z.add(m2, Sa1);
-      z.fold();
-      z.add(m3, Sa2);
-      F[4] = fx_mul96(fx_split<1>(z.get()), Q);
+      F[1] = vel(Sa0, m1, 0);
+      F[2] = vel(Sa1, m2, 1);
+      F[3] = vel(Sa2, m3, 2);
+      long long zz;  // mu_m . S_a
+      if constexpr (ST) {
+        zz = (FxSum(m1, Sa0, r.hz[0]).get() >> r.sz[0]) + (FxSum(m2, Sa1, r.hz[1]).get() >> r.sz[1]) +
+             (FxSum(m3, Sa2, r.hz[2]).get() >> r.sz[2]);
+      } else {
+        FxSum z(m1, Sa0);
+        z.add(m2, Sa1);
+        z.fold();
+        z.add(m3, Sa2);
+        zz = z.get();
+      }
+      F[4] = fx_mul96(fx_split<1>(zz), Q);
       F[5] = fx_mul96(Sr, fx_split<0>(fx_mul(Qv, m4)));
 #pragma unroll
       for (int v = 0; v < 6; ++v) {
@@ -198,10 +275,11 @@ __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sL
 #pragma unroll
       for (int v = 0; v < 6; ++v) {
         // to FP64, with as many of the low bits as there is room for
-        const long long r = acc[v] + (low[v] >> 27);
-        const int k = min(max(__clzll(r ^ (r >> 63)) - 2, 0), 27);
-        const long long w = (r << k) + ((low[v] & 0x7ffffffu) >> (27 - k));
-        const double x = fx_double(w, f.eg[v == 0 ? 0 : (v < 4 ? 1 : v - 2)] - k);
+        const long long s = acc[v] + (low[v] >> 27);
+        const int k = min(max(__clzll(s ^ (s >> 63)) - 2, 0), 27);
+        const long long w = (s << k) + ((low[v] & 0x7ffffffu) >> (27 - k));
+        const int eg = ST && v > 0 && v < 4 ? r.eg[v - 1] : f.eg[v == 0 ? 0 : (v < 4 ? 1 : v - 2)];
+        const double x = fx_double(w, eg - k);
         sG[v * n3 + ms] = dir == 0 ? x : x + sG[v * n3 + ms];
       }
     }
@@ -232,7 +310,8 @@ __device__ __noinline__ void adj_volume_fp64(double* smem, const MeshDev<double>
 // elements: the element kernel with the pairs in FP64 1181 us (FP64 pipe 86 %
 // busy); 495 us without them and 233 us here (issue 47 %, integer pipes 36 %,
 // FP64 pipe 32 %, of which the recovery of the primitives and its transpose).
-template <int N>
+// GEN: for meshes with stretched elements.
+template <int N, bool GEN>
 __global__ void __launch_bounds__(VolShape<N>::THREADS, (resident_ctas(VolShape<N>::THREADS, AdjFxShape<N>::SMEM, 1024)))
 k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const MeshDev<double> m, const PhysDev ph,
              const Tables<N> tab, const FxTab<N> ft, double* __restrict__ gV) {
@@ -240,6 +319,7 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int sEx[AX_NUM];
   __shared__ AdjFxPlan sF;
+  __shared__ AdjFxRows sRows;
   Fx* sQ = reinterpret_cast<Fx*>(smem_raw);
   Fx* sL = sQ + 6 * n3;
   Fx* sLt = sL + 5 * n3;
@@ -263,19 +343,21 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
   __syncthreads();
   {
     const bool in = t < n3;
-    const int ex[AX_NUM] = {fx_mag(q.rho), max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w)), fx_mag(q.h), fx_mag(l[0]),
-                            max(max(fx_mag(l[1]), fx_mag(l[2])), fx_mag(l[3])), fx_mag(l[4]),
-                            in ? 0x7fffffff - fx_mag(q.rho) : 0, in ? 0x7fffffff - fx_mag(q.h) : 0};
+    const int mu = max(max(fx_mag(q.u), fx_mag(q.v)), fx_mag(q.w)), ml = max(max(fx_mag(l[1]), fx_mag(l[2])), fx_mag(l[3]));
+    const int ex[AX_NUM] = {fx_mag(q.rho), GEN ? fx_mag(q.u) : mu, fx_mag(q.h), fx_mag(l[0]), GEN ? fx_mag(l[1]) : ml,
+                            fx_mag(l[4]), in ? 0x7fffffff - fx_mag(q.rho) : 0, in ? 0x7fffffff - fx_mag(q.h) : 0,
+                            fx_mag(q.v), fx_mag(q.w), fx_mag(l[2]), fx_mag(l[3])};
 #pragma unroll
-    for (int x = 0; x < AX_NUM; ++x) {
+    for (int x = 0; x < (GEN ? AX_NUM : AX_V); ++x) {
       const int mx = __reduce_max_sync(0xffffffffu, ex[x]);
       if ((t & 31) == 0) atomicMax(&sEx[x], mx);
     }
   }
   __syncthreads();
-  if (t == 0) sF = adj_fx_plan(sEx, m.JaX_max[e], ft.eW + 1 - AdjFxShape<N>::LSH);
+  if (t == 0) sF = adj_fx_plan<GEN>(sEx, m.JaX_max[e], ft.eW + 1 - AdjFxShape<N>::LSH, &sRows);
   __syncthreads();
   const AdjFxPlan f = sF;
+  const bool st = GEN && m.JaX_max[e].kind == FX_STRETCHED;
   // node slots: swizzled in fixed point (vslot), natural in FP64
   if (t < n3) {
     const int ts = f.ok ? vslot<N, double>(t) : t;
@@ -283,17 +365,18 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
       if (!f.ok) reinterpret_cast<double*>(sQ)[v * n3 + ts] = x[v];
-      else if (v < 5) sQ[v * n3 + ts] = fx_of(x[v], v == 0 ? f.bR : (v < 4 ? f.bU : f.bH));
+      else if (v < 5) sQ[v * n3 + ts] = fx_of(x[v], v == 0 ? f.bR : (v < 4 ? (st ? sRows.bU[v - 1] : f.bU) : f.bH));
     }
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       if (!f.ok) reinterpret_cast<double*>(sL)[v * n3 + ts] = l[v];
-      else sL[v * n3 + ts] = fx_of(l[v], v == 0 ? f.bL0 : (v < 4 ? f.bLM : f.bLE));
+      else sL[v * n3 + ts] = fx_of(l[v], v == 0 ? f.bL0 : (v < 4 ? (st ? sRows.bLM[v - 1] : f.bLM) : f.bLE));
     }
   }
   if (f.ok) {
     __syncthreads();
-    adj_passes_fx<N>(sQ, sL, sLt, sA, sG, sT, sW, m.JaX, S, e0, f, t);
+    if (st) adj_passes_fx<N, GEN>(sQ, sL, sLt, sA, sG, sT, sW, m.JaX, S, e0, f, sRows, t);
+    else adj_passes_fx<N, false>(sQ, sL, sLt, sA, sG, sT, sW, m.JaX, S, e0, f, sRows, t);
   } else {
     adj_volume_fp64<N>(reinterpret_cast<double*>(smem_raw), m, ph, tab, e, t);
   }

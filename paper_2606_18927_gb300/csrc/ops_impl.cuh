@@ -347,9 +347,9 @@ static int run_vjp_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
   if (phase == 3 || phase == 14) {
     if (part && ph.viscous) k_adj_halo_in<N><<<halo_blocks, 128, 0, s>>>(m, m.halo_G, a.gGf);
     if (!ec) {
-      cudaFuncSetAttribute(k_adj_volume<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, AdjFxShape<N>::SMEM);
-      k_adj_volume<N><<<a.K, VolShape<N>::THREADS, AdjFxShape<N>::SMEM, s>>>(a.Uin, a.lam, m, ph, tab, fx_tab<N>(),
-                                                                             a.gV);
+      auto kv = a.stretched ? k_adj_volume<N, true> : k_adj_volume<N, false>;
+      cudaFuncSetAttribute(kv, cudaFuncAttributeMaxDynamicSharedMemorySize, AdjFxShape<N>::SMEM);
+      kv<<<a.K, VolShape<N>::THREADS, AdjFxShape<N>::SMEM, s>>>(a.Uin, a.lam, m, ph, tab, fx_tab<N>(), a.gV);
     }
     kel<<<a.K, AdjShape<N>::THREADS, smem, s>>>(a.Uin, a.lam, m, ph, tab, a.gGf, a.gV, a.gU, a.gWf, sendU);
   }

@@ -8,6 +8,7 @@ import pytest
 from paper_2606_18927_gb300 import dg, inputs as I
 from gpu_helpers import torch_cuda
 from test_gpu_adjoint_fx import cotangent, operator, vjp
+from test_gpu_stretched import inner, stretched_case
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +71,52 @@ def test_density_contrast(ora, N, contrast):
     e = np.abs(got[cols] - ref) / scale
     print(N, contrast, e.max(), np.sqrt((e * e).mean()))
     assert e.max() <= 4e-15
+
+
+def two_elements(ora, N, ratio, along):
+    """Two of the twelve elements of the stretched box, joined in x, between outflow boundaries."""
+    phys = I.phys_params(Ma=0.3, Re=1600.0, inviscid=True)
+    spec, X, U = stretched_case(N, ratio, phys, ora.lgl(N)[0], along)
+    X, U = (np.ascontiguousarray(a.reshape(-1, 12, (N + 1) ** 3)[:, :2]) for a in (X, U))
+    nbr = np.full((2, 6), -3, dtype=np.int32)
+    nbr[0, 1], nbr[1, 0] = 1, 0
+    return dict(phys, p_out=phys["p0"]), X, U, nbr
+
+
+@pytest.mark.parametrize("N", [2, 3, 5, 7])
+@pytest.mark.parametrize("ratio,along", [((1, 3, 1), True), ((1, 30, 1), True), ((1, 3, 1), False), ((1, 30, 1), False),
+                                         ((1, 300, 30), False), ((300, 1, 300), False)])
+def test_stretched_elements(ora, N, ratio, along):
+    """Elements with sides far apart, with velocities along the sides or alike; sampled columns
+    of the oracle, bound as above.  (Velocities 300 apart beside one pressure: FP64's recovery
+    of p from the energy exceeds that bound, so they are in the next test.)"""
+    torch = torch_cuda()
+    phys, X, U, nbr = two_elements(ora, N, ratio, along)
+    g = dg.Operator(N, X, nbr, phys, surf_flux=1, viscous=0)
+    o = ora.Oracle(N, X, nbr, phys, vol_flux=0, surf_flux=1, viscous=0, extended=True)
+    lam = I.random_direction(U.shape, 44)
+    got = vjp(torch, g, U, lam).ravel()
+    cols = np.concatenate([v * U[0].size + np.arange(3 + v, U[0].size, max(1, U[0].size // 10)) for v in range(5)])
+    ref, scale = columns(ora, o, U, lam, cols)
+    e = np.abs(got[cols] - ref) / scale
+    print(N, ratio, along, e.max(), np.sqrt((e * e).mean()))
+    assert e.max() <= 4e-15
+
+
+@pytest.mark.parametrize("N", [2, 3, 5, 7])
+def test_mass_cotangent_keeps_its_bits(ora, N):
+    """Stretched by powers of two with the velocities along, the gradients of the mass row at the
+    nodes inside the elements (volume terms alone) scale by powers of two: the same bits at every
+    ratio, as in FP64."""
+    torch = torch_cuda()
+    rows = []
+    for ratio in ((1, 8, 1), (1, 256, 8), (64, 1, 1024), (16, 16, 1)):
+        phys, X, U, nbr = two_elements(ora, N, ratio, True)
+        g = dg.Operator(N, X, nbr, phys, surf_flux=1, viscous=0)
+        lam = np.zeros(U.shape)
+        lam[0] = I.random_direction(U[0].shape, 45)
+        r = vjp(torch, g, U, lam)[:4, :, inner(N)]
+        rows.append(r / np.array((1.0,) + ratio)[:, None, None])
+    for r in rows[1:]:
+        print(N, np.abs(r - rows[0]).max() / np.abs(rows[0]).max())
+        assert np.array_equal(r, rows[0])
