@@ -114,7 +114,7 @@ __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& 
   f.eg[3] = E + eX[AX_LE] + eW + eX[AX_RHO] - 57;
   const bool even = (ex[AX_RHO] >> 20) - ((0x7fffffff - ex[AX_NRHO]) >> 20) <= 2 &&
                     (ex[AX_H] >> 20) - ((0x7fffffff - ex[AX_NH]) >> 20) <= 2;
-  f.ok = ok && even && abs(eA) < 200 && mt.kind != FX_GRADED;
+  f.ok = ok && even && abs(eA) < 200 && mt.kind < FX_GRADED;
   return f;
 }
 

@@ -2209,10 +2209,15 @@ __device__ __forceinline__ int vslot(int node) {
 }
 
 // the values of one node that the two-point flux of a direction reads
-template <class R>
+// (M: of the metrics)
+template <class R, class M>
 struct VolNode {
-  R rho, u, v, w, p4, hh, p2, ib, irh, a0, a1, a2;
+  R rho, u, v, w, p4, hh, p2, ib, irh;
+  M a0, a1, a2;
 };
+// the sum of two nodes' metrics (fixed-point ones: volume_fx.cuh)
+__device__ __forceinline__ float metric_sum(float a, float b, int) { return a + b; }
+__device__ __forceinline__ double metric_sum(double a, double b, int) { return a + b; }
 
 template <int N>
 struct VolShape {
@@ -2229,25 +2234,28 @@ struct VolShape {
 };
 
 // shared-memory arrays of the volume kernel
-template <typename R>
+template <typename R, typename M = R>
 struct VolSmem {
   R* sQ;    // [QS][n3] node values: rho u v w 4p' h|e 2p (KG) (+ FP32: ul vl wl); EC see k_volume
-  R* sA;    // [9][n3] Ja (dir*3+comp)
+  M* sA;    // [9][n3] Ja (dir*3+comp)
   R* sR;    // [5][n3] residual
   R* sC8;   // [n2] DVS / 8
   R* sC16;  // [n2] DVS / 16
   R* sC1;   // [n2] DVS
+  int eA[3] = {0, 0, 0};  // fixed-point metrics: the units' exponents by component
 };
 
 // The three direction passes over the lines of element e, from the staged node
 // values: leaves each node's sum (with R_v) in sm.sR.
-template <int N, typename R, bool EC>
-__device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDev<R>& m, const PhysDev& ph,
+template <int N, typename R, bool EC, typename M = R>
+__device__ __forceinline__ void volume_passes(const VolSmem<R, M>& sm, const MeshDev<R>& m, const PhysDev& ph,
                                               const R* __restrict__ Rv, int e, int t) {
   using Sh = VolShape<N>;
   constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW;
   constexpr bool F32 = std::is_same<R, float>::value;
-  R *sQ = sm.sQ, *sA = sm.sA, *sR = sm.sR, *sC8 = sm.sC8, *sC16 = sm.sC16, *sC1 = sm.sC1;
+  R *sQ = sm.sQ, *sR = sm.sR, *sC8 = sm.sC8, *sC16 = sm.sC16, *sC1 = sm.sC1;
+  M* sA = sm.sA;
+  using Node = VolNode<R, M>;
   const size_t S = (size_t)m.K * n3;
   const bool kg = ph.vol_flux == 1;
   const bool dif = F32 && !EC && ph.fs_diff;
@@ -2265,7 +2273,7 @@ __device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDe
   };
   auto load_node = [&](int nd, int dir) {
     const int node = vslot<N, R>(nd);
-    VolNode<R> X;
+    Node X;
     X.rho = sQ[node]; X.u = sQ[n3 + node]; X.v = sQ[2 * n3 + node]; X.w = sQ[3 * n3 + node];
     X.p4 = sQ[4 * n3 + node]; X.hh = sQ[5 * n3 + node];
     X.p2 = (kg || EC) ? sQ[6 * n3 + node] : R(0);
@@ -2277,8 +2285,9 @@ __device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDe
   };
   // symmetric two-point flux F#(A, B) . 4 {Ja} in the scaled form of the
   // coefficient tables (mass row against DVS / 8, the others against DVS / 16)
-  auto sym_flux = [&](const VolNode<R>& A, const VolNode<R>& B, R F[5]) {
-    const R Sa0 = A.a0 + B.a0, Sa1 = A.a1 + B.a1, Sa2 = A.a2 + B.a2;
+  auto sym_flux = [&](const Node& A, const Node& B, R F[5]) {
+    const R Sa0 = metric_sum(A.a0, B.a0, sm.eA[0]), Sa1 = metric_sum(A.a1, B.a1, sm.eA[1]),
+            Sa2 = metric_sum(A.a2, B.a2, sm.eA[2]);
     const R Sr = A.rho + B.rho, Su = A.u + B.u, Sv = A.v + B.v, Sw = A.w + B.w;
     const R Sp = A.p4 + B.p4;
     const R ua = Su * Sa0 + Sv * Sa1 + Sw * Sa2;  // 4 {u}.{a}
@@ -2334,13 +2343,13 @@ __device__ __forceinline__ void volume_passes(const VolSmem<R>& sm, const MeshDe
   constexpr bool HALF = std::is_same<R, double>::value && n == 8 && Sh::WARPS_LINES % 2 == 0;
   constexpr int DMAX = HALF ? n / 2 - 1 : n / 2;
   constexpr int HW = Sh::WARPS_LINES / 2, NX = HW * LPW * (n / 2);
-  R* sX = sA;  // [5][NX] zeta pair fluxes handed to the second half of the warps
+  R* sX = reinterpret_cast<R*>(sA);  // [5][NX] zeta pair fluxes handed to the second half of the warps
   R carry[5] = {R(0), R(0), R(0), R(0), R(0)};
 #pragma unroll 1
   for (int dir = 0; dir < 3; ++dir) {
     const int me = node_at(dir, pos);
     const int ms = vslot<N, R>(me);
-    const VolNode<R> A = load_node(me, dir);
+    const Node A = load_node(me, dir);
     // FP32 difference form: the low parts of this lane's node velocity
     float Aul = 0.f, Avl = 0.f, Awl = 0.f;
     if constexpr (F32 && !EC) {

@@ -203,7 +203,8 @@ struct FxRows {
 // column and every velocity component has its own, and the products are shifted
 // to the largest one's.  FX_GRADED: some column is below an eighth of its largest at
 // some node (thin at one end); its lines there would lose as much: summed in FP64.
-enum { FX_EVEN, FX_STRETCHED, FX_GRADED };
+// FX_THIN: below a 64th.
+enum { FX_EVEN, FX_STRETCHED, FX_GRADED, FX_THIN };
 struct FxMetric {
   int col[3], kind;
 };
@@ -333,7 +334,7 @@ __device__ __forceinline__ FxPlan fx_plan(const int* ex, const FxMetric& mt, int
       }
     }
   }
-  f.ok = finite && range && even && mt.kind != FX_GRADED && (eU - eUt <= 5 || xU >> 20 == 0);
+  f.ok = finite && range && even && mt.kind < FX_GRADED && (eU - eUt <= 5 || xU >> 20 == 0);
   return f;
 }
 
@@ -342,9 +343,9 @@ __device__ __forceinline__ FxPlan fx_plan(const int* ex, const FxMetric& mt, int
 // has room).  One block per element, once per mesh; *kinds collects the kinds.
 static __global__ void k_metric_fx(int n3, long long S, const double* __restrict__ Ja, Fx* __restrict__ JaX,
                                    FxMetric* __restrict__ mt, int* __restrict__ kinds) {
-  __shared__ int mx[3], graded;
+  __shared__ int mx[3], graded, thin;
   if (threadIdx.x < 3) mx[threadIdx.x] = 100 << 20;
-  if (threadIdx.x == 3) graded = 0;
+  if (threadIdx.x == 3) graded = thin = 0;
   __syncthreads();
   const size_t e0 = (size_t)blockIdx.x * n3;
   auto column = [&](int t, int c) {
@@ -362,14 +363,16 @@ static __global__ void k_metric_fx(int n3, long long S, const double* __restrict
   const bool even = most - least <= 1 << 20;
   for (int t = threadIdx.x; t < n3; t += blockDim.x) {
     for (int c = 0; c < 3; ++c) {
-      if (mx[c] - column(t, c) > 3 << 20) graded = 1;
+      const int below = mx[c] - column(t, c);
+      if (below > 3 << 20) graded = 1;
+      if (below > 6 << 20) thin = 1;
       const int eb = ((even ? most : mx[c]) >> 20) + 1;
       for (int d = 0; d < 3; ++d) JaX[(d * 3 + c) * S + e0 + t] = fx_of(Ja[(d * 3 + c) * S + e0 + t], eb);
     }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int kind = graded ? FX_GRADED : (even ? FX_EVEN : FX_STRETCHED);
+    const int kind = thin ? FX_THIN : (graded ? FX_GRADED : (even ? FX_EVEN : FX_STRETCHED));
     mt[blockIdx.x] = FxMetric{{even ? most : mx[0], even ? most : mx[1], even ? most : mx[2]}, kind};
     if (kind != FX_EVEN) atomicOr(kinds, 1 << kind);
   }
@@ -509,8 +512,18 @@ __device__ __forceinline__ void volume_passes_fx(const Fx* sQ, const Fx* sA, lon
   }
 }
 
-// an element summed in FP64 (fx_plan); rare, so kept out of line
-template <int N, int VF>
+// the double nearest to the sum of two fixed-point metrics in units of 2^e
+__device__ __forceinline__ double metric_sum(Fx a, Fx b, int e) {
+  return fx_double(((long long)(a.h + b.h) << 31) + (a.l + b.l), e);
+}
+
+// An element summed in FP64 (fx_plan); rare, so kept out of line.  The FP64 pipe
+// bounds it (30 operations a pair; KEP flux, N = 7, 12^3 elements all of them: 601 us
+// with the metrics' sums added on it), so these three are formed from the staged
+// fixed-point metrics on the integer pipes (545; 539 when such meshes kept the
+// pairs' sums in memory, 252 bytes a node).  Ja read again in FP64 (FXM false) where a
+// column falls so far below its largest that its limbs hold less than FP64's 53 bits.
+template <int N, int VF, bool FXM>
 __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<double>& m, const PhysDev& ph,
                                                 const Tables<N>& tab, const double* __restrict__ Rv, int e, int t) {
   constexpr int n3 = VolShape<N>::n3, n2 = VolShape<N>::n2, T = VolShape<N>::THREADS;
@@ -520,13 +533,22 @@ __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<doub
     sC16[x] = 0.5 * tab.DVS8[x];
     sC1[x] = 8.0 * tab.DVS8[x];
   }
-  if (t < n3) {
-    const int ts = vslot<N, double>(t);
+  if constexpr (!FXM) {
+    if (t < n3) {
+      const int ts = vslot<N, double>(t);
 #pragma unroll
-    for (int c = 0; c < 9; ++c) sA[c * n3 + ts] = m.Ja[(size_t)c * ((size_t)m.K * n3) + (size_t)e * n3 + t];
+      for (int c = 0; c < 9; ++c) sA[c * n3 + ts] = m.Ja[(size_t)c * ((size_t)m.K * n3) + (size_t)e * n3 + t];
+    }
+    __syncthreads();
+    volume_passes<N, double, VF == FX_EC>(VolSmem<double>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
+  } else {
+    const FxMetric& mt = m.JaX_max[e];
+    VolSmem<double, Fx> sm{sQ, reinterpret_cast<Fx*>(sA), sR, sC8, sC16, sC1};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sm.eA[c] = (mt.col[c] >> 20) - 1022 - 59;
+    __syncthreads();
+    volume_passes<N, double, VF == FX_EC, Fx>(sm, m, ph, Rv, e, t);
   }
-  __syncthreads();
-  volume_passes<N, double, VF == FX_EC>(VolSmem<double>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
 }
 
 // k_volume of the FP64 form: one CTA per element, the passes in fixed point
@@ -632,7 +654,21 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
         if constexpr (VF == FX_KG) sQ[6 * n3 + ts] = fx_of(be, f.bZ);
       }
     } else {
-      stage_node<N, double, EC>(reinterpret_cast<double*>(smem_raw), ts, q, ph, false);
+      // as stage_node, from this kernel's own e and reciprocals
+      double* d = reinterpret_cast<double*>(smem_raw) + ts;
+      d[0] = q.rho; d[n3] = q.u; d[2 * n3] = q.v; d[3 * n3] = q.w;
+      d[4 * n3] = 4.0 * q.p;
+      if constexpr (EC) {
+        const double beta = be * ph.rgm1;
+        d[4 * n3] = 8.0 * beta * q.p;
+        d[5 * n3] = beta;
+        d[6 * n3] = q.u * q.u + q.v * q.v + q.w * q.w;
+        d[7 * n3] = en * ph.gm1;  // 1 / (2 beta)
+        d[8 * n3] = irh;
+      } else {
+        d[5 * n3] = VF == FX_KG ? en : q.h;
+        if constexpr (VF == FX_KG) d[6 * n3] = be;
+      }
     }
   }
   if (fx) {
@@ -640,7 +676,9 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
     if (GEN && m.JaX_max[e].kind == FX_STRETCHED) volume_passes_fx<N, VF, GEN>(sQ, sA, sR, sT, sW, sH, f, sRows, t);
     else volume_passes_fx<N, VF, false>(sQ, sA, sR, sT, sW, sH, f, sRows, t);
   } else {
-    volume_passes_fp64<N, VF>(reinterpret_cast<double*>(smem_raw), m, ph, tab, Rv, e, t);
+    double* smem = reinterpret_cast<double*>(smem_raw);
+    if (GEN && m.JaX_max[e].kind == FX_THIN) volume_passes_fp64<N, VF, !GEN>(smem, m, ph, tab, Rv, e, t);
+    else volume_passes_fp64<N, VF, true>(smem, m, ph, tab, Rv, e, t);
   }
   volume_epilogue<N, double, MODE>(
       Uin, m, ph, tab, Fs, Out, dU, Uout, st, status, e, t, [&](int nd, size_t gn, double acc[5]) {

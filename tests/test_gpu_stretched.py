@@ -97,16 +97,16 @@ def test_rows_against_the_extended_oracle(ora, vol, N, ratio, along):
         assert e <= bound
 
 
-@pytest.mark.parametrize("N", [4, 7])
-def test_elements_thin_at_one_end(ora, N):
-    """y graded 16 : 1 along the elements, a flow across it: the lines at the thin end
-    have their own, small, fluxes.  The bound above, line by line."""
+@pytest.mark.parametrize("N,grade", [(4, 0.88), (7, 0.88), (7, 0.98)])
+def test_elements_thin_at_one_end(ora, N, grade):
+    """y graded 16 : 1 (99 : 1) along the elements, a flow across it: the lines at the thin
+    end have their own, small, fluxes.  The bound above, line by line."""
     torch = torch_cuda()
     phys = I.phys_params(Ma=0.3, Re=1600.0, inviscid=True)
     x, w, D = ora.lgl(N)
     n = N + 1
     spec, X, U = stretched_case(N, (1, 1, 1), phys, x)
-    X[1] += 0.88 * np.sin(X[1])
+    X[1] += grade * np.sin(X[1])
     X = np.ascontiguousarray(X)
     U[2] *= 1e-3
     nbr = I.connectivity(spec)
@@ -122,5 +122,5 @@ def test_elements_thin_at_one_end(ora, N):
     bound = np.sqrt(8.0 * D2 * total) * 2.0 ** -54 / J
     sel = np.tile(inner(N), (spec.K, 1))
     e = np.sqrt((((a[0] - ref[0]) / bound)[sel] ** 2).mean())
-    print(N, e)
+    print(N, grade, e)
     assert e <= 1.0
