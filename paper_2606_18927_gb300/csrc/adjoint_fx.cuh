@@ -13,7 +13,7 @@
 // added in FP64: the error against the extended-precision oracle's J^T lam
 // stays at FP64's.  Elements out of range (non-finite values; a value's or a
 // cotangent's largest magnitude beyond 2^200 or below 2^-200 without being zero;
-// density or enthalpy differing by more than a factor 8 over the nodes: the gradients
+// density or enthalpy differing by more than a factor 4 over the nodes: the gradients
 // at the light ones are divided by their own density) are summed in FP64.
 #pragma once
 #include "adjoint.cuh"
@@ -112,8 +112,8 @@ __device__ __forceinline__ AdjFxPlan adj_fx_plan(const int* ex, const FxMetric& 
   f.eg[1] = et + eX[AX_RHO] + eA + 2;
   f.eg[2] = (st ? Z : eX[AX_LM] + eA) + eW - 58;
   f.eg[3] = E + eX[AX_LE] + eW + eX[AX_RHO] - 57;
-  const bool even = (ex[AX_RHO] >> 20) - ((0x7fffffff - ex[AX_NRHO]) >> 20) <= 2 &&
-                    (ex[AX_H] >> 20) - ((0x7fffffff - ex[AX_NH]) >> 20) <= 2;
+  const bool even = (ex[AX_RHO] >> 20) - ((0x7fffffff - ex[AX_NRHO]) >> 20) <= 1 &&
+                    (ex[AX_H] >> 20) - ((0x7fffffff - ex[AX_NH]) >> 20) <= 1;
   f.ok = ok && even && abs(eA) < 200 && mt.kind < FX_GRADED;
   return f;
 }
