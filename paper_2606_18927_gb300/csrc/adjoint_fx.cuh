@@ -149,7 +149,7 @@ struct AdjFxShape {
 // memory as in volume_passes_fx).
 template <int N, bool ST>
 __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sLt, Fx* sA, double* sG, const Fx* sT,
-                                              const long long* sW, const Fx* __restrict__ JaX, size_t S, size_t e0,
+                                              const long long* sW, const MeshDev<double>& m, size_t S, size_t e0, int e,
                                               const AdjFxPlan& f, const volatile AdjFxRows& r, int t) {
   using Sh = VolShape<N>;
   constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, LPW = Sh::LPW;
@@ -175,7 +175,8 @@ __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sL
       }
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        a[c] = JaX[(size_t)(dir * 3 + c) * S + e0 + me];
+        const size_t x = (size_t)(dir * 3 + c) * S + e0 + me;
+        a[c] = STORED_FX<N> ? m.JaX[x] : metric_fx(m.Ja[x], m.JaX_max[e], c);
         if (active) sA[c * n3 + ms] = a[c];
       }
     }
@@ -375,8 +376,8 @@ k_adj_volume(const double* __restrict__ U, const double* __restrict__ lam, const
   }
   if (f.ok) {
     __syncthreads();
-    if (st) adj_passes_fx<N, GEN>(sQ, sL, sLt, sA, sG, sT, sW, m.JaX, S, e0, f, sRows, t);
-    else adj_passes_fx<N, false>(sQ, sL, sLt, sA, sG, sT, sW, m.JaX, S, e0, f, sRows, t);
+    if (st) adj_passes_fx<N, GEN>(sQ, sL, sLt, sA, sG, sT, sW, m, S, e0, e, f, sRows, t);
+    else adj_passes_fx<N, false>(sQ, sL, sLt, sA, sG, sT, sW, m, S, e0, e, f, sRows, t);
   } else {
     adj_volume_fp64<N>(reinterpret_cast<double*>(smem_raw), m, ph, tab, e, t);
   }

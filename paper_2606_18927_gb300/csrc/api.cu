@@ -58,8 +58,8 @@ struct dg_ctx {
   // (Ja Ja^T) / J [24][S] and of the lifted primitives [4][S]
   float2* lift_M2 = nullptr;
   float2* lift_W2 = nullptr;
-  dg::Fx* JaX = nullptr;    // FP64: [9][S] metrics in fixed point (volume kernel), and
-  dg::FxMetric* JaX_max = nullptr;  // the elements' largest magnitudes and kinds [K]
+  dg::Fx* JaX = nullptr;    // FP64, N = 7: [9][S] metrics in fixed point (volume kernel), and
+  dg::FxMetric* JaX_max = nullptr;  // FP64: the elements' largest magnitudes and kinds [K]
   int stretched = 0;        // some element is not FX_EVEN
   double* wm_t = nullptr;  // wall-law warm start per wall node (NaN: none yet)
   // partitioned meshes: halo buffers [n_halo][5][n2] (state traces, FP64) and
@@ -73,7 +73,7 @@ struct dg_ctx {
   double* U = nullptr;
   double* dU = nullptr;
   double* io = nullptr;   // staging of a host input
-  double* io2 = nullptr;  // staging of a host output
+  double* io2 = nullptr;  // staging of a host output; the adjoint's gV (calls on one stream follow each other)
   void* Ja = nullptr;
   void* invJ = nullptr;
   double* fgeo = nullptr;
@@ -101,7 +101,6 @@ struct dg_ctx {
   double* wJ = nullptr;        // w_i w_j w_k J per node (kinetic-energy integral)
   double vol = 0.0;
   // adjoint scratch (allocated on the first dg_vjp)
-  double* gV = nullptr;
   double* gUf = nullptr;
   double* gGf = nullptr;
   double* gWf = nullptr;
@@ -169,7 +168,7 @@ void free_all(dg_ctx* c) {
   c->cp_in = c->cp_out = nullptr;
   void* ptrs[] = {c->U, c->dU, c->io, c->io2, c->Ja, c->invJ, c->fgeo, c->nbr, c->elem_face, c->faces,
                   c->ws_elem, c->ws_lag, c->Rv, c->Gf, c->Fs, c->tau, c->status,
-                  c->gV, c->gUf, c->gGf, c->gWf, c->gUs, c->gtheta, c->wq, c->ro_ckpt, c->ro_stage, c->ro_work,
+                  c->gUf, c->gGf, c->gWf, c->gUs, c->gtheta, c->wq, c->ro_ckpt, c->ro_stage, c->ro_work,
                   c->ro_scalar, c->wJ, c->W32, c->W64, c->JaJ, c->Mj, c->lift_M2, c->lift_W2, c->JaX, c->JaX_max, c->halo_U, c->send_U,
                   c->halo_G, c->send_G,
                   c->wm_t};
@@ -688,7 +687,7 @@ int dg_init_mesh(dg_ctx** out, const dg_mesh_desc* m, const dg_phys* p, const dg
   if (e != cudaSuccess) { free_all(c); delete c; return cuda_fail(nullptr, e, "dg_init_mesh: upload"); }
   // FP64: the volume kernel's metrics in fixed point
   if (o->precision == DG_FP64) {
-    chk(alloc(&c->JaX, 9 * S));
+    if (c->N == 7 && dg::STORED_FX<7>) chk(alloc(&c->JaX, 9 * S));
     chk(alloc(&c->JaX_max, (size_t)c->K));
     if (e == cudaSuccess) {
       // (status is free until the first evaluation)
@@ -995,7 +994,6 @@ static int ensure_adjoint_scratch(dg_ctx* c) {
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   const size_t kn2 = (size_t)c->K * 6 * c->n2;
-  if (c->opts.vol_flux != DG_VOL_EC_CHANDRASHEKAR) chk(alloc(&c->gV, 5 * c->S));
   chk(alloc(&c->gUf, 5 * kn2));
   chk(alloc(&c->gGf, 4 * kn2));
   chk(alloc(&c->gWf, 4 * kn2));
@@ -1013,7 +1011,7 @@ static dg::OpArgs adjoint_args(dg_ctx* c, const double* U, const double* lam, do
   a.faces = c->faces; a.ws_elem = c->ws_elem; a.ws_lag = c->ws_lag;
   a.D = c->geo.basis.D.data(); a.w = c->geo.basis.w.data();
   a.Uin = U; a.status = c->status;
-  a.lam = lam; a.gU = gU; a.gV = c->gV; a.gUf = c->gUf; a.gGf = c->gGf; a.gWf = c->gWf; a.gUs = c->gUs; a.gtheta = gth;
+  a.lam = lam; a.gU = gU; a.gV = c->io2; a.gUf = c->gUf; a.gGf = c->gGf; a.gWf = c->gWf; a.gUs = c->gUs; a.gtheta = gth;
   a.JaJ = c->JaJ; a.Mj = c->Mj;
   a.JaX = c->JaX; a.JaX_max = c->JaX_max; a.stretched = c->stretched;
   a.n_halo = c->geo.n_halo;

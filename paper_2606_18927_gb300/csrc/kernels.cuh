@@ -91,6 +91,10 @@ struct Fx {
   int h, l;
 };
 struct FxMetric;  // volume_fx.cuh
+// whether the fixed-point metrics are kept in memory (72 bytes a node) or formed from
+// Ja in the kernels that read them
+template <int N>
+constexpr bool STORED_FX = N == 7;
 
 struct PhysDev {
   double gamma, gm1, R, mu, Pr, cp, kcond, rcp_R;
@@ -159,8 +163,8 @@ struct MeshDev {
   // written by k_prim64 (null unless that lifting is selected)
   const float2* lift_M2;
   float2* lift_W2;
-  const Fx* JaX;         // FP64 form: [9][K*n3] metrics in fixed point (volume_fx.cuh) and their largest
-  const FxMetric* JaX_max;  // magnitudes [K]
+  const Fx* JaX;         // FP64 form: metrics in fixed point [9][K*n3] (STORED_FX) and
+  const FxMetric* JaX_max;  // the elements' largest magnitudes [K] (volume_fx.cuh)
   double* wm_t;          // [n_wall*n2] last wall-law solution per wall node (warm start; may be null)
   int* status;           // device status flags (index checks of the bounds-checking build)
 };

@@ -59,8 +59,8 @@ struct OpArgs {
   // [24][K n^3] and of the lifted primitives [4][K n^3] (null: not selected)
   const float2* lift_M2;
   float2* lift_W2;
-  const Fx* JaX;        // FP64 form: [9][K n^3] metrics in fixed point and their largest
-  const FxMetric* JaX_max;  // magnitudes [K]
+  const Fx* JaX;        // FP64 form: metrics in fixed point [9][K n^3] (null: formed in the kernels) and
+  const FxMetric* JaX_max;  // the elements' largest magnitudes [K]
   int stretched;        // some element's metrics are not FX_EVEN
   double* wm_t;  // wall-law warm-start values per wall node (null: cold solves)
   // partitioned meshes: n_halo halo faces (the last faces), remote traces in

@@ -340,12 +340,16 @@ __device__ __forceinline__ FxPlan fx_plan(const int* ex, const FxMetric& mt, int
   return f;
 }
 
-// The metrics Ja of every element in its units: limbs [9][K n3] and FxMetric [K]
-// (one bit below fx_of's bound, so that a pair's sum of three products S_u . S_a
-// has room).  One block per element, once per mesh; *kinds collects the kinds.
+// A metric Ja^d_c in the element's unit, one bit below fx_of's bound, so that a
+// pair's sum of three products S_u . S_a has room
+__device__ __forceinline__ Fx metric_fx(double a, const FxMetric& mt, int c) { return fx_of(a, (mt.col[c] >> 20) + 1); }
+
+// The elements' FxMetric [K], and with JaX the metrics in their units, limbs
+// [9][K n3].  One block per element, once per mesh; *kinds collects the kinds.
 static __global__ void k_metric_fx(int n3, long long S, const double* __restrict__ Ja, Fx* __restrict__ JaX,
                                    FxMetric* __restrict__ mt, int* __restrict__ kinds) {
   __shared__ int mx[3], graded, thin;
+  __shared__ FxMetric my;
   if (threadIdx.x < 3) mx[threadIdx.x] = 100 << 20;
   if (threadIdx.x == 3) graded = thin = 0;
   __syncthreads();
@@ -363,21 +367,23 @@ static __global__ void k_metric_fx(int n3, long long S, const double* __restrict
   __syncthreads();
   const int most = max(mx[0], max(mx[1], mx[2])), least = min(mx[0], min(mx[1], mx[2]));
   const bool even = most - least <= 1 << 20;
-  for (int t = threadIdx.x; t < n3; t += blockDim.x) {
+  for (int t = threadIdx.x; t < n3; t += blockDim.x)
     for (int c = 0; c < 3; ++c) {
       const int below = mx[c] - column(t, c);
       if (below > 3 << 20) graded = 1;
       if (below > 6 << 20) thin = 1;
-      const int eb = ((even ? most : mx[c]) >> 20) + 1;
-      for (int d = 0; d < 3; ++d) JaX[(d * 3 + c) * S + e0 + t] = fx_of(Ja[(d * 3 + c) * S + e0 + t], eb);
     }
-  }
   __syncthreads();
   if (threadIdx.x == 0) {
     const int kind = thin ? FX_THIN : (graded ? FX_GRADED : (even ? FX_EVEN : FX_STRETCHED));
-    mt[blockIdx.x] = FxMetric{{even ? most : mx[0], even ? most : mx[1], even ? most : mx[2]}, kind};
+    my = FxMetric{{even ? most : mx[0], even ? most : mx[1], even ? most : mx[2]}, kind};
+    mt[blockIdx.x] = my;
     if (kind != FX_EVEN) atomicOr(kinds, 1 << kind);
   }
+  __syncthreads();
+  if (JaX)
+    for (int t = threadIdx.x; t < n3; t += blockDim.x)
+      for (int x = 0; x < 9; ++x) JaX[x * S + e0 + t] = metric_fx(Ja[x * S + e0 + t], my, x % 3);
 }
 
 template <int N, int VF>
@@ -586,7 +592,8 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
     q = m.W64 ? load_prim64(m.W64, S, g) : primitive<double>(Uin[g], Uin[S + g], Uin[2 * S + g], Uin[3 * S + g], Uin[4 * S + g], ph);
     const int ts = vslot<N, double>(t);
 #pragma unroll
-    for (int c = 0; c < 9; ++c) sA[c * n3 + ts] = m.JaX[(size_t)c * S + g];
+    for (int c = 0; c < 9; ++c)
+      sA[c * n3 + ts] = STORED_FX<N> ? m.JaX[(size_t)c * S + g] : metric_fx(m.Ja[(size_t)c * S + g], m.JaX_max[e], c % 3);
     if constexpr (EC) {
       const double ir = rcp_pos(q.rho);
       // (the quotient's remainder added back: half an ulp instead of two)
