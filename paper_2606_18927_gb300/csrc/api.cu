@@ -999,7 +999,14 @@ static int ensure_adjoint_scratch(dg_ctx* c) {
   chk(alloc(&c->gWf, 4 * kn2));
   chk(alloc(&c->gUs, (size_t)c->geo.n_wall * c->n2 * 5 + 1));
   chk(alloc(&c->gtheta, 2));
-  if (e != cudaSuccess) return cuda_fail(c, e, "adjoint scratch allocation");
+  if (e != cudaSuccess) {
+    // leave no half of it behind: a later call would take it for the whole
+    for (double** p : {&c->gUf, &c->gGf, &c->gWf, &c->gUs, &c->gtheta}) {
+      if (*p) cudaFree(*p);
+      *p = nullptr;
+    }
+    return cuda_fail(c, e, "adjoint scratch allocation");
+  }
   return DG_OK;
 }
 
