@@ -1053,12 +1053,13 @@ static __device__ float solve_utau_f(int law, float u, float h, float nu, float 
 // the bracketed solve from scratch.  The state changes little between stages
 // and the FP32 solution is good to 1e-6, so two evaluations of F usually
 // suffice instead of about eight (an evaluation is some 170 FP64 operations,
-// the solve a serial chain).  *t_out receives the converged t.
+// the solve a serial chain).  Caps near what a solve needs (below 32) count its
+// own evaluations alone: no FP32 start.  *t_out receives the converged t.
 static __device__ double solve_utau_warm(int law, double u, double h, double nu, double kap, double B, int maxit,
                                          double t_prev, double* t_out, bool* ok) {
   *ok = true;
   if (!(u > 0.0)) { *t_out = t_prev; return 0.0; }
-  if (!(t_prev == t_prev)) {
+  if (!(t_prev == t_prev) && maxit >= 32) {
     bool okf;
     const float utf = solve_utau_f(law, (float)u, (float)h, (float)nu, (float)kap, (float)B, maxit, &okf);
     if (okf) t_prev = law == 1 ? logf(utf * (float)h / (float)nu) : logf((float)u / utf);
