@@ -17,13 +17,12 @@
 //   k_halo_face FP32: faces shared with another rank of a partitioned mesh;
 //   k_wall      wall face nodes: mirror state and the wall-stress model (may
 //               run on a side stream beside k_lift and k_face);
-//   k_volume_fx (volume_fx.cuh; FP64 form, KEP fluxes) and
-//   k_volume    one CTA per element: two-point flux differencing (KEP or
+//   k_volume_fx (volume_fx.cuh; FP64 form: pair fluxes in fixed point) and
+//   k_volume    (FP32-mixed) one CTA per element: two-point flux differencing (KEP or
 //               entropy-conserving) with the split-form matrix DVS = 2D - B/w
 //               (zero corners), the surface integral, 1/J scaling, body force,
 //               and either Ut or the LSERK4 register update of U and dU (N = 7:
-//               swizzled shared-memory node slots, vslot; FP64: each pair at
-//               distance n/2 formed once).
+//               swizzled shared-memory node slots, vslot).
 // R is the arithmetic type of the fluxes and their sums (double, or float in
 // the mixed form); the state U, dU, the pressure recovery and the RK update
 // are always double.  The FP32 form also keeps per-stage FP32 primitives
@@ -2231,9 +2230,9 @@ struct VolShape {
   static constexpr int WARPS_LINES = (n2 + LPW - 1) / LPW;  // warps for one direction
   static constexpr int WARPS_NODES = (n3 + 31) / 32;
   static constexpr int THREADS = 32 * (WARPS_LINES > WARPS_NODES ? WARPS_LINES : WARPS_NODES);
-  // shared memory (in units of R): 7 prim slots (9 with the entropy-
-  // conserving flux, 10 in the FP32 form of the KEP fluxes: the low parts of
-  // the velocity), 9 metric, 5 residual per node, three coefficient tables
+  // k_volume's shared memory (floats): 10 prim slots (the velocity's low parts
+  // among them; 9 with the entropy-conserving flux), 9 metric, 5 residual per
+  // node, three coefficient tables
   static constexpr int SMEM_R_EC = 23 * n3 + 3 * n2;
   static constexpr int SMEM_R_F32 = 24 * n3 + 3 * n2;
 };
@@ -2567,27 +2566,27 @@ __device__ __forceinline__ void volume_epilogue(const double* __restrict__ Uin, 
 }
 
 // a node's values in the volume kernel's shared memory
-template <int N, typename R, bool EC>
-__device__ __forceinline__ void stage_node(R* sQ, int ts, const Prim<R>& q, const PhysDev& ph, bool dif) {
+template <int N, bool EC>
+__device__ __forceinline__ void stage_node(float* sQ, int ts, const Prim<float>& q, const PhysDev& ph, bool dif) {
   constexpr int n3 = VolShape<N>::n3;
   const bool kg = ph.vol_flux == 1;
   sQ[ts] = q.rho; sQ[n3 + ts] = q.u; sQ[2 * n3 + ts] = q.v; sQ[3 * n3 + ts] = q.w;
-  sQ[4 * n3 + ts] = dif ? q.p : R(4) * q.p;
+  sQ[4 * n3 + ts] = dif ? q.p : 4.0f * q.p;
   if constexpr (EC) {
-    const R pf = q.p + cR<R>(ph.p_ref, ph.f32c.p_ref);
-    const R beta = R(0.5) * q.rho * rcp_t<R>(pf);
-    const R irho = rcp_t<R>(q.rho);
-    sQ[4 * n3 + ts] = R(8) * beta * q.p;
+    const float pf = q.p + ph.f32c.p_ref;
+    const float beta = 0.5f * q.rho * rcp_t<float>(pf);
+    const float irho = rcp_t<float>(q.rho);
+    sQ[4 * n3 + ts] = 8.0f * beta * q.p;
     sQ[5 * n3 + ts] = beta;
     sQ[6 * n3 + ts] = q.u * q.u + q.v * q.v + q.w * q.w;
     sQ[7 * n3 + ts] = pf * irho;      // 1 / (2 beta)
-    sQ[8 * n3 + ts] = R(0.5) * irho;  // 1 / (2 rho)
+    sQ[8 * n3 + ts] = 0.5f * irho;    // 1 / (2 rho)
   } else if (!kg) {
     sQ[5 * n3 + ts] = q.h;
   } else {
-    const R pf = q.p + cR<R>(ph.p_ref, ph.f32c.p_ref);
+    const float pf = q.p + ph.f32c.p_ref;
     sQ[5 * n3 + ts] = q.h - pf / q.rho;  // e = E / rho
-    sQ[6 * n3 + ts] = R(2) * pf;
+    sQ[6 * n3 + ts] = 2.0f * pf;
   }
 }
 
@@ -2597,66 +2596,57 @@ constexpr int vol_min_blocks() {
   return DENSE ? resident_ctas(T, (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4, 1536) : (T > 512 ? 1 : 2);
 }
 
-template <int N, typename R, int MODE, bool EC, bool DENSE>
+// k_volume: the FP32-mixed form (the FP64 form: k_volume_fx, volume_fx.cuh)
+template <int N, int MODE, bool EC, bool DENSE>
 __global__ void __launch_bounds__(VolShape<N>::THREADS, (vol_min_blocks<N, EC, DENSE>()))
-k_volume(const double* __restrict__ Uin, const MeshDev<R> m, const PhysDev ph, const Tables<N> tab,
-         const R* __restrict__ Rv, const R* __restrict__ Fs, double* __restrict__ Out,
+k_volume(const double* __restrict__ Uin, const MeshDev<float> m, const PhysDev ph, const Tables<N> tab,
+         const float* __restrict__ Rv, const float* __restrict__ Fs, double* __restrict__ Out,
          double* __restrict__ dU, double* __restrict__ Uout, const StageArgs st, int* __restrict__ status) {
   using Sh = VolShape<N>;
-  constexpr int n = Sh::n, n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS;
+  constexpr int n2 = Sh::n2, n3 = Sh::n3, T = Sh::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr bool F32 = std::is_same<R, float>::value;
-  constexpr int QS = EC ? 9 : (F32 ? 10 : 7);
-  R* sQ = reinterpret_cast<R*>(smem_raw);  // [QS][n3]: rho u v w 4p' h|e 2p (KG) (+ FP32: ul vl wl); EC see above
-  R* sA = sQ + QS * n3;                     // [9][n3]: Ja (dir*3+comp)
-  R* sR = sA + 9 * n3;                      // [5][n3]: residual
-  R* sC8 = sR + 5 * n3;                     // [n2]: DVS / 8
-  R* sC16 = sC8 + n2;                       // [n2]: DVS / 16
-  R* sC1 = sC16 + n2;                       // [n2]: DVS
+  constexpr int QS = EC ? 9 : 10;
+  float* sQ = reinterpret_cast<float*>(smem_raw);  // [QS][n3]: rho u v w 4p' h|e 2p (KG) ul vl wl; EC see stage_node
+  float* sA = sQ + QS * n3;                         // [9][n3]: Ja (dir*3+comp)
+  float* sR = sA + 9 * n3;                          // [5][n3]: residual
+  float* sC8 = sR + 5 * n3;                         // [n2]: DVS / 8
+  float* sC16 = sC8 + n2;                           // [n2]: DVS / 16
+  float* sC1 = sC16 + n2;                           // [n2]: DVS
   const int e = blockIdx.x, t = threadIdx.x;
   const size_t S = (size_t)m.K * n3;
-  const bool kg = ph.vol_flux == 1;
-  // FP32 Pirozzoli form: flux differences G(i -> m) and per-side surface
+  // Pirozzoli form: flux differences G(i -> m) and per-side surface
   // differences F* - F(U_i) (see flux_delta)
-  const bool dif = std::is_same<R, float>::value && !EC && ph.fs_diff;
+  const bool dif = !EC && ph.fs_diff;
   for (int x = t; x < n2; x += T) {
-    sC8[x] = (R)tab.DVS8[x];
-    sC16[x] = (R)(0.5 * tab.DVS8[x]);
-    sC1[x] = (R)(8.0 * tab.DVS8[x]);
+    sC8[x] = (float)tab.DVS8[x];
+    sC16[x] = (float)(0.5 * tab.DVS8[x]);
+    sC1[x] = (float)(8.0 * tab.DVS8[x]);
   }
-  // prologue: node t (the FP32-mixed form reads the stage's FP32 primitives
-  // and loads the FP64 state only in the epilogue)
+  // prologue: node t (the stage's FP32 primitives; the FP64 state is loaded
+  // only in the epilogue)
   if (t < n3) {
     const size_t g = (size_t)e * n3 + t;
-    Prim<R> q;
-    if constexpr (F32) {
-      // the difference form works on the storage form (shifted rho, h) and
-      // the velocity's low parts
-      q = dif ? load_prim32(m.W32, S, g) : load_prim32_full(m.W32, S, g, ph);
-      if constexpr (!EC) {
-        if (dif) {
-          const int ts = vslot<N, R>(t);
-          const Lo3 l = load_lo32(m.W32, S, g);
-          sQ[7 * n3 + ts] = l.u; sQ[8 * n3 + ts] = l.v; sQ[9 * n3 + ts] = l.w;
-        }
+    const int ts = vslot<N, float>(t);
+    // the difference form works on the storage form (shifted rho, h) and
+    // the velocity's low parts
+    const Prim<float> q = dif ? load_prim32(m.W32, S, g) : load_prim32_full(m.W32, S, g, ph);
+    if constexpr (!EC) {
+      if (dif) {
+        const Lo3 l = load_lo32(m.W32, S, g);
+        sQ[7 * n3 + ts] = l.u; sQ[8 * n3 + ts] = l.v; sQ[9 * n3 + ts] = l.w;
       }
-    } else if (m.W64) {
-      q = load_prim64(m.W64, S, g);
-    } else {
-      q = primitive<R>(Uin[g], Uin[S + g], Uin[2 * S + g], Uin[3 * S + g], Uin[4 * S + g], ph);
     }
-    const int ts = vslot<N, R>(t);
-    stage_node<N, R, EC>(sQ, ts, q, ph, dif);
+    stage_node<N, EC>(sQ, ts, q, ph, dif);
 #pragma unroll
     for (int c = 0; c < 9; ++c) sA[c * n3 + ts] = m.Ja[(size_t)c * S + g];
   }
   __syncthreads();
-  volume_passes<N, R, EC>(VolSmem<R>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
-  volume_epilogue<N, R, MODE>(Uin, m, ph, tab, Fs, Out, dU, Uout, st, status, e, t,
-                              [&](int nd, size_t, R acc[5]) {
+  volume_passes<N, float, EC>(VolSmem<float>{sQ, sA, sR, sC8, sC16, sC1}, m, ph, Rv, e, t);
+  volume_epilogue<N, float, MODE>(Uin, m, ph, tab, Fs, Out, dU, Uout, st, status, e, t,
+                                  [&](int nd, size_t, float acc[5]) {
 #pragma unroll
-                                for (int v = 0; v < 5; ++v) acc[v] = sR[v * n3 + vslot<N, R>(nd)];
-                              });
+                                    for (int v = 0; v < 5; ++v) acc[v] = sR[v * n3 + vslot<N, float>(nd)];
+                                  });
 }
 
 }  // namespace dg
