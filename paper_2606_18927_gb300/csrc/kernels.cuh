@@ -77,11 +77,12 @@ constexpr int resident_ctas(int threads, int smem, int resident) {
 // are more than those CTAs, by 1.1 to 1.6; below it the spills (36 to 144 bytes)
 // only lengthen the kernels: FP32-mixed steps of 64 to 729 elements were up to
 // 13 % slower (N = 5, entropy-conserving, 6^3 elements: k_volume 14.8 against 16.8
-// us).  The entropy-conserving kernel spills most and needs five elements per SM
-// at least (dense against the other: N = 4 1.02 at 8.8 elements per SM, N = 5 0.96
-// at 4.8 and 1.02 at 18, N = 6 0.88 at 3.4 and 1.0 at 11).
+// us).  The entropy-conserving kernel spills most.  Its dense form against the other,
+// swept over 0.5 to 24 elements per SM: N = 7 0.97 at 2.5 and 0.88 at 16; N = 3 1.04 to
+// 1.10 up to 11, 0.97 and 1.01 at 16 and 24; N = 4 0.95 and 0.88 there; N = 5 1.06 to 1.24
+// up to 11, 1.02 and 0.95; N = 6 1.02 to 1.10, 1.01 and 0.97; N = 2, 8 no difference.
 constexpr bool dense_mesh(long long K, int threads, bool ec) {
-  const int ctas = 819 / threads, least = ec ? 5 : 1;
+  const int ctas = 819 / threads, least = ec ? (threads < 512 ? 20 : 2) : 1;
   return K > 152LL * (ctas > least ? ctas : least);
 }
 
