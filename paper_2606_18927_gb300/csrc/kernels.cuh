@@ -77,10 +77,14 @@ constexpr int resident_ctas(int threads, int smem, int resident) {
 // are more than those CTAs, by 1.1 to 1.6; below it the spills (36 to 144 bytes)
 // only lengthen the kernels: FP32-mixed steps of 64 to 729 elements were up to
 // 13 % slower (N = 5, entropy-conserving, 6^3 elements: k_volume 14.8 against 16.8
-// us).  The entropy-conserving kernel spills most.  Its dense form against the other,
-// swept over 0.5 to 24 elements per SM: N = 7 0.97 at 2.5 and 0.88 at 16; N = 3 1.04 to
-// 1.10 up to 11, 0.97 and 1.01 at 16 and 24; N = 4 0.95 and 0.88 there; N = 5 1.06 to 1.24
-// up to 11, 1.02 and 0.95; N = 6 1.02 to 1.10, 1.01 and 0.97; N = 2, 8 no difference.
+// us).  The entropy-conserving kernel spills most and takes the dense budget only at
+// N = 7 from 2 elements per SM (0.97 of the other's time at 2.5, 0.88 at 16) and at N = 6
+// from 20 (0.97; 1.02 to 1.10 up to 11).  At N = 4 and 5 it has one of its own: 64
+// registers (1024 threads, no spills and 20 bytes) instead of 74 and 80, so that five and
+// four CTAs fit instead of four and three (0.89 and 0.85 from 11 elements per SM; the
+// dense form 1.00 and 0.95 at 24).
+template <int N>
+constexpr bool EC_DENSE = N >= 6;
 constexpr bool dense_mesh(long long K, int threads, bool ec) {
   const int ctas = 819 / threads, least = ec ? (threads < 512 ? 20 : 2) : 1;
   return K > 152LL * (ctas > least ? ctas : least);
@@ -2594,7 +2598,9 @@ __device__ __forceinline__ void stage_node(float* sQ, int ts, const Prim<float>&
 template <int N, bool EC, bool DENSE>
 constexpr int vol_min_blocks() {
   constexpr int T = VolShape<N>::THREADS;
-  return DENSE ? resident_ctas(T, (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4, 1536) : (T > 512 ? 1 : 2);
+  constexpr int smem = (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4;
+  if (DENSE) return resident_ctas(T, smem, 1536);
+  return EC && (N == 4 || N == 5) ? resident_ctas(T, smem, 1024) : (T > 512 ? 1 : 2);
 }
 
 // k_volume: the FP32-mixed form (the FP64 form: k_volume_fx, volume_fx.cuh)

@@ -276,7 +276,8 @@ static int run_typed(const OpArgs& a, const PhysDev& ph, cudaStream_t s) {
     };
     auto form = [&](auto dense) {
       constexpr bool D = decltype(dense)::value;
-      if (ec) volume(a.mode == 0 ? k_volume<N, 0, true, D> : k_volume<N, 1, true, D>);
+      constexpr bool DE = D && EC_DENSE<N>;
+      if (ec) volume(a.mode == 0 ? k_volume<N, 0, true, DE> : k_volume<N, 1, true, DE>);
       else volume(a.mode == 0 ? k_volume<N, 0, false, D> : k_volume<N, 1, false, D>);
     };
     if (dense_mesh(a.K, VolShape<N>::THREADS, ec)) form(std::true_type{});
