@@ -82,11 +82,13 @@ constexpr int resident_ctas(int threads, int smem, int resident) {
 // from 20 (0.97; 1.02 to 1.10 up to 11).  At N = 4 and 5 it has one of its own: 64
 // registers (1024 threads, no spills and 20 bytes) instead of 74 and 80, so that five and
 // four CTAs fit instead of four and three (0.89 and 0.85 from 11 elements per SM; the
-// dense form 1.00 and 0.95 at 24).
+// dense form 1.00 and 0.95 at 24).  At N = 3 that budget (59 registers instead of 78)
+// is the dense form, from 14 elements per SM (1.04 at 11, 0.84 at 16, 1.01 at 24, 0.91
+// at 32 and 48).
 template <int N>
-constexpr bool EC_DENSE = N >= 6;
+constexpr bool EC_DENSE = N == 3 || N >= 6;
 constexpr bool dense_mesh(long long K, int threads, bool ec) {
-  const int ctas = 819 / threads, least = ec ? (threads < 512 ? 20 : 2) : 1;
+  const int ctas = 819 / threads, least = ec ? (threads <= 64 ? 14 : threads < 512 ? 20 : 2) : 1;
   return K > 152LL * (ctas > least ? ctas : least);
 }
 
@@ -2599,7 +2601,7 @@ template <int N, bool EC, bool DENSE>
 constexpr int vol_min_blocks() {
   constexpr int T = VolShape<N>::THREADS;
   constexpr int smem = (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4;
-  if (DENSE) return resident_ctas(T, smem, 1536);
+  if (DENSE) return resident_ctas(T, smem, EC && N == 3 ? 1024 : 1536);
   return EC && (N == 4 || N == 5) ? resident_ctas(T, smem, 1024) : (T > 512 ? 1 : 2);
 }
 
