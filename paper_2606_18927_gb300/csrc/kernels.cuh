@@ -77,18 +77,21 @@ constexpr int resident_ctas(int threads, int smem, int resident) {
 // are more than those CTAs, by 1.1 to 1.6; below it the spills (36 to 144 bytes)
 // only lengthen the kernels: FP32-mixed steps of 64 to 729 elements were up to
 // 13 % slower (N = 5, entropy-conserving, 6^3 elements: k_volume 14.8 against 16.8
-// us).  The entropy-conserving kernel spills most and takes the dense budget only at
-// N = 7 from 2 elements per SM (0.97 of the other's time at 2.5, 0.88 at 16) and at N = 6
-// from 20 (0.97; 1.02 to 1.10 up to 11).  At N = 4 and 5 it has one of its own: 64
-// registers (1024 threads, no spills and 20 bytes) instead of 74 and 80, so that five and
-// four CTAs fit instead of four and three (0.89 and 0.85 from 11 elements per SM; the
-// dense form 1.00 and 0.95 at 24).  At N = 3 that budget (59 registers instead of 78)
-// is the dense form, from 14 elements per SM (1.04 at 11, 0.84 at 16, 1.01 at 24, 0.91
-// at 32 and 48).
+// us).  The entropy-conserving kernel spills most; what pays for it, and from how
+// many elements per SM (time against the other form, or N = 4's against 74 registers):
+//   N = 3  64 registers (no spills) from 14: 0.84 at 15 and 16, 0.92 at 28, 0.87 at 61,
+//          1.0 between; 1.04 at 11
+//   N = 4  64 registers (no spills) always: five CTAs fit instead of four; 1.0 up to 5,
+//          0.75 to 0.95 beyond (with 40: 1.0 at 24)
+//   N = 5  64 registers (20 bytes) from 3, the other form's three CTAs: 0.96 at 4, 0.85
+//          at 24 (with 40: 1.06 to 1.14 up to 11, 0.95 at 24)
+//   N = 6  40 from 20: 0.97; 1.02 to 1.10 up to 11
+//   N = 7  40 from 5: the operator alone 0.98, a stage 0.94; at 3 1.03 and 0.97
+//   N = 2, 8  no difference
 template <int N>
-constexpr bool EC_DENSE = N == 3 || N >= 6;
+constexpr bool EC_DENSE = N != 4;
 constexpr bool dense_mesh(long long K, int threads, bool ec) {
-  const int ctas = 819 / threads, least = ec ? (threads <= 64 ? 14 : threads < 512 ? 20 : 2) : 1;
+  const int ctas = 819 / threads, least = !ec ? 1 : threads <= 64 ? 14 : threads <= 256 ? 3 : threads < 512 ? 20 : 5;
   return K > 152LL * (ctas > least ? ctas : least);
 }
 
@@ -2601,8 +2604,8 @@ template <int N, bool EC, bool DENSE>
 constexpr int vol_min_blocks() {
   constexpr int T = VolShape<N>::THREADS;
   constexpr int smem = (EC ? VolShape<N>::SMEM_R_EC : VolShape<N>::SMEM_R_F32) * 4;
-  if (DENSE) return resident_ctas(T, smem, EC && N == 3 ? 1024 : 1536);
-  return EC && (N == 4 || N == 5) ? resident_ctas(T, smem, 1024) : (T > 512 ? 1 : 2);
+  if (DENSE) return resident_ctas(T, smem, EC && (N == 3 || N == 5) ? 1024 : 1536);
+  return EC && N == 4 ? resident_ctas(T, smem, 1024) : (T > 512 ? 1 : 2);
 }
 
 // k_volume: the FP32-mixed form (the FP64 form: k_volume_fx, volume_fx.cuh)

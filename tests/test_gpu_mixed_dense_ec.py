@@ -1,5 +1,5 @@
 """The entropy-conserving FP32-mixed kernel on either side of the mesh size at which it
-takes the dense register budget (14 elements per SM at N = 3, 20 at N = 6, 2 at N = 7): one
+takes the dense register budget (14 elements per SM at N = 3, 3 at N = 5, 20 at N = 6, 5 at N = 7): one
 period of a flow against many, as for the other kernels, bound 2e-5."""
 import pytest
 
@@ -11,7 +11,7 @@ from gpu_helpers import torch_cuda
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N,per_sm", [(3, 14), (6, 20), (7, 2)])
+@pytest.mark.parametrize("N,per_sm", [(3, 14), (5, 3), (6, 20), (7, 5)])
 def test_both_budgets(N, per_sm):
     torch = torch_cuda()
     phys = I.phys_params(Ma=0.1, Re=1600.0)
