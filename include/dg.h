@@ -173,8 +173,8 @@ int dg_lgl_nodes(int N, double* xi, double* w);
  * sampling points) on the host, validates it, allocates the device storage
  * and uploads it.  stream: cudaStream_t (may be 0).  On success *out owns
  * everything; free it with dg_destroy.  Device storage at N = 7: about 800
- * bytes per DOF in the FP64 viscous form (state, RK register, metrics, also in
- * fixed point, the stored products Ja / J and (Ja Ja^T) / J, the lifting's float
+ * bytes per DOF in the FP64 viscous form (state, RK register, metrics, there also
+ * in fixed point, the stored products Ja / J and (Ja Ja^T) / J, the lifting's float
  * pairs, the stored primitives, scratch),
  * about 290 in the FP32-mixed form.  Errors: DG_ERR_ARG, DG_ERR_MESH,
  * DG_ERR_OOM, DG_ERR_CUDA (the message is then available through
@@ -243,6 +243,9 @@ int dg_rk_steps(dg_ctx* c, double t, double dt, int nsteps);
  * exterior state's dependence on the interior one) (else
  * DG_ERR_NOT_IMPLEMENTED); partitioned contexts run it in phases
  * (dg_vjp_phase; dg_vjp answers DG_ERR_ARG there).
+ * Densities, temperatures, sound speeds and their squares lie in FP32's normal
+ * range (1e-38 to 3e38; the operator's own recovery of the primitives and its Riemann
+ * fluxes need the same): reciprocals and roots are refined from FP32 ones.
  * The first call allocates the adjoint scratch of the context. */
 int dg_vjp(dg_ctx* c, const double* U, const double* lam, double* gU, double* gtheta);
 

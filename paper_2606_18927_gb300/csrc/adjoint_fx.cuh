@@ -309,8 +309,8 @@ __device__ __noinline__ void adj_volume_fp64(double* smem, const MeshDev<double>
 // k_adj_volume: one CTA per element; gV = the volume integral's and the body
 // force's part of gU (through the primitives).  Measured at N = 7, 10^3
 // elements: the element kernel with the pairs in FP64 1181 us (FP64 pipe 86 %
-// busy); 495 us without them and 233 us here (issue 47 %, integer pipes 36 %,
-// FP64 pipe 32 %, of which the recovery of the primitives and its transpose).
+// busy); 497 us without them and 231 us here (issue 51 %, integer pipes 39 %,
+// FP64 pipe 30 %, of which the recovery of the primitives and its transpose).
 // GEN: for meshes with stretched elements.
 template <int N, bool GEN>
 __global__ void __launch_bounds__(VolShape<N>::THREADS, (resident_ctas(VolShape<N>::THREADS, AdjFxShape<N>::SMEM, 1024)))

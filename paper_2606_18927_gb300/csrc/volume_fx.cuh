@@ -560,9 +560,9 @@ __device__ __noinline__ void volume_passes_fp64(double* smem, const MeshDev<doub
 }
 
 // k_volume of the FP64 form: one CTA per element, the passes in fixed point
-// (elements out of fx_plan's range: in FP64), the epilogue in FP64.  Measured at N = 7, 32^3 elements: KEP flux 10.08 ms with
-// FP64 pair fluxes (FP64 pipe 90 % busy), 3.07 ms in fixed point (issue 52 %,
-// integer pipes 37 %, FP64 pipe 30 %).
+// (elements out of fx_plan's range: in FP64), the epilogue in FP64.  Measured at N = 7,
+// 32^3 elements: KEP flux 10.08 ms with FP64 pair fluxes (FP64 pipe 90 % busy), 3.04 ms
+// in fixed point (16^3: issue 55 %, integer pipes 41 and 21 %, FP64 pipe 45 %).
 // GEN: for meshes with stretched elements (their passes beside the others').
 template <int N, int MODE, int VF, bool GEN>
 __global__ void __launch_bounds__(VolShape<N>::THREADS, (resident_ctas(VolShape<N>::THREADS, VolFxShape<N, VF>::SMEM, 1024)))
