@@ -222,7 +222,11 @@ int dg_time_derivative(dg_ctx* c, const double* U, double* Ut, double t, int on_
  * applies the update in registers, in place. */
 int dg_rk_stage(dg_ctx* c, int s, double t, double dt);
 
-/* nsteps full LSERK4 steps from time t. */
+/* nsteps full LSERK4 steps from time t.  (The calls below may be captured into a
+ * caller's own CUDA graph where they neither copy to the host nor synchronise.  From
+ * the first such capture on, every evaluation of the context forms its own primitives
+ * instead of taking those that an earlier call stored: replays change the state and
+ * the stored values without a call.) */
 int dg_rk_steps(dg_ctx* c, double t, double dt, int nsteps);
 
 /* Vector-Jacobian product of the operator (the hand-written adjoint):
