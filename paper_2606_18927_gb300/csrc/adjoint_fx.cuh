@@ -176,7 +176,7 @@ __device__ __forceinline__ void adj_passes_fx(const Fx* sQ, const Fx* sL, Fx* sL
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const size_t x = (size_t)(dir * 3 + c) * S + e0 + me;
-        a[c] = STORED_FX<N> ? m.JaX[x] : metric_fx(m.Ja[x], m.JaX_max[e], c);
+        a[c] = N == 7 || m.JaX ? m.JaX[x] : metric_fx(m.Ja[x], m.JaX_max[e], c);
         if (active) sA[c * n3 + ms] = a[c];
       }
     }

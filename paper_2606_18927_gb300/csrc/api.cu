@@ -58,7 +58,7 @@ struct dg_ctx {
   // (Ja Ja^T) / J [24][S] and of the lifted primitives [4][S]
   float2* lift_M2 = nullptr;
   float2* lift_W2 = nullptr;
-  dg::Fx* JaX = nullptr;    // FP64, N = 7: [9][S] metrics in fixed point (volume kernel), and
+  dg::Fx* JaX = nullptr;    // FP64: [9][S] metrics in fixed point (volume kernel; null: stored_fx), and
   dg::FxMetric* JaX_max = nullptr;  // FP64: the elements' largest magnitudes and kinds [K]
   int stretched = 0;        // some element is not FX_EVEN
   double* wm_t = nullptr;  // wall-law warm start per wall node (NaN: none yet)
@@ -687,7 +687,7 @@ int dg_init_mesh(dg_ctx** out, const dg_mesh_desc* m, const dg_phys* p, const dg
   if (e != cudaSuccess) { free_all(c); delete c; return cuda_fail(nullptr, e, "dg_init_mesh: upload"); }
   // FP64: the volume kernel's metrics in fixed point
   if (o->precision == DG_FP64) {
-    if (c->N == 7 && dg::STORED_FX<7>) chk(alloc(&c->JaX, 9 * S));
+    if (dg::stored_fx(c->N, S)) chk(alloc(&c->JaX, 9 * S));
     chk(alloc(&c->JaX_max, (size_t)c->K));
     if (e == cudaSuccess) {
       // (status is free until the first evaluation)

@@ -100,10 +100,12 @@ struct Fx {
   int h, l;
 };
 struct FxMetric;  // volume_fx.cuh
-// whether the fixed-point metrics are kept in memory (72 bytes a node) or formed from
-// Ja in the kernels that read them
-template <int N>
-constexpr bool STORED_FX = N == 7;
+// Whether the fixed-point metrics are kept in memory (72 bytes a node) or formed from
+// Ja in the kernels that read them.  N = 7 keeps them, where 252 bytes of pair sums
+// were; elsewhere meshes up to 75 MB of them, for which their forming shows (N = 3, 4^3
+// elements: the operator 34.0 us with them kept, 34.4 without; N = 4, 565k nodes a step
+// 926 and 935) and which do not fill a device.
+constexpr bool stored_fx(int N, size_t nodes) { return N == 7 || nodes <= (size_t)1 << 20; }
 
 struct PhysDev {
   double gamma, gm1, R, mu, Pr, cp, kcond, rcp_R;
@@ -172,7 +174,7 @@ struct MeshDev {
   // written by k_prim64 (null unless that lifting is selected)
   const float2* lift_M2;
   float2* lift_W2;
-  const Fx* JaX;         // FP64 form: metrics in fixed point [9][K*n3] (STORED_FX) and
+  const Fx* JaX;         // FP64 form: metrics in fixed point [9][K*n3] (null: see stored_fx) and
   const FxMetric* JaX_max;  // the elements' largest magnitudes [K] (volume_fx.cuh)
   double* wm_t;          // [n_wall*n2] last wall-law solution per wall node (warm start; may be null)
   int* status;           // device status flags (index checks of the bounds-checking build)

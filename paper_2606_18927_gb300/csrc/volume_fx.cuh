@@ -593,7 +593,7 @@ k_volume_fx(const double* __restrict__ Uin, const MeshDev<double> m, const PhysD
     const int ts = vslot<N, double>(t);
 #pragma unroll
     for (int c = 0; c < 9; ++c)
-      sA[c * n3 + ts] = STORED_FX<N> ? m.JaX[(size_t)c * S + g] : metric_fx(m.Ja[(size_t)c * S + g], m.JaX_max[e], c % 3);
+      sA[c * n3 + ts] = N == 7 || m.JaX ? m.JaX[(size_t)c * S + g] : metric_fx(m.Ja[(size_t)c * S + g], m.JaX_max[e], c % 3);
     if constexpr (EC) {
       const double ir = rcp_pos(q.rho);
       // (the quotient's remainder added back: half an ulp instead of two)
